@@ -1,0 +1,116 @@
+// Block fixed-point contractions for the FP64 kernels.
+//
+// GB300 retires two FP64 operations per clock and SM, but 64 IMAD.WIDE (32 x 32
+// + 64 bit multiply-adds), on a pipe that runs beside the FP64 pipe: one FP64
+// operation takes the time of 32 of them (measured 2.0 against 55-64 lanes per
+// clock and SM; both together take no longer than the FP64 part alone).  The
+// reference-element contractions sum_a c_a x_a, with constant c and a handful
+// of nodal values x of similar size, therefore run in integers: the x of one
+// sum share an exponent (that of the largest), each is held as two signed
+// parts h 2^28 + l (58 bits with the sign), the constants likewise, and a term
+// takes three IMAD.WIDE:
+//   a += x.h c.h ;  b += x.h c.l + x.l c.h      (x.l c.l < 2^-56 of a is left out)
+// with sum = a + b 2^-28, exact otherwise.  Rounding happens when x is aligned
+// (2^-57 of the largest x or less) and when the result returns to a double:
+// an error below 2^-56 of sum |c| max|x|, against several roundings of 2^-53
+// of the running sum in floating point.
+//
+// Ranges.  A group whose largest value is below 2^-823 is taken as zero; one
+// with a value of 2^957 or above (infinities and NaN among them) makes its
+// results NaN, so a non-finite state stays non-finite.
+#pragma once
+#include <cmath>
+#include <cstdint>
+#include <cuda_runtime.h>
+
+namespace dgswe {
+
+struct Fx {
+  int32_t h, l;  // h 2^28 + l, |h| < 2^30, |l| < 2^28
+};
+struct FxAcc {
+  long long a, b;
+};
+// How results leave: exponent step kk (in the high word), and masks that make
+// every result of the group zero (am = 0) or NaN (om).
+struct FxScale {
+  int kk, am, om;
+};
+
+constexpr int kFxLo = 28;
+constexpr int kFxMinExp = 200, kFxMaxExp = 1980;  // biased exponents of a group's largest value
+
+__device__ __forceinline__ int fx_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+
+// x in units of 2^(E - 1075 - SH), E the group's largest biased exponent:
+// |x| < 2^(53 + SH).  SH = 5 uses the format's full range; smaller SH leave
+// room for sums of x.
+template <int SH>
+__device__ __forceinline__ Fx fx_from(double v, int E) {
+  const int hi = __double2hiint(v);
+  const unsigned lo = (unsigned)__double2loint(v);
+  // mantissa at bit 62, then down to 53 + SH bits and to the group's exponent;
+  // a shift of 63 leaves nothing (zeros, tiny values, a group below kFxMinExp)
+  const int sh = min((E < kFxMinExp ? 4096 : E) - ((hi >> 20) & 0x7ff) + (10 - SH), 63);
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const unsigned long long m = (((unsigned long long)__funnelshift_l(lo, mh, 10) << 32) | (lo << 10)) >> sh;
+  const int s = hi >> 31;
+  Fx r;
+  r.h = ((int)(m >> kFxLo) ^ s) - s;
+  r.l = ((int)((unsigned)m & ((1u << kFxLo) - 1)) ^ s) - s;
+  return r;
+}
+
+__device__ __forceinline__ long long fx_wide(int a, int b) { return (long long)a * (long long)b; }
+
+__device__ __forceinline__ void fx_mac(FxAcc& s, Fx x, Fx c) {
+  s.a += fx_wide(x.h, c.h);
+  s.b += fx_wide(x.h, c.l);
+  s.b += fx_wide(x.l, c.h);
+}
+// The sum in units of (unit of x)(unit of c) 2^56.
+__device__ __forceinline__ long long fx_sum(const FxAcc& s) { return s.a + (s.b >> kFxLo); }
+// A sum |r| < 2^62 as an operand again, in units of r's 2^4.
+__device__ __forceinline__ Fx fx_operand(long long r) {
+  Fx x;
+  x.h = (int)(r >> 32);
+  x.l = (int)(((unsigned)r >> 4) & ((1u << kFxLo) - 1));
+  return x;
+}
+
+// Scale of results r 2^k (k in binary orders) whose groups' largest exponents
+// were lo..hi (several groups for a product of groups).
+__device__ __forceinline__ FxScale fx_scale(int k, bool finite) {
+  FxScale s;
+  s.kk = (int)((unsigned)k << 20);
+  s.am = k < -1022 ? 0 : -1;
+  s.om = (!finite || k > 960) ? 0x7ff80000 : 0;
+  return s;
+}
+__device__ __forceinline__ double fx_to(long long r, const FxScale& s) {
+  const double d = (double)r;
+  const int hi = ((r != 0 ? __double2hiint(d) + s.kk : 0) & s.am) | s.om;
+  return __hiloint2double(hi, __double2loint(d) & s.am);
+}
+
+// ------------------------------------------------------------------ host: constant tables
+
+// A constant in units of 2^-cs.
+inline Fx fx_const(double c, int cs) {
+  const long long m = std::llround(std::ldexp(c, cs));
+  Fx r;
+  r.h = (int32_t)(m >> kFxLo);
+  r.l = (int32_t)(m - ((long long)r.h << kFxLo));
+  return r;
+}
+// Largest cs at which the constants fit the format (|c| 2^cs < 2^58) and a row
+// of absolute sum `row` keeps |sum| below 2^62 for operands below 2^xbits.
+inline int fx_table_scale(double cmax, double row, int xbits) {
+  int e1 = 0, e2 = 0;
+  std::frexp(cmax, &e1);
+  std::frexp(row, &e2);
+  const int a = 58 - e1, b = 62 + 56 - xbits - e2;
+  return a < b ? a : b;
+}
+
+}  // namespace dgswe

@@ -22,9 +22,12 @@
 // loops unrolled every thread of a warp reads the same entry, a broadcast
 // from the constant bank.
 #pragma once
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "dg_fixed.cuh"
 #include "dg_host.h"
 
 namespace dgswe {
@@ -70,6 +73,18 @@ struct EstepOps {
   R Dr[S::NP * S::NP];
   R Ds[S::NP * S::NP];
   R LIFT[S::NP * S::NF * S::NFP];
+  int8_t fmask[S::NF * S::NFP];
+};
+
+// FP64: the tables as block fixed-point constants in units of 2^-cs, LIFT with
+// the factor 1/2 of the trace jump folded in.
+template <int DIM, int P>
+struct EstepOps<DIM, P, double> {
+  using S = Sh<DIM, P>;
+  Fx Dr[S::NP * S::NP];
+  Fx Ds[S::NP * S::NP];
+  Fx LIFT[S::NP * S::NF * S::NFP];
+  int cs;
   int8_t fmask[S::NF * S::NFP];
 };
 
@@ -312,6 +327,139 @@ __device__ __forceinline__ void q_normal(R h, const R* E, const R* n, const Phys
 
 // ------------------------------------------------------------------ kernels
 
+// E-step of element e, FP64: every contraction in block fixed point (dg_fixed.cuh).
+// Per velocity component j the nodal values and the neighbours' traces share an
+// exponent; the reference derivatives and the lifted jumps w_f(a) =
+// sum_k LIFT_a,fk [u_j]_k / 2 stay integers and are combined with the element's
+// metric terms and sc n_i (one more exponent) before they return to doubles:
+// 4 NP conversions and 9 products are the FP64 pipe's share (2D), of 417
+// FP64 instructions in floating point at p = 2.  524,288 triangles, p = 2:
+// 411 -> 180 us; p = 1: 167 -> 67 us; 8,192 triangles, p = 2: 20.6 -> 12.5 us.
+template <int DIM, int P, bool COH, bool PRE>
+__device__ __forceinline__ void estep_element_fx(int e, int K, const double* __restrict__ V, double* __restrict__ E,
+                                                 const double* __restrict__ geo, const int32_t* __restrict__ nbr,
+                                                 const int8_t* __restrict__ nbrf, const double* __restrict__ fn,
+                                                 const double* __restrict__ fsj,
+                                                 const EstepOps<DIM, P, double>& ops,
+                                                 const BCEntry<double>* __restrict__ bct, const int* pnb,
+                                                 const int* pnbf) {
+  using S = Sh<DIM, P>;
+  constexpr int NP = S::NP, NF = S::NF, NFP = S::NFP;
+  const size_t KN = (size_t)K * NP;
+  double u[DIM][NP], ub[DIM][NF][NFP];
+#pragma unroll
+  for (int j = 0; j < DIM; ++j)
+#pragma unroll
+    for (int a = 0; a < NP; ++a) u[j][a] = DG_LDC(COH, V, (1 + j) * KN + (size_t)e * NP + a);
+  double G[DIM][DIM], sn[NF][DIM];
+  const double Jinv = geo[6 * K + e];
+#pragma unroll
+  for (int r = 0; r < DIM; ++r)
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) G[r][i] = geo[(2 * r + i) * K + e];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    const int e2 = PRE ? pnb[f] : nbr[f * K + e];
+    double n[DIM];
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) n[i] = fn[(f * DIM + i) * K + e];
+    const double sc = fsj[f * K + e] * Jinv;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) sn[f][i] = sc * n[i];
+    if (e2 >= 0) {
+      const int f2 = PRE ? pnbf[f] : nbrf[f * K + e];
+#pragma unroll
+      for (int k = 0; k < NFP; ++k) {
+        const int b = ops.fmask[f2 * NFP + (NFP - 1 - k)];
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) ub[j][f][k] = DG_LDC(COH, V, (1 + j) * KN + (size_t)e2 * NP + b);
+      }
+    } else {
+      const BCEntry<double> bc = bct[-1 - e2];
+#pragma unroll
+      for (int k = 0; k < NFP; ++k) {
+        double Vm[DIM + 1], Vp[DIM + 1];
+        Vm[0] = 1.0;
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) Vm[1 + j] = u[j][face_node(DIM, P, f, k)];
+        ghost_V<DIM, double>(Vm, n, bc, Vp);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) ub[j][f][k] = Vp[1 + j];
+      }
+    }
+  }
+  int eg = 0;
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
+#pragma unroll
+    for (int r = 0; r < DIM; ++r) eg = max(eg, fx_exp(G[r][i]));
+#pragma unroll
+    for (int f = 0; f < NF; ++f) eg = max(eg, fx_exp(sn[f][i]));
+  }
+  Fx Gx[DIM][DIM], snx[NF][DIM];
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) {
+#pragma unroll
+    for (int r = 0; r < DIM; ++r) Gx[r][i] = fx_from<5>(G[r][i], eg);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) snx[f][i] = fx_from<5>(sn[f][i], eg);
+  }
+#pragma unroll
+  for (int j = 0; j < DIM; ++j) {
+    int eu = 0;
+#pragma unroll
+    for (int a = 0; a < NP; ++a) eu = max(eu, fx_exp(u[j][a]));
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+      for (int k = 0; k < NFP; ++k) eu = max(eu, fx_exp(ub[j][f][k]));
+    Fx ux[NP], gx[NF][NFP];  // |ux| < 2^57, jumps < 2^58
+#pragma unroll
+    for (int a = 0; a < NP; ++a) ux[a] = fx_from<4>(u[j][a], eu);
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+      for (int k = 0; k < NFP; ++k) {
+        const Fx o = ux[face_node(DIM, P, f, k)], b = fx_from<4>(ub[j][f][k], eu);
+        gx[f][k].h = b.h - o.h;
+        gx[f][k].l = b.l - o.l;
+      }
+    // results in units of 2^(eu - 1079) 2^-cs 2^56 2^4 2^(eg - 1080) 2^56
+    const FxScale s = fx_scale(eu + eg - 2043 - ops.cs, eu <= kFxMaxExp && eg <= kFxMaxExp);
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      FxAcc dr{0, 0}, ds{0, 0}, out[DIM];
+#pragma unroll
+      for (int b = 0; b < NP; ++b) {
+        fx_mac(dr, ux[b], ops.Dr[a * NP + b]);
+        if constexpr (DIM == 2) fx_mac(ds, ux[b], ops.Ds[a * NP + b]);
+      }
+      const Fx drx = fx_operand(fx_sum(dr));
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) {
+        out[i] = FxAcc{0, 0};
+        fx_mac(out[i], drx, Gx[0][i]);
+      }
+      if constexpr (DIM == 2) {
+        const Fx dsx = fx_operand(fx_sum(ds));
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) fx_mac(out[i], dsx, Gx[DIM - 1][i]);
+      }
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        FxAcc w{0, 0};
+#pragma unroll
+        for (int k = 0; k < NFP; ++k) fx_mac(w, gx[f][k], ops.LIFT[a * (NF * NFP) + f * NFP + k]);
+        const Fx wx = fx_operand(fx_sum(w));
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) fx_mac(out[i], wx, snx[f][i]);
+      }
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) E[(DIM * i + j) * KN + (size_t)e * NP + a] = fx_to(fx_sum(out[i]), s);
+    }
+  }
+}
+
 // E-step of element e (the body of estep_kernel).  PRE: the element's face
 // neighbours and their local faces arrive preloaded in pnb / pnbf (one per
 // face) instead of being read from nbr / nbrf.
@@ -324,94 +472,73 @@ __device__ __forceinline__ void estep_element(int e, int K, const R* __restrict_
                                               const int* pnbf = nullptr) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NF = S::NF, NFP = S::NFP, NE = S::NE;
-  const size_t KN = (size_t)K * NP;
-  R u[DIM][NP];
+  if constexpr (sizeof(R) == 8) {
+    estep_element_fx<DIM, P, COH, PRE>(e, K, V, E, geo, nbr, nbrf, fn, fsj, ops, bct, pnb, pnbf);
+  } else {
+    const size_t KN = (size_t)K * NP;
+    R u[DIM][NP];
 #pragma unroll
-  for (int j = 0; j < DIM; ++j)
+    for (int j = 0; j < DIM; ++j)
 #pragma unroll
-    for (int a = 0; a < NP; ++a) u[j][a] = DG_LDC(COH, V, (1 + j) * KN + (size_t)e * NP + a);
-  R G[2][2];
-  G[0][0] = geo[e];
-  if constexpr (DIM == 2) {
-    G[0][1] = geo[K + e];
-    G[1][0] = geo[2 * K + e];
-    G[1][1] = geo[3 * K + e];
-  }
-  const R Jinv = geo[6 * K + e];
-  R Eo[NE][NP];
-#pragma unroll
-  for (int a = 0; a < NP; ++a) {
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) {
-      R dr = R(0), ds = R(0);
-#pragma unroll
-      for (int b = 0; b < NP; ++b) {
-        dr += ops.Dr[a * NP + b] * u[j][b];
-        if constexpr (DIM == 2) ds += ops.Ds[a * NP + b] * u[j][b];
-      }
-#pragma unroll
-      for (int i = 0; i < DIM; ++i) {
-        R v = G[0][i] * dr;
-        if constexpr (DIM == 2) v += G[1][i] * ds;
-        Eo[DIM * i + j][a] = v;
-      }
+      for (int a = 0; a < NP; ++a) u[j][a] = DG_LDC(COH, V, (1 + j) * KN + (size_t)e * NP + a);
+    R G[2][2];
+    G[0][0] = geo[e];
+    if constexpr (DIM == 2) {
+      G[0][1] = geo[K + e];
+      G[1][0] = geo[2 * K + e];
+      G[1][1] = geo[3 * K + e];
     }
-  }
+    const R Jinv = geo[6 * K + e];
+    R Eo[NE][NP];
 #pragma unroll
-  for (int f = 0; f < NF; ++f) {
-    const int e2 = PRE ? pnb[f] : nbr[f * K + e];
-    R n[DIM];
+    for (int a = 0; a < NP; ++a) {
 #pragma unroll
-    for (int i = 0; i < DIM; ++i) n[i] = fn[(f * DIM + i) * K + e];
-    const R sc = fsj[f * K + e] * Jinv;
-    R gj[NFP][DIM];
-    if (e2 >= 0) {
-      const int f2 = PRE ? pnbf[f] : nbrf[f * K + e];
+      for (int j = 0; j < DIM; ++j) {
+        R dr = R(0), ds = R(0);
 #pragma unroll
-      for (int k = 0; k < NFP; ++k) {
-        const int a = face_node(DIM, P, f, k);
-        const int b = ops.fmask[f2 * NFP + (NFP - 1 - k)];
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) gj[k][j] = R(0.5) * (DG_LDC(COH, V, (1 + j) * KN + (size_t)e2 * NP + b) - u[j][a]);
-      }
-    } else {
-      const BCEntry<R> bc = bct[-1 - e2];
-#pragma unroll
-      for (int k = 0; k < NFP; ++k) {
-        const int a = face_node(DIM, P, f, k);
-        R Vm[DIM + 1], Vp[DIM + 1];
-        Vm[0] = R(1);
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) Vm[1 + j] = u[j][a];
-        ghost_V<DIM, R>(Vm, n, bc, Vp);
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) gj[k][j] = R(0.5) * (Vp[1 + j] - Vm[1 + j]);
-      }
-    }
-    if constexpr (sizeof(R) == 8) {
-      // FP64 (bound by the FP64 pipe): lift each velocity jump once,
-      // w_j(a) = sum_k LIFT_a,fk [u_j]_k / 2, then scale by sc n_i: NP DIM
-      // (NFP + DIM) multiply-adds per face instead of NP NFP DIM DIM
-      R sn[DIM];
-#pragma unroll
-      for (int i = 0; i < DIM; ++i) sn[i] = sc * n[i];
-#pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        R w[DIM];
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) w[j] = R(0);
-#pragma unroll
-        for (int k = 0; k < NFP; ++k) {
-          const R L = ops.LIFT[a * (NF * NFP) + f * NFP + k];
-#pragma unroll
-          for (int j = 0; j < DIM; ++j) w[j] += L * gj[k][j];
+        for (int b = 0; b < NP; ++b) {
+          dr += ops.Dr[a * NP + b] * u[j][b];
+          if constexpr (DIM == 2) ds += ops.Ds[a * NP + b] * u[j][b];
         }
 #pragma unroll
-        for (int i = 0; i < DIM; ++i)
-#pragma unroll
-          for (int j = 0; j < DIM; ++j) Eo[DIM * i + j][a] += sn[i] * w[j];
+        for (int i = 0; i < DIM; ++i) {
+          R v = G[0][i] * dr;
+          if constexpr (DIM == 2) v += G[1][i] * ds;
+          Eo[DIM * i + j][a] = v;
+        }
       }
-    } else {
+    }
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const int e2 = PRE ? pnb[f] : nbr[f * K + e];
+      R n[DIM];
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) n[i] = fn[(f * DIM + i) * K + e];
+      const R sc = fsj[f * K + e] * Jinv;
+      R gj[NFP][DIM];
+      if (e2 >= 0) {
+        const int f2 = PRE ? pnbf[f] : nbrf[f * K + e];
+#pragma unroll
+        for (int k = 0; k < NFP; ++k) {
+          const int a = face_node(DIM, P, f, k);
+          const int b = ops.fmask[f2 * NFP + (NFP - 1 - k)];
+#pragma unroll
+          for (int j = 0; j < DIM; ++j) gj[k][j] = R(0.5) * (DG_LDC(COH, V, (1 + j) * KN + (size_t)e2 * NP + b) - u[j][a]);
+        }
+      } else {
+        const BCEntry<R> bc = bct[-1 - e2];
+#pragma unroll
+        for (int k = 0; k < NFP; ++k) {
+          const int a = face_node(DIM, P, f, k);
+          R Vm[DIM + 1], Vp[DIM + 1];
+          Vm[0] = R(1);
+#pragma unroll
+          for (int j = 0; j < DIM; ++j) Vm[1 + j] = u[j][a];
+          ghost_V<DIM, R>(Vm, n, bc, Vp);
+#pragma unroll
+          for (int j = 0; j < DIM; ++j) gj[k][j] = R(0.5) * (Vp[1 + j] - Vm[1 + j]);
+        }
+      }
       // FP32: the face's jump terms sc n_i [u_j]/2, scaled once per face node
       R gt[NFP][DIM][DIM];
 #pragma unroll
@@ -434,11 +561,11 @@ __device__ __forceinline__ void estep_element(int e, int K, const R* __restrict_
         }
       }
     }
+#pragma unroll
+    for (int c = 0; c < NE; ++c)
+#pragma unroll
+      for (int a = 0; a < NP; ++a) E[c * KN + (size_t)e * NP + a] = Eo[c][a];
   }
-#pragma unroll
-  for (int c = 0; c < NE; ++c)
-#pragma unroll
-    for (int a = 0; a < NP; ++a) E[c * KN + (size_t)e * NP + a] = Eo[c][a];
 }
 
 template <int DIM, int P, typename R>
@@ -2051,12 +2178,41 @@ template <int DIM, int P, typename R>
 void fill_ops(const RefOps& o, EstepOps<DIM, P, R>& eo, FaceOps<DIM, P, R>& fo, VolOps<DIM, P, R>& vo) {
   using S = Sh<DIM, P>;
   const int NP = S::NP, NQ = S::NQ;
-  for (int i = 0; i < NP * NP; ++i) {
-    eo.Dr[i] = (R)o.Dr[i];
-    eo.Ds[i] = (R)o.Ds[i];
-    vo.Minv[i] = (R)o.Minv[i];
+  for (int i = 0; i < NP * NP; ++i) vo.Minv[i] = (R)o.Minv[i];
+  if constexpr (sizeof(R) == 8) {
+    // one scale for the three tables: derivative rows act on operands below
+    // 2^57, lift rows (1/2 LIFT, per face) on jumps below 2^58
+    eo.cs = 60;
+    for (int a = 0; a < NP; ++a) {
+      double m = 0.0, r1 = 0.0, r2 = 0.0, lm = 0.0;
+      for (int b = 0; b < NP; ++b) {
+        m = std::max({m, std::fabs(o.Dr[a * NP + b]), std::fabs(o.Ds[a * NP + b])});
+        r1 += std::fabs(o.Dr[a * NP + b]);
+        r2 += std::fabs(o.Ds[a * NP + b]);
+      }
+      eo.cs = std::min(eo.cs, fx_table_scale(m, std::max(r1, r2), 57));
+      for (int f = 0; f < S::NF; ++f) {
+        double r = 0.0;
+        for (int k = 0; k < S::NFP; ++k) {
+          const double c = 0.5 * std::fabs(o.LIFT[a * (S::NF * S::NFP) + f * S::NFP + k]);
+          r += c;
+          lm = std::max(lm, c);
+        }
+        eo.cs = std::min(eo.cs, fx_table_scale(lm, r, 58));
+      }
+    }
+    for (int i = 0; i < NP * NP; ++i) {
+      eo.Dr[i] = fx_const(o.Dr[i], eo.cs);
+      eo.Ds[i] = fx_const(o.Ds[i], eo.cs);
+    }
+    for (int i = 0; i < NP * S::NF * S::NFP; ++i) eo.LIFT[i] = fx_const(0.5 * o.LIFT[i], eo.cs);
+  } else {
+    for (int i = 0; i < NP * NP; ++i) {
+      eo.Dr[i] = (R)o.Dr[i];
+      eo.Ds[i] = (R)o.Ds[i];
+    }
+    for (int i = 0; i < NP * S::NF * S::NFP; ++i) eo.LIFT[i] = (R)o.LIFT[i];
   }
-  for (int i = 0; i < NP * S::NF * S::NFP; ++i) eo.LIFT[i] = (R)o.LIFT[i];
   for (int i = 0; i < S::NF * S::NFP; ++i) {
     eo.fmask[i] = (int8_t)o.fmask[i];
     fo.fmask[i] = (int8_t)o.fmask[i];
