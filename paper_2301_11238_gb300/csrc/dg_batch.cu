@@ -166,6 +166,7 @@ struct GDrv final : GroupDrv {
   EstepOps<DIM, P, R> eo{};
   FaceOps<DIM, P, R> fo{};
   VolOps<DIM, P, R> vo{};
+  VolArg<DIM, P, R> va{};  // operator tables of the volume pass
   bool tc = false;
   std::unique_ptr<tc::Launcher<(P >= 2 ? P : 2), true>> tcl;
   int n_sm = 0;
@@ -176,6 +177,8 @@ struct GDrv final : GroupDrv {
   void persistent_step(dg_batch* b, Group& g, cudaStream_t s) override;
   explicit GDrv(const RefOps& o, bool use_tc) {
     fill_ops<DIM, P, R>(o, eo, fo, vo);
+    if constexpr (sizeof(R) == 8) fill_vol_fx<DIM, P>(o, va);
+    else va = vo;
     if constexpr (kTcForm) {
       tc = use_tc;
       if (tc) tcl.reset(new tc::Launcher<P, true>());
@@ -307,7 +310,7 @@ struct GDrv final : GroupDrv {
           K, F, b->at<R>(g.off.V[vin]), b->at<R>(g.off.V[0]), b->at<R>(g.off.V[vout]), b->at<R>(g.off.E),
           g.has_bed ? b->at<R>(g.off.bed) : nullptr, g.has_bed ? b->at<R>(g.off.src) : nullptr,
           b->at<R>(g.off.geo), b->at<int32_t>(g.off.fid),
-          b->at<R>(g.off.wflux), vo, ptab(b), b->at<int32_t>(g.off.inst), (R)c0, (R)c1,
+          b->at<R>(g.off.wflux), va, ptab(b), b->at<int32_t>(g.off.inst), (R)c0, (R)c1,
           b->at<DevScalars>(b->off_sc));
       return;
     }
@@ -316,7 +319,7 @@ struct GDrv final : GroupDrv {
         K, F, b->at<R>(g.off.V[vin]), b->at<R>(g.off.V[0]), b->at<R>(g.off.V[vout]), b->at<R>(g.off.E),
         g.has_bed ? b->at<R>(g.off.bed) : nullptr, g.has_bed ? b->at<R>(g.off.src) : nullptr,
           b->at<R>(g.off.geo), b->at<int32_t>(g.off.fid),
-        b->at<R>(g.off.wflux), vo, Phys<R>{}, ptab(b), b->at<int32_t>(g.off.inst), 1, (R)c0, (R)c1,
+        b->at<R>(g.off.wflux), va, Phys<R>{}, ptab(b), b->at<int32_t>(g.off.inst), 1, (R)c0, (R)c1,
         b->at<DevScalars>(b->off_sc));
   }
   // the volume pass in mode 2 (r_V of V[vin] into V[vout]): the tensor-core
@@ -337,7 +340,7 @@ struct GDrv final : GroupDrv {
     volume_kernel<DIM, P, R, true><<<(K + T - 1) / T, T, 0, s>>>(
         K, F, b->at<R>(g.off.V[vin]), nullptr, b->at<R>(g.off.V[vout]), b->at<R>(g.off.E),
         g.has_bed ? b->at<R>(g.off.bed) : nullptr, g.has_bed ? b->at<R>(g.off.src) : nullptr, b->at<R>(g.off.geo),
-        b->at<int32_t>(g.off.fid), b->at<R>(g.off.wflux), vo, Phys<R>{}, ptab(b), b->at<int32_t>(g.off.inst), 2, R(0),
+        b->at<int32_t>(g.off.fid), b->at<R>(g.off.wflux), va, Phys<R>{}, ptab(b), b->at<int32_t>(g.off.inst), 2, R(0),
         R(0), b->at<DevScalars>(b->off_sc));
   }
   void dt(dg_batch* b, Group& g, cudaStream_t s) override {
@@ -414,7 +417,7 @@ void GDrv<DIM, P, R>::persistent_step(dg_batch* b, Group& g, cudaStream_t s) {
   const int total = g.p_pstart[persist::kPhases];
   const int grid = std::max(1, std::min(total, persist_grid));
   cudaMemsetAsync(pl.done, 0, (size_t)(nm * persist::kPhases + 1) * sizeof(int), s);
-  persist::step_kernel<DIM, P, R><<<grid, persist::kThreads, 0, s>>>(pl, A, eo, fo, vo);
+  persist::step_kernel<DIM, P, R><<<grid, persist::kThreads, 0, s>>>(pl, A, eo, fo, va);
 }
 
 template <typename R>

@@ -70,13 +70,25 @@ __device__ __forceinline__ void fx_mac(FxAcc& s, Fx x, Fx c) {
 }
 // The sum in units of (unit of x)(unit of c) 2^56.
 __device__ __forceinline__ long long fx_sum(const FxAcc& s) { return s.a + (s.b >> kFxLo); }
-// A sum |r| < 2^62 as an operand again, in units of r's 2^4.
+// Moves what b has above one unit of a into a: sums of more than 15 terms do
+// this every 15, so that b (two products below 2^58 a term) stays below 2^63.
+__device__ __forceinline__ void fx_fold(FxAcc& s) {
+  s.a += s.b >> kFxLo;
+  s.b &= (1ll << kFxLo) - 1;
+}
+// A sum |r| < 2^RB as an operand |x| < 2^58 again, in units of r's 2^(RB - 58), rounded.
+template <int RB>
 __device__ __forceinline__ Fx fx_operand(long long r) {
+  const long long t = r + (1ll << (RB - 59));
   Fx x;
-  x.h = (int)(r >> 32);
-  x.l = (int)(((unsigned)r >> 4) & ((1u << kFxLo) - 1));
+  x.h = (int)(t >> (RB - 30));
+  x.l = (int)((unsigned)(t >> (RB - 58)) & ((1u << kFxLo) - 1));
   return x;
 }
+// Left shift that brings the sums whose magnitudes were or-ed into m (fx_mag)
+// up to 2^61 .. 2^62.
+__device__ __forceinline__ unsigned long long fx_mag(long long r) { return (unsigned long long)(r ^ (r >> 63)); }
+__device__ __forceinline__ int fx_norm(unsigned long long m) { return max(__clzll((long long)(m | 1)) - 2, 0); }
 
 // Scale of results r 2^k (k in binary orders) whose groups' largest exponents
 // were lo..hi (several groups for a product of groups).
@@ -103,8 +115,8 @@ inline Fx fx_const(double c, int cs) {
   r.l = (int32_t)(m - ((long long)r.h << kFxLo));
   return r;
 }
-// Largest cs at which the constants fit the format (|c| 2^cs < 2^58) and a row
-// of absolute sum `row` keeps |sum| below 2^62 for operands below 2^xbits.
+// Largest cs at which the constants are below 2^58 units and a row of absolute
+// sum `row` keeps |sum| below 2^62 for operands below 2^xbits.
 inline int fx_table_scale(double cmax, double row, int xbits) {
   int e1 = 0, e2 = 0;
   std::frexp(cmax, &e1);

@@ -203,32 +203,48 @@ __device__ __forceinline__ R viscous_eta(R s, const Phys<R>& ph) {
   return ph.hb ? ph.eta * pow(fmax(s, ph.hb_floor), ph.hb_n - R(1)) : ph.eta;
 }
 
+// x < y for x >= 0, y > 0 (a NaN x is not less).  FP64: as integers, which
+// order such values alike and leave the FP64 pipe alone.
+template <typename R>
+__device__ __forceinline__ bool less_pos(R x, R y) { return x < y; }
+template <>
+__device__ __forceinline__ bool less_pos<double>(double x, double y) {
+  return __double_as_longlong(x) < __double_as_longlong(y);
+}
+
+// Stress coefficient mu: sigma = mu 2 E in 1D, mu (D + tr D I) in 2D with
+// s2 = ||D||_c^2 / 2.
+template <typename R>
+__device__ __forceinline__ R stress_mu1(R e, const Phys<R>& ph) {
+  return R(2) * viscous_eta<R>(fabs(e), ph) + bingham_coef<R>(fabs(e), ph);
+}
+template <typename R>
+__device__ __forceinline__ R stress_mu2(R s2, const Phys<R>& ph) {
+  if (ph.reg == 5 && !ph.hb) {
+    // bi-viscosity with the Newtonian viscous part: gamma below the yield
+    // rate (gamma s < sigma0, tested on s^2) and sigma0 / s above it, so
+    // the reciprocal square root is taken only where the material yields
+    const R g = ph.gamma, s0 = ph.sigma0;
+    const R coef = s0 == R(0) ? R(0) : (less_pos<R>(g * g * s2, s0 * s0) ? g : s0 * dg_rsqrt<R>(s2));
+    return R(2) * ph.eta + coef;
+  }
+  // s = sqrt(nc2 / 2) and 1 / s from one reciprocal square root
+  const R s_inv = s2 > R(0) ? dg_rsqrt<R>(s2) : R(0);
+  const R s = s2 * s_inv;
+  return R(2) * viscous_eta<R>(s, ph) + bingham_coef<R>(s, s_inv, ph);
+}
+
 // sigma from E (component 2i+j = du_j/dx_i); returns sig[i][j].
 template <int DIM, typename R>
 __device__ __forceinline__ void stress(const R* E, const Phys<R>& ph, R sig[DIM][DIM]) {
   if constexpr (DIM == 1) {
     R e = E[0];
-    R mu = R(2) * viscous_eta<R>(fabs(e), ph) + bingham_coef<R>(fabs(e), ph);
-    sig[0][0] = mu * R(2) * e;
+    sig[0][0] = stress_mu1<R>(e, ph) * R(2) * e;
   } else {
     R d11 = E[0], d22 = E[3], d12 = R(0.5) * (E[1] + E[2]);
     R tr = d11 + d22;
     R nc2 = d11 * d11 + R(2) * d12 * d12 + d22 * d22 + tr * tr;
-    const R s2 = R(0.5) * nc2;
-    R mu;
-    if (ph.reg == 5 && !ph.hb) {
-      // bi-viscosity with the Newtonian viscous part: gamma below the yield
-      // rate (gamma s < sigma0, tested on s^2) and sigma0 / s above it, so
-      // the reciprocal square root is taken only where the material yields
-      const R g = ph.gamma, s0 = ph.sigma0;
-      const R coef = s0 == R(0) ? R(0) : (g * g * s2 < s0 * s0 ? g : s0 * dg_rsqrt<R>(s2));
-      mu = R(2) * ph.eta + coef;
-    } else {
-      // s = sqrt(nc2 / 2) and 1 / s from one reciprocal square root
-      const R s_inv = s2 > R(0) ? dg_rsqrt<R>(s2) : R(0);
-      const R s = s2 * s_inv;
-      mu = R(2) * viscous_eta<R>(s, ph) + bingham_coef<R>(s, s_inv, ph);
-    }
+    const R mu = stress_mu2<R>(R(0.5) * nc2, ph);
     sig[0][0] = mu * (d11 + tr);
     sig[1][1] = mu * (d22 + tr);
     sig[0][1] = mu * d12;
@@ -346,12 +362,8 @@ __device__ __forceinline__ void estep_element_fx(int e, int K, const double* __r
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NF = S::NF, NFP = S::NFP;
   const size_t KN = (size_t)K * NP;
-  double u[DIM][NP], ub[DIM][NF][NFP];
-#pragma unroll
-  for (int j = 0; j < DIM; ++j)
-#pragma unroll
-    for (int a = 0; a < NP; ++a) u[j][a] = DG_LDC(COH, V, (1 + j) * KN + (size_t)e * NP + a);
   double G[DIM][DIM], sn[NF][DIM];
+  int nb[NF], nf[NF];
   const double Jinv = geo[6 * K + e];
 #pragma unroll
   for (int r = 0; r < DIM; ++r)
@@ -359,34 +371,11 @@ __device__ __forceinline__ void estep_element_fx(int e, int K, const double* __r
     for (int i = 0; i < DIM; ++i) G[r][i] = geo[(2 * r + i) * K + e];
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
-    const int e2 = PRE ? pnb[f] : nbr[f * K + e];
-    double n[DIM];
-#pragma unroll
-    for (int i = 0; i < DIM; ++i) n[i] = fn[(f * DIM + i) * K + e];
+    nb[f] = PRE ? pnb[f] : nbr[f * K + e];
+    nf[f] = PRE ? pnbf[f] : (int)nbrf[f * K + e];
     const double sc = fsj[f * K + e] * Jinv;
 #pragma unroll
-    for (int i = 0; i < DIM; ++i) sn[f][i] = sc * n[i];
-    if (e2 >= 0) {
-      const int f2 = PRE ? pnbf[f] : nbrf[f * K + e];
-#pragma unroll
-      for (int k = 0; k < NFP; ++k) {
-        const int b = ops.fmask[f2 * NFP + (NFP - 1 - k)];
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) ub[j][f][k] = DG_LDC(COH, V, (1 + j) * KN + (size_t)e2 * NP + b);
-      }
-    } else {
-      const BCEntry<double> bc = bct[-1 - e2];
-#pragma unroll
-      for (int k = 0; k < NFP; ++k) {
-        double Vm[DIM + 1], Vp[DIM + 1];
-        Vm[0] = 1.0;
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) Vm[1 + j] = u[j][face_node(DIM, P, f, k)];
-        ghost_V<DIM, double>(Vm, n, bc, Vp);
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) ub[j][f][k] = Vp[1 + j];
-      }
-    }
+    for (int i = 0; i < DIM; ++i) sn[f][i] = sc * fn[(f * DIM + i) * K + e];
   }
   int eg = 0;
 #pragma unroll
@@ -404,29 +393,57 @@ __device__ __forceinline__ void estep_element_fx(int e, int K, const double* __r
 #pragma unroll
     for (int f = 0; f < NF; ++f) snx[f][i] = fx_from<5>(sn[f][i], eg);
   }
-#pragma unroll
+  // one component at a time: both at once take 192 registers (p = 2) and half the warps
+#pragma unroll 1
   for (int j = 0; j < DIM; ++j) {
+    double u[NP], ub[NF][NFP];
     int eu = 0;
 #pragma unroll
-    for (int a = 0; a < NP; ++a) eu = max(eu, fx_exp(u[j][a]));
+    for (int a = 0; a < NP; ++a) u[a] = DG_LDC(COH, V, (1 + j) * KN + (size_t)e * NP + a);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      if (nb[f] >= 0) {
+#pragma unroll
+        for (int k = 0; k < NFP; ++k)
+          ub[f][k] = DG_LDC(COH, V, (1 + j) * KN + (size_t)nb[f] * NP + ops.fmask[nf[f] * NFP + (NFP - 1 - k)]);
+      } else {
+        const BCEntry<double> bc = bct[-1 - nb[f]];
+        double n[DIM];
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) n[i] = fn[(f * DIM + i) * K + e];
+#pragma unroll
+        for (int k = 0; k < NFP; ++k) {
+          double Vm[DIM + 1], Vp[DIM + 1];
+          Vm[0] = 1.0;
+#pragma unroll
+          for (int i = 0; i < DIM; ++i)
+            Vm[1 + i] = DG_LDC(COH, V, (1 + i) * KN + (size_t)e * NP + face_node(DIM, P, f, k));
+          ghost_V<DIM, double>(Vm, n, bc, Vp);
+          ub[f][k] = Vp[1];
+          if constexpr (DIM == 2) ub[f][k] = j == 0 ? Vp[1] : Vp[DIM];
+        }
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < NP; ++a) eu = max(eu, fx_exp(u[a]));
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
-      for (int k = 0; k < NFP; ++k) eu = max(eu, fx_exp(ub[j][f][k]));
+      for (int k = 0; k < NFP; ++k) eu = max(eu, fx_exp(ub[f][k]));
     Fx ux[NP], gx[NF][NFP];  // |ux| < 2^57, jumps < 2^58
 #pragma unroll
-    for (int a = 0; a < NP; ++a) ux[a] = fx_from<4>(u[j][a], eu);
+    for (int a = 0; a < NP; ++a) ux[a] = fx_from<4>(u[a], eu);
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
       for (int k = 0; k < NFP; ++k) {
-        const Fx o = ux[face_node(DIM, P, f, k)], b = fx_from<4>(ub[j][f][k], eu);
+        const Fx o = ux[face_node(DIM, P, f, k)], b = fx_from<4>(ub[f][k], eu);
         gx[f][k].h = b.h - o.h;
         gx[f][k].l = b.l - o.l;
       }
     // results in units of 2^(eu - 1079) 2^-cs 2^56 2^4 2^(eg - 1080) 2^56
     const FxScale s = fx_scale(eu + eg - 2043 - ops.cs, eu <= kFxMaxExp && eg <= kFxMaxExp);
-#pragma unroll
+#pragma unroll (P == 3 ? 1 : 2)
     for (int a = 0; a < NP; ++a) {
       FxAcc dr{0, 0}, ds{0, 0}, out[DIM];
 #pragma unroll
@@ -434,14 +451,14 @@ __device__ __forceinline__ void estep_element_fx(int e, int K, const double* __r
         fx_mac(dr, ux[b], ops.Dr[a * NP + b]);
         if constexpr (DIM == 2) fx_mac(ds, ux[b], ops.Ds[a * NP + b]);
       }
-      const Fx drx = fx_operand(fx_sum(dr));
+      const Fx drx = fx_operand<62>(fx_sum(dr));
 #pragma unroll
       for (int i = 0; i < DIM; ++i) {
         out[i] = FxAcc{0, 0};
         fx_mac(out[i], drx, Gx[0][i]);
       }
       if constexpr (DIM == 2) {
-        const Fx dsx = fx_operand(fx_sum(ds));
+        const Fx dsx = fx_operand<62>(fx_sum(ds));
 #pragma unroll
         for (int i = 0; i < DIM; ++i) fx_mac(out[i], dsx, Gx[DIM - 1][i]);
       }
@@ -450,7 +467,7 @@ __device__ __forceinline__ void estep_element_fx(int e, int K, const double* __r
         FxAcc w{0, 0};
 #pragma unroll
         for (int k = 0; k < NFP; ++k) fx_mac(w, gx[f][k], ops.LIFT[a * (NF * NFP) + f * NFP + k]);
-        const Fx wx = fx_operand(fx_sum(w));
+        const Fx wx = fx_operand<62>(fx_sum(w));
 #pragma unroll
         for (int i = 0; i < DIM; ++i) fx_mac(out[i], wx, snx[f][i]);
       }
@@ -568,8 +585,16 @@ __device__ __forceinline__ void estep_element(int e, int K, const R* __restrict_
   }
 }
 
+// Resident blocks of 256 threads the E-step asks the compiler to fit per SM:
+// two in FP64 (at most 128 registers a thread): its integer chains wait on one
+// another, and 16 warps cover what 8 do not.
+template <typename R>
+constexpr int estep_min_blocks() {
+  return sizeof(R) == 8 ? 2 : 1;
+}
+
 template <int DIM, int P, typename R>
-__global__ void __launch_bounds__(256) estep_kernel(int K, const R* __restrict__ V, R* __restrict__ E,
+__global__ void __launch_bounds__(256, estep_min_blocks<R>()) estep_kernel(int K, const R* __restrict__ V, R* __restrict__ E,
                                                     const R* __restrict__ geo, const int32_t* __restrict__ nbr,
                                                     const int8_t* __restrict__ nbrf, const R* __restrict__ fn,
                                                     const R* __restrict__ fsj, const EstepOps<DIM, P, R> ops,
@@ -819,7 +844,7 @@ __global__ void __launch_bounds__(256, face_pf_min_blocks<DIM, P, R>())
 // element is computed, so the neighbour-trace gathers need no dependent
 // round trip to the connectivity first.  Same arithmetic as estep_kernel.
 template <int DIM, int P, typename R>
-__global__ void __launch_bounds__(256) estep_pf_kernel(int K, const R* __restrict__ V, R* __restrict__ E,
+__global__ void __launch_bounds__(256, estep_min_blocks<R>()) estep_pf_kernel(int K, const R* __restrict__ V, R* __restrict__ E,
                                                        const R* __restrict__ geo, const int32_t* __restrict__ nbr,
                                                        const int8_t* __restrict__ nbrf, const R* __restrict__ fn,
                                                        const R* __restrict__ fsj, const EstepOps<DIM, P, R> ops,
@@ -1028,22 +1053,11 @@ __device__ __forceinline__ void conservative_stage(const R (&Vn)[Sh<DIM, P>::NV]
 // dV = -M(V)^{-1} r, i.e. M dh/dt = -r_h and M_h du/dt = -r_u - M_u dh/dt,
 // with M_h = <psi, max(h, h_floor) psi> and M_u = <psi, u psi> at the volume
 // quadrature points; r in physical scaling, Jinv = 1 / J.
-// STASH: the depth and velocity at the volume points arrive in Vqs (kept
-// from the volume-integral loop) instead of being interpolated again, and
-// M_h is assembled as sum_q max(h_q, h_floor) (w_q l_a l_b), the products
-// w_q l_a l_b read from pm (mass_products: the shared operator table) or,
-// with pm = nullptr, formed in the same order here.
 template <int DIM, int P, typename R>
-__host__ __device__ constexpr int mass_products_pad() {
-  return (int)(((Sh<DIM, P>::NP * (Sh<DIM, P>::NP + 1) / 2 * sizeof(R) + 15) / 16) * 16 / sizeof(R));
-}
-template <int DIM, int P, typename R, bool STASH = false>
 __device__ __forceinline__ void mass_solve_element(const R (&Vn)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
                                                    const R (&r)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
                                                    const VolOps<DIM, P, R>& ops, R h_floor, R Jinv,
-                                                   R (&dV)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
-                                                   const R (*Vqs)[Sh<DIM, P>::NV] = nullptr,
-                                                   const R* pm = nullptr) {
+                                                   R (&dV)[Sh<DIM, P>::NV][Sh<DIM, P>::NP]) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NQ = S::NQ;
 #pragma unroll
@@ -1065,62 +1079,26 @@ __device__ __forceinline__ void mass_solve_element(const R (&Vn)[Sh<DIM, P>::NV]
 #pragma unroll 1
   for (int q = 0; q < NQ; ++q) {
     R hq = R(0), hdq = R(0), uq[DIM];
-    if constexpr (STASH) {
-      hq = Vqs[q][0];
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) uq[j] = Vqs[q][1 + j];
+    for (int j = 0; j < DIM; ++j) uq[j] = R(0);
 #pragma unroll
-      for (int a = 0; a < NP; ++a) hdq += ops.Vq[q * NP + a] * dV[0][a];
-    } else {
+    for (int a = 0; a < NP; ++a) {
+      const R l = ops.Vq[q * NP + a];
+      hq += l * Vn[0][a];
+      hdq += l * dV[0][a];
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) uq[j] = R(0);
-#pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        const R l = ops.Vq[q * NP + a];
-        hq += l * Vn[0][a];
-        hdq += l * dV[0][a];
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) uq[j] += l * Vn[1 + j][a];
-      }
+      for (int j = 0; j < DIM; ++j) uq[j] += l * Vn[1 + j][a];
     }
     const R wd = ops.wq[q] * hdq;
-    if constexpr (STASH) {
-      const R hf = fmax(hq, h_floor);
-      constexpr int MPAD = mass_products_pad<DIM, P, R>();
-      R pq[MPAD];
-      if (pm) {
-        const double2* p2 = reinterpret_cast<const double2*>(pm + q * MPAD);
+    const R wh = ops.wq[q] * fmax(hq, h_floor);
 #pragma unroll
-        for (int c = 0; c < MPAD / 2; ++c) {
-          const double2 v = p2[c];
-          pq[2 * c] = v.x;
-          pq[2 * c + 1] = v.y;
-        }
-      } else {
+    for (int a = 0; a < NP; ++a) {
+      const R la = ops.Vq[q * NP + a];
+      const R t = wh * la;
 #pragma unroll
-        for (int a = 0, i = 0; a < NP; ++a)
+      for (int b = 0; b <= a; ++b) Mh[a][b] += t * ops.Vq[q * NP + b];
 #pragma unroll
-          for (int b = 0; b <= a; ++b, ++i) pq[i] = (ops.wq[q] * ops.Vq[q * NP + a]) * ops.Vq[q * NP + b];
-      }
-#pragma unroll
-      for (int a = 0, i = 0; a < NP; ++a) {
-#pragma unroll
-        for (int b = 0; b <= a; ++b, ++i) Mh[a][b] += hf * pq[i];
-        const R la = ops.Vq[q * NP + a];
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) rhs[j][a] -= wd * uq[j] * la;
-      }
-    } else {
-      const R wh = ops.wq[q] * fmax(hq, h_floor);
-#pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        const R la = ops.Vq[q * NP + a];
-        const R t = wh * la;
-#pragma unroll
-        for (int b = 0; b <= a; ++b) Mh[a][b] += t * ops.Vq[q * NP + b];
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) rhs[j][a] -= wd * uq[j] * la;
-      }
+      for (int j = 0; j < DIM; ++j) rhs[j][a] -= wd * uq[j] * la;
     }
   }
   // Cholesky of the reference-scaled M_h (lower triangle); the diagonal is
@@ -1282,87 +1260,44 @@ __device__ __forceinline__ void mass_solve_dispatch(const R (&Vn)[Sh<DIM, P>::NV
   mass_solve_element<DIM, P, R>(Vn, r, ops, ph.h_floor, Jinv, dV);
 }
 
-// Per-volume-point operator rows (Vq, Wr, Ws, Wm) of the direct
-// FP64 2D volume kernel, copied once per block into shared memory with each
-// row padded to 16 bytes, so that a row arrives in 128-bit loads instead of
-// one constant-bank load per value (FP64 headline volume kernel: 0.401 ->
-// 0.389 ms).  FP32 keeps the constant-bank reads, which measured faster
-// there (0.252 vs 0.386 ms on 2M triangles); so does the staged kernel,
-// whose shared memory holds its element tiles (tab = nullptr), and 1D,
-// where the fill cost more than it saved (200-element dam break: -5 %).
+}  // namespace dgswe
+
+#include "dg_volume_fx.cuh"
+
+namespace dgswe {
+
+// The volume pass's operator tables (a kernel parameter) and, for FP64
+// triangles, their shared-memory copy.
 template <int DIM, int P, typename R>
-struct QTab {
-  static constexpr int NP = Sh<DIM, P>::NP, NQ = Sh<DIM, P>::NQ, ROWS = 4;
-  static constexpr int PAD = (int)(((NP * sizeof(R) + 15) / 16) * 16 / sizeof(R));
-  static constexpr bool USED = sizeof(R) == 8 && DIM == 2;
-  // after the rows: per volume point the mass products w_q l_a l_b (b <= a,
-  // row by row) of the FP64 mass solve, padded to 16 bytes
-  static constexpr int MBASE = NQ * ROWS * PAD, MPAD = mass_products_pad<DIM, P, R>();
-  static constexpr int SIZE = USED ? MBASE + NQ * MPAD : 2;
+struct VolArgT {
+  using type = VolOps<DIM, P, R>;
+  static constexpr int TAB = 2;
+};
+template <int DIM, int P>
+struct VolArgT<DIM, P, double> {
+  using type = VolFx<DIM, P>;
+  static constexpr int TAB = FxTab<DIM, P>::SIZE;
 };
 template <int DIM, int P, typename R>
-__device__ __forceinline__ void qtab_fill(R* tab, const VolOps<DIM, P, R>& ops) {
-  using T = QTab<DIM, P, R>;
-  if constexpr (T::USED) {
-    for (int i = threadIdx.x; i < T::MBASE; i += blockDim.x) {
-      const int q = i / (T::ROWS * T::PAD), k = (i / T::PAD) % T::ROWS, a = i % T::PAD;
-      R v = R(0);
-      if (a < T::NP) {
-        const int j = q * T::NP + a;
-        v = k == 0 ? ops.Vq[j] : k == 1 ? ops.Wr[j] : k == 2 ? ops.Ws[j] : ops.Wm[j];
-      }
-      tab[i] = v;
-    }
-    for (int i = threadIdx.x; i < T::NQ * T::MPAD; i += blockDim.x) {
-      const int q = i / T::MPAD, idx = i % T::MPAD;
-      R v = R(0);
-      if (idx < T::NP * (T::NP + 1) / 2) {
-        int a = 0;
-        while ((a + 1) * (a + 2) / 2 <= idx) ++a;
-        const int b = idx - a * (a + 1) / 2;
-        v = (ops.wq[q] * ops.Vq[q * T::NP + a]) * ops.Vq[q * T::NP + b];
-      }
-      tab[T::MBASE + i] = v;
-    }
+using VolArg = typename VolArgT<DIM, P, R>::type;
+// Shared table of a kernel that runs volume passes (all threads of the block).
+template <int DIM, int P, typename R>
+__device__ __forceinline__ void vol_table(Fx* tab, const VolArg<DIM, P, R>& ops) {
+  if constexpr (sizeof(R) == 8) {
+    fxtab_fill<DIM, P>(tab, ops);
+    if constexpr (FxTab<DIM, P>::USED) __syncthreads();
   }
-}
-// Row ROW of volume point q: from the shared table (FP64) or the operator
-// parameters (FP32).
-template <int DIM, int P, int ROW, typename R>
-__device__ __forceinline__ void op_row(const VolOps<DIM, P, R>& ops, const R* tab, int q,
-                                       R (&out)[Sh<DIM, P>::NP]) {
-  using T = QTab<DIM, P, R>;
-  constexpr int NP = T::NP;
-  if constexpr (T::USED) {
-    if (tab) {
-      const double2* p = reinterpret_cast<const double2*>(tab + (q * T::ROWS + ROW) * T::PAD);
-      double tmp[T::PAD];
-#pragma unroll
-      for (int c = 0; c < T::PAD / 2; ++c) {
-        const double2 v = p[c];
-        tmp[2 * c] = v.x;
-        tmp[2 * c + 1] = v.y;
-      }
-#pragma unroll
-      for (int a = 0; a < NP; ++a) out[a] = tmp[a];
-      return;
-    }
-  }
-  const R* tabsrc = ROW == 0 ? ops.Vq : ROW == 1 ? ops.Wr : ROW == 2 ? ops.Ws : ops.Wm;
-#pragma unroll
-  for (int a = 0; a < NP; ++a) out[a] = tabsrc[q * NP + a];
 }
 
 // Everything the volume kernels do for one element e once its nodal values
 // are in registers: volume integrals, face lift, mass solve and output.
 // Bed and slope source S_j = -g_c h dH/dx_j - g_s h delta_1j (Eq. Sterm).
-// FP64 contexts read the coefficients c_j = -g_c dH/dx_j - g_s delta_1j at the
-// volume points from src ([DIM * NQ][K], host-computed once since the bed does
-// not change), which saves the FP64 kernels (bound by the FP64 pipe) the
-// interpolation of the bed gradient; FP32 contexts (latency-bound, where the
-// extra global loads inside the point loop cost more than the arithmetic)
-// interpolate the gradient from the element's nodal bed bed_e.  Both nullptr:
-// flat bed (the slope term -g_s h remains).  V0e[v]: the
+// FP64 contexts (volume_element_fx, dg_volume_fx.cuh) read the coefficients
+// c_j = -g_c dH/dx_j - g_s delta_1j at the volume points from src
+// ([DIM * NQ][K], host-computed once since the bed does not change); FP32
+// contexts (latency-bound, where the extra global loads inside the point loop
+// cost more than the arithmetic) interpolate the gradient from the element's
+// nodal bed bed_e.  nullptr: flat bed (the slope term -g_s h remains).  V0e[v]: the
 // element's values of field v of the stage's first state (read in mode 1
 // when c0 != 0).  mode 0: write dV/dt to out; mode 1: out = c0 * V0 + c1 * (Vin +
 // dt * dV/dt); mode 2: write the spatial residual r_V of Eq. WeakForm51
@@ -1370,13 +1305,13 @@ __device__ __forceinline__ void op_row(const VolOps<DIM, P, R>& ops, const R* ta
 template <int DIM, int P, typename R, bool COH = false>
 __device__ __forceinline__ void volume_element(int e, int K, int F, const R (&Vn)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
                                                const R (&En)[Sh<DIM, P>::NE][Sh<DIM, P>::NP],
-                                               const R* __restrict__ bed_e, const R* __restrict__ src,
+                                               const R* __restrict__ bed_e,
                                                const R* const (&V0e)[Sh<DIM, P>::NV],
                                                R* out,
                                                const R* __restrict__ geo, const int32_t* __restrict__ fid,
                                                const R* __restrict__ wflux, const VolOps<DIM, P, R>& ops,
                                                const Phys<R>& ph, int ins, int mode, R c0, R c1,
-                                               const DevScalars* __restrict__ sc, const R* tab) {
+                                               const DevScalars* __restrict__ sc) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NQ = S::NQ, NF = S::NF, NFP = S::NFP, NFQ = S::NFQ, NV = S::NV, NE = S::NE;
   const size_t KN = (size_t)K * NP;
@@ -1395,14 +1330,7 @@ __device__ __forceinline__ void volume_element(int e, int K, int F, const R (&Vn
 #pragma unroll
     for (int a = 0; a < NP; ++a) r[v][a] = R(0);
 
-  const bool has_src = sizeof(R) == 8 && src != nullptr;
-  const bool has_bed = sizeof(R) == 4 && bed_e != nullptr;
-  // FP64: the depth and velocity at the volume points, kept for the mass
-  // solve (per-thread local memory; saves its interpolation of them).  The
-  // FP32 kernels, issue-bound, ran slower with it (8.4M-triangle slump
-  // volume 0.97 -> 1.07 ms) and interpolate again.
-  constexpr bool kStash = sizeof(R) == 8;
-  R Vqs[kStash ? NQ : 1][NV];
+  const bool has_bed = bed_e != nullptr;
   R Hn[NP];
 #pragma unroll
   for (int a = 0; a < NP; ++a) Hn[a] = has_bed ? bed_e[a] : R(0);
@@ -1416,18 +1344,6 @@ __device__ __forceinline__ void volume_element(int e, int K, int F, const R (&Vn
 #pragma unroll
     for (int c = 0; c < NE; ++c) Eq[c] = R(0);
     R Hr = R(0), Hs = R(0);
-    if constexpr (QTab<DIM, P, R>::USED) {
-    R rvq[NP];
-    op_row<DIM, P, 0>(ops, tab, q, rvq);
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      const R l = rvq[a];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Vq[v] += l * Vn[v][a];
-#pragma unroll
-      for (int c = 0; c < NE; ++c) Eq[c] += l * En[c][a];
-    }
-    } else {
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
       const R l = ops.Vq[q * NP + a];
@@ -1439,11 +1355,6 @@ __device__ __forceinline__ void volume_element(int e, int K, int F, const R (&Vn
         Hr += ops.Drq[q * NP + a] * Hn[a];
         if constexpr (DIM == 2) Hs += ops.Dsq[q * NP + a] * Hn[a];
       }
-    }
-    }
-    if constexpr (kStash) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Vqs[q][v] = Vq[v];
     }
     const R h = Vq[0];
     const R hr = h * ph.rho_inv;
@@ -1459,20 +1370,15 @@ __device__ __forceinline__ void volume_element(int e, int K, int F, const R (&Vn
     }
     R Sv[NV];
     Sv[0] = R(0);
-    if (has_src) {
+    R dH[DIM];
 #pragma unroll
-      for (int jj = 0; jj < DIM; ++jj) Sv[1 + jj] = h * src[(size_t)(jj * NQ + q) * K + e];
-    } else {
-      R dH[DIM];
-#pragma unroll
-      for (int i = 0; i < DIM; ++i) {
-        dH[i] = G[0][i] * Hr;
-        if constexpr (DIM == 2) dH[i] += G[1][i] * Hs;
-      }
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) Sv[1 + j] = -ph.gc * h * dH[j];
-      Sv[1] -= ph.gs * h;
+    for (int i = 0; i < DIM; ++i) {
+      dH[i] = G[0][i] * Hr;
+      if constexpr (DIM == 2) dH[i] += G[1][i] * Hs;
     }
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) Sv[1 + j] = -ph.gc * h * dH[j];
+    Sv[1] -= ph.gs * h;
     R fr[NV], fs[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -1483,17 +1389,11 @@ __device__ __forceinline__ void volume_element(int e, int K, int F, const R (&Vn
         fs[v] = G[1][0] * fx[0][v] + G[1][1] * fx[1][v];
       }
     }
-    R rwr[NP], rws[NP], rwm[NP];
-    if constexpr (QTab<DIM, P, R>::USED) {
-      op_row<DIM, P, 1>(ops, tab, q, rwr);
-      if constexpr (DIM == 2) op_row<DIM, P, 2>(ops, tab, q, rws);
-      op_row<DIM, P, 3>(ops, tab, q, rwm);
-    }
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
-      const R wr = QTab<DIM, P, R>::USED ? rwr[a] : ops.Wr[q * NP + a];
-      const R ws = DIM == 1 ? R(0) : QTab<DIM, P, R>::USED ? rws[a] : ops.Ws[q * NP + a];
-      const R wm = QTab<DIM, P, R>::USED ? rwm[a] : ops.Wm[q * NP + a];
+      const R wr = ops.Wr[q * NP + a];
+      const R ws = DIM == 1 ? R(0) : ops.Ws[q * NP + a];
+      const R wm = ops.Wm[q * NP + a];
       // accumulated straight into r, three fused multiply-adds per entry
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
@@ -1547,11 +1447,7 @@ __device__ __forceinline__ void volume_element(int e, int K, int F, const R (&Vn
 
   // ---- mass solve: M dh/dt = -r_h ; M_h du/dt = -r_u - M_u dh/dt
   R dV[NV][NP];
-  if constexpr (kStash)
-    mass_solve_element<DIM, P, R, true>(Vn, r, ops, ph.h_floor, geo[6 * K + e], dV, Vqs,
-                                        (QTab<DIM, P, R>::USED && tab) ? tab + QTab<DIM, P, R>::MBASE : nullptr);
-  else
-    mass_solve_dispatch<DIM, P, R>(Vn, r, ops, ph, geo[6 * K + e], dV);
+  mass_solve_dispatch<DIM, P, R>(Vn, r, ops, ph, geo[6 * K + e], dV);
 
   // ---- output
   if (mode == 0) {
@@ -1577,14 +1473,31 @@ __device__ __forceinline__ void volume_element(int e, int K, int F, const R (&Vn
   }
 }
 
-// Register cap of the direct volume kernel: 168 for FP32 at p = 3, the most
-// that keeps three warps on each SM sub-partition (16,384 registers each; the
-// autotuner picks 32-thread blocks for this kernel).  Left to the compiler
-// it took 171 (176 allocated), two warps per sub-partition, and the p = 3
-// bump volume pass ran 0.40 instead of 0.30 ms.  Otherwise no cap.
+template <int DIM, int P, typename R, bool COH = false>
+__device__ __forceinline__ void volume_any(int e, int K, int F, const R (&Vn)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
+                                           const R (&En)[Sh<DIM, P>::NE][Sh<DIM, P>::NP],
+                                           const R* __restrict__ bed_e, const R* __restrict__ src,
+                                           const R* const (&V0e)[Sh<DIM, P>::NV], R* out,
+                                           const R* __restrict__ geo, const int32_t* __restrict__ fid,
+                                           const R* __restrict__ wflux, const VolArg<DIM, P, R>& ops,
+                                           const Phys<R>& ph, int ins, int mode, R c0, R c1,
+                                           const DevScalars* __restrict__ sc, const Fx* tab) {
+  if constexpr (sizeof(R) == 8)
+    volume_element_fx<DIM, P, COH>(e, K, F, Vn, En, src, V0e, out, geo, fid, wflux, ops, ph, ins, mode, c0, c1, sc,
+                                   tab);
+  else
+    volume_element<DIM, P, R, COH>(e, K, F, Vn, En, bed_e, V0e, out, geo, fid, wflux, ops, ph, ins, mode, c0, c1, sc);
+}
+
+// Register cap of the direct volume kernel: 168, the most that keeps three
+// warps on each SM sub-partition (16,384 registers each), for FP32 at p = 3
+// (left to the compiler it took 171, and the p = 3 bump volume pass ran 0.40
+// instead of 0.30 ms) and FP64 triangles at p = 2 (230 registers left to the
+// compiler: 1004 us against 929 on 524,288 triangles, with 156 bytes spilled; on
+// 8,192 triangles, one warp a sub-partition, 56 against 61 us).  Otherwise no cap.
 template <int DIM, int P, typename R>
 constexpr int volume_max_regs() {
-  return (sizeof(R) == 4 && P == 3) ? 168 : 255;
+  return (DIM == 2 && P == (sizeof(R) == 4 ? 3 : 2)) ? 168 : 255;
 }
 
 // One thread per element; nodal values read straight from global memory.
@@ -1593,15 +1506,14 @@ __global__ void __launch_bounds__(256) __maxnreg__((volume_max_regs<DIM, P, R>()
                                                      const R* V0, R* out,
                                                      const R* __restrict__ E, const R* __restrict__ bed, const R* __restrict__ src,
                                                      const R* __restrict__ geo, const int32_t* __restrict__ fid,
-                                                     const R* __restrict__ wflux, const VolOps<DIM, P, R> ops,
+                                                     const R* __restrict__ wflux, const VolArg<DIM, P, R> ops,
                                                      const Phys<R> ph0, const Phys<R>* __restrict__ ptab,
                                                      const int32_t* __restrict__ inst, int mode, R c0, R c1,
                                                      const DevScalars* __restrict__ sc) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV, NE = S::NE;
-  __shared__ __align__(16) R tab[QTab<DIM, P, R>::SIZE];
-  qtab_fill<DIM, P, R>(tab, ops);
-  if constexpr (QTab<DIM, P, R>::USED) __syncthreads();
+  __shared__ __align__(16) Fx tab[VolArgT<DIM, P, R>::TAB];
+  vol_table<DIM, P, R>(tab, ops);
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= K) return;
   const int ins = BATCH ? inst[e] : 0;
@@ -1620,7 +1532,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((volume_max_regs<DIM, P, R>()
   const R* V0e[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) V0e[v] = V0 ? V0 + v * KN + eo : nullptr;
-  volume_element<DIM, P, R>(e, K, F, Vn, En, bed ? bed + eo : nullptr, src, V0e, out, geo, fid, wflux, ops, ph, ins, mode,
+  volume_any<DIM, P, R>(e, K, F, Vn, En, bed ? bed + eo : nullptr, src, V0e, out, geo, fid, wflux, ops, ph, ins, mode,
                             c0, c1, sc, tab);
 }
 
@@ -1850,7 +1762,7 @@ __global__ void __launch_bounds__(256) volume_staged_kernel(int K, int F, const 
                                                             R* out, const R* __restrict__ E,
                                                             const R* __restrict__ bed, const R* __restrict__ src, const R* __restrict__ geo,
                                                             const int32_t* __restrict__ fid,
-                                                            const R* __restrict__ wflux, const VolOps<DIM, P, R> ops,
+                                                            const R* __restrict__ wflux, const VolArg<DIM, P, R> ops,
                                                             const Phys<R>* __restrict__ ptab,
                                                             const int32_t* __restrict__ inst, R c0, R c1,
                                                             DevScalars* sc) {
@@ -1950,7 +1862,7 @@ __global__ void __launch_bounds__(256) volume_staged_kernel(int K, int F, const 
       const R* V0e[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) V0e[v] = sV[NV + NE + 1 + v];
-      volume_element<DIM, P, R>(e, K, F, Vn, En, (sizeof(R) == 4 && bed) ? sV[NV + NE] : nullptr, src, V0e, out, geo, fid, wflux, ops, ph,
+      volume_any<DIM, P, R>(e, K, F, Vn, En, (sizeof(R) == 4 && bed) ? sV[NV + NE] : nullptr, src, V0e, out, geo, fid, wflux, ops, ph,
                                 ins, 1, c0, c1, sc, nullptr);
     }
     __syncthreads();

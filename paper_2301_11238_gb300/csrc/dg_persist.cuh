@@ -104,13 +104,13 @@ __device__ __forceinline__ bool wait_count(const int* counter, int need) {
 template <int DIM, int P, typename R>
 __global__ void __launch_bounds__(kThreads) step_kernel(const Plan pl, const Arrays<R> A,
                                                         const EstepOps<DIM, P, R> eo, const FaceOps<DIM, P, R> fo,
-                                                        const VolOps<DIM, P, R> vo) {
+                                                        const VolArg<DIM, P, R> vo) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV, NE = S::NE, NFQ = S::NFQ;
-  __shared__ __align__(16) R tab[QTab<DIM, P, R>::SIZE];
+  __shared__ __align__(16) Fx tab[VolArgT<DIM, P, R>::TAB];
   __shared__ double red[kThreads / 32];
   __shared__ int s_item, s_ok;
-  qtab_fill<DIM, P, R>(tab, vo);
+  vol_table<DIM, P, R>(tab, vo);
   const int tid = threadIdx.x;
   const int K = A.K, F = A.F;
   const size_t KN = (size_t)K * NP;
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kThreads) step_kernel(const Plan pl, const Arr
           const R* V0e[NV];
 #pragma unroll
           for (int v = 0; v < NV; ++v) V0e[v] = A.V[0] + v * KN + eo2;
-          volume_element<DIM, P, R, true>((int)e, K, F, Vn, En, A.bed ? A.bed + eo2 : nullptr, A.src, V0e, A.V[vout],
+          volume_any<DIM, P, R, true>((int)e, K, F, Vn, En, A.bed ? A.bed + eo2 : nullptr, A.src, V0e, A.V[vout],
                                           A.geo, A.fid, A.wflux, vo, phy, ins, 1, c0, c1, A.sc, tab);
         }
       }

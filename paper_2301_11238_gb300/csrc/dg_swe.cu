@@ -89,12 +89,15 @@ struct Impl final : Driver {
   EstepOps<DIM, P, R> eo{};
   FaceOps<DIM, P, R> fo{};
   VolOps<DIM, P, R> vo{};
+  VolArg<DIM, P, R> va{};  // operator tables of the volume pass
   Phys<R> ph{};
   bool tc = false;
   std::unique_ptr<tc::Launcher<(P >= 2 ? P : 2), false>> tcl;
 
   explicit Impl(const dg_swe_ctx& c) {
     fill_ops<DIM, P, R>(c.ops, eo, fo, vo);
+    if constexpr (sizeof(R) == 8) fill_vol_fx<DIM, P>(c.ops, va);
+    else va = vo;
     ph = make_phys<R>(c.prm, c.reg);
     if constexpr (kTcForm) {
       tc = c.prec == DG_PREC_FP32_TC;
@@ -137,7 +140,7 @@ struct Impl final : Driver {
         K, F, (const R*)Vin, (const R*)V0, (R*)out, c->at<R>(c->off.E),
         c->has_bed ? c->at<R>(c->off.bed) : nullptr, c->has_bed ? c->at<R>(c->off.src) : nullptr,
         c->at<R>(c->off.geo), c->at<int32_t>(c->off.fid),
-        c->at<R>(c->off.wflux), vo, ph, nullptr, nullptr, mode, (R)c0, (R)c1, c->at<DevScalars>(c->off.sc));
+        c->at<R>(c->off.wflux), va, ph, nullptr, nullptr, mode, (R)c0, (R)c1, c->at<DevScalars>(c->off.sc));
   }
   void wetdry_stage(dg_swe_ctx* c, const void* Vin, const void* V0, const void* rbuf, void* out, double c0,
                     double c1, cudaStream_t s) override {
@@ -172,7 +175,7 @@ struct Impl final : Driver {
     volume_kernel<DIM, P, R, false><<<(K + kBlock - 1) / kBlock, kBlock, 0, s>>>(
         K, F, (const R*)V, nullptr, (R*)out, (const R*)E, c->has_bed ? c->at<R>(c->off.bed) : nullptr,
         c->has_bed ? c->at<R>(c->off.src) : nullptr,
-        c->at<R>(c->off.geo), c->at<int32_t>(c->off.fid), (const R*)wflux, vo, ph, nullptr, nullptr, 0, R(0), R(0),
+        c->at<R>(c->off.geo), c->at<int32_t>(c->off.fid), (const R*)wflux, va, ph, nullptr, nullptr, 0, R(0), R(0),
         c->at<DevScalars>(c->off.sc));
   }
   void dt_partial(dg_swe_ctx* c, const void* V, cudaStream_t s) override {
