@@ -12,16 +12,16 @@
  * with the quadrature, fluxes and boundary ghosts of dg_swe.h.  The Jacobian
  * uses the Appendix A tangent terms with the HLL wave speeds held fixed; it
  * is block tridiagonal for a left-to-right ordered mesh (element e's right
- * neighbour is e + 1) and is solved by block Thomas elimination with partial
- * pivoting (the paper does not name its linear solver), either in FP64 or
- * factored in FP32 and refined in FP64 (linear_solver).  Newton stops when
+ * neighbour is e + 1) and is solved by block cyclic reduction with partial
+ * pivoting inside the blocks (the paper does not name its linear solver), either
+ * in FP64 or in FP32 refined in FP64 (linear_solver).  Newton stops when
  * ||R||_2 <= rtol ||R^0||_2, ||R||_2 <= atol or
  * ||dx||_inf <= xtol (1 + ||x||_inf), after at most max_it iterations
  * (the paper uses 10, Sec. 6).  Residual and Jacobian are FP64.
  *
  * The whole integration (time steps x Newton iterations: assembly, solve,
- * update, convergence test) runs in one persistent launch with one thread
- * block per instance.  Conventions (status, workspace, stream) follow
+ * update, convergence test) runs in one persistent launch of one thread-block
+ * cluster (up to eight blocks) per instance.  Conventions (status, workspace, stream) follow
  * dg_swe.h.
  */
 #ifndef DG_IMPLICIT_H
@@ -42,8 +42,8 @@ typedef struct {
   int32_t on_fail_continue;  /* 1: keep going after max_it (the paper's runs);
                                 0: stop and report DG_ERR_NEWTON                  */
   double rtol, atol, xtol;   /* stopping rule above                               */
-  int32_t linear_solver;     /* 0: FP64 block Thomas (partial pivoting);
-                                1: FP32 block-Thomas factorization with two FP64
+  int32_t linear_solver;     /* 0: FP64 block elimination (partial pivoting);
+                                1: FP32 block elimination with two FP64
                                    iterative-refinement rounds (residual of the
                                    linear system in FP64); needs
                                    2(p+1) + m3 + 1 <= 10                           */

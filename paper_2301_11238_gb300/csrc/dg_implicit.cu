@@ -1,6 +1,6 @@
 // Backward Euler + Newton-Raphson for the 1D scheme (Sec. 5.1, Appendix A):
-// one persistent thread block per instance runs time steps x Newton
-// iterations (assembly, block-Thomas solve, update, convergence test).
+// one persistent thread-block cluster per instance runs time steps x Newton
+// iterations (assembly, block cyclic reduction, update, convergence test).
 // See include/dg_implicit.h.
 #include <cmath>
 #include <cstring>
@@ -38,13 +38,14 @@ struct ImplArgs {
   int max_it, on_fail_continue;
   int n_gamma;    // > 1: continuation in gamma within each time step (Sec. 6.3)
   double gamma0;
-  int mixed;  // 1: FP32 block-Thomas factorization + FP64 iterative refinement
+  int mixed;  // 1: FP32 block factorization + FP64 iterative refinement
   BCEntry<double> bcL, bcR;
-  double *X, *Uold, *R, *D, *L, *U, *W, *Y, *DX;
-  float *Wf, *Af;    // mixed: W_e = A_e^-1 U_e and A_e^-1 per element (FP32)
-  double *Rr, *Dx2;  // mixed: refinement residual and correction
+  double *X, *Uold, *R, *D, *L, *U, *Y, *DX;
+  double *pt, *fc;               // pointwise data (volume_point, face_data)
+  float *Df, *Lf, *Uf, *bf, *xf;  // mixed: FP32 copies of the system, its solution
+  double* Rr;                    // mixed: refinement residual
   const double *J, *bed;
-  double* red;  // per-block partials of the residual norm / dx norms
+  double* red;  // reduction slots of the cluster
   dg_implicit_stats* st;
 };
 
@@ -101,479 +102,423 @@ __device__ __forceinline__ double block_sum(double v, double* sred) {
   return t;
 }
 
-__device__ __forceinline__ double block_max(double v, double* sred) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) sred[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t = fmax(t, sred[i]);
-  return t;
+// ------------------------------------------------------------------ thread-block cluster helpers
+// The integrator runs on one cluster of thread blocks (up to eight SMs): a
+// warp-wide FP64 instruction holds its sub-partition for 64 clocks however many
+// of its lanes are active (measured 64-72), so the independent pieces of a
+// Newton iteration are spread over the cluster's sub-partitions, and phases are
+// separated by the cluster barrier (about 360 clocks, five FP64 instructions).
+
+constexpr int kThreads = 256, kWarps = kThreads / 32, kMaxCluster = 8;
+
+__device__ __forceinline__ int cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ int cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return (int)r;
+}
+// All threads of the cluster; orders their global-memory accesses.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Residual and Jacobian blocks of element e at X (thread per element).
-// Returns the element's squared residual norm.
+// Position of the thread in the cluster, and the reduction slots.
+struct Team {
+  int rank, size, tid, threads, warp, warps, lane;
+  double* red;  // [4][kMaxCluster] global; slots used in turn
+  int slot;
+};
+
+// Sum (MAX: maximum, NaNs skipped) over the cluster, the same value in every
+// thread; blocks in rank order, so repeated runs agree.  Contains a cluster barrier.
+template <bool MAX>
+__device__ double team_reduce(double v, Team& t, double* sred) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double w = __shfl_down_sync(0xffffffffu, v, o);
+    v = MAX ? fmax(v, w) : v + w;
+  }
+  __syncthreads();
+  if (t.lane == 0) sred[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double* slot = t.red + t.slot * kMaxCluster;
+  if (threadIdx.x == 0) {
+    double s = sred[0];
+    for (int i = 1; i < kWarps; ++i) s = MAX ? fmax(s, sred[i]) : s + sred[i];
+    slot[t.rank] = s;
+  }
+  cluster_sync();
+  double s = slot[0];
+  for (int i = 1; i < t.size; ++i) s = MAX ? fmax(s, slot[i]) : s + slot[i];
+  t.slot = (t.slot + 1) & 3;
+  return s;
+}
+
+// 1 / x of either sign
+__device__ __forceinline__ double rcp_any(double x) {
+  const double r = rcp_pos(fabs(x));
+  return __hiloint2double(__double2hiint(r) | (__double2hiint(x) & (int)0x80000000u), __double2loint(r));
+}
+__device__ __forceinline__ float rcp_any(float x) { return 1.0f / x; }
+
+// ------------------------------------------------------------------ assembly
+
+// Pointwise data of a Newton iterate, one item per thread (kPt doubles a volume
+// point, kFc a face): every face is evaluated once.
+constexpr int kPt = 5;   // h, u, sigma, sigma', dH/dx
+constexpr int kFc = 17;  // F_h, F_u, G; d(F_h, F_u)/d(h, u) left and right; dF_u/dE left, right; dG/du left, right
+
 template <int P, int M3>
-__device__ double assemble(int e, const ImplArgs& a, const ImplOps<P, M3>& o) {
+__device__ void volume_point(int i, const ImplArgs& a, const ImplOps<P, M3>& o) {
   using S = IS<P, M3>;
   constexpr int NP = S::NP, NE = S::NE, NB = S::NB, NQ = S::NQ;
-  const int K = a.K;
+  const int e = i / NQ, q = i - e * NQ;
   const double* x = a.X + (size_t)e * NB;
-  const double J = a.J[e];
-  double h[NP], u[NP], E[NE];
+  double h = 0, u = 0, ee = 0, dH = 0;
 #pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    h[i] = x[i];
-    u[i] = x[NP + i];
+  for (int k = 0; k < NP; ++k) {
+    h += o.Vq[q * NP + k] * x[k];
+    u += o.Vq[q * NP + k] * x[NP + k];
+    if (a.bed) dH += o.dVq[q * NP + k] * a.bed[(size_t)e * NP + k];
   }
 #pragma unroll
-  for (int i = 0; i < NE; ++i) E[i] = x[2 * NP + i];
-  // ---- pointwise quantities at volume points
-  double qh[NQ], qu[NQ], qs[NQ], qds[NQ], qdH[NQ];
+  for (int c = 0; c < NE; ++c) ee += o.VEq[q * NE + c] * x[2 * NP + c];
+  double* p = a.pt + (size_t)i * kPt;
+  p[0] = h;
+  p[1] = u;
+  sigma1d(ee, a, p[2], p[3]);
+  p[4] = a.bed ? dH / a.J[e] : 0.0;
+}
+
+// Face i between elements i - 1 and i, normal +1: numerical flux F (HLL minus
+// the central flux of Q), central G, and their derivatives with the HLL speeds
+// held fixed.  At the ends the missing side is the ghost state, its derivatives
+// taken through the ghost's dependence on the inner state.
+template <int P, int M3>
+__device__ void face_data(int i, const ImplArgs& a, const ImplOps<P, M3>& o) {
+  using S = IS<P, M3>;
+  constexpr int NP = S::NP, NE = S::NE, NB = S::NB;
+  double h[2], u[2], ee[2];                          // left, right
+  double dh[2] = {1, 1}, du[2] = {1, 1}, de[2] = {1, 1};  // d ghost / d inner
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int e = i - 1 + s, f = 1 - s;  // the left element's face 1, the right one's face 0
+    h[s] = u[s] = ee[s] = 0.0;
+    if (e >= 0 && e < a.K) {
+      const double* x = a.X + (size_t)e * NB;
+#pragma unroll
+      for (int k = 0; k < NP; ++k) {
+        h[s] += o.lf[f * NP + k] * x[k];
+        u[s] += o.lf[f * NP + k] * x[NP + k];
+      }
+#pragma unroll
+      for (int c = 0; c < NE; ++c) ee[s] += o.lEf[f * NE + c] * x[2 * NP + c];
+    }
+  }
+  if (i == 0 || i == a.K) {
+    const int g = i == 0 ? 0 : 1, in = 1 - g;  // ghost side, inner side
+    const BCEntry<double>& b = i == 0 ? a.bcL : a.bcR;
+    const bool d0 = b.mode[0] == 1, d1 = b.mode[1] == 1, w = b.mode[1] == 2, d2 = b.mode[2] == 1;
+    const double gh = d0 ? b.val[0] : h[in], gu = d1 ? b.val[1] : w ? -u[in] : u[in], ge = d2 ? b.val[2] : ee[in];
+    const double fh = d0 ? 0.0 : 1.0, fu = d1 ? 0.0 : w ? -1.0 : 1.0, fe = d2 ? 0.0 : 1.0;
+    if (g == 0) {
+      h[0] = gh, u[0] = gu, ee[0] = ge, dh[0] = fh, du[0] = fu, de[0] = fe;
+    } else {
+      h[1] = gh, u[1] = gu, ee[1] = ge, dh[1] = fh, du[1] = fu, de[1] = fe;
+    }
+  }
+  double c[2], F0[2], F1[2], sg[2], ds[2];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    c[s] = sqrt_pos(a.gc * fmax(h[s], a.h_floor));
+    F0[s] = h[s] * u[s];
+    F1[s] = F0[s] * u[s] + (0.5 * a.gc) * h[s] * h[s];
+    sigma1d(ee[s], a, sg[s], ds[s]);
+  }
+  const double SL = fmin(u[0] - c[0], u[1] - c[1]), SR = fmax(u[0] + c[0], u[1] + c[1]);
+  // F = x F_left + y F_right + z (U_right - U_left)
+  double x = 1.0, y = 0.0, z = 0.0;
+  if (SL >= 0.0) {
+  } else if (SR <= 0.0) {
+    x = 0.0;
+    y = 1.0;
+  } else {
+    const double inv = rcp_pos(SR - SL);
+    x = SR * inv;
+    y = -SL * inv;
+    z = SL * x;
+  }
+  double* p = a.fc + (size_t)i * kFc;
+  const double hr = 0.5 * a.rho_inv;
+  p[0] = x * F0[0] + (y * F0[1] + z * (h[1] - h[0]));
+  p[1] = x * F1[0] + (y * F1[1] + z * (F0[1] - F0[0])) - hr * (h[0] * sg[0] + h[1] * sg[1]);
+  p[2] = 0.5 * (u[0] + u[1]);
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const double wf = s == 0 ? x : y, wu = s == 0 ? -z : z;  // weights of dF and dU of the side
+    double* A = p + 3 + 4 * s;
+    A[0] = (wf * u[s] + wu) * dh[s];
+    A[1] = (wf * h[s]) * du[s];
+    A[2] = (wf * (u[s] * u[s] + a.gc * h[s]) + wu * u[s] - hr * sg[s]) * dh[s];
+    A[3] = (wf * (2.0 * h[s] * u[s]) + wu * h[s]) * du[s];
+    p[11 + s] = -hr * h[s] * ds[s] * de[s];
+    p[13 + s] = 0.5 * du[s];
+  }
+}
+
+// Row r of element e: residual entry and the rows of the blocks D (own), L (left
+// neighbour), U (right neighbour).  Returns the residual entry.
+template <int P, int M3>
+__device__ double assemble_row(int e, int r, const ImplArgs& a, const ImplOps<P, M3>& o) {
+  using S = IS<P, M3>;
+  constexpr int NP = S::NP, NE = S::NE, NB = S::NB, NQ = S::NQ;
+  const double J = a.J[e];
+  const int rb = r < NP ? 0 : (r < 2 * NP ? 1 : 2);  // row block: h, u, E
+  const int ri = rb < 2 ? r - rb * NP : r - 2 * NP;
+  double res = rb < 2 ? -a.Uold[(size_t)e * 2 * NP + r] * a.inv_dt : 0.0;
+  double D[NB];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) D[c] = 0.0;
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
-    double hh = 0, uu = 0, ee = 0, dH = 0;
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      hh += o.Vq[q * NP + i] * h[i];
-      uu += o.Vq[q * NP + i] * u[i];
-      if (a.bed) dH += o.dVq[q * NP + i] * a.bed[(size_t)e * NP + i];
-    }
-#pragma unroll
-    for (int c = 0; c < NE; ++c) ee += o.VEq[q * NE + c] * E[c];
-    qh[q] = hh;
-    qu[q] = uu;
-    sigma1d(ee, a, qs[q], qds[q]);
-    qdH[q] = dH / J;
-  }
-  // ---- face data: traces, fluxes and their derivatives (frozen HLL speeds)
-  double Fh[2], Fu[2], Gb[2];              // F_bar.n (h, u rows incl. -Q_bar.n), G_bar.n
-  double Am[2][2][2], Ap[2][2][2];         // d flux(h,u rows)/d (h,u) of - and + side
-  double BEm[2], BEp[2], GVm[2], GVp[2];   // d u-row/dE-, dE+;  d(-Gbar n)/du-, du+
-  int nb_e[2];
-#pragma unroll
-  for (int f = 0; f < 2; ++f) {
-    const double n = f == 0 ? -1.0 : 1.0;
-    double hm = 0, um = 0, em = 0;
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      hm += o.lf[f * NP + i] * h[i];
-      um += o.lf[f * NP + i] * u[i];
-    }
-#pragma unroll
-    for (int c = 0; c < NE; ++c) em += o.lEf[f * NE + c] * E[c];
-    double hp, up, ep, dVh = 1.0, dVu = 1.0, dEp = 1.0;
-    const int e2 = f == 0 ? e - 1 : e + 1;
-    if (e2 >= 0 && e2 < K) {
-      const double* x2 = a.X + (size_t)e2 * NB;
-      const int f2 = 1 - f;
-      hp = up = ep = 0.0;
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        hp += o.lf[f2 * NP + i] * x2[i];
-        up += o.lf[f2 * NP + i] * x2[NP + i];
-      }
-#pragma unroll
-      for (int c = 0; c < NE; ++c) ep += o.lEf[f2 * NE + c] * x2[2 * NP + c];
-      nb_e[f] = e2;
+    const double* p = a.pt + ((size_t)e * NQ + q) * kPt;
+    const double h = p[0], u = p[1], w = o.wq[q];
+    const double m = w * J * (rb < 2 ? o.Vq[q * NP + ri] : o.VEq[q * NE + ri]);
+    const double d = w * (rb < 2 ? o.dVq[q * NP + ri] : o.dVEq[q * NE + ri]);
+    double ch = 0.0, cu = 0.0, ce = 0.0;
+    if (rb == 0) {
+      const double mt = m * a.inv_dt;
+      ch = mt - d * u;
+      cu = -d * h;
+      res += ch * h;
+    } else if (rb == 1) {
+      const double mt = m * a.inv_dt, s = p[2] * a.rho_inv, f = a.gs + a.gc * p[4], hu = h * u;
+      ch = mt * u + d * (s - (u * u + a.gc * h)) + m * f;
+      cu = mt * h - 2.0 * d * hu;
+      ce = d * (h * p[3] * a.rho_inv);
+      res += mt * hu + d * (h * s - (hu * u + 0.5 * a.gc * h * h)) + m * f * h;
     } else {
-      const BCEntry<double>& b = f == 0 ? a.bcL : a.bcR;
-      hp = b.mode[0] == 1 ? b.val[0] : hm;
-      dVh = b.mode[0] == 1 ? 0.0 : 1.0;
-      if (b.mode[1] == 1) {
-        up = b.val[1];
-        dVu = 0.0;
-      } else if (b.mode[1] == 2) {
-        up = -um;
-        dVu = -1.0;
-      } else {
-        up = um;
-      }
-      ep = b.mode[2] == 1 ? b.val[2] : em;
-      dEp = b.mode[2] == 1 ? 0.0 : 1.0;
-      nb_e[f] = -1;
-    }
-    const double cm = sqrt(a.gc * fmax(hm, a.h_floor)), cp = sqrt(a.gc * fmax(hp, a.h_floor));
-    const double unm = um * n, unp = up * n;
-    const double SL = fmin(unm - cm, unp - cp), SR = fmax(unm + cm, unp + cp);
-    const double Fm0 = hm * unm, Fm1 = (hm * um * um + 0.5 * a.gc * hm * hm) * n;
-    const double Fp0 = hp * unp, Fp1 = (hp * up * up + 0.5 * a.gc * hp * hp) * n;
-    const double dFm[2][2] = {{um * n, hm * n}, {(um * um + a.gc * hm) * n, 2.0 * hm * um * n}};
-    const double dFp[2][2] = {{up * n, hp * n}, {(up * up + a.gc * hp) * n, 2.0 * hp * up * n}};
-    const double dUm[2][2] = {{1.0, 0.0}, {um, hm}};
-    const double dUp[2][2] = {{1.0, 0.0}, {up, hp}};
-    double F0, F1;
-    if (SL >= 0.0) {
-      F0 = Fm0;
-      F1 = Fm1;
-      for (int r = 0; r < 2; ++r)
-        for (int c = 0; c < 2; ++c) {
-          Am[f][r][c] = dFm[r][c];
-          Ap[f][r][c] = 0.0;
-        }
-    } else if (SR <= 0.0) {
-      F0 = Fp0;
-      F1 = Fp1;
-      for (int r = 0; r < 2; ++r)
-        for (int c = 0; c < 2; ++c) {
-          Am[f][r][c] = 0.0;
-          Ap[f][r][c] = dFp[r][c];
-        }
-    } else {
-      const double inv = 1.0 / (SR - SL);
-      F0 = (SR * Fm0 - SL * Fp0 + SL * SR * (hp - hm)) * inv;
-      F1 = (SR * Fm1 - SL * Fp1 + SL * SR * (hp * up - hm * um)) * inv;
-      for (int r = 0; r < 2; ++r)
-        for (int c = 0; c < 2; ++c) {
-          Am[f][r][c] = (SR * dFm[r][c] - SL * SR * dUm[r][c]) * inv;
-          Ap[f][r][c] = (-SL * dFp[r][c] + SL * SR * dUp[r][c]) * inv;
-        }
-    }
-    double sm, dsm, sp, dsp;
-    sigma1d(em, a, sm, dsm);
-    sigma1d(ep, a, sp, dsp);
-    Fh[f] = F0;
-    Fu[f] = F1 - 0.5 * (hm * sm + hp * sp) * a.rho_inv * n;
-    Gb[f] = 0.5 * (um + up) * n;
-    Am[f][1][0] -= 0.5 * sm * a.rho_inv * n;
-    Ap[f][1][0] -= 0.5 * sp * a.rho_inv * n;
-    BEm[f] = -0.5 * hm * dsm * a.rho_inv * n;
-    BEp[f] = -0.5 * hp * dsp * a.rho_inv * n;
-    GVm[f] = -0.5 * n;
-    GVp[f] = -0.5 * n;
-    // chain rule through boundary ghosts (dV+/dV- diagonal)
-    if (nb_e[f] < 0) {
-      for (int r = 0; r < 2; ++r) {
-        Ap[f][r][0] *= dVh;
-        Ap[f][r][1] *= dVu;
-      }
-      BEp[f] *= dEp;
-      GVp[f] *= dVu;
-    }
-  }
-  // ---- residual
-  double Rl[NB];
-  const double* uo = a.Uold + (size_t)e * 2 * NP;
-  double nrm = 0.0;
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    double rh = 0, ru = 0;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      const double w = o.wq[q], l = o.Vq[q * NP + i], dl = o.dVq[q * NP + i];
-      rh += w * J * l * qh[q] * a.inv_dt - w * dl * qh[q] * qu[q];
-      ru += w * J * l * qh[q] * qu[q] * a.inv_dt
-            + w * dl * (qh[q] * qs[q] * a.rho_inv - (qh[q] * qu[q] * qu[q] + 0.5 * a.gc * qh[q] * qh[q]))
-            + w * J * l * (a.gs * qh[q] + a.gc * qh[q] * qdH[q]);
-    }
-    rh -= uo[i] * a.inv_dt;
-    ru -= uo[NP + i] * a.inv_dt;
-#pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      rh += o.lf[f * NP + i] * Fh[f];
-      ru += o.lf[f * NP + i] * Fu[f];
-    }
-    Rl[i] = rh;
-    Rl[NP + i] = ru;
-  }
-#pragma unroll
-  for (int c = 0; c < NE; ++c) {
-    double r = 0.0;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
+      cu = d;
+      ce = m;
       double ee = 0.0;
 #pragma unroll
-      for (int d = 0; d < NE; ++d) ee += o.VEq[q * NE + d] * E[d];
-      r += o.wq[q] * J * o.VEq[q * NE + c] * ee + o.wq[q] * o.dVEq[q * NE + c] * qu[q];
+      for (int c = 0; c < NE; ++c) ee += o.VEq[q * NE + c] * a.X[(size_t)e * NB + 2 * NP + c];
+      res += m * ee + d * u;
     }
 #pragma unroll
-    for (int f = 0; f < 2; ++f) r -= o.lEf[f * NE + c] * Gb[f];
-    Rl[2 * NP + c] = r;
-  }
+    for (int c = 0; c < NP; ++c) {
+      D[c] += ch * o.Vq[q * NP + c];
+      D[NP + c] += cu * o.Vq[q * NP + c];
+    }
 #pragma unroll
-  for (int i = 0; i < NB; ++i) {
-    a.R[(size_t)e * NB + i] = Rl[i];
-    nrm += Rl[i] * Rl[i];
+    for (int c = 0; c < NE; ++c) D[2 * NP + c] += ce * o.VEq[q * NE + c];
   }
-  // ---- Jacobian blocks: D (own), L (left neighbour), U (right neighbour)
-  double* Dm = a.D + (size_t)e * NB * NB;
-  double* Lm = a.L + (size_t)e * NB * NB;
-  double* Um = a.U + (size_t)e * NB * NB;
-  for (int r = 0; r < NB; ++r) {
-    const int rb = r < NP ? 0 : (r < 2 * NP ? 1 : 2);  // row block: h, u, E
-    const int ri = rb < 2 ? r - rb * NP : r - 2 * NP;
+  // faces: 0 (left, the face data's right side is own) and 1
+  double* Dm = a.D + ((size_t)e * NB + r) * NB;
+  double* Lm = a.L + ((size_t)e * NB + r) * NB;
+  double* Um = a.U + ((size_t)e * NB + r) * NB;
+#pragma unroll
+  for (int f = 0; f < 2; ++f) {
+    const double* p = a.fc + (size_t)(e + f) * kFc;
+    const double fr = (f == 0 ? -1.0 : 1.0) * (rb < 2 ? o.lf[f * NP + ri] : o.lEf[f * NE + ri]);
+    const int own = 1 - f, out = f;  // side of the own and of the outer state
+    double vo[3] = {0, 0, 0}, vx[3] = {0, 0, 0};  // d/d(h, u, E) of the own and the outer trace
+    if (rb < 2) {
+      res += fr * p[rb];
+      vo[0] = fr * p[3 + 4 * own + 2 * rb];
+      vo[1] = fr * p[3 + 4 * own + 2 * rb + 1];
+      vx[0] = fr * p[3 + 4 * out + 2 * rb];
+      vx[1] = fr * p[3 + 4 * out + 2 * rb + 1];
+      if (rb == 1) {
+        vo[2] = fr * p[11 + own];
+        vx[2] = fr * p[11 + out];
+      }
+    } else {
+      res -= fr * p[2];
+      vo[1] = -fr * p[13 + own];
+      vx[1] = -fr * p[13 + out];
+    }
+    const bool end = f == 0 ? e == 0 : e == a.K - 1;  // the outer state is the ghost of the own one
+    double* N = f == 0 ? Lm : Um;
+#pragma unroll
     for (int c = 0; c < NB; ++c) {
       const int cb = c < NP ? 0 : (c < 2 * NP ? 1 : 2);
       const int ci = cb < 2 ? c - cb * NP : c - 2 * NP;
-      double dv = 0.0, lv = 0.0, uv = 0.0;
-      for (int q = 0; q < NQ; ++q) {
-        const double w = o.wq[q];
-        const double lr = rb < 2 ? o.Vq[q * NP + ri] : o.VEq[q * NE + ri];
-        const double dlr = rb < 2 ? o.dVq[q * NP + ri] : o.dVEq[q * NE + ri];
-        const double lc = cb < 2 ? o.Vq[q * NP + ci] : o.VEq[q * NE + ci];
-        const double hq = qh[q], uq = qu[q];
-        if (rb == 0 && cb == 0) dv += w * J * lr * lc * a.inv_dt - w * dlr * uq * lc;
-        else if (rb == 0 && cb == 1) dv += -w * dlr * hq * lc;
-        else if (rb == 1 && cb == 0)
-          dv += w * J * lr * uq * lc * a.inv_dt - w * dlr * (uq * uq + a.gc * hq) * lc + w * dlr * qs[q] * a.rho_inv * lc
-                + w * J * lr * (a.gs + a.gc * qdH[q]) * lc;
-        else if (rb == 1 && cb == 1) dv += w * J * lr * hq * lc * a.inv_dt - w * dlr * 2.0 * hq * uq * lc;
-        else if (rb == 1 && cb == 2) dv += w * dlr * hq * qds[q] * a.rho_inv * lc;
-        else if (rb == 2 && cb == 2) dv += w * J * lr * lc;
-        else if (rb == 2 && cb == 1) dv += w * dlr * lc;
-      }
-      for (int f = 0; f < 2; ++f) {
-        const double fr = rb < 2 ? o.lf[f * NP + ri] : o.lEf[f * NE + ri];
-        const double fcm = cb < 2 ? o.lf[f * NP + ci] : o.lEf[f * NE + ci];
-        const int f2 = 1 - f;
-        const double fcp = cb < 2 ? o.lf[f2 * NP + ci] : o.lEf[f2 * NE + ci];
-        double vm = 0.0, vp = 0.0;
-        if (rb < 2 && cb < 2) {
-          vm = Am[f][rb][cb];
-          vp = Ap[f][rb][cb];
-        } else if (rb == 1 && cb == 2) {
-          vm = BEm[f];
-          vp = BEp[f];
-        } else if (rb == 2 && cb == 1) {
-          vm = GVm[f];
-          vp = GVp[f];
-        }
-        dv += fr * fcm * vm;
-        if (nb_e[f] < 0) {
-          dv += fr * fcm * vp;  // ghost depends on this element's own trace
-        } else if (f == 0) {
-          lv += fr * fcp * vp;
-        } else {
-          uv += fr * fcp * vp;
-        }
-      }
-      Dm[r * NB + c] = dv;
-      Lm[r * NB + c] = lv;
-      Um[r * NB + c] = uv;
+      const double lo = cb < 2 ? o.lf[f * NP + ci] : o.lEf[f * NE + ci];
+      const double lx = cb < 2 ? o.lf[(1 - f) * NP + ci] : o.lEf[(1 - f) * NE + ci];
+      D[c] += (end ? vo[cb] + vx[cb] : vo[cb]) * lo;
+      N[c] = end ? 0.0 : vx[cb] * lx;
     }
   }
-  return nrm;
+#pragma unroll
+  for (int c = 0; c < NB; ++c) Dm[c] = D[c];
+  a.R[(size_t)e * NB + r] = res;
+  return res;
 }
 
-// Block Thomas elimination with one warp: lane c owns column c of the
-// augmented block [A | U_e | b] (2 NB + 1 <= 32 columns); Gauss-Jordan with
-// partial pivoting by shuffles.  Solves J dx = -R; writes dx to a.DX.
-template <int NB>
-__device__ void thomas_warp(int K, const ImplArgs& a) {
-  const int lane = threadIdx.x & 31;
-  double col[NB];
+// ------------------------------------------------------------------ block cyclic reduction
+
+// Block-tridiagonal system in T: blocks D, L, U [K][NB][NB] and right-hand side
+// b [K][NB], overwritten; solution x.  Cyclic reduction: at stride s the rows
+// i = s - 1, 3 s - 1, .. of those left are eliminated (P = D^-1 L, Q = D^-1 U,
+// r = D^-1 b replace L, U, b) and the rows between them updated, so a solve is
+// log2 K elimination steps deep instead of K; a row's elimination is a
+// Gauss-Jordan with partial pivoting of [D | L | U | b] by one warp, a column
+// per lane (two per lane beyond 32 columns).
+template <typename T>
+struct BTri {
+  T *D, *L, *U, *b;
+  int K;
+};
+
+template <typename T, int NB>
+struct BCols {
+  static constexpr int N = 3 * NB + 1, NC = (N + 31) / 32;
+};
+
+// Gauss-Jordan of the warp's columns; columns 0 .. NB - 1 become the identity.
+template <typename T, int NB>
+__device__ __forceinline__ void gauss_jordan(T (&col)[BCols<T, NB>::NC][NB]) {
+  constexpr int NC = BCols<T, NB>::NC;
 #pragma unroll
-  for (int r = 0; r < NB; ++r) col[r] = 0.0;
-  for (int e = 0; e < K; ++e) {
-    const double* D = a.D + (size_t)e * NB * NB;
-    const double* L = a.L + (size_t)e * NB * NB;
-    const double* U = a.U + (size_t)e * NB * NB;
-    // previous W_{e-1} column (lane NB + c) for lanes c < NB; y_{e-1} stays on lane 2 NB
-    double prev[NB];
+  for (int k = 0; k < NB; ++k) {
+    int piv = k;
+    T best = fabs(col[0][k]);
 #pragma unroll
-    for (int j = 0; j < NB; ++j) prev[j] = __shfl_sync(0xffffffffu, col[j], lane < NB ? NB + lane : lane);
-    double nc[NB];
-#pragma unroll
-    for (int r = 0; r < NB; ++r) {
-      double v = 0.0;
-      if (lane < NB) v = D[r * NB + lane];
-      else if (lane < 2 * NB) v = U[r * NB + (lane - NB)];
-      else if (lane == 2 * NB) v = -a.R[(size_t)e * NB + r];
-      if (e > 0 && (lane < NB || lane == 2 * NB)) {
-        double s = 0.0;
-#pragma unroll
-        for (int j = 0; j < NB; ++j) s += L[r * NB + j] * prev[j];
-        v -= s;
+    for (int r = k + 1; r < NB; ++r) {
+      const T v = fabs(col[0][r]);
+      if (less_pos<T>(best, v)) {
+        best = v;
+        piv = r;
       }
-      nc[r] = v;
     }
+    piv = __shfl_sync(0xffffffffu, piv, k);
 #pragma unroll
-    for (int r = 0; r < NB; ++r) col[r] = nc[r];
-    // Gauss-Jordan on the augmented block
-#pragma unroll
-    for (int k = 0; k < NB; ++k) {
-      int piv = k;
-      double best = fabs(col[k]);
-#pragma unroll
-      for (int r = k + 1; r < NB; ++r)
-        if (fabs(col[r]) > best) {
-          best = fabs(col[r]);
-          piv = r;
-        }
-      piv = __shfl_sync(0xffffffffu, piv, k);
+    for (int c = 0; c < NC; ++c) {
 #pragma unroll
       for (int r = k + 1; r < NB; ++r)
         if (r == piv) {
-          const double t = col[k];
-          col[k] = col[r];
-          col[r] = t;
+          const T t = col[c][k];
+          col[c][k] = col[c][r];
+          col[c][r] = t;
         }
-      const double pv = __shfl_sync(0xffffffffu, col[k], k);
-      col[k] = col[k] / pv;
+    }
+    T f[NB];
+#pragma unroll
+    for (int r = 0; r < NB; ++r) f[r] = __shfl_sync(0xffffffffu, col[0][r], k);
+    const T inv = rcp_any(f[k]);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      col[c][k] *= inv;
+#pragma unroll
+      for (int r = 0; r < NB; ++r)
+        if (r != k) col[c][r] -= f[r] * col[c][k];
+    }
+  }
+}
+
+// Row i: update by its eliminated neighbours i - s, i + s (s = 0: none), then,
+// if elim, elimination.
+template <typename T, int NB>
+__device__ void bcr_row(const BTri<T>& A, int i, int s, bool elim, int lane) {
+  constexpr int NC = BCols<T, NB>::NC, B2 = NB * NB;
+  const int lft = i - s, rgt = i + s;
+  const bool hr = s > 0 && rgt < A.K;
+  T col[NC][NB];
+  T* Di = A.D + (size_t)i * B2;
+  T* Li = A.L + (size_t)i * B2;
+  T* Ui = A.U + (size_t)i * B2;
+#pragma unroll
+  for (int cc = 0; cc < NC; ++cc) {
+    const int c = lane + 32 * cc, kind = c < NB ? 0 : c < 2 * NB ? 1 : c < 3 * NB ? 2 : 3, j = c - kind * NB;
+    const bool in = c < 3 * NB + 1;
+    // base column, and the neighbours' columns that L_i and U_i multiply
+    const T* base = kind == 0 ? Di + j : kind == 1 ? Li + j : kind == 2 ? Ui + j : A.b + (size_t)i * NB;
+    const int st = kind == 3 ? 1 : NB;
+    const bool keep = s == 0 || kind == 0 || kind == 3;
+#pragma unroll
+    for (int r = 0; r < NB; ++r) col[cc][r] = in && keep ? base[r * st] : T(0);
+    if (s > 0) {
+      T v[NB], w[NB];
+      const T* vp = kind == 0 ? A.U + (size_t)lft * B2 + j : kind == 1 ? A.L + (size_t)lft * B2 + j : A.b + (size_t)lft * NB;
+      const T* wp = kind == 0 ? A.L + (size_t)rgt * B2 + j : kind == 2 ? A.U + (size_t)rgt * B2 + j : A.b + (size_t)rgt * NB;
+      const bool hv = in && kind != 2, hw = in && hr && kind != 1;
+#pragma unroll
+      for (int m = 0; m < NB; ++m) {
+        v[m] = hv ? vp[m * st] : T(0);
+        w[m] = hw ? wp[m * st] : T(0);
+      }
 #pragma unroll
       for (int r = 0; r < NB; ++r) {
-        if (r == k) continue;
-        const double fct = __shfl_sync(0xffffffffu, col[r], k);
-        col[r] -= fct * col[k];
-      }
-    }
-    // store W_e (lanes NB..2NB-1, column-major) and y_e (lane 2NB)
-    if (lane >= NB && lane <= 2 * NB) {
-      double* dst = lane < 2 * NB ? a.W + (size_t)e * NB * NB + (size_t)(lane - NB) * NB : a.Y + (size_t)e * NB;
+        T t = col[cc][r];
 #pragma unroll
-      for (int r = 0; r < NB; ++r) dst[r] = col[r];
+        for (int m = 0; m < NB; ++m) t -= Li[r * NB + m] * v[m];
+        if (hr) {
+#pragma unroll
+          for (int m = 0; m < NB; ++m) t -= Ui[r * NB + m] * w[m];
+        }
+        col[cc][r] = t;
+      }
     }
   }
-  __syncwarp();
-  // back substitution: dx_{K-1} = y_{K-1}; dx_e = y_e - W_e dx_{e+1}
-  double nxt[NB];
+  __syncwarp();  // every lane has read the row's blocks
+  if (elim) gauss_jordan<T, NB>(col);
 #pragma unroll
-  for (int r = 0; r < NB; ++r) nxt[r] = 0.0;
-  for (int e = K - 1; e >= 0; --e) {
-    double v = 0.0;
-    if (lane < NB) {
-      v = a.Y[(size_t)e * NB + lane];
-      if (e < K - 1) {
-        const double* W = a.W + (size_t)e * NB * NB;
+  for (int cc = 0; cc < NC; ++cc) {
+    const int c = lane + 32 * cc, kind = c < NB ? 0 : c < 2 * NB ? 1 : c < 3 * NB ? 2 : 3, j = c - kind * NB;
+    if (c >= 3 * NB + 1 || (elim && kind == 0)) continue;
+    T* dst = kind == 0 ? Di + j : kind == 1 ? Li + j : kind == 2 ? Ui + j : A.b + (size_t)i * NB;
+    const int st = kind == 3 ? 1 : NB;
 #pragma unroll
-        for (int j = 0; j < NB; ++j) v -= W[j * NB + lane] * nxt[j];
-      }
-      a.DX[(size_t)e * NB + lane] = v;
-    }
-#pragma unroll
-    for (int j = 0; j < NB; ++j) nxt[j] = __shfl_sync(0xffffffffu, v, j);
+    for (int r = 0; r < NB; ++r) dst[r * st] = col[cc][r];
   }
 }
 
-// Mixed-precision block Thomas, factorization (one warp): lane c owns
-// column c of [A_e | U_e | I] in FP32 (3 NB <= 32 columns) with
-// A_e = D_e - L_e W_{e-1}; Gauss-Jordan leaves W_e = A_e^-1 U_e on lanes
-// NB..2NB-1 and A_e^-1 on lanes 2NB..3NB-1, both stored.
-template <int NB>
-__device__ void thomas_factor_f32(int K, const ImplArgs& a) {
-  const int lane = threadIdx.x & 31;
-  float col[NB];
+// x of the system; all threads of the cluster (blocks, b written and ordered
+// before the call; x is ordered for all threads after it).
+template <typename T, int NB>
+__device__ void bcr_solve(const BTri<T>& A, T* x, const Team& t) {
+  const int K = A.K;
+  // stride s: the rows left are s - 1, 2 s - 1, ..; n of them.  A row left at
+  // stride s was updated by those eliminated at s / 2.
+  int s = 1;
+  for (;; s *= 2) {
+    const int n = K / s;
+    for (int k = t.warp; k < n; k += t.warps)
+      if ((k & 1) == 0 || s > 1) bcr_row<T, NB>(A, (k + 1) * s - 1, s / 2, (k & 1) == 0, t.lane);
+    cluster_sync();
+    if (n <= 1) break;
+  }
+  // back: rows eliminated at stride s, whose neighbours at distance s are known
+  for (; s >= 1; s /= 2) {
+    const int n = (K / s + 1) / 2 * NB;  // eliminated rows times unknowns
+    for (int k = t.tid; k < n; k += t.threads) {
+      const int i = (2 * (k / NB) + 1) * s - 1, r = k % NB;
+      T v = A.b[(size_t)i * NB + r];
+      const T* Pm = A.L + ((size_t)i * NB + r) * NB;
+      const T* Qm = A.U + ((size_t)i * NB + r) * NB;
+      if (i - s >= 0) {
 #pragma unroll
-  for (int r = 0; r < NB; ++r) col[r] = 0.f;
-  for (int e = 0; e < K; ++e) {
-    const double* D = a.D + (size_t)e * NB * NB;
-    const double* L = a.L + (size_t)e * NB * NB;
-    const double* U = a.U + (size_t)e * NB * NB;
-    float prev[NB];
-#pragma unroll
-    for (int j = 0; j < NB; ++j) prev[j] = __shfl_sync(0xffffffffu, col[j], lane < NB ? NB + lane : lane);
-#pragma unroll
-    for (int r = 0; r < NB; ++r) {
-      float v = 0.f;
-      if (lane < NB) {
-        v = (float)D[r * NB + lane];
-        if (e > 0) {
-          float sacc = 0.f;
-#pragma unroll
-          for (int j = 0; j < NB; ++j) sacc += (float)L[r * NB + j] * prev[j];
-          v -= sacc;
-        }
-      } else if (lane < 2 * NB) {
-        v = (float)U[r * NB + (lane - NB)];
-      } else if (lane < 3 * NB) {
-        v = (r == lane - 2 * NB) ? 1.f : 0.f;
+        for (int m = 0; m < NB; ++m) v -= Pm[m] * x[(size_t)(i - s) * NB + m];
       }
-      col[r] = v;
-    }
+      if (i + s < K) {
 #pragma unroll
-    for (int k = 0; k < NB; ++k) {
-      int piv = k;
-      float best = fabsf(col[k]);
-#pragma unroll
-      for (int r = k + 1; r < NB; ++r)
-        if (fabsf(col[r]) > best) {
-          best = fabsf(col[r]);
-          piv = r;
-        }
-      piv = __shfl_sync(0xffffffffu, piv, k);
-#pragma unroll
-      for (int r = k + 1; r < NB; ++r)
-        if (r == piv) {
-          const float t = col[k];
-          col[k] = col[r];
-          col[r] = t;
-        }
-      const float pv = __shfl_sync(0xffffffffu, col[k], k);
-      col[k] = col[k] / pv;
-#pragma unroll
-      for (int r = 0; r < NB; ++r) {
-        if (r == k) continue;
-        const float fct = __shfl_sync(0xffffffffu, col[r], k);
-        col[r] -= fct * col[k];
+        for (int m = 0; m < NB; ++m) v -= Qm[m] * x[(size_t)(i + s) * NB + m];
       }
+      x[(size_t)i * NB + r] = v;
     }
-    if (lane >= NB && lane < 3 * NB) {
-      float* dst = lane < 2 * NB ? a.Wf + ((size_t)e * NB + (lane - NB)) * NB
-                                 : a.Af + ((size_t)e * NB + (lane - 2 * NB)) * NB;
-#pragma unroll
-      for (int r = 0; r < NB; ++r) dst[r] = col[r];  // column-major blocks
-    }
+    cluster_sync();
   }
 }
 
-// Solve J x = b with the stored FP32 factors (one warp; lane r < NB owns row
-// r): forward y_e = A_e^-1 (b_e - L_e y_{e-1}), back x_e = y_e - W_e x_{e+1}.
-// b and x are FP64 arrays [K][NB]; y is kept in a.Y.
+// FP64 residual of the linear system, r = -R - J dx (block tridiagonal).
 template <int NB>
-__device__ void thomas_apply_f32(int K, const ImplArgs& a, const double* b, double* x) {
-  const int lane = threadIdx.x & 31;
-  float yp[NB];
-#pragma unroll
-  for (int j = 0; j < NB; ++j) yp[j] = 0.f;
-  for (int e = 0; e < K; ++e) {
-    float t = 0.f;
-    if (lane < NB) {
-      t = (float)b[(size_t)e * NB + lane];
-      if (e > 0) {
-        const double* L = a.L + (size_t)e * NB * NB + (size_t)lane * NB;
-#pragma unroll
-        for (int j = 0; j < NB; ++j) t -= (float)L[j] * yp[j];
-      }
-    }
-    float tt[NB];
-#pragma unroll
-    for (int j = 0; j < NB; ++j) tt[j] = __shfl_sync(0xffffffffu, t, j);
-    float y = 0.f;
-    if (lane < NB) {
-      const float* Ai = a.Af + (size_t)e * NB * NB;
-#pragma unroll
-      for (int j = 0; j < NB; ++j) y += Ai[j * NB + lane] * tt[j];
-      a.Y[(size_t)e * NB + lane] = (double)y;
-    }
-#pragma unroll
-    for (int j = 0; j < NB; ++j) yp[j] = __shfl_sync(0xffffffffu, y, j);
-  }
-  __syncwarp();
-  float nx[NB];
-#pragma unroll
-  for (int j = 0; j < NB; ++j) nx[j] = 0.f;
-  for (int e = K - 1; e >= 0; --e) {
-    float v = 0.f;
-    if (lane < NB) {
-      v = (float)a.Y[(size_t)e * NB + lane];
-      if (e < K - 1) {
-        const float* Wm = a.Wf + (size_t)e * NB * NB;
-#pragma unroll
-        for (int j = 0; j < NB; ++j) v -= Wm[j * NB + lane] * nx[j];
-      }
-      x[(size_t)e * NB + lane] = (double)v;
-    }
-#pragma unroll
-    for (int j = 0; j < NB; ++j) nx[j] = __shfl_sync(0xffffffffu, v, j);
-  }
-}
-
-// FP64 residual of the linear system, r = -R - J dx (block tridiagonal), all threads.
-template <int NB>
-__device__ void linear_residual_f64(int K, const ImplArgs& a) {
-  for (int i = threadIdx.x; i < K * NB; i += blockDim.x) {
+__device__ void linear_residual_f64(const ImplArgs& a, const Team& t) {
+  for (int i = t.tid; i < a.K * NB; i += t.threads) {
     const int e = i / NB, r = i - e * NB;
     double v = -a.R[i];
     const double* D = a.D + (size_t)e * NB * NB + (size_t)r * NB;
@@ -585,7 +530,7 @@ __device__ void linear_residual_f64(int K, const ImplArgs& a) {
 #pragma unroll
       for (int j = 0; j < NB; ++j) v -= L[j] * x[j - NB];
     }
-    if (e < K - 1) {
+    if (e < a.K - 1) {
       const double* U = a.U + (size_t)e * NB * NB + (size_t)r * NB;
 #pragma unroll
       for (int j = 0; j < NB; ++j) v -= U[j] * x[j + NB];
@@ -594,23 +539,49 @@ __device__ void linear_residual_f64(int K, const ImplArgs& a) {
   }
 }
 
+// FP32 block factorization and solve of J x = b (b in FP64), on float copies of
+// the blocks.
+template <int NB>
+__device__ void solve_f32(const ImplArgs& a, const double* b, float* x, const Team& t) {
+  const BTri<float> A{a.Df, a.Lf, a.Uf, a.bf, a.K};
+  for (int i = t.tid; i < a.K * NB * NB; i += t.threads) {
+    a.Df[i] = (float)a.D[i];
+    a.Lf[i] = (float)a.L[i];
+    a.Uf[i] = (float)a.U[i];
+    if (i < a.K * NB) a.bf[i] = (float)b[i];
+  }
+  cluster_sync();
+  bcr_solve<float, NB>(A, x, t);
+}
+
 constexpr int kRefinements = 2;
 
 // Newton iteration for one time level (and one continuation stage): returns
 // the iteration count, whether it converged and max |x|.
 template <int P, int M3>
-__device__ void newton_solve(const ImplArgs& a, const ImplOps<P, M3>& o, double* sred, int& its_out,
+__device__ void newton_solve(const ImplArgs& a, const ImplOps<P, M3>& o, Team& t, double* sred, int& its_out,
                              bool& conv_out, double& xmax_out) {
   using S = IS<P, M3>;
-  constexpr int NB = S::NB;
+  constexpr int NB = S::NB, NQ = S::NQ;
   const int K = a.K;
   double r0 = 0.0, dxmax = 0.0, xmax = 0.0;
   int its = 0;
   bool conv = false;
   for (int it = 0;; ++it) {
+    // faces first (the longer items), volume points after them
+    for (int i = t.tid; i < K + 1 + K * NQ; i += t.threads) {
+      if (i <= K) face_data<P, M3>(i, a, o);
+      else volume_point<P, M3>(i - K - 1, a, o);
+    }
+    cluster_sync();
     double part = 0.0;
-    for (int e = threadIdx.x; e < K; e += blockDim.x) part += assemble<P, M3>(e, a, o);
-    const double rn = sqrt(block_sum(part, sred));
+    for (int i = t.tid; i < K * NB; i += t.threads) {
+      const int r = i / K, e = i - r * K;  // a warp's rows are of one kind
+      const double v = assemble_row<P, M3>(e, r, a, o);
+      part += v * v;
+      (a.mixed ? a.Rr : a.Y)[(size_t)e * NB + r] = -v;
+    }
+    const double rn = sqrt(team_reduce<false>(part, t, sred));
     if (it == 0) {
       r0 = rn;
       if (rn <= a.atol) {
@@ -627,79 +598,77 @@ __device__ void newton_solve(const ImplArgs& a, const ImplOps<P, M3>& o, double*
       its = it;
       break;
     }
-    __syncthreads();
-    if constexpr (3 * NB <= 32) {
-      if (a.mixed) {
-        // -R into Rr, FP32 factor + solve, then FP64 residual / correction rounds
-        for (int i = threadIdx.x; i < K * NB; i += blockDim.x) a.Rr[i] = -a.R[i];
-        __syncthreads();
-        if (threadIdx.x < 32) {
-          thomas_factor_f32<NB>(K, a);
-          __syncwarp();
-          thomas_apply_f32<NB>(K, a, a.Rr, a.DX);
-        }
-        __syncthreads();
-        for (int ref = 0; ref < kRefinements; ++ref) {
-          linear_residual_f64<NB>(K, a);
-          __syncthreads();
-          if (threadIdx.x < 32) thomas_apply_f32<NB>(K, a, a.Rr, a.Dx2);
-          __syncthreads();
-          for (int i = threadIdx.x; i < K * NB; i += blockDim.x) a.DX[i] += a.Dx2[i];
-          __syncthreads();
-        }
-      } else {
-        if (threadIdx.x < 32) thomas_warp<NB>(K, a);
-        __syncthreads();
+    double dm = 0.0, xm = 0.0;
+    if (a.mixed) {
+      // FP32 factorization and solve, then rounds of FP64 residual and FP32 correction
+      solve_f32<NB>(a, a.Rr, a.xf, t);
+      for (int i = t.tid; i < K * NB; i += t.threads) a.DX[i] = (double)a.xf[i];
+      cluster_sync();
+      for (int ref = 0; ref < kRefinements; ++ref) {
+        linear_residual_f64<NB>(a, t);
+        cluster_sync();
+        solve_f32<NB>(a, a.Rr, a.xf, t);
+        for (int i = t.tid; i < K * NB; i += t.threads) a.DX[i] += (double)a.xf[i];
+        cluster_sync();
       }
     } else {
-      if (threadIdx.x < 32) thomas_warp<NB>(K, a);
-      __syncthreads();
+      bcr_solve<double, NB>(BTri<double>{a.D, a.L, a.U, a.Y, K}, a.DX, t);
     }
-    double dm = 0.0, xm = 0.0;
-    for (int i = threadIdx.x; i < K * NB; i += blockDim.x) {
+    for (int i = t.tid; i < K * NB; i += t.threads) {
       const double d = a.DX[i];
       const double xn = a.X[i] + d;
       a.X[i] = xn;
       dm = fmax(dm, fabs(d));
       xm = fmax(xm, fabs(xn));
     }
-    dxmax = block_max(dm, sred);
-    xmax = block_max(xm, sred);
-    __syncthreads();
+    dxmax = team_reduce<true>(dm, t, sred);
+    xmax = team_reduce<true>(xm, t, sred);
   }
-  __syncthreads();
   its_out = its;
   conv_out = conv;
   xmax_out = xmax;
 }
 
 template <int P, int M3>
-__global__ void __launch_bounds__(256) implicit_kernel(ImplArgs a, ImplOps<P, M3> o, long long n_steps) {
+__global__ void __launch_bounds__(kThreads) implicit_kernel(ImplArgs a, ImplOps<P, M3> o, long long n_steps) {
   using S = IS<P, M3>;
   constexpr int NP = S::NP, NB = S::NB, NQ = S::NQ;
-  __shared__ double sred[32];
+  __shared__ double sred[kWarps];
   const int K = a.K;
+  Team t;
+  t.rank = cluster_rank();
+  t.size = cluster_size();
+  // consecutive warps of items go to different blocks, then to different sub-partitions
+  t.lane = threadIdx.x & 31;
+  t.warp = (threadIdx.x >> 5) * t.size + t.rank;
+  t.warps = kWarps * t.size;
+  t.tid = t.warp * 32 + t.lane;
+  t.threads = t.warps * 32;
+  t.red = a.red;
+  t.slot = 0;
   for (long long step = 0; step < n_steps; ++step) {
     // <N_V, U(V^{k-1})>
-    for (int e = threadIdx.x; e < K; e += blockDim.x) {
+    for (int i = t.tid; i < K * NP; i += t.threads) {
+      const int e = i / NP, k = i - e * NP;
       const double* x = a.X + (size_t)e * NB;
       const double J = a.J[e];
-      for (int i = 0; i < NP; ++i) {
-        double s0 = 0, s1 = 0;
-        for (int q = 0; q < NQ; ++q) {
-          double hh = 0, uu = 0;
-          for (int j = 0; j < NP; ++j) {
-            hh += o.Vq[q * NP + j] * x[j];
-            uu += o.Vq[q * NP + j] * x[NP + j];
-          }
-          s0 += o.wq[q] * J * o.Vq[q * NP + i] * hh;
-          s1 += o.wq[q] * J * o.Vq[q * NP + i] * hh * uu;
+      double s0 = 0, s1 = 0;
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        double hh = 0, uu = 0;
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+          hh += o.Vq[q * NP + j] * x[j];
+          uu += o.Vq[q * NP + j] * x[NP + j];
         }
-        a.Uold[(size_t)e * 2 * NP + i] = s0;
-        a.Uold[(size_t)e * 2 * NP + NP + i] = s1;
+        const double w = o.wq[q] * J * o.Vq[q * NP + k];
+        s0 += w * hh;
+        s1 += w * (hh * uu);
       }
+      a.Uold[(size_t)e * 2 * NP + k] = s0;
+      a.Uold[(size_t)e * 2 * NP + NP + k] = s1;
     }
-    __syncthreads();
+    // (Uold is read after the first barrier of newton_solve)
     // continuation in gamma (Sec. 6.3): gamma_i = gamma0 + (i-1)(gamma-gamma0)/(n_gamma-1)
     const int ng = a.n_gamma > 1 ? a.n_gamma : 1;
     int its = 0;
@@ -710,11 +679,11 @@ __global__ void __launch_bounds__(256) implicit_kernel(ImplArgs a, ImplOps<P, M3
       if (ng > 1) b.gamma = a.gamma0 + ic * (a.gamma - a.gamma0) / (ng - 1);
       int it_s;
       bool cv_s;
-      newton_solve<P, M3>(b, o, sred, it_s, cv_s, xmax);
+      newton_solve<P, M3>(b, o, t, sred, it_s, cv_s, xmax);
       its += it_s;
       conv = conv && cv_s;
     }
-    if (threadIdx.x == 0) {
+    if (t.tid == 0) {
       dg_implicit_stats& st = *a.st;
       st.steps += 1;
       st.t += a.dt;
@@ -724,7 +693,7 @@ __global__ void __launch_bounds__(256) implicit_kernel(ImplArgs a, ImplOps<P, M3
       if (!(xmax == xmax)) st.status = DG_ERR_NONFINITE;
       else if (!conv && !a.on_fail_continue) st.status = DG_ERR_NEWTON;
     }
-    __syncthreads();
+    cluster_sync();
     if (a.st->status != 0) break;
   }
 }
@@ -833,7 +802,7 @@ struct dg_implicit {
   size_t ws_need = 0;
   char* ws = nullptr;
   struct {
-    size_t X, Uold, R, D, L, U, W, Y, DX, J, bed, red, st, MEinv, act, Wf, Af, Rr, Dx2;
+    size_t X, Uold, R, D, L, U, Y, DX, J, bed, red, st, MEinv, act, pt, fc, Df, Lf, Uf, bf, xf, Rr;
   } off{};
   cudaStream_t stream = nullptr;
   std::unique_ptr<ImplDrv> drv;
@@ -879,10 +848,14 @@ ImplArgs make_args(dg_implicit* s) {
   a.mixed = s->ip.linear_solver == 1 ? 1 : 0;
   a.n_gamma = s->ip.n_gamma;
   a.gamma0 = s->ip.gamma0;
-  a.Wf = s->at<float>(s->off.Wf);
-  a.Af = s->at<float>(s->off.Af);
+  a.Df = s->at<float>(s->off.Df);
+  a.Lf = s->at<float>(s->off.Lf);
+  a.Uf = s->at<float>(s->off.Uf);
+  a.bf = s->at<float>(s->off.bf);
+  a.xf = s->at<float>(s->off.xf);
   a.Rr = s->at<double>(s->off.Rr);
-  a.Dx2 = s->at<double>(s->off.Dx2);
+  a.pt = s->at<double>(s->off.pt);
+  a.fc = s->at<double>(s->off.fc);
   a.bcL = s->bcL;
   a.bcR = s->bcR;
   a.X = s->at<double>(s->off.X);
@@ -891,7 +864,6 @@ ImplArgs make_args(dg_implicit* s) {
   a.D = s->at<double>(s->off.D);
   a.L = s->at<double>(s->off.L);
   a.U = s->at<double>(s->off.U);
-  a.W = s->at<double>(s->off.W);
   a.Y = s->at<double>(s->off.Y);
   a.DX = s->at<double>(s->off.DX);
   a.J = s->at<double>(s->off.J);
@@ -919,7 +891,19 @@ struct IDrv final : ImplDrv {
     for (int i = 0; i < 2 * S::NE; ++i) o.lEf[i] = s.lEf[i];
   }
   void run(dg_implicit* s, long long n, cudaStream_t st) override {
-    implicit_kernel<P, M3><<<1, 256, 0, st>>>(make_args(s), o, n);
+    // one cluster: eight blocks from 12 elements on, where the phases have work
+    // for several warps; below, one block and its cheaper barrier
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = s->K >= 12 ? kMaxCluster : 1;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(at.val.clusterDim.x);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, implicit_kernel<P, M3>, make_args(s), o, n);
   }
   void init_E(dg_implicit* s, cudaStream_t st) override {
     const int K = (int)s->K;
@@ -1118,7 +1102,6 @@ dg_status dg_implicit_init(const dg_swe_mesh* mesh, int order, int regularizatio
   s->off.D = take(K * NB * NB * 8);
   s->off.L = take(K * NB * NB * 8);
   s->off.U = take(K * NB * NB * 8);
-  s->off.W = take(K * NB * NB * 8);
   s->off.Y = take(K * NB * 8);
   s->off.DX = take(K * NB * 8);
   s->off.J = take(K * 8);
@@ -1127,10 +1110,15 @@ dg_status dg_implicit_init(const dg_swe_mesh* mesh, int order, int regularizatio
   s->off.st = take(sizeof(dg_implicit_stats));
   s->off.MEinv = take(NE * NE * 8);
   s->off.act = take(8);
-  s->off.Wf = take(K * NB * NB * 4);
-  s->off.Af = take(K * NB * NB * 4);
-  s->off.Rr = take(K * NB * 8);
-  s->off.Dx2 = take(K * NB * 8);
+  s->off.pt = take(K * NQ * kPt * 8);
+  s->off.fc = take((K + 1) * kFc * 8);
+  const size_t mixed = s->ip.linear_solver == 1 ? 1 : 0;
+  s->off.Df = take(mixed * K * NB * NB * 4);
+  s->off.Lf = take(mixed * K * NB * NB * 4);
+  s->off.Uf = take(mixed * K * NB * NB * 4);
+  s->off.bf = take(mixed * K * NB * 4);
+  s->off.xf = take(mixed * K * NB * 4);
+  s->off.Rr = take(mixed * K * NB * 8);
   s->ws_need = off;
   *out = s.release();
   return DG_OK;
