@@ -349,8 +349,8 @@ struct GDrv final : GroupDrv {
                                                     b->at<int32_t>(g.off.blk_gid), b->at<R>(g.off.V[0]),
                                                     b->at<R>(g.off.geo), b->at<double>(b->off_iparm),
                                                     b->at<double>(g.off.partial));
-    dt_members_kernel<<<(nm + 7) / 8, 256, 0, s>>>(nm, b->at<int32_t>(g.off.mblk), b->at<int32_t>(g.off.gid),
-                                                   b->at<double>(g.off.partial), b->at<DevScalars>(b->off_sc));
+    dt_members_kernel<<<nm, 256, 0, s>>>(b->at<int32_t>(g.off.mblk), b->at<int32_t>(g.off.gid),
+                                         b->at<double>(g.off.partial), b->at<DevScalars>(b->off_sc));
   }
   void mass(dg_batch* b, Group& g, int first, int count, int set_ref, cudaStream_t s) override {
     if (count <= 0) return;

@@ -108,6 +108,9 @@ __device__ __forceinline__ double block_sum(double v, double* sred) {
 // of its lanes are active (measured 64-72), so the independent pieces of a
 // Newton iteration are spread over the cluster's sub-partitions, and phases are
 // separated by the cluster barrier (about 360 clocks, five FP64 instructions).
+// 100 elements, p = 1, constant E, 3 Newton iterations a step: 2513 -> 265 us a
+// step (one block with a one-warp block Thomas sweep before); FP32 elimination
+// 1773 -> 330 us; p = 2, m3 = 2: 13.8 -> 1.1 ms; 400 elements: 33.3 -> 1.5 ms.
 
 constexpr int kThreads = 256, kWarps = kThreads / 32, kMaxCluster = 8;
 

@@ -1922,49 +1922,138 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Per-element stable step (see dg_swe_step), block minimum to partial[block].
-// A non-finite state sets partial to -1 (flag).
-template <int DIM, int P, typename R>
-__global__ void __launch_bounds__(256) dt_partial_kernel(int K, const R* __restrict__ V, const R* __restrict__ geo,
-                                                         double gc, double h_floor, double cfl, double nu,
-                                                         double* __restrict__ partial) {
-  constexpr int NP = Sh<DIM, P>::NP;
-  __shared__ double red[8];
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  double dte = 1e300;
-  if (e < K) {
-    const size_t KN = (size_t)K * NP;
-    // wave speeds in the state's precision, step and reduction in FP64
-    R lam = R(0);
-    bool bad = false;
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      const R h = V[(size_t)e * NP + a];
-      R sp2 = R(0);
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) {
-        const R u = V[(1 + j) * KN + (size_t)e * NP + a];
-        sp2 += u * u;
-      }
-      const R l = sqrt(sp2) + sqrt((R)gc * fmax(h, (R)h_floor));
-      if (!isfinite(l) || !isfinite(h)) bad = true;
-      lam = fmax(lam, l);
-    }
-    // per-element bound in the state's precision; min and time sum in FP64
-    const R dx = geo[5 * K + e];
-    const R qq = R(2 * P + 1);
-    dte = (double)((R)cfl * dx / (qq * lam + qq * qq * R(2) * (R)nu / dx));
-    if (bad) dte = -1.0;
-  }
-  double v = warp_min(dte);
+// Minimum over a warp of values that are positive or exactly -1 (a flag, the
+// smallest): such values order as their bits, so the reduction runs on the
+// integer pipe (redux) instead of five FP64 minima of 64 clocks each.
+__device__ __forceinline__ float warp_min_flag(float v) {
+  return __int_as_float(__reduce_min_sync(0xffffffffu, __float_as_int(v)));
+}
+__device__ __forceinline__ double warp_min_flag(double v) {
+  const int hi = __reduce_min_sync(0xffffffffu, __double2hiint(v));
+  const unsigned lo = __double2hiint(v) == hi ? (unsigned)__double2loint(v) : 0xffffffffu;
+  return __hiloint2double(hi, (int)__reduce_min_sync(0xffffffffu, lo));
+}
+template <typename R>
+__device__ __forceinline__ R min_flag(R x, R y) { return x < y ? x : y; }
+template <>
+__device__ __forceinline__ double min_flag<double>(double x, double y) {
+  return __double_as_longlong(x) < __double_as_longlong(y) ? x : y;
+}
+// Minimum over the block (whole warps), valid in thread 0; red: one slot a warp.
+template <typename R>
+__device__ __forceinline__ R block_min_flag(R v, R* red) {
+  v = warp_min_flag(v);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (lane == 0) red[w] = v;
   __syncthreads();
   if (w == 0) {
-    v = lane < (int)(blockDim.x >> 5) ? red[lane] : 1e300;
-    v = warp_min(v);
-    if (lane == 0) partial[blockIdx.x] = v;
+    v = red[lane < (int)(blockDim.x >> 5) ? lane : 0];
+    v = warp_min_flag(v);
   }
+  return v;
+}
+
+// A float near x (FP64: by the integer pipe; 0 or infinity outside the float range).
+__device__ __forceinline__ float near_f32(float x) { return x; }
+__device__ __forceinline__ float near_f32(double x) {
+  const int hi = __double2hiint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  const unsigned m = ((unsigned)(hi & 0x7fffffff) - (896u << 20)) << 3 | (unsigned)__double2loint(x) >> 29;
+  const unsigned b = e <= 896 ? 0u : e >= 1151 ? 0x7f800000u : m;
+  return __uint_as_float(b | ((unsigned)hi & 0x80000000u));
+}
+__device__ __forceinline__ bool not_finite(float x) { return (__float_as_uint(x) & 0x7f800000u) == 0x7f800000u; }
+__device__ __forceinline__ bool not_finite(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
+__device__ __forceinline__ float sqrt_nonneg(float x) { return sqrtf(x); }
+__device__ __forceinline__ double sqrt_nonneg(double x) {
+  return __double_as_longlong(x) == 0 ? 0.0 : sqrt_pos(x);
+}
+
+template <typename R>
+__device__ __forceinline__ R huge_dt() { return sizeof(R) == 8 ? R(1e300) : R(3e38); }
+
+// Stable step of element e (see dg_swe_step), -1 for a non-finite state.  The
+// largest wave speed is found in two steps: fast single-precision speeds at all
+// nodes, then the speed in the state's precision at the nodes within 1e-5 of
+// their largest (usually one), so that the value is that of the plain maximum.
+// With the minimum on the integer pipe: FP64, 524,288 triangles, p = 2 179 -> 77 us
+// (bound by 84 FP64 root and sum instructions an element before); FP32, 2,097,152
+// triangles 81 -> 52 us (ten FP64 minima a warp before).
+template <int DIM, int P, typename R, bool COH = false>
+__device__ __forceinline__ R element_dt(size_t e, int K, const R* __restrict__ V, const R* __restrict__ geo, R gc,
+                                        R h_floor, R cfl, R nu) {
+  constexpr int NP = Sh<DIM, P>::NP;
+  const size_t KN = (size_t)K * NP;
+  R h[NP], u[DIM][NP];
+  float l[NP], top = 0.f;
+  const float gcf = near_f32(gc), hf = near_f32(h_floor);
+  bool bad = false;
+#pragma unroll
+  for (int a = 0; a < NP; ++a) {
+    h[a] = DG_LDC(COH, V, e * NP + a);
+    bad = bad || not_finite(h[a]);
+    float s2 = 0.f;
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) {
+      u[j][a] = DG_LDC(COH, V, (1 + j) * KN + e * NP + a);
+      bad = bad || not_finite(u[j][a]);
+      const float x = near_f32(u[j][a]);
+      s2 += x * x;
+    }
+    l[a] = dg_sqrt<float>(s2) + dg_sqrt<float>(gcf * fmaxf(near_f32(h[a]), hf));
+    top = fmaxf(top, l[a]);
+  }
+  if (bad) return R(-1);
+  const float near_top = top * (1.f - 1e-5f);
+  unsigned cand = 0;
+#pragma unroll
+  for (int a = 0; a < NP; ++a) cand |= l[a] < near_top ? 0u : 1u << a;
+  R lam = R(0);
+  while (cand) {
+    const int c = __ffs(cand) - 1;
+    R hc = h[0], uc[DIM];
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) uc[j] = u[j][0];
+#pragma unroll
+    for (int a = 1; a < NP; ++a)
+      if (a == c) {
+        hc = h[a];
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) uc[j] = u[j][a];
+      }
+    cand &= cand - 1;
+    // nodes equal to this one give the same speed
+#pragma unroll
+    for (int a = 1; a < NP; ++a) {
+      bool same = h[a] == hc;
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) same = same && u[j][a] == uc[j];
+      if (same) cand &= ~(1u << a);
+    }
+    R sp2 = R(0);
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) sp2 += uc[j] * uc[j];
+    const R v = sqrt_nonneg(sp2) + sqrt_nonneg(gc * fmax(hc, h_floor));
+    if (not_finite(v)) return R(-1);
+    lam = fmax(lam, v);
+  }
+  const R dx = geo[5 * (size_t)K + e];
+  const R qq = R(2 * P + 1);
+  return cfl * dx / (qq * lam + qq * qq * R(2) * nu / dx);
+}
+
+// Per-element stable step, block minimum to partial[block] (-1 flags a
+// non-finite state).
+template <int DIM, int P, typename R>
+__global__ void __launch_bounds__(256) dt_partial_kernel(int K, const R* __restrict__ V, const R* __restrict__ geo,
+                                                         double gc, double h_floor, double cfl, double nu,
+                                                         double* __restrict__ partial) {
+  __shared__ R red[8];
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  R dte = huge_dt<R>();
+  if (e < K) dte = element_dt<DIM, P, R>(e, K, V, geo, (R)gc, (R)h_floor, (R)cfl, (R)nu);
+  const R v = block_min_flag(dte, red);
+  if (threadIdx.x == 0) partial[blockIdx.x] = (double)v;
 }
 
 // Final step size: fixed dt (> 0) or min of the partials; advances t and the
@@ -1973,14 +2062,9 @@ static __global__ void dt_finalize_kernel(int nblocks, const double* __restrict_
                                    DevScalars* __restrict__ sc) {
   __shared__ double red[32];
   double v = 1e300;
-  for (int i = threadIdx.x; i < nblocks; i += blockDim.x) v = fmin(v, partial[i]);
-  v = warp_min(v);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) red[w] = v;
-  __syncthreads();
+  for (int i = threadIdx.x; i < nblocks; i += blockDim.x) v = min_flag(v, partial[i]);
+  double m = block_min_flag(v, red);
   if (threadIdx.x == 0) {
-    double m = 1e300;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) m = fmin(m, red[i]);
     if (m < 0.0) {
       sc->status = 4;
       m = 0.0;
@@ -2019,19 +2103,43 @@ __global__ void __launch_bounds__(256) mass_partial_kernel(int K, const R* __res
   }
 }
 
-// Compensated (Kahan) sum of the block partials; which = 0 -> mass, 1 -> mass0 too.
-static __global__ void mass_finalize_kernel(int nblocks, const double* __restrict__ partial, int set_ref,
-                                     DevScalars* __restrict__ sc) {
-  if (threadIdx.x != 0) return;
+// s + e = a + b exactly (Knuth's two-sum).
+__device__ __forceinline__ void two_sum(double a, double b, double& s, double& e) {
+  s = a + b;
+  const double t = s - a;
+  e = (a - (s - t)) + (b - t);
+}
+
+// Compensated sum of the block partials (one block of 256 threads): each thread
+// adds a contiguous share, then the shares are added in a fixed tree; the
+// rounding errors are carried along.  set_ref: mass0 too.  (One thread adding
+// all of them took 70 clocks an addition, four additions a partial.)
+static __global__ void __launch_bounds__(256) mass_finalize_kernel(int nblocks, const double* __restrict__ partial,
+                                                                   int set_ref, DevScalars* __restrict__ sc) {
+  __shared__ double sh[256], sl[256];
+  const int t = threadIdx.x, per = (nblocks + 255) / 256;
   double s = 0.0, c = 0.0;
-  for (int i = 0; i < nblocks; ++i) {
-    double y = partial[i] - c;
-    double t = s + y;
-    c = (t - s) - y;
-    s = t;
+  for (int i = t * per; i < min((t + 1) * per, nblocks); ++i) {
+    double e;
+    two_sum(s, partial[i], s, e);
+    c += e;
   }
-  sc->mass = s;
-  if (set_ref) sc->mass0 = s;
+  sh[t] = s;
+  sl[t] = c;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (t < o && t + o < nblocks) {
+      double e;
+      two_sum(sh[t], sh[t + o], sh[t], e);
+      sl[t] += sl[t + o] + e;
+    }
+    __syncthreads();
+  }
+  if (t == 0) {
+    const double m = sh[0] + sl[0];
+    sc->mass = m;
+    if (set_ref) sc->mass0 = m;
+  }
 }
 
 
@@ -2046,59 +2154,30 @@ __global__ void __launch_bounds__(256) dt_block_kernel(int K, const int64_t* __r
                                                        const R* __restrict__ V, const R* __restrict__ geo,
                                                        const double* __restrict__ iparm,
                                                        double* __restrict__ partial) {
-  constexpr int NP = Sh<DIM, P>::NP;
-  __shared__ double red[8];
+  __shared__ R red[8];
   const int b = blockIdx.x;
   const int g = blk_gid[b];
   const int64_t e = blk_e[b] + threadIdx.x;
-  const double gc = iparm[4 * g + 0], h_floor = iparm[4 * g + 1], cfl = iparm[4 * g + 2], nu = iparm[4 * g + 3];
-  double dte = 1e300;
-  if (e < blk_e[b + 1]) {
-    const size_t KN = (size_t)K * NP;
-    R lam = R(0);
-    bool bad = false;
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      const R h = V[(size_t)e * NP + a];
-      R sp2 = R(0);
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) {
-        const R u = V[(1 + j) * KN + (size_t)e * NP + a];
-        sp2 += u * u;
-      }
-      const R l = sqrt(sp2) + sqrt((R)gc * fmax(h, (R)h_floor));
-      if (!isfinite(l) || !isfinite(h)) bad = true;
-      lam = fmax(lam, l);
-    }
-    // per-element bound in the state's precision; min and time sum in FP64
-    const R dx = geo[5 * K + e];
-    const R qq = R(2 * P + 1);
-    dte = (double)((R)cfl * dx / (qq * lam + qq * qq * R(2) * (R)nu / dx));
-    if (bad) dte = -1.0;
-  }
-  double v = warp_min(dte);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  if (w == 0) {
-    v = lane < (int)(blockDim.x >> 5) ? red[lane] : 1e300;
-    v = warp_min(v);
-    if (lane == 0) partial[b] = v;
-  }
+  R dte = huge_dt<R>();
+  if (e < blk_e[b + 1])
+    dte = element_dt<DIM, P, R>((size_t)e, K, V, geo, (R)iparm[4 * g + 0], (R)iparm[4 * g + 1], (R)iparm[4 * g + 2],
+                                (R)iparm[4 * g + 3]);
+  const R v = block_min_flag(dte, red);
+  if (threadIdx.x == 0) partial[b] = (double)v;
 }
 
-// One warp per instance of a group: minimum of its block partials (exact,
-// so independent of order), then dt, t, step count and dt_min/max.
-static __global__ void dt_members_kernel(int n_members, const int32_t* __restrict__ mblk,
-                                         const int32_t* __restrict__ gid, const double* __restrict__ partial,
-                                         DevScalars* __restrict__ sc) {
-  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (i >= n_members) return;
-  double m = 1e300;
-  for (int b = mblk[i] + lane; b < mblk[i + 1]; b += 32) m = fmin(m, partial[b]);
-  m = warp_min(m);
-  if (lane == 0) {
+// One block per instance of a group: minimum of its block partials (exact, so
+// independent of order), then dt, t, step count and dt_min/max.
+static __global__ void __launch_bounds__(256) dt_members_kernel(const int32_t* __restrict__ mblk,
+                                                                const int32_t* __restrict__ gid,
+                                                                const double* __restrict__ partial,
+                                                                DevScalars* __restrict__ sc) {
+  __shared__ double red[8];
+  const int i = blockIdx.x;
+  double v = 1e300;
+  for (int b = mblk[i] + threadIdx.x; b < mblk[i + 1]; b += blockDim.x) v = min_flag(v, partial[b]);
+  double m = block_min_flag(v, red);
+  if (threadIdx.x == 0) {
     DevScalars& s = sc[gid[i]];
     if (m < 0.0) {
       s.status = 4;

@@ -150,33 +150,14 @@ __global__ void __launch_bounds__(kThreads) step_kernel(const Plan pl, const Arr
     if (ph == 0) {
       // step bound of one 128-element tile (dt_block_kernel's per-element bound)
       const int64_t e = e_lo + (int64_t)t * kThreads + tid;
-      double dte = 1e300;
+      R dte = huge_dt<R>();
       if (e < e_hi) {
         const int g = pl.gid[m];
-        const double gc = A.iparm[4 * g + 0], h_floor = A.iparm[4 * g + 1], cfl = A.iparm[4 * g + 2],
-                     nu = A.iparm[4 * g + 3];
-        R lam = R(0);
-        bool bad = false;
-#pragma unroll
-        for (int a = 0; a < NP; ++a) {
-          const R h = DG_LDC(true, A.V[0], (size_t)e * NP + a);
-          R sp2 = R(0);
-#pragma unroll
-          for (int jj = 0; jj < DIM; ++jj) {
-            const R u = DG_LDC(true, A.V[0], (1 + jj) * KN + (size_t)e * NP + a);
-            sp2 += u * u;
-          }
-          const R l = sqrt(sp2) + sqrt((R)gc * fmax(h, (R)h_floor));
-          if (!isfinite(l) || !isfinite(h)) bad = true;
-          lam = fmax(lam, l);
-        }
-        const R dx = A.geo[5 * K + e];
-        const R qq = R(2 * P + 1);
-        dte = (double)((R)cfl * dx / (qq * lam + qq * qq * R(2) * (R)nu / dx));
-        if (bad) dte = -1.0;
+        dte = element_dt<DIM, P, R, true>((size_t)e, K, A.V[0], A.geo, (R)A.iparm[4 * g + 0], (R)A.iparm[4 * g + 1],
+                                          (R)A.iparm[4 * g + 2], (R)A.iparm[4 * g + 3]);
       }
-      double v = warp_min(dte);
-      if ((tid & 31) == 0) red[tid >> 5] = v;
+      const R v = warp_min_flag(dte);
+      if ((tid & 31) == 0) red[tid >> 5] = (double)v;
       __syncthreads();
       if (tid == 0) {
         double mn = red[0];

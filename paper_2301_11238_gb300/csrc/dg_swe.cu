@@ -235,7 +235,7 @@ void enqueue_step(dg_swe_ctx* c, double fixed_dt, cudaStream_t s) {
 
 void enqueue_mass(dg_swe_ctx* c, int set_ref, cudaStream_t s) {
   c->drv->mass_partial(c, c->ws + c->off.V0, s);
-  mass_finalize_kernel<<<1, 32, 0, s>>>(c->nblk_mass, c->at<double>(c->off.partial), set_ref,
+  mass_finalize_kernel<<<1, 256, 0, s>>>(c->nblk_mass, c->at<double>(c->off.partial), set_ref,
                                         c->at<DevScalars>(c->off.sc));
 }
 
