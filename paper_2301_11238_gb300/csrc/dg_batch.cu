@@ -123,6 +123,9 @@ __global__ void __launch_bounds__(256) mass_block_kernel(int K, int b0, const in
                                                          const R* __restrict__ V, const R* __restrict__ geo,
                                                          const double* __restrict__ wint,
                                                          double* __restrict__ partial) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(V);
   __shared__ double red[8];
   const int b = b0 + blockIdx.x;
   const int64_t e = blk_e[b] + threadIdx.x;
@@ -147,6 +150,9 @@ __global__ void __launch_bounds__(256) mass_block_kernel(int K, int b0, const in
 static __global__ void mass_members_kernel(int first, int count, const int32_t* __restrict__ mblk,
                                            const int32_t* __restrict__ gid, const double* __restrict__ partial,
                                            int set_ref, DevScalars* __restrict__ sc) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(partial);
   const int i = first + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (i >= first + count) return;
@@ -251,13 +257,13 @@ struct GDrv final : GroupDrv {
     if (g.tile[0] < 0) {
       const int T = -g.tile[0];
       const int grid = std::max(1, std::min((K + T - 1) / T, estep_pf_blocks(T)));
-      estep_pf_kernel<DIM, P, R><<<grid, T, 0, s>>>(
+      launch_after(estep_pf_kernel<DIM, P, R>, grid, T, 0, s,
           K, b->at<R>(g.off.V[vin]), b->at<R>(g.off.E), b->at<R>(g.off.geo), b->at<int32_t>(g.off.nbr),
           b->at<int8_t>(g.off.nbrf), b->at<R>(g.off.fn), b->at<R>(g.off.fsj), eo, bct(b));
       return;
     }
     const int T = g.tile[0];
-    estep_kernel<DIM, P, R><<<(K + T - 1) / T, T, 0, s>>>(
+    launch_after(estep_kernel<DIM, P, R>, (K + T - 1) / T, T, 0, s,
         K, b->at<R>(g.off.V[vin]), b->at<R>(g.off.E), b->at<R>(g.off.geo), b->at<int32_t>(g.off.nbr),
         b->at<int8_t>(g.off.nbrf), b->at<R>(g.off.fn), b->at<R>(g.off.fsj), eo, bct(b));
   }
@@ -266,7 +272,7 @@ struct GDrv final : GroupDrv {
     const int K = (int)g.K, F = (int)g.F, T = g.tile[1] > 0 ? g.tile[1] : -g.tile[1];
     if (g.tile[1] > 0) {
       const long long n = (long long)F * S::NFQ;
-      face_kernel<DIM, P, R, true, false><<<(unsigned)((n + T - 1) / T), T, 0, s>>>(
+      launch_after(face_kernel<DIM, P, R, true, false>, (unsigned)((n + T - 1) / T), T, 0, s,
           K, F, b->at<R>(g.off.V[vin]), b->at<R>(g.off.E), b->at<int32_t>(g.off.fe1), b->at<int8_t>(g.off.ff1),
           b->at<int32_t>(g.off.fe2), b->at<int8_t>(g.off.ff2), b->at<R>(g.off.fnrm), b->at<R>(g.off.fsjf),
           b->at<R>(g.off.wflux), fo, Phys<R>{}, ptab(b), b->at<int32_t>(g.off.inst), bct(b));
@@ -274,7 +280,7 @@ struct GDrv final : GroupDrv {
       // one thread per face in a grid-stride loop over the resident blocks
       // (the next face's connectivity loads while the current one computes)
       const int grid = std::max(1, std::min((F + T - 1) / T, face_pf_blocks(T)));
-      face_pf_kernel<DIM, P, R><<<(unsigned)grid, T, 0, s>>>(
+      launch_after(face_pf_kernel<DIM, P, R>, (unsigned)grid, T, 0, s,
           K, F, b->at<R>(g.off.V[vin]), b->at<R>(g.off.E), b->at<int32_t>(g.off.fe1), b->at<int8_t>(g.off.ff1),
           b->at<int32_t>(g.off.fe2), b->at<int8_t>(g.off.ff2), b->at<R>(g.off.fnrm), b->at<R>(g.off.fsjf),
           b->at<R>(g.off.wflux), fo, ptab(b), b->at<int32_t>(g.off.inst), bct(b));
@@ -288,7 +294,7 @@ struct GDrv final : GroupDrv {
       // conservative stage from it
       const int rb = vout != 0 ? vout : 1;
       residual(b, g, vin, rb, s);
-      wetdry_stage_kernel<DIM, P, R, true><<<(K + 127) / 128, 128, 0, s>>>(
+      launch_after(wetdry_stage_kernel<DIM, P, R, true>, (K + 127) / 128, 128, 0, s,
           K, b->at<R>(g.off.V[vin]), b->at<R>(g.off.V[0]), b->at<R>(g.off.V[rb]), b->at<R>(g.off.V[vout]),
           b->at<R>(g.off.geo), vo, Phys<R>{}, ptab(b), b->at<int32_t>(g.off.inst), (R)c0, (R)c1,
           b->at<DevScalars>(b->off_sc));
@@ -308,7 +314,7 @@ struct GDrv final : GroupDrv {
       const int ntiles = (K + T - 1) / T;
       const int grid = std::min(ntiles, staged_blocks(T));
       if (grid <= 0) return;
-      volume_staged_kernel<DIM, P, R><<<grid, T, staged_smem_bytes<DIM, P, R>(T), s>>>(
+      launch_after(volume_staged_kernel<DIM, P, R>, grid, T, staged_smem_bytes<DIM, P, R>(T), s,
           K, F, b->at<R>(g.off.V[vin]), b->at<R>(g.off.V[0]), b->at<R>(g.off.V[vout]), b->at<R>(g.off.E),
           g.has_bed ? b->at<R>(g.off.bed) : nullptr, g.has_bed ? b->at<R>(g.off.src) : nullptr,
           b->at<R>(g.off.geo), b->at<int32_t>(g.off.fid),
@@ -317,7 +323,7 @@ struct GDrv final : GroupDrv {
       return;
     }
     const int T = g.tile[2];
-    volume_kernel<DIM, P, R, true><<<(K + T - 1) / T, T, 0, s>>>(
+    launch_after(volume_kernel<DIM, P, R, true>, (K + T - 1) / T, T, 0, s,
         K, F, b->at<R>(g.off.V[vin]), b->at<R>(g.off.V[0]), b->at<R>(g.off.V[vout]), b->at<R>(g.off.E),
         g.has_bed ? b->at<R>(g.off.bed) : nullptr, g.has_bed ? b->at<R>(g.off.src) : nullptr,
           b->at<R>(g.off.geo), b->at<int32_t>(g.off.fid),
@@ -339,7 +345,7 @@ struct GDrv final : GroupDrv {
       }
     }
     const int T = g.tile[2] > 0 ? g.tile[2] : -g.tile[2];
-    volume_kernel<DIM, P, R, true><<<(K + T - 1) / T, T, 0, s>>>(
+    launch_after(volume_kernel<DIM, P, R, true>, (K + T - 1) / T, T, 0, s,
         K, F, b->at<R>(g.off.V[vin]), nullptr, b->at<R>(g.off.V[vout]), b->at<R>(g.off.E),
         g.has_bed ? b->at<R>(g.off.bed) : nullptr, g.has_bed ? b->at<R>(g.off.src) : nullptr, b->at<R>(g.off.geo),
         b->at<int32_t>(g.off.fid), b->at<R>(g.off.wflux), va, Phys<R>{}, ptab(b), b->at<int32_t>(g.off.inst), 2, R(0),
@@ -347,21 +353,21 @@ struct GDrv final : GroupDrv {
   }
   void dt(dg_batch* b, Group& g, cudaStream_t s) override {
     const int nblk = (int)g.blk_gid.size(), nm = (int)g.members.size();
-    dt_block_kernel<DIM, P, R><<<nblk, 256, 0, s>>>((int)g.K, b->at<int64_t>(g.off.blk_e),
+    launch_after(dt_block_kernel<DIM, P, R>, nblk, 256, 0, s, (int)g.K, b->at<int64_t>(g.off.blk_e),
                                                     b->at<int32_t>(g.off.blk_gid), b->at<R>(g.off.V[0]),
                                                     b->at<R>(g.off.geo), b->at<double>(b->off_iparm),
                                                     b->at<double>(g.off.partial));
-    dt_members_kernel<<<nm, 256, 0, s>>>(b->at<int32_t>(g.off.mblk), b->at<int32_t>(g.off.gid),
+    launch_after(dt_members_kernel, nm, 256, 0, s, b->at<int32_t>(g.off.mblk), b->at<int32_t>(g.off.gid),
                                          b->at<double>(g.off.partial), b->at<DevScalars>(b->off_sc));
   }
   void mass(dg_batch* b, Group& g, int first, int count, int set_ref, cudaStream_t s) override {
     if (count <= 0) return;
     const int b0 = g.mblk[first], nb = g.mblk[first + count] - b0;
     if (nb > 0)
-      mass_block_kernel<S::NP, R><<<(unsigned)nb, 256, 0, s>>>((int)g.K, b0, b->at<int64_t>(g.off.blk_e),
+      launch_after(mass_block_kernel<S::NP, R>, (unsigned)nb, 256, 0, s, (int)g.K, b0, b->at<int64_t>(g.off.blk_e),
                                                               b->at<R>(g.off.V[0]), b->at<R>(g.off.geo),
                                                               b->at<double>(g.off.wint), b->at<double>(g.off.partial));
-    mass_members_kernel<<<(unsigned)((count + 7) / 8), 256, 0, s>>>(first, count, b->at<int32_t>(g.off.mblk),
+    launch_after(mass_members_kernel, (unsigned)((count + 7) / 8), 256, 0, s, first, count, b->at<int32_t>(g.off.mblk),
                                                                    b->at<int32_t>(g.off.gid),
                                                                    b->at<double>(g.off.partial), set_ref,
                                                                    b->at<DevScalars>(b->off_sc));
@@ -537,7 +543,7 @@ dg_status check(dg_batch* b) {
 
 template <typename Rin, typename Rout>
 void conv(const void* in, void* out, size_t n, cudaStream_t s) {
-  if (n) convert_kernel<Rin, Rout><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, (const Rin*)in, (Rout*)out);
+  if (n) launch_after(convert_kernel<Rin, Rout>, (unsigned)((n + 255) / 256), 256, 0, s, n, (const Rin*)in, (Rout*)out);
 }
 
 dg_status read_stats(dg_batch* b, dg_swe_stats* st) {
@@ -902,7 +908,7 @@ dg_status dg_batch_set_workspace(dg_batch* b, void* ptr, size_t bytes) {
   BK(up(b->off_ptab, b->h_phys.data(), b->h_phys.size()));
   BK(up(b->off_bct, b->h_bc.data(), b->h_bc.size()));
   BK(up(b->off_iparm, b->h_iparm.data(), b->h_iparm.size() * 8));
-  reset_scalars_array_kernel<<<(b->n + 127) / 128, 128, 0, s>>>(b->n, b->at<DevScalars>(b->off_sc));
+  launch_after(reset_scalars_array_kernel, (b->n + 127) / 128, 128, 0, s, b->n, b->at<DevScalars>(b->off_sc));
   BK(cudaGetLastError());
   BK(cudaStreamSynchronize(s));
   return DG_OK;
@@ -930,7 +936,7 @@ dg_status dg_batch_set_state(dg_batch* b, int i, const double* V, int on_device)
       BK(cudaStreamSynchronize(s));
     }
   }
-  reset_scalars_array_kernel<<<1, 1, 0, s>>>(1, b->at<DevScalars>(b->off_sc) + i);
+  launch_after(reset_scalars_array_kernel, 1, 1, 0, s, 1, b->at<DevScalars>(b->off_sc) + i);
   g.drv->mass(b, g, mi, 1, 1, s);
   BK(cudaGetLastError());
   if (!on_device) BK(cudaStreamSynchronize(s));

@@ -29,6 +29,7 @@
 
 #include "dg_fixed.cuh"
 #include "dg_host.h"
+#include "dg_launch.cuh"
 #include "dg_math64.cuh"
 
 namespace dgswe {
@@ -623,6 +624,9 @@ __global__ void __launch_bounds__(256, estep_min_blocks<R>()) estep_kernel(int K
                                                     const int8_t* __restrict__ nbrf, const R* __restrict__ fn,
                                                     const R* __restrict__ fsj, const EstepOps<DIM, P, R> ops,
                                                     const BCEntry<R>* __restrict__ bct) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(V);
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= K) return;
   estep_element<DIM, P, R>(e, K, V, E, geo, nbr, nbrf, fn, fsj, ops, bct);
@@ -768,6 +772,9 @@ __global__ void __launch_bounds__(256, face_min_blocks<DIM, P, R>())
                                                    const Phys<R> ph0, const Phys<R>* __restrict__ ptab,
                                                    const int32_t* __restrict__ inst,
                                                    const BCEntry<R>* __restrict__ bct) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(V, E);
   constexpr int NFQ = Sh<DIM, P>::NFQ;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long nthreads = PERFACE ? (long long)F : (long long)F * NFQ;
@@ -841,6 +848,9 @@ __global__ void __launch_bounds__(256, face_pf_min_blocks<DIM, P, R>())
                    const R* __restrict__ fnrm, const R* __restrict__ fsj, R* __restrict__ wflux,
                    const FaceOps<DIM, P, R> ops, const Phys<R>* __restrict__ ptab, const int32_t* __restrict__ inst,
                    const BCEntry<R>* __restrict__ bct) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(V, E);
   const int stride = gridDim.x * blockDim.x;
   int fc = blockIdx.x * blockDim.x + threadIdx.x;
   if (fc >= F) return;
@@ -888,6 +898,9 @@ __global__ void __launch_bounds__(256, estep_min_blocks<R>()) estep_pf_kernel(in
                                                        const int8_t* __restrict__ nbrf, const R* __restrict__ fn,
                                                        const R* __restrict__ fsj, const EstepOps<DIM, P, R> ops,
                                                        const BCEntry<R>* __restrict__ bct) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(V);
   constexpr int NF = Sh<DIM, P>::NF;
   const int stride = gridDim.x * blockDim.x;
   int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1549,10 +1562,13 @@ __global__ void __launch_bounds__(256) __maxnreg__((volume_max_regs<DIM, P, R>()
                                                      const Phys<R> ph0, const Phys<R>* __restrict__ ptab,
                                                      const int32_t* __restrict__ inst, int mode, R c0, R c1,
                                                      const DevScalars* __restrict__ sc) {
+  pdl_trigger();
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV, NE = S::NE;
   __shared__ __align__(16) Fx tab[VolArgT<DIM, P, R>::TAB];
   vol_table<DIM, P, R>(tab, ops);
+  pdl_wait();
+  after_wait(Vin, V0, E, wflux, sc);
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= K) return;
   const int ins = BATCH ? inst[e] : 0;
@@ -1587,6 +1603,9 @@ __global__ void __launch_bounds__(128) wetdry_stage_kernel(int K, const R* __res
                                                            const Phys<R>* __restrict__ ptab,
                                                            const int32_t* __restrict__ inst, R c0, R c1,
                                                            const DevScalars* __restrict__ sc) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(Vin, V0, rbuf, sc);
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1805,6 +1824,9 @@ __global__ void __launch_bounds__(256) volume_staged_kernel(int K, int F, const 
                                                             const Phys<R>* __restrict__ ptab,
                                                             const int32_t* __restrict__ inst, R c0, R c1,
                                                             DevScalars* sc) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(Vin, V0, E, wflux);
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV, NE = S::NE;
   constexpr int NARR = staged_arrays<DIM, P>();
@@ -2048,6 +2070,9 @@ template <int DIM, int P, typename R>
 __global__ void __launch_bounds__(256) dt_partial_kernel(int K, const R* __restrict__ V, const R* __restrict__ geo,
                                                          double gc, double h_floor, double cfl, double nu,
                                                          double* __restrict__ partial) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(V);
   __shared__ R red[8];
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   R dte = huge_dt<R>();
@@ -2060,6 +2085,9 @@ __global__ void __launch_bounds__(256) dt_partial_kernel(int K, const R* __restr
 // step counter.  A negative partial latches DG_ERR_NONFINITE (4).
 static __global__ void dt_finalize_kernel(int nblocks, const double* __restrict__ partial, double fixed_dt,
                                    DevScalars* __restrict__ sc) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(partial);
   __shared__ double red[32];
   double v = 1e300;
   for (int i = threadIdx.x; i < nblocks; i += blockDim.x) v = min_flag(v, partial[i]);
@@ -2083,6 +2111,9 @@ template <int NP, typename R>
 __global__ void __launch_bounds__(256) mass_partial_kernel(int K, const R* __restrict__ V, const R* __restrict__ geo,
                                                            const double* __restrict__ wint,
                                                            double* __restrict__ partial) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(V);
   __shared__ double red[8];
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   double m = 0.0;
@@ -2116,6 +2147,9 @@ __device__ __forceinline__ void two_sum(double a, double b, double& s, double& e
 // all of them took 70 clocks an addition, four additions a partial.)
 static __global__ void __launch_bounds__(256) mass_finalize_kernel(int nblocks, const double* __restrict__ partial,
                                                                    int set_ref, DevScalars* __restrict__ sc) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(partial);
   __shared__ double sh[256], sl[256];
   const int t = threadIdx.x, per = (nblocks + 255) / 256;
   double s = 0.0, c = 0.0;
@@ -2154,6 +2188,9 @@ __global__ void __launch_bounds__(256) dt_block_kernel(int K, const int64_t* __r
                                                        const R* __restrict__ V, const R* __restrict__ geo,
                                                        const double* __restrict__ iparm,
                                                        double* __restrict__ partial) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(V);
   __shared__ R red[8];
   const int b = blockIdx.x;
   const int g = blk_gid[b];
@@ -2172,6 +2209,9 @@ static __global__ void __launch_bounds__(256) dt_members_kernel(const int32_t* _
                                                                 const int32_t* __restrict__ gid,
                                                                 const double* __restrict__ partial,
                                                                 DevScalars* __restrict__ sc) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(partial);
   __shared__ double red[8];
   const int i = blockIdx.x;
   double v = 1e300;
@@ -2192,6 +2232,9 @@ static __global__ void __launch_bounds__(256) dt_members_kernel(const int32_t* _
 }
 
 static __global__ void reset_scalars_array_kernel(int n, DevScalars* sc) {
+  pdl_trigger();
+  pdl_wait();
+
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   sc[i].dt = 0.0;
@@ -2306,11 +2349,17 @@ inline double max_bingham_slope(int reg, double sigma0, double gamma, double pap
 
 template <typename Rin, typename Rout>
 __global__ void convert_kernel(size_t n, const Rin* __restrict__ in, Rout* __restrict__ out) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(in);
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = (Rout)in[i];
 }
 
 static __global__ void reset_scalars_kernel(DevScalars* sc) {
+  pdl_trigger();
+  pdl_wait();
+
   sc->dt = 0.0;
   sc->t = 0.0;
   sc->dt_min = 1e300;

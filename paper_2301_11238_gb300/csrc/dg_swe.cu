@@ -120,14 +120,14 @@ struct Impl final : Driver {
 
   void estep(dg_swe_ctx* c, const void* V, void* E, cudaStream_t s) override {
     const int K = (int)c->mesh.K;
-    estep_kernel<DIM, P, R><<<(K + kBlock - 1) / kBlock, kBlock, 0, s>>>(
+    launch_after(estep_kernel<DIM, P, R>, (K + kBlock - 1) / kBlock, kBlock, 0, s,
         K, (const R*)V, (R*)E, c->at<R>(c->off.geo), c->at<int32_t>(c->off.nbr), c->at<int8_t>(c->off.nbrf),
         c->at<R>(c->off.fn), c->at<R>(c->off.fsj), eo, c->at<BCEntry<R>>(c->off.bct));
   }
   void face(dg_swe_ctx* c, const void* V, const void* E, cudaStream_t s) override {
     const int K = (int)c->mesh.K, F = (int)c->mesh.F;
     const long long n = (long long)F * S::NFQ;
-    face_kernel<DIM, P, R, false, false><<<(unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s>>>(
+    launch_after(face_kernel<DIM, P, R, false, false>, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s,
         K, F, (const R*)V, (const R*)E, c->at<int32_t>(c->off.fe1), c->at<int8_t>(c->off.ff1),
         c->at<int32_t>(c->off.fe2), c->at<int8_t>(c->off.ff2), c->at<R>(c->off.fnrm), c->at<R>(c->off.fsjf),
         c->at<R>(c->off.wflux), fo, ph, nullptr, nullptr, c->at<BCEntry<R>>(c->off.bct));
@@ -136,7 +136,7 @@ struct Impl final : Driver {
               cudaStream_t s) override {
     if (volume_tc(c, Vin, V0, out, c->ws + c->off.E, c->ws + c->off.wflux, mode, c0, c1, s)) return;
     const int K = (int)c->mesh.K, F = (int)c->mesh.F;
-    volume_kernel<DIM, P, R, false><<<(K + kBlock - 1) / kBlock, kBlock, 0, s>>>(
+    launch_after(volume_kernel<DIM, P, R, false>, (K + kBlock - 1) / kBlock, kBlock, 0, s,
         K, F, (const R*)Vin, (const R*)V0, (R*)out, c->at<R>(c->off.E),
         c->has_bed ? c->at<R>(c->off.bed) : nullptr, c->has_bed ? c->at<R>(c->off.src) : nullptr,
         c->at<R>(c->off.geo), c->at<int32_t>(c->off.fid),
@@ -145,14 +145,14 @@ struct Impl final : Driver {
   void wetdry_stage(dg_swe_ctx* c, const void* Vin, const void* V0, const void* rbuf, void* out, double c0,
                     double c1, cudaStream_t s) override {
     const int K = (int)c->mesh.K;
-    wetdry_stage_kernel<DIM, P, R, false><<<(K + kWetDryBlock - 1) / kWetDryBlock, kWetDryBlock, 0, s>>>(
+    launch_after(wetdry_stage_kernel<DIM, P, R, false>, (K + kWetDryBlock - 1) / kWetDryBlock, kWetDryBlock, 0, s,
         K, (const R*)Vin, (const R*)V0, (const R*)rbuf, (R*)out, c->at<R>(c->off.geo), vo, ph, nullptr, nullptr,
         (R)c0, (R)c1, c->at<DevScalars>(c->off.sc));
   }
   void face_into(dg_swe_ctx* c, const void* V, const void* E, void* wflux, cudaStream_t s) override {
     const int K = (int)c->mesh.K, F = (int)c->mesh.F;
     const long long n = (long long)F * S::NFQ;
-    face_kernel<DIM, P, R, false, false><<<(unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s>>>(
+    launch_after(face_kernel<DIM, P, R, false, false>, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s,
         K, F, (const R*)V, (const R*)E, c->at<int32_t>(c->off.fe1), c->at<int8_t>(c->off.ff1),
         c->at<int32_t>(c->off.fe2), c->at<int8_t>(c->off.ff2), c->at<R>(c->off.fnrm), c->at<R>(c->off.fsjf),
         (R*)wflux, fo, ph, nullptr, nullptr, c->at<BCEntry<R>>(c->off.bct));
@@ -172,7 +172,7 @@ struct Impl final : Driver {
                      cudaStream_t s) override {
     if (volume_tc(c, V, nullptr, out, E, wflux, 0, 0.0, 0.0, s)) return;
     const int K = (int)c->mesh.K, F = (int)c->mesh.F;
-    volume_kernel<DIM, P, R, false><<<(K + kBlock - 1) / kBlock, kBlock, 0, s>>>(
+    launch_after(volume_kernel<DIM, P, R, false>, (K + kBlock - 1) / kBlock, kBlock, 0, s,
         K, F, (const R*)V, nullptr, (R*)out, (const R*)E, c->has_bed ? c->at<R>(c->off.bed) : nullptr,
         c->has_bed ? c->at<R>(c->off.src) : nullptr,
         c->at<R>(c->off.geo), c->at<int32_t>(c->off.fid), (const R*)wflux, va, ph, nullptr, nullptr, 0, R(0), R(0),
@@ -183,13 +183,13 @@ struct Impl final : Driver {
     const auto& p = c->prm;
     const double slope = max_bingham_slope(c->reg, p.sigma0, p.gamma, p.pap_m);
     const double nu = (4.0 * max_viscous_eta(p) + slope) / p.rho;
-    dt_partial_kernel<DIM, P, R><<<c->nblk_dt, kRedBlock, 0, s>>>(
+    launch_after(dt_partial_kernel<DIM, P, R>, c->nblk_dt, kRedBlock, 0, s,
         K, (const R*)V, c->at<R>(c->off.geo), p.g * std::cos(p.alpha), p.h_floor, p.cfl, nu,
         c->at<double>(c->off.partial));
   }
   void mass_partial(dg_swe_ctx* c, const void* V, cudaStream_t s) override {
     const int K = (int)c->mesh.K;
-    mass_partial_kernel<S::NP, R><<<c->nblk_mass, kRedBlock, 0, s>>>(
+    launch_after(mass_partial_kernel<S::NP, R>, c->nblk_mass, kRedBlock, 0, s,
         K, (const R*)V, c->at<R>(c->off.geo), c->at<double>(c->off.wint), c->at<double>(c->off.partial));
   }
 };
@@ -226,7 +226,7 @@ void enqueue_step(dg_swe_ctx* c, double fixed_dt, cudaStream_t s) {
   void* V1 = c->ws + c->off.V1;
   void* V2 = c->ws + c->off.V2;
   c->drv->dt_partial(c, V0, s);
-  dt_finalize_kernel<<<1, 256, 0, s>>>(c->nblk_dt, c->at<double>(c->off.partial), fixed_dt,
+  launch_after(dt_finalize_kernel, 1, 256, 0, s, c->nblk_dt, c->at<double>(c->off.partial), fixed_dt,
                                        c->at<DevScalars>(c->off.sc));
   enqueue_stage(c, V0, V0, V1, V1, 0.0, 1.0, s);
   enqueue_stage(c, V1, V0, V2, V2, 0.75, 0.25, s);
@@ -235,7 +235,7 @@ void enqueue_step(dg_swe_ctx* c, double fixed_dt, cudaStream_t s) {
 
 void enqueue_mass(dg_swe_ctx* c, int set_ref, cudaStream_t s) {
   c->drv->mass_partial(c, c->ws + c->off.V0, s);
-  mass_finalize_kernel<<<1, 256, 0, s>>>(c->nblk_mass, c->at<double>(c->off.partial), set_ref,
+  launch_after(mass_finalize_kernel, 1, 256, 0, s, c->nblk_mass, c->at<double>(c->off.partial), set_ref,
                                         c->at<DevScalars>(c->off.sc));
 }
 
@@ -248,7 +248,7 @@ dg_status check_ws(dg_swe_ctx* c) {
 template <typename Rin, typename Rout>
 void convert(const void* in, void* out, size_t n, cudaStream_t s) {
   if (n == 0) return;
-  convert_kernel<Rin, Rout><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, (const Rin*)in, (Rout*)out);
+  launch_after(convert_kernel<Rin, Rout>, (unsigned)((n + 255) / 256), 256, 0, s, n, (const Rin*)in, (Rout*)out);
 }
 
 void destroy_graphs(dg_swe_ctx* c) {
@@ -460,7 +460,7 @@ dg_status dg_swe_set_workspace(dg_swe_ctx* c, void* ptr, size_t bytes) {
     CK(cudaStreamSynchronize(s));
   }
   CK(cudaMemsetAsync(c->ws + c->off.E, 0, (size_t)c->dim * c->dim * K * c->ops.Np * c->rsize, s));
-  reset_scalars_kernel<<<1, 1, 0, s>>>(c->at<DevScalars>(c->off.sc));
+  launch_after(reset_scalars_kernel, 1, 1, 0, s, c->at<DevScalars>(c->off.sc));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   return DG_OK;
@@ -498,7 +498,7 @@ dg_status dg_swe_set_state(dg_swe_ctx* c, const double* V, int on_device) {
     CK(cudaMemcpyAsync(V0, f.data(), n * 4, cudaMemcpyHostToDevice, s));
     CK(cudaStreamSynchronize(s));
   }
-  reset_scalars_kernel<<<1, 1, 0, s>>>(c->at<DevScalars>(c->off.sc));
+  launch_after(reset_scalars_kernel, 1, 1, 0, s, c->at<DevScalars>(c->off.sc));
   enqueue_mass(c, 1, s);
   CK(cudaGetLastError());
   if (!on_device) CK(cudaStreamSynchronize(s));
