@@ -309,6 +309,7 @@ struct GDrv final : GroupDrv {
         return;
       }
     }
+    if (g.tile[2] > 0 && split(b, g, vin, vout, 1, c0, c1, s)) return;
     if (g.tile[2] < 0) {
       const int T = -g.tile[2];
       const int ntiles = (K + T - 1) / T;
@@ -330,6 +331,21 @@ struct GDrv final : GroupDrv {
         b->at<R>(g.off.wflux), va, Phys<R>{}, ptab(b), b->at<int32_t>(g.off.inst), 1, (R)c0, (R)c1,
         b->at<DevScalars>(b->off_sc));
   }
+  // the FP64 volume pass of a small group, in place of the direct form; false if not used
+  bool split(dg_batch* b, Group& g, int vin, int vout, int mode, double c0, double c1, cudaStream_t s) {
+    if constexpr (sizeof(R) == 8) {
+      const int K = (int)g.K, F = (int)g.F;
+      if (!volume_split(K, sizeof(R))) return false;
+      constexpr int EB = kSplitBlock / split_lanes<DIM, P>();  // elements a block
+      launch_after(volume_split_kernel<DIM, P, true>, (K + EB - 1) / EB, kSplitBlock, 0, s, K, F,
+                   b->at<double>(g.off.V[vin]), mode == 1 ? b->at<double>(g.off.V[0]) : nullptr,
+                   b->at<double>(g.off.V[vout]), b->at<double>(g.off.E), g.has_bed ? b->at<double>(g.off.src) : nullptr,
+                   b->at<double>(g.off.geo), b->at<int32_t>(g.off.fid), b->at<double>(g.off.wflux), va, Phys<double>{},
+                   ptab(b), b->at<int32_t>(g.off.inst), mode, c0, c1, b->at<DevScalars>(b->off_sc));
+      return true;
+    }
+    return false;
+  }
   // the volume pass in mode 2 (r_V of V[vin] into V[vout]): the tensor-core
   // form or the direct kernel (the staged form has no mode 2; a negative
   // block size is taken by its magnitude)
@@ -344,6 +360,7 @@ struct GDrv final : GroupDrv {
         return;
       }
     }
+    if (split(b, g, vin, vout, 2, 0.0, 0.0, s)) return;
     const int T = g.tile[2] > 0 ? g.tile[2] : -g.tile[2];
     launch_after(volume_kernel<DIM, P, R, true>, (K + T - 1) / T, T, 0, s,
         K, F, b->at<R>(g.off.V[vin]), nullptr, b->at<R>(g.off.V[vout]), b->at<R>(g.off.E),

@@ -1591,6 +1591,54 @@ __global__ void __launch_bounds__(256) __maxnreg__((volume_max_regs<DIM, P, R>()
                             c0, c1, sc, tab);
 }
 
+// FP64 volume pass for small meshes: T neighbouring lanes per element (see
+// volume_element_fx).  With one thread per element a mesh of up to 152 SMs x 4
+// sub-partitions x 32 lanes = 19,456 elements leaves each sub-partition at most
+// one warp, and the pass takes as long as one element's chain of instructions (a
+// warp-wide FP64 instruction 64 clocks, whatever the lanes); T lanes shorten the
+// chain, and the chip has room for them.
+template <int DIM, int P>
+constexpr int split_lanes() {
+  return DIM == 1 ? (P == 1 ? 2 : 4) : 4;
+}
+constexpr int kSplitBlock = 64;
+inline bool volume_split(int64_t K, size_t rsize) { return rsize == 8 && K <= 152 * 4 * 32; }
+
+template <int DIM, int P, bool BATCH>
+__global__ void __launch_bounds__(kSplitBlock) volume_split_kernel(
+    int K, int F, const double* __restrict__ Vin, const double* V0, double* out, const double* __restrict__ E,
+    const double* __restrict__ src, const double* __restrict__ geo, const int32_t* __restrict__ fid,
+    const double* __restrict__ wflux, const VolFx<DIM, P> ops, const Phys<double> ph0,
+    const Phys<double>* __restrict__ ptab, const int32_t* __restrict__ inst, int mode, double c0, double c1,
+    const DevScalars* __restrict__ sc) {
+  using S = Sh<DIM, P>;
+  constexpr int NP = S::NP, NV = S::NV, NE = S::NE, T = split_lanes<DIM, P>();
+  pdl_trigger();
+  __shared__ __align__(16) Fx tab[FxTab<DIM, P>::SIZE];
+  vol_table<DIM, P, double>(tab, ops);
+  pdl_wait();
+  after_wait(Vin, V0, E, wflux, sc);
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool live = g / T < K;
+  const int e = live ? g / T : K - 1;
+  const int ins = BATCH ? inst[e] : 0;
+  const Phys<double> ph = BATCH ? ptab[ins] : ph0;
+  const size_t KN = (size_t)K * NP, eo = (size_t)e * NP;
+  double Vn[NV][NP], En[NE][NP];
+#pragma unroll
+  for (int a = 0; a < NP; ++a) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Vn[v][a] = Vin[v * KN + eo + a];
+#pragma unroll
+    for (int c = 0; c < NE; ++c) En[c][a] = E[c * KN + eo + a];
+  }
+  const double* V0e[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) V0e[v] = V0 ? V0 + v * KN + eo : nullptr;
+  volume_element_fx<DIM, P, false, T>(e, K, F, Vn, En, src, V0e, out, geo, fid, wflux, ops, ph, ins, mode, c0, c1, sc,
+                                      tab, g % T, live);
+}
+
 // Stage update of wet/dry mode, one thread per element: after a volume pass
 // in mode 2 has written the residual r_V of the stage's input state to rbuf,
 // out = the conservative stage (conservative_stage) from Vin, V0 and rbuf.

@@ -118,6 +118,22 @@ struct Impl final : Driver {
     return false;
   }
 
+  // the FP64 volume pass of a small mesh (mode as volume_kernel); false if not used
+  bool split(dg_swe_ctx* c, const void* Vin, const void* V0, void* out, const void* E, const void* wflux, int mode,
+             double c0, double c1, cudaStream_t s) {
+    if constexpr (sizeof(R) == 8) {
+      const int K = (int)c->mesh.K, F = (int)c->mesh.F;
+      if (!volume_split(K, sizeof(R))) return false;
+      constexpr int EB = kSplitBlock / split_lanes<DIM, P>();  // elements a block
+      launch_after(volume_split_kernel<DIM, P, false>, (K + EB - 1) / EB, kSplitBlock, 0, s, K, F, (const double*)Vin,
+                   (const double*)V0, (double*)out, (const double*)E, c->has_bed ? c->at<double>(c->off.src) : nullptr,
+                   c->at<double>(c->off.geo), c->at<int32_t>(c->off.fid), (const double*)wflux, va, ph, nullptr,
+                   nullptr, mode, c0, c1, c->at<DevScalars>(c->off.sc));
+      return true;
+    }
+    return false;
+  }
+
   void estep(dg_swe_ctx* c, const void* V, void* E, cudaStream_t s) override {
     const int K = (int)c->mesh.K;
     launch_after(estep_kernel<DIM, P, R>, (K + kBlock - 1) / kBlock, kBlock, 0, s,
@@ -136,6 +152,7 @@ struct Impl final : Driver {
               cudaStream_t s) override {
     if (volume_tc(c, Vin, V0, out, c->ws + c->off.E, c->ws + c->off.wflux, mode, c0, c1, s)) return;
     const int K = (int)c->mesh.K, F = (int)c->mesh.F;
+    if (split(c, Vin, V0, out, c->ws + c->off.E, c->ws + c->off.wflux, mode, c0, c1, s)) return;
     launch_after(volume_kernel<DIM, P, R, false>, (K + kBlock - 1) / kBlock, kBlock, 0, s,
         K, F, (const R*)Vin, (const R*)V0, (R*)out, c->at<R>(c->off.E),
         c->has_bed ? c->at<R>(c->off.bed) : nullptr, c->has_bed ? c->at<R>(c->off.src) : nullptr,
@@ -172,6 +189,7 @@ struct Impl final : Driver {
                      cudaStream_t s) override {
     if (volume_tc(c, V, nullptr, out, E, wflux, 0, 0.0, 0.0, s)) return;
     const int K = (int)c->mesh.K, F = (int)c->mesh.F;
+    if (split(c, V, nullptr, out, E, wflux, 0, 0.0, 0.0, s)) return;
     launch_after(volume_kernel<DIM, P, R, false>, (K + kBlock - 1) / kBlock, kBlock, 0, s,
         K, F, (const R*)V, nullptr, (R*)out, (const R*)E, c->has_bed ? c->at<R>(c->off.bed) : nullptr,
         c->has_bed ? c->at<R>(c->off.src) : nullptr,

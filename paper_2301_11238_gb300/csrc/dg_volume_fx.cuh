@@ -83,8 +83,36 @@ __device__ __forceinline__ void fx_row(const VolFx<DIM, P>& ops, const Fx* tab, 
   for (int a = 0; a < N; ++a) out[a] = src[q * N + a];
 }
 
-// Arguments and modes as volume_element (dg_kernels.cuh).
-template <int DIM, int P, bool COH>
+// Sums and maxima over the T neighbouring lanes that share an element.
+// (the sum's two parts apart, so that it is exactly that of T = 1)
+template <int T>
+__device__ __forceinline__ long long lanes_sum(FxAcc v) {
+  if constexpr (T > 1) {
+    fx_fold(v);
+    int low = (int)v.b;
+#pragma unroll
+    for (int o = 1; o < T; o *= 2) {
+      v.a += __shfl_xor_sync(0xffffffffu, v.a, o);
+      low += __shfl_xor_sync(0xffffffffu, low, o);
+    }
+    v.b = low;
+  }
+  return fx_sum(v);
+}
+template <int T>
+__device__ __forceinline__ int lanes_max(int v) {
+#pragma unroll
+  for (int o = 1; o < T; o *= 2) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+// Arguments and modes as volume_element (dg_kernels.cuh).  T = 1: one thread per
+// element.  T = 2, 4: T neighbouring lanes share one (tl: the thread's place
+// among them; all lanes of a warp come here, live = false for those past the
+// last element): each takes every T-th volume point and face, the integer sums
+// are added across the lanes (exactly, so the results are those of T = 1), and
+// each writes every T-th node.
+template <int DIM, int P, bool COH, int T = 1>
 __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
                                                   const double (&Vn)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
                                                   const double (&En)[Sh<DIM, P>::NE][Sh<DIM, P>::NP],
@@ -93,17 +121,19 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
                                                   const double* __restrict__ geo, const int32_t* __restrict__ fid,
                                                   const double* __restrict__ wflux, const VolFx<DIM, P>& ops,
                                                   const Phys<double>& ph, int ins, int mode, double c0, double c1,
-                                                  const DevScalars* __restrict__ sc, const Fx* tab) {
+                                                  const DevScalars* __restrict__ sc, const Fx* tab, int tl = 0,
+                                                  bool live = true) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NQ = S::NQ, NF = S::NF, NFP = S::NFP, NFQ = S::NFQ, NV = S::NV;
+  constexpr int NS = (NQ + T - 1) / T;  // volume points of a thread
   constexpr int NM = VolFx<DIM, P>::NM;
   constexpr int ND = DIM == 1 ? 1 : 3;  // gradient components the stress needs
   constexpr int NT = DIM == 1 ? 1 : 3;  // momentum flux tensor (symmetric)
   const size_t KN = (size_t)K * NP;
   const size_t eo = (size_t)e * NP;
 
-  double hu_s[NQ][DIM], T_s[NQ][NT], S_s[NQ][DIM], u_s[NQ][DIM];
-  Fx hm_s[NQ];
+  double hu_s[NS][DIM], T_s[NS][NT], S_s[NS][DIM], u_s[NS][DIM];
+  Fx hm_s[NS];
   int eH = 0, eT = 0, eS = 0;  // largest exponents of h u, the flux tensor and the source
   // bound of the exponent of max(h, h_floor) at the volume points (Lebesgue constants below 4)
   int eM = 0;
@@ -153,7 +183,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       sd[2 % ND] = fx_scale(e12 - 1023 - ops.cs_v, e12 <= kFxMaxExp);
     }
 #pragma unroll 1
-    for (int q = 0; q < NQ; ++q) {
+    for (int q = tl, i = 0; q < NQ; q += T, ++i) {
       Fx row[NP];
       fx_row<DIM, P, 0>(ops, tab, q, row);
       double Vq[NV], d[ND];
@@ -174,40 +204,43 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       const double h = Vq[0];
       // max(h, h_floor) as integers: h_floor > 0, so a negative h orders below it
       const double hm = __longlong_as_double(max(__double_as_longlong(h), __double_as_longlong(ph.h_floor)));
-      hm_s[q] = fx_from<5>(hm, eM);
-      double hu[DIM], T[NT], Sv[DIM];
+      hm_s[i] = fx_from<5>(hm, eM);
+      double hu[DIM], Tq[NT], Sv[DIM];
 #pragma unroll
       for (int j = 0; j < DIM; ++j) hu[j] = -h * Vq[1 + j];
       const double p = (0.5 * ph.gc * h) * h;
       if constexpr (DIM == 1) {
-        T[0] = h * ph.rho_inv * stress_mu1<double>(d[0], ph) * (2.0 * d[0]) + (hu[0] * Vq[1] - p);
+        Tq[0] = h * ph.rho_inv * stress_mu1<double>(d[0], ph) * (2.0 * d[0]) + (hu[0] * Vq[1] - p);
       } else {
         constexpr int Y = 1 % ND, XY = 2 % ND, U2 = 2 % NV;
         const double tr = d[0] + d[Y];
         // ||D||_c^2 / 2
         const double s2 = 0.5 * (d[0] * d[0] + d[Y] * d[Y] + tr * tr) + 0.25 * (d[XY] * d[XY]);
         const double m = h * ph.rho_inv * stress_mu2<double>(s2, ph);
-        T[0] = m * (d[0] + tr) + (hu[0] * Vq[1] - p);
-        T[1 % NT] = m * (0.5 * d[XY]) + hu[0] * Vq[U2];
-        T[2 % NT] = m * (d[Y] + tr) + (hu[1 % DIM] * Vq[U2] - p);
+        Tq[0] = m * (d[0] + tr) + (hu[0] * Vq[1] - p);
+        Tq[1 % NT] = m * (0.5 * d[XY]) + hu[0] * Vq[U2];
+        Tq[2 % NT] = m * (d[Y] + tr) + (hu[1 % DIM] * Vq[U2] - p);
       }
 #pragma unroll
       for (int j = 0; j < DIM; ++j) {
         if (src) Sv[j] = h * src[(size_t)(j * NQ + q) * K + e];
         else Sv[j] = j == 0 ? -ph.gs * h : 0.0;
-        hu_s[q][j] = hu[j];
-        S_s[q][j] = Sv[j];
-        u_s[q][j] = Vq[1 + j];
+        hu_s[i][j] = hu[j];
+        S_s[i][j] = Sv[j];
+        u_s[i][j] = Vq[1 + j];
         eH = max(eH, fx_exp(hu[j]));
         eS = max(eS, fx_exp(Sv[j]));
       }
 #pragma unroll
       for (int c = 0; c < NT; ++c) {
-        T_s[q][c] = T[c];
-        eT = max(eT, fx_exp(T[c]));
+        T_s[i][c] = Tq[c];
+        eT = max(eT, fx_exp(Tq[c]));
       }
     }
   }
+  eH = lanes_max<T>(eH);
+  eT = lanes_max<T>(eT);
+  eS = lanes_max<T>(eS);
 
   // ---- pass 2: J times (metric transform, test functions, face lift)
   FxAcc r[NV][NP];
@@ -233,6 +266,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
   const size_t FQ = (size_t)F * NFQ;
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
+    if (T > 1 && f % T != tl) continue;
     const uint32_t raw = (uint32_t)fid[f * K + e];
     const bool own = (raw & 0x80000000u) == 0;
     const size_t base = (size_t)(raw & 0x7fffffffu) * NFQ;
@@ -245,6 +279,8 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
         eW[v > 0] = max(eW[v > 0], fx_exp(x));
       }
   }
+  eW[0] = lanes_max<T>(eW[0]);
+  eW[1] = lanes_max<T>(eW[1]);
   // one unit per group of rows (depth, momentum): operands below
   // 2^(tot - 2043) in units of 2^(tot - 2101)
   const int tot0 = max(eH + eG, eW[0] + 1021), tot1 = max(max(eT + eG, eS + eJ), eW[1] + 1021);
@@ -256,6 +292,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
     for (int v = 0; v < NV; ++v)
 #pragma unroll
       for (int m = 0; m < NFQ; ++m) {
+        if (T > 1 && f % T != tl) continue;
         const Fx x = fx_from<5>(fv[f][v][m], (v > 0 ? tot1 : tot0) - 1021);
 #pragma unroll
         for (int k = 0; k < NFP; ++k) fx_mac(r[v][face_node(DIM, P, f, k)], x, ops.LfT[k * NFQ + m]);
@@ -270,8 +307,8 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
     // at most 2 NFQ + 5 (DIM + 1) terms before the first fold, 5 (DIM + 1) after it
     static_assert(2 * S::NFQ <= 15, "the lift terms need a fold of their own");
 #pragma unroll 1
-    for (int q = 0; q < NQ; ++q) {
-      if (DIM == 2 && q % 5 == 0) {
+    for (int q = tl, k = 0; q < NQ; q += T, ++k) {
+      if (DIM == 2 && k % 5 == 0) {
 #pragma unroll
         for (int v = 0; v < NV; ++v)
 #pragma unroll
@@ -287,7 +324,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
         Fx x[DIM];
 #pragma unroll
         for (int i = 0; i < DIM; ++i)
-          x[i] = v == 0 ? fx_from<5>(hu_s[q][i], tot0 - eG) : fx_from<5>(T_s[q][(v - 1 + i) % (NT + 1)], tot1 - eG);
+          x[i] = v == 0 ? fx_from<5>(hu_s[k][i], tot0 - eG) : fx_from<5>(T_s[k][(v - 1 + i) % (NT + 1)], tot1 - eG);
         FxAcc fr{0, 0}, fs{0, 0};
 #pragma unroll
         for (int i = 0; i < DIM; ++i) {
@@ -299,7 +336,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
         if constexpr (DIM == 2) fsx = fx_operand<61>(fx_sum(fs));
         if (v > 0) {
           FxAcc s{0, 0};
-          fx_mac(s, fx_from<5>(S_s[q][(v + DIM - 1) % DIM], tot1 - eJ), Jx);
+          fx_mac(s, fx_from<5>(S_s[k][(v + DIM - 1) % DIM], tot1 - eJ), Jx);
           sx = fx_operand<61>(fx_sum(s));
         }
 #pragma unroll
@@ -311,6 +348,11 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       }
     }
   }
+  long long rs[NV][NP];
+#pragma unroll
+  for (int v = 0; v < NV; ++v)
+#pragma unroll
+    for (int a = 0; a < NP; ++a) rs[v][a] = lanes_sum<T>(r[v][a]);
   const FxScale s0 = fx_scale(tot0 - 2045 - ops.cs_w, finite), s1 = fx_scale(tot1 - 2045 - ops.cs_w, finite);
 
   // mode 2: the spatial residual r_V itself (physical scaling), for the
@@ -319,7 +361,8 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
 #pragma unroll
     for (int v = 0; v < NV; ++v)
 #pragma unroll
-      for (int a = 0; a < NP; ++a) out[v * KN + eo + a] = fx_to(fx_sum(r[v][a]), v > 0 ? s1 : s0);
+      for (int a = 0; a < NP; ++a)
+        if (live && (T == 1 || a % T == tl)) out[v * KN + eo + a] = fx_to(rs[v][a], v > 0 ? s1 : s0);
     return;
   }
 
@@ -333,10 +376,10 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
     unsigned long long m = 0;
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
-      rh[a] = fx_sum(r[0][a]);
+      rh[a] = rs[0][a];
       m |= fx_mag(rh[a]);
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) ru[j][a] = fx_to(fx_sum(r[1 + j][a]), s1);
+      for (int j = 0; j < DIM; ++j) ru[j][a] = fx_to(rs[1 + j][a], s1);
     }
     int n = fx_norm(m);
     Fx rx[NP];
@@ -363,7 +406,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
   const FxScale sq = fx_scale(kh, finite);
   int eZ = 0;
 #pragma unroll 1
-  for (int q = 0; q < NQ; ++q) {
+  for (int q = tl, k = 0; q < NQ; q += T, ++k) {
     Fx row[NP];
     fx_row<DIM, P, 0>(ops, tab, q, row);
     FxAcc s{0, 0};
@@ -372,11 +415,12 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
     const double dq = fx_to(fx_sum(s), sq);
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
-      const double z = dq * u_s[q][j];
-      u_s[q][j] = z;
+      const double z = dq * u_s[k][j];
+      u_s[k][j] = z;
       eZ = max(eZ, fx_exp(z));
     }
   }
+  eZ = lanes_max<T>(eZ);
   const FxScale sm = fx_scale(eM - 1024 - ops.cs_m, finite),
                 sz = fx_scale(eZ - 1024 - ops.cs_w, finite && eZ <= kFxMaxExp);
   // -r_u - <psi, x_h u>, and after it M_h (one after the other: their
@@ -388,10 +432,10 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
 #pragma unroll
       for (int a = 0; a < NP; ++a) za[j][a] = FxAcc{0, 0};
 #pragma unroll 1
-    for (int q = 0; q < NQ; ++q) {
+    for (int q = tl, k = 0; q < NQ; q += T, ++k) {
       Fx wm[NP];
       fx_row<DIM, P, 3>(ops, tab, q, wm);
-      if (NQ > 15 && q % 12 == 0) {
+      if (NS > 15 && k % 12 == 0) {
 #pragma unroll
         for (int j = 0; j < DIM; ++j)
 #pragma unroll
@@ -399,7 +443,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       }
 #pragma unroll
       for (int j = 0; j < DIM; ++j) {
-        const Fx z = fx_from<5>(u_s[q][j], eZ);
+        const Fx z = fx_from<5>(u_s[k][j], eZ);
 #pragma unroll
         for (int a = 0; a < NP; ++a) fx_mac(za[j][a], z, wm[a]);
       }
@@ -407,17 +451,17 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
 #pragma unroll
     for (int j = 0; j < DIM; ++j)
 #pragma unroll
-      for (int a = 0; a < NP; ++a) ru[j][a] = fx_to(fx_sum(za[j][a]), sz) - ru[j][a];
+      for (int a = 0; a < NP; ++a) ru[j][a] = fx_to(lanes_sum<T>(za[j][a]), sz) - ru[j][a];
   }
   FxAcc Ma[NM];
 #pragma unroll
   for (int i = 0; i < NM; ++i) Ma[i] = FxAcc{0, 0};
 #pragma unroll 1
-  for (int q = 0; q < NQ; ++q) {
+  for (int q = tl, k = 0; q < NQ; q += T, ++k) {
     Fx mp[NM];
     fx_row<DIM, P, 4>(ops, tab, q, mp);
-    const Fx hm = hm_s[q];
-    if (NQ > 15 && q % 12 == 0) {
+    const Fx hm = hm_s[k];
+    if (NS > 15 && k % 12 == 0) {
 #pragma unroll
       for (int i = 0; i < NM; ++i) fx_fold(Ma[i]);
     }
@@ -431,7 +475,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
 #pragma unroll
   for (int a = 0, i = 0; a < NP; ++a) {
 #pragma unroll
-    for (int b = 0; b <= a; ++b, ++i) Mh[a][b] = fx_to(fx_sum(Ma[i]), sm);
+    for (int b = 0; b <= a; ++b, ++i) Mh[a][b] = fx_to(lanes_sum<T>(Ma[i]), sm);
 #pragma unroll
     for (int b = 0; b < a; ++b) {
       double s = Mh[a][b];
@@ -469,7 +513,8 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
 #pragma unroll
     for (int v = 0; v < NV; ++v)
 #pragma unroll
-      for (int a = 0; a < NP; ++a) out[v * KN + eo + a] = Jinv * x[v][a];
+      for (int a = 0; a < NP; ++a)
+        if (live && (T == 1 || a % T == tl)) out[v * KN + eo + a] = Jinv * x[v][a];
     return;
   }
   const double cx = DG_LDC(COH, &sc[ins].dt, 0) * Jinv;
@@ -477,6 +522,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
   for (int v = 0; v < NV; ++v)
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
+      if (T > 1 && a % T != tl) continue;
       double y = c1 * (Vn[v][a] + cx * x[v][a]);
       if (c0 != 0.0) y += c0 * DG_LDC(COH, V0e[v], a);
       x[v][a] = y;
@@ -484,7 +530,8 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
 #pragma unroll
   for (int v = 0; v < NV; ++v)
 #pragma unroll
-    for (int a = 0; a < NP; ++a) out[v * KN + eo + a] = x[v][a];
+    for (int a = 0; a < NP; ++a)
+      if (live && (T == 1 || a % T == tl)) out[v * KN + eo + a] = x[v][a];
 }
 
 // ------------------------------------------------------------------ host: tables
