@@ -31,11 +31,13 @@ struct Driver {
   virtual void face_into(dg_swe_ctx* c, const void* V, const void* E, void* wflux, cudaStream_t s) = 0;
   virtual void residual_from(dg_swe_ctx* c, const void* V, const void* E, const void* wflux, void* out,
                              cudaStream_t s) = 0;
-  // Backward-Euler support (dg_newton.h): <l_a, U(V)> (mode 0) or
-  // out += (<l_a, U(V)> - Uold) * inv_dt (mode 1); z = scale M(V)^{-1} x.
-  virtual void be_time(dg_swe_ctx* c, const void* V, const void* Uold, void* out, double inv_dt, int mode,
-                       cudaStream_t s) = 0;
-  virtual void precond(dg_swe_ctx* c, const void* V, const void* x, void* z, double scale, cudaStream_t s) = 0;
+  // Backward-Euler support (dg_newton.h, FP64 only): be_time_kernel,
+  // mass_factor_kernel and mass_apply_kernel (dg_newton_kernels.cuh).
+  virtual void be_time(dg_swe_ctx* c, const double* V, const double* Uold, double* out, double inv_dt, int mode,
+                       const double* R0, const double* eps, cudaStream_t s) = 0;
+  virtual void mass_factor(dg_swe_ctx* c, const double* V, double* mats, cudaStream_t s) = 0;
+  virtual void mass_apply(dg_swe_ctx* c, const double* x, const double* mats, double scale, const double* nrm2,
+                          double* xn, double* out, bool add, cudaStream_t s) = 0;
 };
 struct DriverDeleter {
   void operator()(Driver* d) const;

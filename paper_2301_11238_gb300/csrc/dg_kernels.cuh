@@ -1709,83 +1709,11 @@ __global__ void __launch_bounds__(128) wetdry_stage_kernel(int K, const R* __res
   conservative_stage<DIM, P, R, double>(Vn, r, V0e, c0, c1, dt, ops, ph.h_floor, Jinv, out, KN, eo);
 }
 
-// ------------------------------------------------------------------ backward Euler (Newton-Krylov)
+}  // namespace dgswe
 
-// <l_a, U_v(V)> per element in physical scaling, with U = (h, h u_1, ..,
-// h u_d) (Eq. Uterm) at the volume quadrature points.  mode 0: out = that;
-// mode 1: out += (that - Uold) * inv_dt, which adds the backward-Euler time
-// term of Eq. WeakForm7 to the spatial residual already in out.
-template <int DIM, int P, typename R>
-__global__ void __launch_bounds__(256) be_time_kernel(int K, const R* __restrict__ V, const R* __restrict__ Uold,
-                                                      R* __restrict__ out, const R* __restrict__ geo,
-                                                      const VolOps<DIM, P, R> ops, R inv_dt, int mode) {
-  using S = Sh<DIM, P>;
-  constexpr int NP = S::NP, NQ = S::NQ, NV = S::NV;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= K) return;
-  const size_t KN = (size_t)K * NP, eo = (size_t)e * NP;
-  R Vn[NV][NP], acc[NV][NP];
-#pragma unroll
-  for (int v = 0; v < NV; ++v)
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      Vn[v][a] = V[v * KN + eo + a];
-      acc[v][a] = R(0);
-    }
-  const R J = geo[4 * K + e];
-#pragma unroll 1
-  for (int q = 0; q < NQ; ++q) {
-    R Vq[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      R t = R(0);
-#pragma unroll
-      for (int a = 0; a < NP; ++a) t += ops.Vq[q * NP + a] * Vn[v][a];
-      Vq[v] = t;
-    }
-    const R w = ops.wq[q] * J;
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      const R wl = w * ops.Vq[q * NP + a];
-      acc[0][a] += wl * Vq[0];
-#pragma unroll
-      for (int j = 1; j < NV; ++j) acc[j][a] += wl * (Vq[0] * Vq[j]);
-    }
-  }
-#pragma unroll
-  for (int v = 0; v < NV; ++v)
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      const size_t i = v * KN + eo + a;
-      out[i] = mode == 0 ? acc[v][a] : out[i] + (acc[v][a] - Uold[i]) * inv_dt;
-    }
-}
+#include "dg_newton_kernels.cuh"
 
-// z = scale * M(V)^{-1} x per element, M(V) the primitive-variable mass
-// matrix (Appendix A, dU/dV): the preconditioner of the Newton-Krylov solve.
-template <int DIM, int P, typename R>
-__global__ void __launch_bounds__(256) mass_precond_kernel(int K, const R* __restrict__ V, const R* __restrict__ x,
-                                                           R* __restrict__ z, const R* __restrict__ geo,
-                                                           const VolOps<DIM, P, R> ops, R h_floor, R scale) {
-  using S = Sh<DIM, P>;
-  constexpr int NP = S::NP, NV = S::NV;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= K) return;
-  const size_t KN = (size_t)K * NP, eo = (size_t)e * NP;
-  R Vn[NV][NP], xr[NV][NP], dV[NV][NP];
-#pragma unroll
-  for (int v = 0; v < NV; ++v)
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      Vn[v][a] = V[v * KN + eo + a];
-      xr[v][a] = x[v * KN + eo + a];
-    }
-  mass_solve_element<DIM, P, R>(Vn, xr, ops, h_floor, geo[6 * K + e], dV);
-#pragma unroll
-  for (int v = 0; v < NV; ++v)
-#pragma unroll
-    for (int a = 0; a < NP; ++a) z[v * KN + eo + a] = -scale * dV[v][a];
-}
+namespace dgswe {
 
 // ------------------------------------------------------------------ staged volume kernel
 // Bulk asynchronous copies (global -> shared, completion counted in bytes on

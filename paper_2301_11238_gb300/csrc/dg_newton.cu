@@ -26,49 +26,81 @@ inline size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // ------------------------------------------------------------------ FP64 vector kernels
 
-// partial[i * G + b] = block b's share of <x, Y_i>, Y_i = Y + i * n.
-__global__ void __launch_bounds__(kVecBlock) dots_partial_kernel(size_t n, const double* __restrict__ x,
-                                                                 const double* __restrict__ Y,
-                                                                 double* __restrict__ partial) {
+// Block sum of v in thread 0 (kVecBlock threads, fixed order).
+__device__ __forceinline__ double vec_block_sum(double v, double* sh) {
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < 32) t = warp_sum(threadIdx.x < kVecBlock / 32 ? sh[threadIdx.x] : 0.0);
+  return t;
+}
+// The grid's last block to finish adds the partials of every dot in a fixed
+// order: dot i = sum of partial[i * G + b] over its G blocks, a warp a dot.
+// counter is zero before and after.
+__device__ __forceinline__ void vec_finish(int G, int cnt, const double* partial, double* out, unsigned* counter) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x * gridDim.y - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int i = threadIdx.x >> 5; i < cnt; i += kVecBlock / 32) {
+    double acc = 0.0;
+    for (int b = threadIdx.x & 31; b < G; b += 32) acc += __ldcg(partial + (size_t)i * G + b);
+    acc = warp_sum(acc);
+    if ((threadIdx.x & 31) == 0) out[i] = acc;
+  }
+  if (threadIdx.x == 0) *counter = 0;
+}
+
+// out[i] = <x, Y_i>, Y_i = Y + i * n; grid (G, number of dots).
+__global__ void __launch_bounds__(kVecBlock) dots_kernel(size_t n, const double* __restrict__ x,
+                                                         const double* __restrict__ Y, double* __restrict__ partial,
+                                                         double* __restrict__ out, unsigned* counter) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(x, Y);
+  __shared__ double sh[kVecBlock / 32];
   const int i = blockIdx.y;
   const double* y = Y + (size_t)i * n;
   double acc = 0.0;
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x)
     acc += x[j] * y[j];
+  acc = vec_block_sum(acc, sh);
+  if (threadIdx.x == 0) partial[(size_t)i * gridDim.x + blockIdx.x] = acc;
+  vec_finish(gridDim.x, gridDim.y, partial, out, counter);
+}
+
+// w -= sum_i c[i] Y_i; nrm2 given: and *nrm2 = <w, w>.
+__global__ void __launch_bounds__(kVecBlock) multi_axpy_kernel(size_t n, int k, const double* __restrict__ c,
+                                                               const double* __restrict__ Y, double* __restrict__ w,
+                                                               double* __restrict__ partial, double* __restrict__ nrm2,
+                                                               unsigned* counter) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(c, Y, w);
   __shared__ double sh[kVecBlock / 32];
-  acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < kVecBlock / 32 ? sh[threadIdx.x] : 0.0;
-    v = warp_sum(v);
-    if (threadIdx.x == 0) partial[(size_t)i * gridDim.x + blockIdx.x] = v;
-  }
-}
-
-// out[i] = sum over the G partials of dot i (fixed order).
-__global__ void dots_finalize_kernel(int G, int k, const double* __restrict__ partial, double* __restrict__ out) {
-  const int i = blockIdx.x;
-  if (i >= k) return;
   double acc = 0.0;
-  for (int b = threadIdx.x; b < G; b += 32) acc += partial[(size_t)i * G + b];
-  acc = warp_sum(acc);
-  if (threadIdx.x == 0) out[i] = acc;
-}
-
-// w -= sum_i c[i] Y_i
-__global__ void multi_axpy_kernel(size_t n, int k, const double* __restrict__ c, const double* __restrict__ Y,
-                                  double* __restrict__ w) {
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x) {
     double s = w[j];
     for (int i = 0; i < k; ++i) s -= c[i] * Y[(size_t)i * n + j];
     w[j] = s;
+    acc += s * s;
   }
+  if (!nrm2) return;
+  acc = vec_block_sum(acc, sh);
+  if (threadIdx.x == 0) partial[blockIdx.x] = acc;
+  vec_finish(gridDim.x, 1, partial, nrm2, counter);
 }
 
 // out = sum_i c[i] Y_i
-__global__ void combine_kernel(size_t n, int k, const double* __restrict__ c, const double* __restrict__ Y,
-                               double* __restrict__ out) {
+__global__ void __launch_bounds__(kVecBlock) combine_kernel(size_t n, int k, const double* __restrict__ c,
+                                                            const double* __restrict__ Y, double* __restrict__ out) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(c, Y);
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x) {
     double s = 0.0;
     for (int i = 0; i < k; ++i) s += c[i] * Y[(size_t)i * n + j];
@@ -77,44 +109,33 @@ __global__ void combine_kernel(size_t n, int k, const double* __restrict__ c, co
 }
 
 // y = a * x
-__global__ void scale_kernel(size_t n, double a, const double* __restrict__ x, double* __restrict__ y) {
-  for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x)
-    y[j] = a * x[j];
-}
-
-// y = x / sqrt(*nrm2)
-__global__ void normalize_kernel(size_t n, const double* __restrict__ nrm2, const double* __restrict__ x,
-                                 double* __restrict__ y) {
-  const double a = 1.0 / sqrt(*nrm2);
+__global__ void __launch_bounds__(kVecBlock) scale_kernel(size_t n, double a, const double* __restrict__ x,
+                                                          double* __restrict__ y) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(x);
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x)
     y[j] = a * x[j];
 }
 
 // eps = sqrt(1e-16) (1 + ||V||) / ||z|| ; Vp = V + eps z
-__global__ void fd_point_kernel(size_t n, const double* __restrict__ V, const double* __restrict__ z,
-                                const double* __restrict__ vn2, const double* __restrict__ zn2,
-                                double* __restrict__ Vp, double* __restrict__ eps_out) {
+__global__ void __launch_bounds__(kVecBlock) fd_point_kernel(size_t n, const double* __restrict__ V,
+                                                             const double* __restrict__ z,
+                                                             const double* __restrict__ vn2,
+                                                             const double* __restrict__ zn2, double* __restrict__ Vp,
+                                                             double* __restrict__ eps_out) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(V, z, vn2, zn2);
   const double eps = 1e-8 * (1.0 + sqrt(*vn2)) / sqrt(*zn2);
   if (blockIdx.x == 0 && threadIdx.x == 0) *eps_out = eps;
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x)
     Vp[j] = V[j] + eps * z[j];
 }
 
-// w = (R1 - R0) / eps
-__global__ void fd_diff_kernel(size_t n, const double* __restrict__ R1, const double* __restrict__ R0,
-                               const double* __restrict__ eps, double* __restrict__ w) {
-  const double a = 1.0 / *eps;
-  for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x)
-    w[j] = (R1[j] - R0[j]) * a;
-}
-
-// V += d
-__global__ void add_kernel(size_t n, const double* __restrict__ d, double* __restrict__ V) {
-  for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x)
-    V[j] += d[j];
-}
-
 __global__ void advance_time_kernel(DevScalars* sc, double dt) {
+  pdl_trigger();
+  pdl_wait();
   sc->t += dt;
   sc->dt = dt;
   sc->dt_min = fmin(sc->dt_min, dt);
@@ -133,10 +154,13 @@ struct dg_newton {
   size_t ws_need = 0;
   char* ws = nullptr;
   struct {
-    size_t Uold, R0, R1, Vp, z, w, u, basis, partial, dots, scal;
+    size_t Uold, R0, Vp, z, w, u, basis, mats, partial, dots, scal, counter;
   } off{};
   dg_newton_stats st{};
   std::string err;
+  // host side of the per-iteration read (pinned, so that the copy is one DMA and
+  // the call does not stage it)
+  double* hbuf = nullptr;
   template <typename T>
   T* at(size_t o) const { return reinterpret_cast<T*>(ws + o); }
 };
@@ -157,7 +181,7 @@ dg_status nfail(dg_newton* k, dg_status s, const std::string& m) {
   } while (0)
 
 // scalar slots
-enum { S_VN2 = 0, S_ZN2 = 1, S_EPS = 2, S_WN2 = 3, S_COUNT = 8 };
+enum { S_VN2 = 0, S_ZN2 = 1, S_EPS = 2, S_COUNT = 8 };
 
 struct Ctx {
   dg_newton* k;
@@ -167,17 +191,26 @@ struct Ctx {
   unsigned grid;
   double* V;  // the context's state
   double* E;
-  void residual(const double* Vx, double* out) {
+  // R(Vx); eps given: its directional difference (R(Vx) - R0) / *eps
+  void residual(const double* Vx, double* out, const double* R0, const double* eps) {
     c->drv->estep(c, Vx, E, s);
     c->drv->face(c, Vx, E, s);
     c->drv->volume(c, Vx, nullptr, out, 2, 0.0, 0.0, s);
-    c->drv->be_time(c, Vx, k->at<double>(k->off.Uold), out, 1.0 / k->prm.dt, 1, s);
+    c->drv->be_time(c, Vx, k->at<double>(k->off.Uold), out, 1.0 / k->prm.dt, eps ? 2 : 1, R0, eps, s);
   }
-  // dots of x against k vectors Y_i into out[0..k) (device)
+  // dots of x against cnt vectors Y_i into out[0..cnt) (device)
   void dots(const double* x, const double* Y, int cnt, double* out) {
-    dots_partial_kernel<<<dim3((unsigned)k->G, (unsigned)cnt), kVecBlock, 0, s>>>(n, x, Y,
-                                                                                 k->at<double>(k->off.partial));
-    dots_finalize_kernel<<<cnt, 32, 0, s>>>(k->G, cnt, k->at<double>(k->off.partial), out);
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)k->G, (unsigned)cnt);
+    cfg.blockDim = dim3(kVecBlock);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, dots_kernel, n, x, Y, k->at<double>(k->off.partial), out,
+                       k->at<unsigned>(k->off.counter));
   }
 };
 
@@ -211,16 +244,22 @@ dg_status dg_newton_init(dg_swe_ctx* c, const dg_newton_params* p, dg_newton** o
   const size_t vb = k->n * sizeof(double);
   k->off.Uold = take(vb);
   k->off.R0 = take(vb);
-  k->off.R1 = take(vb);
   k->off.Vp = take(vb);
   k->off.z = take(vb);
   k->off.w = take(vb);
   k->off.u = take(vb);
   k->off.basis = take((size_t)(k->m + 1) * vb);
+  k->off.mats = take((size_t)(c->dim + 1) * (size_t)c->mesh.K * c->ops.Np * c->ops.Np * sizeof(double));
   k->off.partial = take((size_t)(k->m + 1) * k->G * sizeof(double));
-  k->off.dots = take(2 * (size_t)(k->m + 1) * sizeof(double));
+  k->off.dots = take((2 * (size_t)(k->m + 1) + 1) * sizeof(double));
   k->off.scal = take(S_COUNT * sizeof(double));
+  k->off.counter = take(sizeof(unsigned));
   k->ws_need = o;
+  if (cudaHostAlloc((void**)&k->hbuf, (2 * (size_t)(k->m + 1) + 1) * sizeof(double), cudaHostAllocDefault) !=
+      cudaSuccess) {
+    cudaGetLastError();  // no device here: run needs one anyway
+    k->hbuf = nullptr;
+  }
   *out = k;
   return DG_OK;
 }
@@ -232,6 +271,7 @@ dg_status dg_newton_set_workspace(dg_newton* k, void* ptr, size_t bytes) {
   if (!ptr || ((uintptr_t)ptr & 255) != 0 || bytes < k->ws_need)
     return nfail(k, DG_ERR_WORKSPACE, "workspace missing, misaligned or smaller than dg_newton_workspace_size");
   k->ws = static_cast<char*>(ptr);
+  NK(cudaMemsetAsync(k->ws + k->off.counter, 0, sizeof(unsigned), k->c->stream));
   return DG_OK;
 }
 
@@ -240,33 +280,40 @@ dg_status dg_newton_run(dg_newton* k, int64_t n_steps, dg_newton_stats* stats) {
   dg_swe_ctx* c = k->c;
   if (!k->ws || !c->ws) return nfail(k, DG_ERR_WORKSPACE, "solver or context workspace not set");
   if (n_steps < 0) return nfail(k, DG_ERR_ARG, "n_steps must be >= 0");
+  const size_t nd = 2 * (size_t)(k->m + 1) + 1;
+  if (!k->hbuf) NK(cudaHostAlloc((void**)&k->hbuf, nd * sizeof(double), cudaHostAllocDefault));
   Ctx x{k, c, c->stream, k->n, (unsigned)k->G, c->at<double>(c->off.V0), c->at<double>(c->off.E)};
   const size_t n = k->n;
   const int m = k->m;
   double* Uold = k->at<double>(k->off.Uold);
   double* R0 = k->at<double>(k->off.R0);
-  double* R1 = k->at<double>(k->off.R1);
   double* Vp = k->at<double>(k->off.Vp);
   double* z = k->at<double>(k->off.z);
   double* w = k->at<double>(k->off.w);
   double* u = k->at<double>(k->off.u);
   double* Bv = k->at<double>(k->off.basis);
   double* dots = k->at<double>(k->off.dots);
+  double* wn2 = dots + 2 * (m + 1);  // after the dots, so that one copy brings all
+  double* mats = k->at<double>(k->off.mats);
+  double* partial = k->at<double>(k->off.partial);
+  unsigned* counter = k->at<unsigned>(k->off.counter);
+  double* hbuf = k->hbuf;
   double* sc = k->at<double>(k->off.scal);
   const unsigned G = x.grid;
   cudaStream_t s = x.s;
-  std::vector<double> H((size_t)(m + 1) * m), g(m + 1), cs(m), sn(m), y(m), hbuf(2 * (m + 1) + 1);
+  std::vector<double> H((size_t)(m + 1) * m), g(m + 1), cs(m), sn(m), y(m);
   auto norm2 = [&](const double* v, double* slot, double& host) -> dg_status {
     x.dots(v, v, 1, slot);
-    NK(cudaMemcpyAsync(&host, slot, sizeof(double), cudaMemcpyDeviceToHost, s));
+    NK(cudaMemcpyAsync(hbuf, slot, sizeof(double), cudaMemcpyDeviceToHost, s));
     NK(cudaStreamSynchronize(s));
+    host = hbuf[0];
     return DG_OK;
   };
   for (int64_t step = 0; step < n_steps; ++step) {
-    c->drv->be_time(c, x.V, nullptr, Uold, 0.0, 0, s);
-    x.residual(x.V, R0);
+    c->drv->be_time(c, x.V, nullptr, Uold, 0.0, 0, nullptr, nullptr, s);
+    x.residual(x.V, R0, nullptr, nullptr);
     double r2 = 0.0;
-    dg_status e = norm2(R0, sc + S_WN2, r2);
+    dg_status e = norm2(R0, wn2, r2);
     if (e != DG_OK) return e;
     const double res0 = std::sqrt(r2);
     double res = res0;
@@ -275,27 +322,26 @@ dg_status dg_newton_run(dg_newton* k, int64_t n_steps, dg_newton_stats* stats) {
     while (!ok && its < k->prm.max_newton) {
       if (!std::isfinite(res)) return nfail(k, DG_ERR_NONFINITE, "non-finite Newton residual");
       // ---- GMRES on J d = -R0, right preconditioned by dt M(V)^{-1}
+      c->drv->mass_factor(c, x.V, mats, s);
       x.dots(x.V, x.V, 1, sc + S_VN2);
       const double beta = res;
-      scale_kernel<<<G, kVecBlock, 0, s>>>(n, -1.0 / beta, R0, Bv);
+      launch_after(scale_kernel, G, kVecBlock, 0, s, n, -1.0 / beta, R0, Bv);
       std::fill(g.begin(), g.end(), 0.0);
       g[0] = beta;
       int jn = 0;
       for (int j = 0; j < m; ++j) {
+        // z = dt M^{-1} v_j; from j = 1 on v_j = w / ||w|| of the last round
         double* vj = Bv + (size_t)j * n;
-        c->drv->precond(c, x.V, vj, z, k->prm.dt, s);
+        c->drv->mass_apply(c, j == 0 ? vj : w, mats, k->prm.dt, j == 0 ? nullptr : wn2, vj, z, false, s);
         x.dots(z, z, 1, sc + S_ZN2);
-        fd_point_kernel<<<G, kVecBlock, 0, s>>>(n, x.V, z, sc + S_VN2, sc + S_ZN2, Vp, sc + S_EPS);
-        x.residual(Vp, R1);
-        fd_diff_kernel<<<G, kVecBlock, 0, s>>>(n, R1, R0, sc + S_EPS, w);
+        launch_after(fd_point_kernel, G, kVecBlock, 0, s, n, x.V, z, sc + S_VN2, sc + S_ZN2, Vp, sc + S_EPS);
+        x.residual(Vp, w, R0, sc + S_EPS);
         // classical Gram-Schmidt, twice
         x.dots(w, Bv, j + 1, dots);
-        multi_axpy_kernel<<<G, kVecBlock, 0, s>>>(n, j + 1, dots, Bv, w);
+        launch_after(multi_axpy_kernel, G, kVecBlock, 0, s, n, j + 1, dots, Bv, w, partial, nullptr, counter);
         x.dots(w, Bv, j + 1, dots + (m + 1));
-        multi_axpy_kernel<<<G, kVecBlock, 0, s>>>(n, j + 1, dots + (m + 1), Bv, w);
-        x.dots(w, w, 1, sc + S_WN2);
-        NK(cudaMemcpyAsync(hbuf.data(), dots, 2 * (m + 1) * sizeof(double), cudaMemcpyDeviceToHost, s));
-        NK(cudaMemcpyAsync(hbuf.data() + 2 * (m + 1), sc + S_WN2, sizeof(double), cudaMemcpyDeviceToHost, s));
+        launch_after(multi_axpy_kernel, G, kVecBlock, 0, s, n, j + 1, dots + (m + 1), Bv, w, partial, wn2, counter);
+        NK(cudaMemcpyAsync(hbuf, dots, nd * sizeof(double), cudaMemcpyDeviceToHost, s));
         NK(cudaStreamSynchronize(s));
         for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = hbuf[i] + hbuf[(m + 1) + i];
         const double hn = std::sqrt(hbuf[2 * (m + 1)]);
@@ -318,27 +364,27 @@ dg_status dg_newton_run(dg_newton* k, int64_t n_steps, dg_newton_stats* stats) {
         k->st.krylov_its += 1;
         if (!std::isfinite(g[j + 1])) return nfail(k, DG_ERR_NONFINITE, "non-finite Krylov residual");
         if (std::fabs(g[j + 1]) <= k->prm.krylov_rtol * beta || hn == 0.0) break;
-        if (j + 1 < m) normalize_kernel<<<G, kVecBlock, 0, s>>>(n, sc + S_WN2, w, Bv + (size_t)(j + 1) * n);
       }
       for (int i = jn - 1; i >= 0; --i) {
         double t = g[i];
         for (int l = i + 1; l < jn; ++l) t -= H[(size_t)i * m + l] * y[l];
         y[i] = t / H[(size_t)i * m + i];
       }
-      NK(cudaMemcpyAsync(dots, y.data(), jn * sizeof(double), cudaMemcpyHostToDevice, s));
-      combine_kernel<<<G, kVecBlock, 0, s>>>(n, jn, dots, Bv, u);
-      c->drv->precond(c, x.V, u, z, k->prm.dt, s);
-      add_kernel<<<G, kVecBlock, 0, s>>>(n, z, x.V);
+      // (the last copy into hbuf was waited for; the norm below waits for this one)
+      std::copy(y.begin(), y.begin() + jn, hbuf);
+      NK(cudaMemcpyAsync(dots, hbuf, jn * sizeof(double), cudaMemcpyHostToDevice, s));
+      launch_after(combine_kernel, G, kVecBlock, 0, s, n, jn, dots, Bv, u);
+      c->drv->mass_apply(c, u, mats, k->prm.dt, nullptr, nullptr, x.V, true, s);
       // ---- new residual
-      x.residual(x.V, R0);
-      e = norm2(R0, sc + S_WN2, r2);
+      x.residual(x.V, R0, nullptr, nullptr);
+      e = norm2(R0, wn2, r2);
       if (e != DG_OK) return e;
       res = std::sqrt(r2);
       ++its;
       ok = res <= std::max(k->prm.rtol * res0, k->prm.atol);
     }
     if (!std::isfinite(res)) return nfail(k, DG_ERR_NONFINITE, "non-finite Newton residual");
-    advance_time_kernel<<<1, 1, 0, s>>>(c->at<DevScalars>(c->off.sc), k->prm.dt);
+    launch_after(advance_time_kernel, 1, 1, 0, s, c->at<DevScalars>(c->off.sc), k->prm.dt);
     NK(cudaGetLastError());
     k->st.steps += 1;
     k->st.newton_its += its;
@@ -362,6 +408,9 @@ dg_status dg_newton_run(dg_newton* k, int64_t n_steps, dg_newton_stats* stats) {
 
 const char* dg_newton_last_error(const dg_newton* k) { return k ? k->err.c_str() : "null solver"; }
 
-void dg_newton_destroy(dg_newton* k) { delete k; }
+void dg_newton_destroy(dg_newton* k) {
+  if (k && k->hbuf) cudaFreeHost(k->hbuf);
+  delete k;
+}
 
 }  // extern "C"

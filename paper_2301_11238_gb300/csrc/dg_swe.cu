@@ -174,16 +174,29 @@ struct Impl final : Driver {
         c->at<int32_t>(c->off.fe2), c->at<int8_t>(c->off.ff2), c->at<R>(c->off.fnrm), c->at<R>(c->off.fsjf),
         (R*)wflux, fo, ph, nullptr, nullptr, c->at<BCEntry<R>>(c->off.bct));
   }
-  void be_time(dg_swe_ctx* c, const void* V, const void* Uold, void* out, double inv_dt, int mode,
-               cudaStream_t s) override {
-    const int K = (int)c->mesh.K;
-    be_time_kernel<DIM, P, R><<<(K + kBlock - 1) / kBlock, kBlock, 0, s>>>(
-        K, (const R*)V, (const R*)Uold, (R*)out, c->at<R>(c->off.geo), vo, (R)inv_dt, mode);
+  [[maybe_unused]] static constexpr int kNkElements = kNkBlock / nk_lanes<DIM, P>();
+  void be_time(dg_swe_ctx* c, const double* V, const double* Uold, double* out, double inv_dt, int mode,
+               const double* R0, const double* eps, cudaStream_t s) override {
+    if constexpr (sizeof(R) == 8) {
+      const int K = (int)c->mesh.K;
+      launch_after(be_time_kernel<DIM, P>, (K + kNkElements - 1) / kNkElements, kNkBlock, 0, s, K, V, Uold, out,
+                   c->at<double>(c->off.geo), vo, inv_dt, mode, R0, eps);
+    }
   }
-  void precond(dg_swe_ctx* c, const void* V, const void* x, void* z, double scale, cudaStream_t s) override {
-    const int K = (int)c->mesh.K;
-    mass_precond_kernel<DIM, P, R><<<(K + kBlock - 1) / kBlock, kBlock, 0, s>>>(
-        K, (const R*)V, (const R*)x, (R*)z, c->at<R>(c->off.geo), vo, ph.h_floor, (R)scale);
+  void mass_factor(dg_swe_ctx* c, const double* V, double* mats, cudaStream_t s) override {
+    if constexpr (sizeof(R) == 8) {
+      const int K = (int)c->mesh.K;
+      launch_after(mass_factor_kernel<DIM, P>, (K + kNkElements - 1) / kNkElements, kNkBlock, 0, s, K, V, mats, vo,
+                   ph.h_floor);
+    }
+  }
+  void mass_apply(dg_swe_ctx* c, const double* x, const double* mats, double scale, const double* nrm2, double* xn,
+                  double* out, bool add, cudaStream_t s) override {
+    if constexpr (sizeof(R) == 8) {
+      const int K = (int)c->mesh.K;
+      launch_after(mass_apply_kernel<DIM, P>, (K + kNkElements - 1) / kNkElements, kNkBlock, 0, s, K, x, mats,
+                   c->at<double>(c->off.geo), vo, scale, nrm2, xn, out, add ? 1 : 0);
+    }
   }
   void residual_from(dg_swe_ctx* c, const void* V, const void* E, const void* wflux, void* out,
                      cudaStream_t s) override {
