@@ -186,7 +186,7 @@ struct GDrv final : GroupDrv {
   explicit GDrv(const RefOps& o, bool use_tc) {
     fill_ops<DIM, P, R>(o, eo, fo, vo);
     if constexpr (sizeof(R) == 8) fill_vol_fx<DIM, P>(o, va);
-    else va = vo;
+    else fill_vol_f2<DIM, P>(o, vo, va);
     if constexpr (kTcForm) {
       tc = use_tc;
       if (tc) tcl.reset(new tc::Launcher<P, true>());

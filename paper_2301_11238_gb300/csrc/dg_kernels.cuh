@@ -1314,6 +1314,7 @@ __device__ __forceinline__ void mass_solve_dispatch(const R (&Vn)[Sh<DIM, P>::NV
 
 }  // namespace dgswe
 
+#include "dg_volume_f32.cuh"
 #include "dg_volume_fx.cuh"
 
 namespace dgswe {
@@ -1321,8 +1322,10 @@ namespace dgswe {
 // The volume pass's operator tables (a kernel parameter) and, for FP64
 // triangles, their shared-memory copy.
 template <int DIM, int P, typename R>
-struct VolArgT {
-  using type = VolOps<DIM, P, R>;
+struct VolArgT;
+template <int DIM, int P>
+struct VolArgT<DIM, P, float> {
+  using type = VolF2<DIM, P>;
   static constexpr int TAB = 2;
 };
 template <int DIM, int P>
@@ -1354,191 +1357,34 @@ __device__ __forceinline__ void vol_table(Fx* tab, const VolArg<DIM, P, R>& ops)
 // when c0 != 0).  mode 0: write dV/dt to out; mode 1: out = c0 * V0 + c1 * (Vin +
 // dt * dV/dt); mode 2: write the spatial residual r_V of Eq. WeakForm51
 // (before the mass solve).
+// Vp, Ep: where the element's values of each field lie.
 template <int DIM, int P, typename R, bool COH = false>
-__device__ __forceinline__ void volume_element(int e, int K, int F, const R (&Vn)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
-                                               const R (&En)[Sh<DIM, P>::NE][Sh<DIM, P>::NP],
-                                               const R* __restrict__ bed_e,
-                                               const R* const (&V0e)[Sh<DIM, P>::NV],
-                                               R* out,
-                                               const R* __restrict__ geo, const int32_t* __restrict__ fid,
-                                               const R* __restrict__ wflux, const VolOps<DIM, P, R>& ops,
-                                               const Phys<R>& ph, int ins, int mode, R c0, R c1,
-                                               const DevScalars* __restrict__ sc) {
-  using S = Sh<DIM, P>;
-  constexpr int NP = S::NP, NQ = S::NQ, NF = S::NF, NFP = S::NFP, NFQ = S::NFQ, NV = S::NV, NE = S::NE;
-  const size_t KN = (size_t)K * NP;
-  const size_t eo = (size_t)e * NP;
-  R G[2][2];
-  G[0][0] = geo[e];
-  if constexpr (DIM == 2) {
-    G[0][1] = geo[K + e];
-    G[1][0] = geo[2 * K + e];
-    G[1][1] = geo[3 * K + e];
-  }
-  const R J = geo[4 * K + e];
-  R r[NV][NP];
-#pragma unroll
-  for (int v = 0; v < NV; ++v)
-#pragma unroll
-    for (int a = 0; a < NP; ++a) r[v][a] = R(0);
-
-  const bool has_bed = bed_e != nullptr;
-  R Hn[NP];
-#pragma unroll
-  for (int a = 0; a < NP; ++a) Hn[a] = has_bed ? bed_e[a] : R(0);
-
-  // ---- volume integrals: -<grad N, F - Q> - <N, S>  (Eq. WeakForm51)
-#pragma unroll 1
-  for (int q = 0; q < NQ; ++q) {
-    R Vq[NV], Eq[NE];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) Vq[v] = R(0);
-#pragma unroll
-    for (int c = 0; c < NE; ++c) Eq[c] = R(0);
-    R Hr = R(0), Hs = R(0);
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      const R l = ops.Vq[q * NP + a];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Vq[v] += l * Vn[v][a];
-#pragma unroll
-      for (int c = 0; c < NE; ++c) Eq[c] += l * En[c][a];
-      if (has_bed) {
-        Hr += ops.Drq[q * NP + a] * Hn[a];
-        if constexpr (DIM == 2) Hs += ops.Dsq[q * NP + a] * Hn[a];
-      }
-    }
-    const R h = Vq[0];
-    const R hr = h * ph.rho_inv;
-    R sig[DIM][DIM];
-    stress<DIM, R>(Eq, ph, sig);
-    R fx[DIM][NV];  // (Q - F) in direction i
-#pragma unroll
-    for (int i = 0; i < DIM; ++i) {
-      fx[i][0] = -h * Vq[1 + i];
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) fx[i][1 + j] = -h * Vq[1 + i] * Vq[1 + j] + hr * sig[j][i];
-      fx[i][1 + i] -= R(0.5) * ph.gc * h * h;
-    }
-    R Sv[NV];
-    Sv[0] = R(0);
-    R dH[DIM];
-#pragma unroll
-    for (int i = 0; i < DIM; ++i) {
-      dH[i] = G[0][i] * Hr;
-      if constexpr (DIM == 2) dH[i] += G[1][i] * Hs;
-    }
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) Sv[1 + j] = -ph.gc * h * dH[j];
-    Sv[1] -= ph.gs * h;
-    R fr[NV], fs[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      fr[v] = G[0][0] * fx[0][v];
-      fs[v] = R(0);
-      if constexpr (DIM == 2) {
-        fr[v] += G[0][1] * fx[1][v];
-        fs[v] = G[1][0] * fx[0][v] + G[1][1] * fx[1][v];
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      const R wr = ops.Wr[q * NP + a];
-      const R ws = DIM == 1 ? R(0) : ops.Ws[q * NP + a];
-      const R wm = ops.Wm[q * NP + a];
-      // accumulated straight into r, three fused multiply-adds per entry
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        R t = r[v][a];
-        t += wr * fr[v];
-        if constexpr (DIM == 2) t += ws * fs[v];
-        if (v > 0) t -= wm * Sv[v];  // the depth equation has no source
-        r[v][a] = t;
-      }
-    }
-  }
-#pragma unroll
-  for (int v = 0; v < NV; ++v)
-#pragma unroll
-    for (int a = 0; a < NP; ++a) r[v][a] *= J;
-
-  // ---- face terms <N^-, F_bar.n - Q_bar.n> (weights and sJ folded into wflux)
-  const size_t FQ = (size_t)F * NFQ;
-#pragma unroll
-  for (int f = 0; f < NF; ++f) {
-    const uint32_t raw = (uint32_t)fid[f * K + e];
-    const bool own = (raw & 0x80000000u) == 0;
-    const size_t base = (size_t)(raw & 0x7fffffffu) * NFQ;
-    R fv[NV][NFQ];
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int m = 0; m < NFQ; ++m) {
-        const R x = DG_LDC(COH, wflux, v * FQ + base + (own ? m : NFQ - 1 - m));
-        fv[v][m] = own ? x : -x;
-      }
-#pragma unroll
-    for (int k = 0; k < NFP; ++k) {
-      const int a = face_node(DIM, P, f, k);
-#pragma unroll
-      for (int v = 0; v < NV; ++v)
-#pragma unroll
-        for (int m = 0; m < NFQ; ++m) r[v][a] += ops.LfT[k * NFQ + m] * fv[v][m];
-    }
-  }
-
-  // mode 2: the spatial residual r_V itself (physical scaling), for the
-  // implicit integrators that assemble their own time term
-  if (mode == 2) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int a = 0; a < NP; ++a) out[v * KN + eo + a] = r[v][a];
-    return;
-  }
-
-  // ---- mass solve: M dh/dt = -r_h ; M_h du/dt = -r_u - M_u dh/dt
-  R dV[NV][NP];
-  mass_solve_dispatch<DIM, P, R>(Vn, r, ops, ph, geo[6 * K + e], dV);
-
-  // ---- output
-  if (mode == 0) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int a = 0; a < NP; ++a) out[v * KN + eo + a] = dV[v][a];
-  } else {
-    const R dt = (R)DG_LDC(COH, &sc[ins].dt, 0);
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int a = 0; a < NP; ++a) {
-        const R vi = Vn[v][a];
-        R y = c1 * (vi + dt * dV[v][a]);
-        if (c0 != R(0)) y += c0 * DG_LDC(COH, V0e[v], a);
-        dV[v][a] = y;
-      }
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int a = 0; a < NP; ++a) out[v * KN + eo + a] = dV[v][a];
-  }
-}
-
-template <int DIM, int P, typename R, bool COH = false>
-__device__ __forceinline__ void volume_any(int e, int K, int F, const R (&Vn)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
-                                           const R (&En)[Sh<DIM, P>::NE][Sh<DIM, P>::NP],
-                                           const R* __restrict__ bed_e, const R* __restrict__ src,
-                                           const R* const (&V0e)[Sh<DIM, P>::NV], R* out,
+__device__ __forceinline__ void volume_any(int e, int K, int F, const R* const (&Vp)[Sh<DIM, P>::NV],
+                                           const R* const (&Ep)[Sh<DIM, P>::NE], const R* __restrict__ bed_e,
+                                           const R* __restrict__ src, const R* const (&V0e)[Sh<DIM, P>::NV], R* out,
                                            const R* __restrict__ geo, const int32_t* __restrict__ fid,
                                            const R* __restrict__ wflux, const VolArg<DIM, P, R>& ops,
                                            const Phys<R>& ph, int ins, int mode, R c0, R c1,
                                            const DevScalars* __restrict__ sc, const Fx* tab) {
-  if constexpr (sizeof(R) == 8)
+  using S = Sh<DIM, P>;
+  constexpr int NP = S::NP, NV = S::NV, NE = S::NE;
+  if constexpr (sizeof(R) == 8) {
+    double Vn[NV][NP], En[NE][NP];
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Vn[v][a] = DG_LDC(COH, Vp[v], a);
+#pragma unroll
+      for (int c = 0; c < NE; ++c) En[c][a] = DG_LDC(COH, Ep[c], a);
+    }
     volume_element_fx<DIM, P, COH>(e, K, F, Vn, En, src, V0e, out, geo, fid, wflux, ops, ph, ins, mode, c0, c1, sc,
                                    tab);
-  else
-    volume_element<DIM, P, R, COH>(e, K, F, Vn, En, bed_e, V0e, out, geo, fid, wflux, ops, ph, ins, mode, c0, c1, sc);
+  } else {
+    constexpr int NH = (NP + 1) / 2;
+    float2 V2[NV][NH], E2[DIM == 1 ? 1 : 3][NH];
+    load_element_f32<DIM, P, COH>(Vp, Ep, V2, E2);
+    volume_element_f32<DIM, P, COH>(e, K, F, V2, E2, bed_e, V0e, out, geo, fid, wflux, ops, ph, ins, mode, c0, c1, sc);
+  }
 }
 
 // Register cap of the direct volume kernel: 168, the most that keeps three
@@ -1575,19 +1421,15 @@ __global__ void __launch_bounds__(256) __maxnreg__((volume_max_regs<DIM, P, R>()
   const Phys<R> ph = BATCH ? ptab[ins] : ph0;
   const size_t KN = (size_t)K * NP;
   const size_t eo = (size_t)e * NP;
-  // the element's nodal values, read once (each is used at every volume point)
-  R Vn[NV][NP], En[NE][NP];
+  const R *Vp[NV], *Ep[NE], *V0e[NV];
 #pragma unroll
-  for (int a = 0; a < NP; ++a) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) Vn[v][a] = Vin[v * KN + eo + a];
-#pragma unroll
-    for (int c = 0; c < NE; ++c) En[c][a] = E[c * KN + eo + a];
+  for (int v = 0; v < NV; ++v) {
+    Vp[v] = Vin + v * KN + eo;
+    V0e[v] = V0 ? V0 + v * KN + eo : nullptr;
   }
-  const R* V0e[NV];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) V0e[v] = V0 ? V0 + v * KN + eo : nullptr;
-  volume_any<DIM, P, R>(e, K, F, Vn, En, bed ? bed + eo : nullptr, src, V0e, out, geo, fid, wflux, ops, ph, ins, mode,
+  for (int c = 0; c < NE; ++c) Ep[c] = E + c * KN + eo;
+  volume_any<DIM, P, R>(e, K, F, Vp, Ep, bed ? bed + eo : nullptr, src, V0e, out, geo, fid, wflux, ops, ph, ins, mode,
                             c0, c1, sc, tab);
 }
 
@@ -1888,18 +1730,15 @@ __global__ void __launch_bounds__(256) volume_staged_kernel(int K, int F, const 
         sV[j] = reinterpret_cast<const R*>(dsm + ((size_t)buf * NARR + j) * slot + lead) +
                 (size_t)threadIdx.x * NP;
       }
-      R Vn[NV][NP], En[NE][NP];
+      const R *Vp[NV], *Ep[NE];
 #pragma unroll
-      for (int a = 0; a < NP; ++a) {
+      for (int v = 0; v < NV; ++v) Vp[v] = sV[v];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) Vn[v][a] = sV[v][a];
-#pragma unroll
-        for (int c = 0; c < NE; ++c) En[c][a] = sV[NV + c][a];
-      }
+      for (int c = 0; c < NE; ++c) Ep[c] = sV[NV + c];
       const R* V0e[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) V0e[v] = sV[NV + NE + 1 + v];
-      volume_any<DIM, P, R>(e, K, F, Vn, En, (sizeof(R) == 4 && bed) ? sV[NV + NE] : nullptr, src, V0e, out, geo, fid, wflux, ops, ph,
+      volume_any<DIM, P, R>(e, K, F, Vp, Ep, (sizeof(R) == 4 && bed) ? sV[NV + NE] : nullptr, src, V0e, out, geo, fid, wflux, ops, ph,
                                 ins, 1, c0, c1, sc, nullptr);
     }
     __syncthreads();

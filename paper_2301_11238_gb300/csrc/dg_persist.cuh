@@ -206,18 +206,15 @@ __global__ void __launch_bounds__(kThreads) step_kernel(const Plan pl, const Arr
           const int ins = A.inst[e];
           const Phys<R> phy = A.ptab[ins];
           const size_t eo2 = (size_t)e * NP;
-          R Vn[NV][NP], En[NE][NP];
+          const R *Vp[NV], *Ep[NE];
 #pragma unroll
-          for (int a = 0; a < NP; ++a) {
+          for (int v = 0; v < NV; ++v) Vp[v] = A.V[vin] + v * KN + eo2;
 #pragma unroll
-            for (int v = 0; v < NV; ++v) Vn[v][a] = DG_LDC(true, A.V[vin], v * KN + eo2 + a);
-#pragma unroll
-            for (int c = 0; c < NE; ++c) En[c][a] = DG_LDC(true, A.E, c * KN + eo2 + a);
-          }
+          for (int c = 0; c < NE; ++c) Ep[c] = A.E + c * KN + eo2;
           const R* V0e[NV];
 #pragma unroll
           for (int v = 0; v < NV; ++v) V0e[v] = A.V[0] + v * KN + eo2;
-          volume_any<DIM, P, R, true>((int)e, K, F, Vn, En, A.bed ? A.bed + eo2 : nullptr, A.src, V0e, A.V[vout],
+          volume_any<DIM, P, R, true>((int)e, K, F, Vp, Ep, A.bed ? A.bed + eo2 : nullptr, A.src, V0e, A.V[vout],
                                           A.geo, A.fid, A.wflux, vo, phy, ins, 1, c0, c1, A.sc, tab);
         }
       }

@@ -97,7 +97,7 @@ struct Impl final : Driver {
   explicit Impl(const dg_swe_ctx& c) {
     fill_ops<DIM, P, R>(c.ops, eo, fo, vo);
     if constexpr (sizeof(R) == 8) fill_vol_fx<DIM, P>(c.ops, va);
-    else va = vo;
+    else fill_vol_f2<DIM, P>(c.ops, vo, va);
     ph = make_phys<R>(c.prm, c.reg);
     if constexpr (kTcForm) {
       tc = c.prec == DG_PREC_FP32_TC;
