@@ -224,7 +224,7 @@ struct GDrv final : GroupDrv {
     auto it = pf_grid.find(T);
     if (it != pf_grid.end()) return it->second;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, face_pf_kernel<DIM, P, R>, T, 0) != cudaSuccess || nb < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, face_pf_kernel<DIM, P, R, true>, T, 0) != cudaSuccess || nb < 1)
       nb = 1;
     cudaGetLastError();
     pf_grid[T] = nb * (n_sm > 0 ? n_sm : 1);
@@ -280,10 +280,10 @@ struct GDrv final : GroupDrv {
       // one thread per face in a grid-stride loop over the resident blocks
       // (the next face's connectivity loads while the current one computes)
       const int grid = std::max(1, std::min((F + T - 1) / T, face_pf_blocks(T)));
-      launch_after(face_pf_kernel<DIM, P, R>, (unsigned)grid, T, 0, s,
+      launch_after(face_pf_kernel<DIM, P, R, true>, (unsigned)grid, T, 0, s,
           K, F, b->at<R>(g.off.V[vin]), b->at<R>(g.off.E), b->at<int32_t>(g.off.fe1), b->at<int8_t>(g.off.ff1),
           b->at<int32_t>(g.off.fe2), b->at<int8_t>(g.off.ff2), b->at<R>(g.off.fnrm), b->at<R>(g.off.fsjf),
-          b->at<R>(g.off.wflux), fo, ptab(b), b->at<int32_t>(g.off.inst), bct(b));
+          b->at<R>(g.off.wflux), fo, Phys<R>{}, ptab(b), b->at<int32_t>(g.off.inst), bct(b));
     }
   }
   void volume(dg_batch* b, Group& g, int vin, int vout, double c0, double c1, cudaStream_t s) override {

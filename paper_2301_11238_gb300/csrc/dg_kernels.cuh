@@ -783,7 +783,7 @@ __global__ void __launch_bounds__(256, face_min_blocks<DIM, P, R>())
                                        bct);
 }
 
-// Per-face flux kernel over a grid-stride loop, for batch groups: while a
+// Per-face flux kernel over a grid-stride loop: while a
 // thread gathers and evaluates face fc, the connectivity of its next face
 // (fc + grid size: both elements and local faces, normal, scaled Jacobian)
 // is already on its way, so each face costs one dependent round trip to
@@ -791,16 +791,16 @@ __global__ void __launch_bounds__(256, face_min_blocks<DIM, P, R>())
 // face_kernel (face_point).  The gather and evaluation below restate
 // face_item's after its connectivity loads, so that face_kernel keeps its
 // own compiled form.
-template <int DIM, int P, typename R>
+template <int DIM, int P, typename R, bool BATCH>
 __device__ __forceinline__ void face_pf_body(int fc, int e1, int f1, int e2, int f2, const R (&n)[DIM], R wsj,
                                              int K, int F, const R* __restrict__ V, const R* __restrict__ E,
                                              R* __restrict__ wflux, const FaceOps<DIM, P, R>& ops,
-                                             const Phys<R>* __restrict__ ptab, const int32_t* __restrict__ inst,
-                                             const BCEntry<R>* __restrict__ bct) {
+                                             const Phys<R>& ph0, const Phys<R>* __restrict__ ptab,
+                                             const int32_t* __restrict__ inst, const BCEntry<R>* __restrict__ bct) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NFP = S::NFP, NFQ = S::NFQ, NV = S::NV, NE = S::NE;
   const size_t KN = (size_t)K * NP;
-  const Phys<R> ph = ptab[inst[e1]];
+  const Phys<R> ph = BATCH ? ptab[inst[e1]] : ph0;
   if constexpr (sizeof(R) == 8) {
     face_fx<DIM, P, false>(fc, 0, NFQ, e1, f1, e2, f2, n, wsj, K, F, V, E, wflux, ops, ph, bct);
   } else {
@@ -841,12 +841,12 @@ constexpr int face_pf_min_blocks() {
   return (sizeof(R) == 4 && P <= 2) ? 2 : 1;
 }
 
-template <int DIM, int P, typename R>
+template <int DIM, int P, typename R, bool BATCH>
 __global__ void __launch_bounds__(256, face_pf_min_blocks<DIM, P, R>())
     face_pf_kernel(int K, int F, const R* __restrict__ V, const R* __restrict__ E, const int32_t* __restrict__ fe1,
                    const int8_t* __restrict__ ff1, const int32_t* __restrict__ fe2, const int8_t* __restrict__ ff2,
                    const R* __restrict__ fnrm, const R* __restrict__ fsj, R* __restrict__ wflux,
-                   const FaceOps<DIM, P, R> ops, const Phys<R>* __restrict__ ptab, const int32_t* __restrict__ inst,
+                   const FaceOps<DIM, P, R> ops, const Phys<R> ph0, const Phys<R>* __restrict__ ptab, const int32_t* __restrict__ inst,
                    const BCEntry<R>* __restrict__ bct) {
   pdl_trigger();
   pdl_wait();
@@ -875,7 +875,7 @@ __global__ void __launch_bounds__(256, face_pf_min_blocks<DIM, P, R>())
       for (int i = 0; i < DIM; ++i) nn[i] = fnrm[(size_t)i * F + nx];
       wsjn = fsj[nx];
     }
-    face_pf_body<DIM, P, R>(fc, e1, f1, e2, f2, n, wsj, K, F, V, E, wflux, ops, ptab, inst, bct);
+    face_pf_body<DIM, P, R, BATCH>(fc, e1, f1, e2, f2, n, wsj, K, F, V, E, wflux, ops, ph0, ptab, inst, bct);
     if (!more) break;
     fc = nx;
     e1 = e1n;

@@ -1,5 +1,6 @@
 // C ABI of the GB300 DG shallow-water / regularized-Bingham solver.
 // See include/dg_swe.h for the contract of every entry point.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <memory>
@@ -16,7 +17,19 @@ using namespace dgswe;
 
 namespace {
 
-constexpr int kBlock = 128;
+// Threads a block of the stage kernels: 64 is the fastest size or within 3 % of
+// it for every kernel, order, precision and mesh of 200 to 524,288 elements
+// (128: FP64 1D p = 3 volume 28.5 against 24.6 us, FP32 p = 3 E-step 82 against 73;
+// 32: FP64 volume 63.5 against 53.3 us on 512 triangles).
+constexpr int kBlock = 64;
+// Grid-stride forms (estep_pf_kernel, face_pf_kernel) of a single context, from
+// the number of items a thread each that fills the chip (152 SMs of 256 threads,
+// at the registers these kernels take).  FP32 faces of 2D p >= 2: 13.1 against
+// 14.7 us (p = 2), 20.7 against 31.3 us (p = 3) on 80,000 triangles, 64 against
+// 105 and 103 against 204 us on 524,288, but 5.6 against 4.2 us on 8,192.  FP64
+// faces gain later: equal on 80,000 triangles, 1081 against 1324 us on 524,288
+// (p = 2).  FP32 E-step: p = 3 only, 63 against 73 us on 524,288 triangles.
+constexpr int64_t kFormItems = 152 * 256;
 constexpr int kRedBlock = 256;
 constexpr int kWetDryBlock = 128;
 constexpr int kGraphSteps = 16;
@@ -134,19 +147,35 @@ struct Impl final : Driver {
     return false;
   }
 
+  // resident blocks of a grid-stride kernel times the SMs
+  template <typename Kern>
+  static int resident(Kern k) {
+    int dev = 0, sms = 0, nb = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+      sms = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, kBlock, 0) != cudaSuccess || nb < 1) nb = 1;
+    cudaGetLastError();
+    return nb * sms;
+  }
+  int estep_grid = 0, face_grid = 0;
+
   void estep(dg_swe_ctx* c, const void* V, void* E, cudaStream_t s) override {
     const int K = (int)c->mesh.K;
+    if (DIM == 2 && P == 3 && sizeof(R) == 4 && K >= kFormItems) {
+      if (!estep_grid) estep_grid = resident(estep_pf_kernel<DIM, P, R>);
+      launch_after(estep_pf_kernel<DIM, P, R>, std::min((K + kBlock - 1) / kBlock, estep_grid), kBlock, 0, s,
+                   K, (const R*)V, (R*)E, c->at<R>(c->off.geo), c->at<int32_t>(c->off.nbr),
+                   c->at<int8_t>(c->off.nbrf), c->at<R>(c->off.fn), c->at<R>(c->off.fsj), eo,
+                   c->at<BCEntry<R>>(c->off.bct));
+      return;
+    }
     launch_after(estep_kernel<DIM, P, R>, (K + kBlock - 1) / kBlock, kBlock, 0, s,
-        K, (const R*)V, (R*)E, c->at<R>(c->off.geo), c->at<int32_t>(c->off.nbr), c->at<int8_t>(c->off.nbrf),
-        c->at<R>(c->off.fn), c->at<R>(c->off.fsj), eo, c->at<BCEntry<R>>(c->off.bct));
+                 K, (const R*)V, (R*)E, c->at<R>(c->off.geo), c->at<int32_t>(c->off.nbr), c->at<int8_t>(c->off.nbrf),
+                 c->at<R>(c->off.fn), c->at<R>(c->off.fsj), eo, c->at<BCEntry<R>>(c->off.bct));
   }
   void face(dg_swe_ctx* c, const void* V, const void* E, cudaStream_t s) override {
-    const int K = (int)c->mesh.K, F = (int)c->mesh.F;
-    const long long n = (long long)F * S::NFQ;
-    launch_after(face_kernel<DIM, P, R, false, false>, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s,
-        K, F, (const R*)V, (const R*)E, c->at<int32_t>(c->off.fe1), c->at<int8_t>(c->off.ff1),
-        c->at<int32_t>(c->off.fe2), c->at<int8_t>(c->off.ff2), c->at<R>(c->off.fnrm), c->at<R>(c->off.fsjf),
-        c->at<R>(c->off.wflux), fo, ph, nullptr, nullptr, c->at<BCEntry<R>>(c->off.bct));
+    face_into(c, V, E, c->ws + c->off.wflux, s);
   }
   void volume(dg_swe_ctx* c, const void* Vin, const void* V0, void* out, int mode, double c0, double c1,
               cudaStream_t s) override {
@@ -168,11 +197,19 @@ struct Impl final : Driver {
   }
   void face_into(dg_swe_ctx* c, const void* V, const void* E, void* wflux, cudaStream_t s) override {
     const int K = (int)c->mesh.K, F = (int)c->mesh.F;
+    if (DIM == 2 && P >= 2 && F >= (sizeof(R) == 4 ? 1 : 8) * kFormItems) {
+      if (!face_grid) face_grid = resident(face_pf_kernel<DIM, P, R, false>);
+      launch_after(face_pf_kernel<DIM, P, R, false>, std::min((F + kBlock - 1) / kBlock, face_grid), kBlock, 0, s,
+                   K, F, (const R*)V, (const R*)E, c->at<int32_t>(c->off.fe1), c->at<int8_t>(c->off.ff1),
+                   c->at<int32_t>(c->off.fe2), c->at<int8_t>(c->off.ff2), c->at<R>(c->off.fnrm), c->at<R>(c->off.fsjf),
+                   (R*)wflux, fo, ph, nullptr, nullptr, c->at<BCEntry<R>>(c->off.bct));
+      return;
+    }
     const long long n = (long long)F * S::NFQ;
     launch_after(face_kernel<DIM, P, R, false, false>, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s,
-        K, F, (const R*)V, (const R*)E, c->at<int32_t>(c->off.fe1), c->at<int8_t>(c->off.ff1),
-        c->at<int32_t>(c->off.fe2), c->at<int8_t>(c->off.ff2), c->at<R>(c->off.fnrm), c->at<R>(c->off.fsjf),
-        (R*)wflux, fo, ph, nullptr, nullptr, c->at<BCEntry<R>>(c->off.bct));
+                 K, F, (const R*)V, (const R*)E, c->at<int32_t>(c->off.fe1), c->at<int8_t>(c->off.ff1),
+                 c->at<int32_t>(c->off.fe2), c->at<int8_t>(c->off.ff2), c->at<R>(c->off.fnrm), c->at<R>(c->off.fsjf),
+                 (R*)wflux, fo, ph, nullptr, nullptr, c->at<BCEntry<R>>(c->off.bct));
   }
   [[maybe_unused]] static constexpr int kNkElements = kNkBlock / nk_lanes<DIM, P>();
   void be_time(dg_swe_ctx* c, const double* V, const double* Uold, double* out, double inv_dt, int mode,
