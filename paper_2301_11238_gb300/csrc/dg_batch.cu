@@ -93,6 +93,7 @@ struct dg_batch {
   std::vector<cudaStream_t> side;     // capture streams of the groups after the first
   std::vector<cudaEvent_t> side_ev;
   cudaGraphExec_t g1 = nullptr, gN = nullptr;
+  DevScalars* h_sc = nullptr;  // host side of read_stats, one per instance
   std::string err;
   template <typename T>
   T* at(size_t o) const { return reinterpret_cast<T*>(ws + o); }
@@ -162,7 +163,10 @@ static __global__ void mass_members_kernel(int first, int count, const int32_t* 
   if (lane == 0) {
     DevScalars& d = sc[gid[i]];
     d.mass = m;
-    if (set_ref) d.mass0 = m;
+    if (set_ref) {
+      d.mass0 = m;
+      reset_scalars(d);
+    }
   }
 }
 
@@ -559,13 +563,17 @@ dg_status check(dg_batch* b) {
 }
 
 template <typename Rin, typename Rout>
-void conv(const void* in, void* out, size_t n, cudaStream_t s) {
-  if (n) launch_after(convert_kernel<Rin, Rout>, (unsigned)((n + 255) / 256), 256, 0, s, n, (const Rin*)in, (Rout*)out);
+void fields(int nf, size_t n, const void* in, size_t sin, void* out, size_t sout, cudaStream_t s) {
+  if (n)
+    launch_after(fields_kernel<Rin, Rout>, (unsigned)((n + 255) / 256), 256, 0, s, nf, n, (const Rin*)in, sin,
+                 (Rout*)out, sout);
 }
 
 dg_status read_stats(dg_batch* b, dg_swe_stats* st) {
-  std::vector<DevScalars> h(b->n);
-  BK(cudaMemcpyAsync(h.data(), b->at<DevScalars>(b->off_sc), b->n * sizeof(DevScalars), cudaMemcpyDeviceToHost,
+  // pinned, so that the copy is one DMA in the stream (a pageable one is staged)
+  if (!b->h_sc) BK(cudaHostAlloc((void**)&b->h_sc, b->n * sizeof(DevScalars), cudaHostAllocDefault));
+  const DevScalars* h = b->h_sc;
+  BK(cudaMemcpyAsync(b->h_sc, b->at<DevScalars>(b->off_sc), b->n * sizeof(DevScalars), cudaMemcpyDeviceToHost,
                      b->stream));
   BK(cudaStreamSynchronize(b->stream));
   int bad = -1;
@@ -925,7 +933,7 @@ dg_status dg_batch_set_workspace(dg_batch* b, void* ptr, size_t bytes) {
   BK(up(b->off_ptab, b->h_phys.data(), b->h_phys.size()));
   BK(up(b->off_bct, b->h_bc.data(), b->h_bc.size()));
   BK(up(b->off_iparm, b->h_iparm.data(), b->h_iparm.size() * 8));
-  launch_after(reset_scalars_array_kernel, (b->n + 127) / 128, 128, 0, s, b->n, b->at<DevScalars>(b->off_sc));
+  launch_after(reset_scalars_kernel, (b->n + 127) / 128, 128, 0, s, b->n, b->at<DevScalars>(b->off_sc));
   BK(cudaGetLastError());
   BK(cudaStreamSynchronize(s));
   return DG_OK;
@@ -940,20 +948,24 @@ dg_status dg_batch_set_state(dg_batch* b, int i, const double* V, int on_device)
   const int64_t K = b->K_of[i], Np = b->Np_of[i], eb = g.ebase[mi];
   const int nV = g.dim + 1;
   cudaStream_t s = b->stream;
-  for (int f = 0; f < nV; ++f) {
-    char* dst = b->ws + g.off.V[0] + ((size_t)f * g.K + eb) * Np * b->rsize;
-    const double* src = V + (size_t)f * K * Np;
+  // one launch for a device state; a host state field by field
+  const size_t n = (size_t)K * Np, ng = (size_t)g.K * Np;
+  char* dst = b->ws + g.off.V[0] + (size_t)eb * Np * b->rsize;
+  if (on_device) {
+    if (b->rsize == 8) fields<double, double>(nV, n, V, n, dst, ng, s);
+    else fields<double, float>(nV, n, V, n, dst, ng, s);
+  }
+  for (int f = 0; f < nV && !on_device; ++f) {
+    char* df = dst + f * ng * b->rsize;
+    const double* src = V + f * n;
     if (b->rsize == 8) {
-      BK(cudaMemcpyAsync(dst, src, K * Np * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-    } else if (on_device) {
-      conv<double, float>(src, dst, K * Np, s);
+      BK(cudaMemcpyAsync(df, src, n * 8, cudaMemcpyHostToDevice, s));
     } else {
-      std::vector<float> h(src, src + K * Np);
-      BK(cudaMemcpyAsync(dst, h.data(), h.size() * 4, cudaMemcpyHostToDevice, s));
+      std::vector<float> h(src, src + n);
+      BK(cudaMemcpyAsync(df, h.data(), n * 4, cudaMemcpyHostToDevice, s));
       BK(cudaStreamSynchronize(s));
     }
   }
-  launch_after(reset_scalars_array_kernel, 1, 1, 0, s, 1, b->at<DevScalars>(b->off_sc) + i);
   g.drv->mass(b, g, mi, 1, 1, s);
   BK(cudaGetLastError());
   if (!on_device) BK(cudaStreamSynchronize(s));
@@ -969,18 +981,22 @@ dg_status dg_batch_get_state(dg_batch* b, int i, double* V, int on_device) {
   const int64_t K = b->K_of[i], Np = b->Np_of[i], eb = g.ebase[mi];
   const int nV = g.dim + 1;
   cudaStream_t s = b->stream;
-  for (int f = 0; f < nV; ++f) {
-    const char* src = b->ws + g.off.V[0] + ((size_t)f * g.K + eb) * Np * b->rsize;
-    double* dst = V + (size_t)f * K * Np;
+  const size_t n = (size_t)K * Np, ng = (size_t)g.K * Np;
+  const char* src = b->ws + g.off.V[0] + (size_t)eb * Np * b->rsize;
+  if (on_device) {
+    if (b->rsize == 8) fields<double, double>(nV, n, src, ng, V, n, s);
+    else fields<float, double>(nV, n, src, ng, V, n, s);
+  }
+  for (int f = 0; f < nV && !on_device; ++f) {
+    const char* sf = src + f * ng * b->rsize;
+    double* dst = V + f * n;
     if (b->rsize == 8) {
-      BK(cudaMemcpyAsync(dst, src, K * Np * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
-    } else if (on_device) {
-      conv<float, double>(src, dst, K * Np, s);
+      BK(cudaMemcpyAsync(dst, sf, n * 8, cudaMemcpyDeviceToHost, s));
     } else {
-      std::vector<float> h(K * Np);
-      BK(cudaMemcpyAsync(h.data(), src, h.size() * 4, cudaMemcpyDeviceToHost, s));
+      std::vector<float> h(n);
+      BK(cudaMemcpyAsync(h.data(), sf, n * 4, cudaMemcpyDeviceToHost, s));
       BK(cudaStreamSynchronize(s));
-      for (size_t k = 0; k < h.size(); ++k) dst[k] = h[k];
+      for (size_t k = 0; k < n; ++k) dst[k] = h[k];
     }
   }
   BK(cudaGetLastError());
@@ -1191,6 +1207,7 @@ void dg_batch_destroy(dg_batch* b) {
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
   if (b->ev_join) cudaEventDestroy(b->ev_join);
   if (b->priv) cudaStreamDestroy(b->priv);
+  if (b->h_sc) cudaFreeHost(b->h_sc);
   delete b;
 }
 

@@ -67,6 +67,7 @@ struct dg_swe_ctx {
   cudaStream_t priv = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaGraphExec_t g1 = nullptr, gN = nullptr;
+  void* h_sc = nullptr;  // pinned host copy of the scalar block (read_scalars)
   dgswe::DriverPtr drv;
   std::string err;
 

@@ -131,6 +131,16 @@ struct DevScalars {
   int pad;
 };
 
+// Time and step counters of a new state.
+__host__ __device__ inline void reset_scalars(DevScalars& s) {
+  s.dt = 0.0;
+  s.t = 0.0;
+  s.dt_min = 1e300;
+  s.dt_max = 0.0;
+  s.steps = 0;
+  s.status = 0;
+}
+
 // ------------------------------------------------------------------ arithmetic helpers
 // FP64 kernels take the positive reciprocals and roots of dg_math64.cuh and
 // IEEE division elsewhere.  FP32 uses the fast hardware forms
@@ -1958,7 +1968,8 @@ __device__ __forceinline__ void two_sum(double a, double b, double& s, double& e
 
 // Compensated sum of the block partials (one block of 256 threads): each thread
 // adds a contiguous share, then the shares are added in a fixed tree; the
-// rounding errors are carried along.  set_ref: mass0 too.  (One thread adding
+// rounding errors are carried along.  set_ref: mass0 too, and the counters of a
+// new state.  (One thread adding
 // all of them took 70 clocks an addition, four additions a partial.)
 static __global__ void __launch_bounds__(256) mass_finalize_kernel(int nblocks, const double* __restrict__ partial,
                                                                    int set_ref, DevScalars* __restrict__ sc) {
@@ -1987,7 +1998,10 @@ static __global__ void __launch_bounds__(256) mass_finalize_kernel(int nblocks, 
   if (t == 0) {
     const double m = sh[0] + sl[0];
     sc->mass = m;
-    if (set_ref) sc->mass0 = m;
+    if (set_ref) {
+      sc->mass0 = m;
+      reset_scalars(*sc);
+    }
   }
 }
 
@@ -2046,18 +2060,11 @@ static __global__ void __launch_bounds__(256) dt_members_kernel(const int32_t* _
   }
 }
 
-static __global__ void reset_scalars_array_kernel(int n, DevScalars* sc) {
+static __global__ void reset_scalars_kernel(int n, DevScalars* sc) {
   pdl_trigger();
   pdl_wait();
-
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  sc[i].dt = 0.0;
-  sc[i].t = 0.0;
-  sc[i].dt_min = 1e300;
-  sc[i].dt_max = 0.0;
-  sc[i].steps = 0;
-  sc[i].status = 0;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) reset_scalars(sc[i]);
 }
 
 // ------------------------------------------------------------------ host: operator tables
@@ -2162,6 +2169,19 @@ inline double max_bingham_slope(int reg, double sigma0, double gamma, double pap
   }
 }
 
+// nf contiguous fields of n values each between a caller's array (stride n) and a
+// group's (stride ng), converted.
+template <typename Rin, typename Rout>
+__global__ void __launch_bounds__(256) fields_kernel(int nf, size_t n, const Rin* __restrict__ in, size_t sin,
+                                                     Rout* __restrict__ out, size_t sout) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(in);
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n)
+    for (int f = 0; f < nf; ++f) out[f * sout + i] = (Rout)in[f * sin + i];
+}
+
 template <typename Rin, typename Rout>
 __global__ void convert_kernel(size_t n, const Rin* __restrict__ in, Rout* __restrict__ out) {
   pdl_trigger();
@@ -2169,18 +2189,6 @@ __global__ void convert_kernel(size_t n, const Rin* __restrict__ in, Rout* __res
   after_wait(in);
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = (Rout)in[i];
-}
-
-static __global__ void reset_scalars_kernel(DevScalars* sc) {
-  pdl_trigger();
-  pdl_wait();
-
-  sc->dt = 0.0;
-  sc->t = 0.0;
-  sc->dt_min = 1e300;
-  sc->dt_max = 0.0;
-  sc->steps = 0;
-  sc->status = 0;
 }
 
 }  // namespace dgswe

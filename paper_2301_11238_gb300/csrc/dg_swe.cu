@@ -338,8 +338,11 @@ dg_status capture(dg_swe_ctx* c, int nsteps, cudaGraphExec_t* out) {
 }
 
 dg_status read_scalars(dg_swe_ctx* c, DevScalars* h) {
-  CK(cudaMemcpyAsync(h, c->at<DevScalars>(c->off.sc), sizeof(DevScalars), cudaMemcpyDeviceToHost, c->stream));
+  // pinned, so that the copy is one DMA in the stream (a pageable one is staged)
+  if (!c->h_sc) CK(cudaHostAlloc(&c->h_sc, sizeof(DevScalars), cudaHostAllocDefault));
+  CK(cudaMemcpyAsync(c->h_sc, c->at<DevScalars>(c->off.sc), sizeof(DevScalars), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
+  *h = *static_cast<DevScalars*>(c->h_sc);
   return DG_OK;
 }
 
@@ -528,7 +531,7 @@ dg_status dg_swe_set_workspace(dg_swe_ctx* c, void* ptr, size_t bytes) {
     CK(cudaStreamSynchronize(s));
   }
   CK(cudaMemsetAsync(c->ws + c->off.E, 0, (size_t)c->dim * c->dim * K * c->ops.Np * c->rsize, s));
-  launch_after(reset_scalars_kernel, 1, 1, 0, s, c->at<DevScalars>(c->off.sc));
+  launch_after(reset_scalars_kernel, 1, 1, 0, s, 1, c->at<DevScalars>(c->off.sc));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
   return DG_OK;
@@ -566,7 +569,6 @@ dg_status dg_swe_set_state(dg_swe_ctx* c, const double* V, int on_device) {
     CK(cudaMemcpyAsync(V0, f.data(), n * 4, cudaMemcpyHostToDevice, s));
     CK(cudaStreamSynchronize(s));
   }
-  launch_after(reset_scalars_kernel, 1, 1, 0, s, c->at<DevScalars>(c->off.sc));
   enqueue_mass(c, 1, s);
   CK(cudaGetLastError());
   if (!on_device) CK(cudaStreamSynchronize(s));
@@ -856,6 +858,7 @@ void dg_swe_destroy(dg_swe_ctx* c) {
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->priv) cudaStreamDestroy(c->priv);
+  if (c->h_sc) cudaFreeHost(c->h_sc);
   delete c;
 }
 
