@@ -529,10 +529,24 @@ __device__ __forceinline__ void estep_element(int e, int K, const R* __restrict_
   } else {
     const size_t KN = (size_t)K * NP;
     R u[DIM][NP];
+    // pairs of nodes in 64-bit loads and stores where NP is even (rows are then
+    // 8-byte aligned): half as many memory instructions of 32 lanes NP words apart
+    constexpr bool kPairs = NP % 2 == 0 && !COH;
 #pragma unroll
-    for (int j = 0; j < DIM; ++j)
+    for (int j = 0; j < DIM; ++j) {
+      if constexpr (kPairs) {
+        const float2* p = reinterpret_cast<const float2*>(V + (1 + j) * KN + (size_t)e * NP);
 #pragma unroll
-      for (int a = 0; a < NP; ++a) u[j][a] = DG_LDC(COH, V, (1 + j) * KN + (size_t)e * NP + a);
+        for (int a = 0; a < NP / 2; ++a) {
+          const float2 x = p[a];
+          u[j][2 * a] = x.x;
+          u[j][2 * a + 1] = x.y;
+        }
+      } else {
+#pragma unroll
+        for (int a = 0; a < NP; ++a) u[j][a] = DG_LDC(COH, V, (1 + j) * KN + (size_t)e * NP + a);
+      }
+    }
     R G[2][2];
     G[0][0] = geo[e];
     if constexpr (DIM == 2) {
@@ -614,9 +628,16 @@ __device__ __forceinline__ void estep_element(int e, int K, const R* __restrict_
       }
     }
 #pragma unroll
-    for (int c = 0; c < NE; ++c)
+    for (int c = 0; c < NE; ++c) {
+      if constexpr (kPairs) {
+        float2* p = reinterpret_cast<float2*>(E + c * KN + (size_t)e * NP);
 #pragma unroll
-      for (int a = 0; a < NP; ++a) E[c * KN + (size_t)e * NP + a] = Eo[c][a];
+        for (int a = 0; a < NP / 2; ++a) p[a] = make_float2(Eo[c][2 * a], Eo[c][2 * a + 1]);
+      } else {
+#pragma unroll
+        for (int a = 0; a < NP; ++a) E[c * KN + (size_t)e * NP + a] = Eo[c][a];
+      }
+    }
   }
 }
 
@@ -941,6 +962,13 @@ __global__ void __launch_bounds__(256, estep_min_blocks<R>()) estep_pf_kernel(in
   }
 }
 
+// Minimum (FP64: as integers, off the FP64 pipe; a NaN is then kept or skipped by
+// its bits, and a stage with one stays non-finite through its other sums).
+template <typename T>
+__device__ __forceinline__ T min_depth(T x, T y) { return fmin(x, y); }
+template <>
+__device__ __forceinline__ double min_depth<double>(double x, double y) { return min_f64(x, y); }
+
 // Unroll factor of the wet/dry stage's loops: full below 2D p = 3, none there.
 template <int DIM, int P>
 constexpr int wd_unroll() {
@@ -960,14 +988,14 @@ __device__ __forceinline__ T limit_depth(T* h, const VolOps<DIM, P, R>& ops) {
 #pragma unroll (wd_unroll<DIM, P>())
   for (int a = 0; a < NP; ++a) {
     hbar += (T)ops.wavg[a] * h[a];
-    m = fmin(m, h[a]);
+    m = min_depth(m, h[a]);
   }
 #pragma unroll (wd_unroll<DIM, P>())
   for (int q = 0; q < NQ; ++q) {
     T hq = T(0);
 #pragma unroll (wd_unroll<DIM, P>())
     for (int a = 0; a < NP; ++a) hq += (T)ops.Vq[q * NP + a] * h[a];
-    m = fmin(m, hq);
+    m = min_depth(m, hq);
   }
 #pragma unroll (wd_unroll<DIM, P>())
   for (int f = 0; f < NF; ++f)
@@ -976,7 +1004,7 @@ __device__ __forceinline__ T limit_depth(T* h, const VolOps<DIM, P, R>& ops) {
       T hf = T(0);
 #pragma unroll (wd_unroll<DIM, P>())
       for (int k = 0; k < NFP; ++k) hf += (T)ops.LfT[k * NFQ + mq] * h[face_node(DIM, P, f, k)];
-      m = fmin(m, hf);
+      m = min_depth(m, hf);
     }
   if (hbar <= T(0)) {
 #pragma unroll (wd_unroll<DIM, P>())
@@ -1086,7 +1114,7 @@ __device__ __forceinline__ void conservative_stage(const R (&Vn)[Sh<DIM, P>::NV]
     T d = Mh[a * NP + a];
 #pragma unroll (wd_unroll<DIM, P>())
     for (int c = 0; c < a; ++c) d -= Mh[a * NP + c] * Mh[a * NP + c];
-    dinv[a] = T(1) / sqrt(d);
+    dinv[a] = dg_rsqrt<T>(d);
   }
   const bool dry = hbar < hf;
 #pragma unroll (wd_unroll<DIM, P>())
