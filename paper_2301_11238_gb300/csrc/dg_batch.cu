@@ -533,6 +533,7 @@ void push_phys(const dg_swe_params& p, int reg, std::vector<char>& out) {
   ph.gamma = (R)p.gamma;
   ph.beta = (R)p.beta;
   ph.half_inv_beta = (R)(0.5 / p.beta);
+  ph.yield_s2 = (R)((p.sigma0 / p.gamma) * (p.sigma0 / p.gamma));
   ph.pap_m = (R)p.pap_m;
   ph.h_floor = (R)p.h_floor;
   ph.h_dry = (R)(kDryFactor * p.h_floor);

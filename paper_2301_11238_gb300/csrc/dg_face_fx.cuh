@@ -2,85 +2,85 @@
 // and the pointwise HLL and central stress fluxes in floating point, written for
 // few FP64 instructions.  Included by dg_kernels.cuh.
 //
-// Bound by the FP64 pipe: about 117 operations a face point in 2D (175 with
+// Bound by the FP64 pipe (84 % busy): about 101 operations a face point in 2D (175 with
 // floating-point interpolation, IEEE division and square root and FP64
 // comparisons); comparisons, minima and maxima run on the integer pipe, the
 // reciprocal and roots start from the FP32 unit (dg_math64.cuh).  524,288
-// triangles, p = 2: 1060 -> 750 us, p = 1: 474 -> 342 us; 8,192 triangles,
+// triangles, p = 2: 1060 -> 587 us, p = 1: 474 -> 305 us; 8,192 triangles,
 // p = 2: 24.7 -> 20.6 us; 200 intervals: 10.3 -> 8.3 us.
 #pragma once
 
 namespace dgswe {
 
-// Symmetric-gradient components the stress needs: du/dx, or (d11, d22, 2 d12).
+// Symmetric-gradient components the stress needs: du/dx, or (d11, d22, d12).
 template <int DIM>
 constexpr int sym_comps() { return DIM == 1 ? 1 : 3; }
 
 // One side of a face point: HLL ingredients and the stress row.
 template <int DIM>
 struct Side64 {
-  double un, c;        // normal velocity, wave speed
-  double U[DIM + 1];   // h, h u
-  double F[DIM + 1];   // normal flux
-  double m, t[DIM];    // -(Q . n)_j / 2 = m t_j
+  double un, c;         // normal velocity, wave speed
+  double h, q, p;       // depth, normal discharge, g_c h^2
+  double m, t[DIM];     // -(Q . n)_j / 2 = m t_j
 };
-// nh = n / 2
 template <int DIM>
-__device__ __forceinline__ void side64(const double* V, const double* d, const double* n, const double* nh,
-                                       const Phys<double>& ph, Side64<DIM>& s) {
+__device__ __forceinline__ void side64(const double* V, const double* d, const double* n, const Phys<double>& ph,
+                                       Side64<DIM>& s) {
   const double h = V[0];
   double un = V[1] * n[0];
   if constexpr (DIM == 2) un += V[2] * n[1];
   const double gh = ph.gc * h;
   s.un = un;
   s.c = sqrt_pos(max_pos(gh, ph.gc * ph.h_floor));
-  const double q = h * un, p = h * gh;
-  s.U[0] = h;
-  s.F[0] = q;
-#pragma unroll
-  for (int j = 0; j < DIM; ++j) {
-    s.U[1 + j] = h * V[1 + j];
-    s.F[1 + j] = q * V[1 + j] + p * nh[j];
-  }
+  s.h = h;
+  s.q = h * un;
+  s.p = h * gh;
   if constexpr (DIM == 1) {
-    s.m = (stress_mu1<double>(d[0], ph) * h) * (-0.5 * ph.rho_inv);
+    s.m = stress_mu1<double>(d[0], ph) * ((-0.5 * ph.rho_inv) * h);
     s.t[0] = (2.0 * d[0]) * n[0];
   } else {
-    const double tr = d[0] + d[1], e = 0.5 * d[2];
-    const double s2 = 0.5 * (d[0] * d[0] + d[1] * d[1] + tr * tr + d[2] * e);
-    s.m = (stress_mu2<double>(s2, ph) * h) * (-0.5 * ph.rho_inv);
-    s.t[0] = (d[0] + tr) * n[0] + e * n[1];
-    s.t[1] = e * n[0] + (d[1] + tr) * n[1];
+    // a_i = d_ii + tr D; d11 a_1 + d22 a_2 = d11^2 + d22^2 + tr^2
+    const double a1 = fma(2.0, d[0], d[1]), a2 = fma(2.0, d[1], d[0]);
+    const double s2 = fma(0.5, fma(d[0], a1, d[1] * a2), d[2] * d[2]);
+    s.m = stress_mu2<double>(s2, ph) * ((-0.5 * ph.rho_inv) * h);
+    s.t[0] = a1 * n[0] + d[2] * n[1];
+    s.t[1] = d[2] * n[0] + a2 * n[1];
   }
 }
 
 // Weighted numerical flux of one point: HLL for F minus the central flux of Q.
+// With F = x F_a + y F_b + z (U_b - U_a) and F = u q + n p / 2 per side, the
+// momentum flux is A u_a + B u_b + n (x p_a + y p_b) / 2 with A = x q_a - z h_a,
+// B = y q_b + z h_b: 16 operations with the depth flux instead of 24 (upwind: x
+// or y = 1, the rest 0).  The depth flux keeps the difference of the depths: it
+// is small against c h in slow flow, A + B would round at c h.
 template <int DIM>
 __device__ __forceinline__ void flux64(const double* Vm, const double* Vp, const double* dm, const double* dp,
                                        const double* n, const Phys<double>& ph, double w, double* out) {
-  double nh[DIM];
-#pragma unroll
-  for (int j = 0; j < DIM; ++j) nh[j] = 0.5 * n[j];
   Side64<DIM> a, b;
-  side64<DIM>(Vm, dm, n, nh, ph, a);
-  side64<DIM>(Vp, dp, n, nh, ph, b);
+  side64<DIM>(Vm, dm, n, ph, a);
+  side64<DIM>(Vp, dp, n, ph, b);
   const double SL = min_f64(a.un - a.c, b.un - b.c), SR = max_f64(a.un + a.c, b.un + b.c);
-  double Fn[DIM + 1];
-  if (__double2hiint(SL) >= 0) {
-#pragma unroll
-    for (int v = 0; v < DIM + 1; ++v) Fn[v] = a.F[v];
-  } else if (__double2hiint(SR) < 0) {
-#pragma unroll
-    for (int v = 0; v < DIM + 1; ++v) Fn[v] = b.F[v];
-  } else {
-    const double inv = rcp_pos(SR - SL);
-    const double x = SR * inv, y = -SL * inv, z = SL * x;
-#pragma unroll
-    for (int v = 0; v < DIM + 1; ++v) Fn[v] = x * a.F[v] + (y * b.F[v] + z * (b.U[v] - a.U[v]));
+  double F0 = a.q, A = a.q, B = 0.0, P = a.p;
+  if (__double2hiint(SL) < 0) {
+    if (__double2hiint(SR) < 0) {
+      A = 0.0;
+      F0 = B = b.q;
+      P = b.p;
+    } else {
+      const double inv = rcp_pos(SR - SL);
+      const double x = SR * inv, y = -SL * inv, z = SL * x;
+      A = fma(x, a.q, -z * a.h);
+      B = fma(y, b.q, z * b.h);
+      P = fma(x, a.p, y * b.p);
+      F0 = fma(x, a.q, fma(y, b.q, z * (b.h - a.h)));
+    }
   }
-  out[0] = w * Fn[0];
+  out[0] = w * F0;
+  const double Ph = 0.5 * P;
 #pragma unroll
-  for (int j = 0; j < DIM; ++j) out[1 + j] = w * (Fn[1 + j] + (a.m * a.t[j] + b.m * b.t[j]));
+  for (int j = 0; j < DIM; ++j)
+    out[1 + j] = w * fma(A, Vm[1 + j], fma(B, Vp[1 + j], fma(Ph, n[j], fma(a.m, a.t[j], b.m * b.t[j]))));
 }
 
 // Traces of one side of a face at its nodes, as operands with one exponent per
@@ -113,7 +113,7 @@ __device__ __forceinline__ void load_trace64(const double* __restrict__ V, const
     for (int k = 0; k < NFP; ++k) t.x[v][k] = fx_from<5>(x[k], e);
     t.e[v] = e - 1024;
   }
-  {  // 2 d12 = E_12 + E_21
+  {  // d12 = (E_12 + E_21) / 2
     double x[NFP], y[NFP];
     int e = 0;
 #pragma unroll
@@ -127,7 +127,7 @@ __device__ __forceinline__ void load_trace64(const double* __restrict__ V, const
       const Fx p = fx_from<4>(x[k], e), q = fx_from<4>(y[k], e);
       t.x[NV + 2][k] = Fx{p.h + q.h, p.l + q.l};
     }
-    t.e[NV + 2] = e - 1023;
+    t.e[NV + 2] = e - 1024;  // (one for the format, less one for the half)
   }
 }
 template <int DIM, int P>
@@ -200,7 +200,7 @@ __device__ __forceinline__ void face_fx(int fc, int m0, int m1, int e1, int f1, 
             x += ops.Lf[m * NFP + k] * DG_LDC(COH, E, KN + a);
             y += ops.Lf[m * NFP + k] * DG_LDC(COH, E, 2 * KN + a);
           }
-          dp[2] = (bc.mode[4] == 1 ? bc.val[4] : x) + (bc.mode[5] == 1 ? bc.val[5] : y);
+          dp[2] = 0.5 * ((bc.mode[4] == 1 ? bc.val[4] : x) + (bc.mode[5] == 1 ? bc.val[5] : y));
         }
       }
       flux64<DIM>(Vm, Vp, dm, dp, n, ph, ops.wf[m] * wsj, out);

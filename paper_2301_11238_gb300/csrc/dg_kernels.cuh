@@ -51,6 +51,7 @@ struct Sh {
 template <typename R>
 struct Phys {
   R gc, gs, rho_inv, eta, sigma0, gamma, beta, pap_m, h_floor;
+  R yield_s2;       // bi-viscosity: (sigma0 / gamma)^2, the s^2 at which the material yields (host-computed)
   R half_inv_beta;  // 1 / (2 beta), the half-width of the regularizations 1 and 2 (host-computed)
   R h_dry;          // FP32 contexts: depth below which an element's mass solve runs in FP64
                     // (kDryFactor x h_floor)
@@ -259,8 +260,8 @@ __device__ __forceinline__ R stress_mu2(R s2, const Phys<R>& ph) {
     // bi-viscosity with the Newtonian viscous part: gamma below the yield
     // rate (gamma s < sigma0, tested on s^2) and sigma0 / s above it, so
     // the reciprocal square root is taken only where the material yields
-    const R g = ph.gamma, s0 = ph.sigma0;
-    const R coef = s0 == R(0) ? R(0) : (less_pos<R>(g * g * s2, s0 * s0) ? g : s0 * dg_rsqrt<R>(s2));
+    const R s0 = ph.sigma0;
+    const R coef = !is_pos<R>(s0) ? R(0) : (less_pos<R>(s2, ph.yield_s2) ? ph.gamma : s0 * dg_rsqrt<R>(s2));
     return R(2) * ph.eta + coef;
   }
   // s = sqrt(nc2 / 2) and 1 / s from one reciprocal square root

@@ -7,8 +7,8 @@
 // floating point took 2065 and kept the FP64 pipe 91 % busy; the contractions
 // (interpolation, metric transform, test functions, face lift, mass matrices)
 // are 1140 integer multiply-adds of three IMAD.WIDE each.  524,288 triangles,
-// p = 2: 1969 -> 929 us, p = 1 691 -> 502 us (with the wet/dry stage kernel);
-// 73,728 triangles, p = 2: 314 -> 167 us; 8,192: 84 -> 61 us.  The FP64 pipe is
+// p = 2: 1969 -> 834 us, p = 1 691 -> 402 us (with the wet/dry stage kernel);
+// 73,728 triangles, p = 2: 314 -> 159 us; 8,192: 84 -> 52 us.  The FP64 pipe is
 // 57 % busy then: few warps (168 to 240 registers a thread) wait for one
 // another's chains.
 //
@@ -162,7 +162,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       for (int a = 0; a < NP; ++a) dx[0][a] = fx_from<5>(En[0][a], ed);
       sd[0] = fx_scale(ed - 1024 - ops.cs_v, ed <= kFxMaxExp);
     } else {
-      // d11, d22 and 2 d12 = E_12 + E_21, summed at the nodes
+      // d11, d22 and d12 = (E_12 + E_21) / 2, summed at the nodes
       constexpr int NE = S::NE;
       int e0 = 0, e3 = 0, e12 = 0;
 #pragma unroll
@@ -180,7 +180,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       }
       sd[0] = fx_scale(e0 - 1024 - ops.cs_v, e0 <= kFxMaxExp);
       sd[1 % ND] = fx_scale(e3 - 1024 - ops.cs_v, e3 <= kFxMaxExp);
-      sd[2 % ND] = fx_scale(e12 - 1023 - ops.cs_v, e12 <= kFxMaxExp);
+      sd[2 % ND] = fx_scale(e12 - 1024 - ops.cs_v, e12 <= kFxMaxExp);
     }
 #pragma unroll 1
     for (int q = tl, i = 0; q < NQ; q += T, ++i) {
@@ -213,13 +213,13 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
         Tq[0] = h * ph.rho_inv * stress_mu1<double>(d[0], ph) * (2.0 * d[0]) + (hu[0] * Vq[1] - p);
       } else {
         constexpr int Y = 1 % ND, XY = 2 % ND, U2 = 2 % NV;
-        const double tr = d[0] + d[Y];
-        // ||D||_c^2 / 2
-        const double s2 = 0.5 * (d[0] * d[0] + d[Y] * d[Y] + tr * tr) + 0.25 * (d[XY] * d[XY]);
+        // a_i = d_ii + tr D; d11 a_1 + d22 a_2 = d11^2 + d22^2 + tr^2; s2 = ||D||_c^2 / 2
+        const double a1 = fma(2.0, d[0], d[Y]), a2 = fma(2.0, d[Y], d[0]);
+        const double s2 = fma(0.5, fma(d[0], a1, d[Y] * a2), d[XY] * d[XY]);
         const double m = h * ph.rho_inv * stress_mu2<double>(s2, ph);
-        Tq[0] = m * (d[0] + tr) + (hu[0] * Vq[1] - p);
-        Tq[1 % NT] = m * (0.5 * d[XY]) + hu[0] * Vq[U2];
-        Tq[2 % NT] = m * (d[Y] + tr) + (hu[1 % DIM] * Vq[U2] - p);
+        Tq[0] = fma(m, a1, fma(hu[0], Vq[1], -p));
+        Tq[1 % NT] = fma(m, d[XY], hu[0] * Vq[U2]);
+        Tq[2 % NT] = fma(m, a2, fma(hu[1 % DIM], Vq[U2], -p));
       }
 #pragma unroll
       for (int j = 0; j < DIM; ++j) {
