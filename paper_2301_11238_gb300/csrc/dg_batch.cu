@@ -339,7 +339,7 @@ struct GDrv final : GroupDrv {
   bool split(dg_batch* b, Group& g, int vin, int vout, int mode, double c0, double c1, cudaStream_t s) {
     if constexpr (sizeof(R) == 8) {
       const int K = (int)g.K, F = (int)g.F;
-      if (!volume_split(K, sizeof(R))) return false;
+      if (!volume_split(K)) return false;
       constexpr int EB = kSplitBlock / split_lanes<DIM, P>();  // elements a block
       launch_after(volume_split_kernel<DIM, P, true>, (K + EB - 1) / EB, kSplitBlock, 0, s, K, F,
                    b->at<double>(g.off.V[vin]), mode == 1 ? b->at<double>(g.off.V[0]) : nullptr,

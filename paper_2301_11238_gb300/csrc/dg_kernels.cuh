@@ -387,8 +387,10 @@ __device__ __forceinline__ void q_normal(R h, const R* E, const R* n, const Phys
 // 4 NP conversions and 9 products are the FP64 pipe's share (2D), of 417
 // FP64 instructions in floating point at p = 2.  524,288 triangles, p = 2:
 // 411 -> 180 us; p = 1: 167 -> 67 us; 8,192 triangles, p = 2: 20.6 -> 12.5 us.
+// The components j0 .. j1 - 1 (small meshes: one a thread).
 template <int DIM, int P, bool COH, bool PRE>
-__device__ __forceinline__ void estep_element_fx(int e, int K, const double* __restrict__ V, double* __restrict__ E,
+__device__ __forceinline__ void estep_element_fx(int j0, int j1,
+                                                 int e, int K, const double* __restrict__ V, double* __restrict__ E,
                                                  const double* __restrict__ geo, const int32_t* __restrict__ nbr,
                                                  const int8_t* __restrict__ nbrf, const double* __restrict__ fn,
                                                  const double* __restrict__ fsj,
@@ -431,7 +433,7 @@ __device__ __forceinline__ void estep_element_fx(int e, int K, const double* __r
   }
   // one component at a time: both at once take 192 registers (p = 2) and half the warps
 #pragma unroll 1
-  for (int j = 0; j < DIM; ++j) {
+  for (int j = j0; j < j1; ++j) {
     double u[NP], ub[NF][NFP];
     int eu = 0;
 #pragma unroll
@@ -526,7 +528,7 @@ __device__ __forceinline__ void estep_element(int e, int K, const R* __restrict_
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NF = S::NF, NFP = S::NFP, NE = S::NE;
   if constexpr (sizeof(R) == 8) {
-    estep_element_fx<DIM, P, COH, PRE>(e, K, V, E, geo, nbr, nbrf, fn, fsj, ops, bct, pnb, pnbf);
+    estep_element_fx<DIM, P, COH, PRE>(0, DIM, e, K, V, E, geo, nbr, nbrf, fn, fsj, ops, bct, pnb, pnbf);
   } else {
     const size_t KN = (size_t)K * NP;
     R u[DIM][NP];
@@ -662,6 +664,24 @@ __global__ void __launch_bounds__(256, estep_min_blocks<R>()) estep_kernel(int K
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= K) return;
   estep_element<DIM, P, R>(e, K, V, E, geo, nbr, nbrf, fn, fsj, ops, bct);
+}
+
+// FP64 E-step of a small mesh, a thread per element and velocity component (see
+// volume_split): 8,192 triangles, p = 2: 10.5 -> 7.4 us.
+template <int DIM, int P>
+__global__ void __launch_bounds__(64) estep_split_kernel(int K, const double* __restrict__ V, double* __restrict__ E,
+                                                         const double* __restrict__ geo,
+                                                         const int32_t* __restrict__ nbr,
+                                                         const int8_t* __restrict__ nbrf,
+                                                         const double* __restrict__ fn, const double* __restrict__ fsj,
+                                                         const EstepOps<DIM, P, double> ops,
+                                                         const BCEntry<double>* __restrict__ bct) {
+  pdl_trigger();
+  pdl_wait();
+  after_wait(V);
+  const int g = blockIdx.x * blockDim.x + threadIdx.x, e = g / DIM, j = g % DIM;
+  if (e >= K) return;
+  estep_element_fx<DIM, P, false, false>(j, j + 1, e, K, V, E, geo, nbr, nbrf, fn, fsj, ops, bct, nullptr, nullptr);
 }
 
 // Numerical flux at one face point m from the traces of both sides at the
@@ -1473,17 +1493,22 @@ __global__ void __launch_bounds__(256) __maxnreg__((volume_max_regs<DIM, P, R>()
 }
 
 // FP64 volume pass for small meshes: T neighbouring lanes per element (see
-// volume_element_fx).  With one thread per element a mesh of up to 152 SMs x 4
-// sub-partitions x 32 lanes = 19,456 elements leaves each sub-partition at most
-// one warp, and the pass takes as long as one element's chain of instructions (a
-// warp-wide FP64 instruction 64 clocks, whatever the lanes); T lanes shorten the
-// chain, and the chip has room for them.
+// volume_element_fx).  A warp-wide FP64 instruction takes 64 clocks whatever the
+// lanes, so while a thread per element leaves each of the chip's 152 x 4
+// sub-partitions at most one warp, the pass takes as long as one element's chain
+// of instructions, and lanes that share an element shorten it.  The line is two
+// warps of four lanes a sub-partition, whose FP64 instructions take the time of
+// the longer chain of one.  Four lanes against a thread per
+// element, triangles, us: p = 2: 128 elements 42 / 57, 4,608 41 / 52, 9,522
+// 48 / 53; p = 1: 9,522 16 / 18; p = 3: 512 95 / 197, 9,522 139 / 220; intervals,
+// p = 1: 200 elements 9.4 / 10.9.
+constexpr int kSplitBlock = 64;
+constexpr int64_t kOneWarpEach = 152 * 4 * 32;  // threads that fill every sub-partition once
 template <int DIM, int P>
 constexpr int split_lanes() {
-  return DIM == 1 ? (P == 1 ? 2 : 4) : 4;
+  return Sh<DIM, P>::NQ < 3 ? 2 : 4;  // no more lanes than volume points
 }
-constexpr int kSplitBlock = 64;
-inline bool volume_split(int64_t K, size_t rsize) { return rsize == 8 && K <= 152 * 4 * 32; }
+inline bool volume_split(int64_t K) { return K * 2 <= kOneWarpEach; }
 
 template <int DIM, int P, bool BATCH>
 __global__ void __launch_bounds__(kSplitBlock) volume_split_kernel(

@@ -137,7 +137,7 @@ struct Impl final : Driver {
              double c0, double c1, cudaStream_t s) {
     if constexpr (sizeof(R) == 8) {
       const int K = (int)c->mesh.K, F = (int)c->mesh.F;
-      if (!volume_split(K, sizeof(R))) return false;
+      if (!volume_split(K)) return false;
       constexpr int EB = kSplitBlock / split_lanes<DIM, P>();  // elements a block
       launch_after(volume_split_kernel<DIM, P, false>, (K + EB - 1) / EB, kSplitBlock, 0, s, K, F, (const double*)Vin,
                    (const double*)V0, (double*)out, (const double*)E, c->has_bed ? c->at<double>(c->off.src) : nullptr,
@@ -170,6 +170,15 @@ struct Impl final : Driver {
                    c->at<int8_t>(c->off.nbrf), c->at<R>(c->off.fn), c->at<R>(c->off.fsj), eo,
                    c->at<BCEntry<R>>(c->off.bct));
       return;
+    }
+    if constexpr (sizeof(R) == 8 && DIM == 2) {
+      if (K * 2 <= kOneWarpEach) {
+        launch_after(estep_split_kernel<DIM, P>, (K * DIM + 63) / 64, 64, 0, s,
+                     K, (const R*)V, (R*)E, c->at<R>(c->off.geo), c->at<int32_t>(c->off.nbr),
+                     c->at<int8_t>(c->off.nbrf), c->at<R>(c->off.fn), c->at<R>(c->off.fsj), eo,
+                     c->at<BCEntry<R>>(c->off.bct));
+        return;
+      }
     }
     launch_after(estep_kernel<DIM, P, R>, (K + kBlock - 1) / kBlock, kBlock, 0, s,
                  K, (const R*)V, (R*)E, c->at<R>(c->off.geo), c->at<int32_t>(c->off.nbr), c->at<int8_t>(c->off.nbrf),
