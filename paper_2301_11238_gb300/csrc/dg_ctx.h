@@ -37,7 +37,10 @@ struct Driver {
                        const double* R0, const double* eps, cudaStream_t s) = 0;
   virtual void mass_factor(dg_swe_ctx* c, const double* V, double* mats, cudaStream_t s) = 0;
   virtual void mass_apply(dg_swe_ctx* c, const double* x, const double* mats, double scale, const double* nrm2,
-                          double* xn, double* out, bool add, cudaStream_t s) = 0;
+                          double* xn, double* out, bool add, double* partial, double* zz, unsigned* counter,
+                          cudaStream_t s) = 0;
+  // blocks of a mass_apply launch (slots of partial)
+  virtual int mass_apply_blocks(dg_swe_ctx* c) = 0;
 };
 struct DriverDeleter {
   void operator()(Driver* d) const;

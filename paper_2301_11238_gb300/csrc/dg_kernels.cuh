@@ -1615,6 +1615,12 @@ __global__ void __launch_bounds__(128) wetdry_stage_kernel(int K, const R* __res
   conservative_stage<DIM, P, R, double>(Vn, r, V0e, c0, c1, dt, ops, ph.h_floor, Jinv, out, KN, eo);
 }
 
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+
 }  // namespace dgswe
 
 #include "dg_newton_kernels.cuh"
@@ -1817,12 +1823,6 @@ __device__ __forceinline__ double warp_min(double v) {
   for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_down_sync(0xffffffffu, v, o));
   return v;
 }
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Minimum over a warp of values that are positive or exactly -1 (a flag, the
 // smallest): such values order as their bits, so the reduction runs on the
 // integer pipe (redux) instead of five FP64 minima of 64 clocks each.

@@ -26,35 +26,6 @@ inline size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // ------------------------------------------------------------------ FP64 vector kernels
 
-// Block sum of v in thread 0 (kVecBlock threads, fixed order).
-__device__ __forceinline__ double vec_block_sum(double v, double* sh) {
-  v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x < 32) t = warp_sum(threadIdx.x < kVecBlock / 32 ? sh[threadIdx.x] : 0.0);
-  return t;
-}
-// The grid's last block to finish adds the partials of every dot in a fixed
-// order: dot i = sum of partial[i * G + b] over its G blocks, a warp a dot.
-// counter is zero before and after.
-__device__ __forceinline__ void vec_finish(int G, int cnt, const double* partial, double* out, unsigned* counter) {
-  __shared__ bool last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x * gridDim.y - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  for (int i = threadIdx.x >> 5; i < cnt; i += kVecBlock / 32) {
-    double acc = 0.0;
-    for (int b = threadIdx.x & 31; b < G; b += 32) acc += __ldcg(partial + (size_t)i * G + b);
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) out[i] = acc;
-  }
-  if (threadIdx.x == 0) *counter = 0;
-}
-
 // out[i] = <x, Y_i>, Y_i = Y + i * n; grid (G, number of dots).
 __global__ void __launch_bounds__(kVecBlock) dots_kernel(size_t n, const double* __restrict__ x,
                                                          const double* __restrict__ Y, double* __restrict__ partial,
@@ -68,9 +39,9 @@ __global__ void __launch_bounds__(kVecBlock) dots_kernel(size_t n, const double*
   double acc = 0.0;
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x)
     acc += x[j] * y[j];
-  acc = vec_block_sum(acc, sh);
+  acc = block_sum_fixed(acc, sh);
   if (threadIdx.x == 0) partial[(size_t)i * gridDim.x + blockIdx.x] = acc;
-  vec_finish(gridDim.x, gridDim.y, partial, out, counter);
+  finish_sums(gridDim.x, gridDim.y, partial, out, counter);
 }
 
 // w -= sum_i c[i] Y_i; nrm2 given: and *nrm2 = <w, w>.
@@ -90,9 +61,9 @@ __global__ void __launch_bounds__(kVecBlock) multi_axpy_kernel(size_t n, int k, 
     acc += s * s;
   }
   if (!nrm2) return;
-  acc = vec_block_sum(acc, sh);
+  acc = block_sum_fixed(acc, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = acc;
-  vec_finish(gridDim.x, 1, partial, nrm2, counter);
+  finish_sums(gridDim.x, 1, partial, nrm2, counter);
 }
 
 // out = sum_i c[i] Y_i
@@ -234,7 +205,8 @@ dg_status dg_newton_init(dg_swe_ctx* c, const dg_newton_params* p, dg_newton** o
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaGetLastError();
-  k->G = std::max(1, std::min(2 * std::max(nsm, 1), (int)((k->n + kVecBlock - 1) / kVecBlock)));
+  // four entries a thread, at most two blocks an SM: few partials to finish
+  k->G = std::max(1, std::min(2 * std::max(nsm, 1), (int)((k->n + 4 * kVecBlock - 1) / (4 * kVecBlock))));
   size_t o = 0;
   auto take = [&](size_t bytes) {
     size_t r = o;
@@ -250,7 +222,7 @@ dg_status dg_newton_init(dg_swe_ctx* c, const dg_newton_params* p, dg_newton** o
   k->off.u = take(vb);
   k->off.basis = take((size_t)(k->m + 1) * vb);
   k->off.mats = take((size_t)(c->dim + 1) * (size_t)c->mesh.K * c->ops.Np * c->ops.Np * sizeof(double));
-  k->off.partial = take((size_t)(k->m + 1) * k->G * sizeof(double));
+  k->off.partial = take(std::max((size_t)(k->m + 1) * k->G, (size_t)c->drv->mass_apply_blocks(c)) * sizeof(double));
   k->off.dots = take((2 * (size_t)(k->m + 1) + 1) * sizeof(double));
   k->off.scal = take(S_COUNT * sizeof(double));
   k->off.counter = take(sizeof(unsigned));
@@ -332,8 +304,8 @@ dg_status dg_newton_run(dg_newton* k, int64_t n_steps, dg_newton_stats* stats) {
       for (int j = 0; j < m; ++j) {
         // z = dt M^{-1} v_j; from j = 1 on v_j = w / ||w|| of the last round
         double* vj = Bv + (size_t)j * n;
-        c->drv->mass_apply(c, j == 0 ? vj : w, mats, k->prm.dt, j == 0 ? nullptr : wn2, vj, z, false, s);
-        x.dots(z, z, 1, sc + S_ZN2);
+        c->drv->mass_apply(c, j == 0 ? vj : w, mats, k->prm.dt, j == 0 ? nullptr : wn2, vj, z, false, partial,
+                           sc + S_ZN2, counter, s);
         launch_after(fd_point_kernel, G, kVecBlock, 0, s, n, x.V, z, sc + S_VN2, sc + S_ZN2, Vp, sc + S_EPS);
         x.residual(Vp, w, R0, sc + S_EPS);
         // classical Gram-Schmidt, twice
@@ -374,7 +346,7 @@ dg_status dg_newton_run(dg_newton* k, int64_t n_steps, dg_newton_stats* stats) {
       std::copy(y.begin(), y.begin() + jn, hbuf);
       NK(cudaMemcpyAsync(dots, hbuf, jn * sizeof(double), cudaMemcpyHostToDevice, s));
       launch_after(combine_kernel, G, kVecBlock, 0, s, n, jn, dots, Bv, u);
-      c->drv->mass_apply(c, u, mats, k->prm.dt, nullptr, nullptr, x.V, true, s);
+      c->drv->mass_apply(c, u, mats, k->prm.dt, nullptr, nullptr, x.V, true, partial, nullptr, counter, s);
       // ---- new residual
       x.residual(x.V, R0, nullptr, nullptr);
       e = norm2(R0, wn2, r2);

@@ -34,14 +34,52 @@ __device__ __forceinline__ void nk_table(NkTab<DIM, P>& t, const VolOps<DIM, P, 
   __syncthreads();
 }
 
+// Block sum of v in thread 0 (whole warps, fixed order); sh: one slot a warp.
+__device__ __forceinline__ double block_sum_fixed(double v, double* sh) {
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < 32) t = warp_sum(threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0);
+  return t;
+}
+// Sums finished by the grid's last block: dot i is the sum of partial[i * G + b]
+// over its G blocks, a warp a dot, in a fixed order.  counter is zero before and
+// after.  Every thread of every block calls this after its block's partial has
+// been written by thread 0.
+__device__ __forceinline__ void finish_sums(int G, int cnt, const double* partial, double* out, unsigned* counter) {
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(counter, 1u) == gridDim.x * gridDim.y - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int i = threadIdx.x >> 5; i < cnt; i += blockDim.x >> 5) {
+    const double* p = partial + (size_t)i * G;
+    // eight loads in flight a lane: their latency, not the additions, was the time
+    double acc = 0.0;
+    for (int b0 = threadIdx.x & 31; b0 < G; b0 += 256) {
+      double v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = b0 + 32 * k < G ? __ldcg(p + b0 + 32 * k) : 0.0;
+      acc += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    }
+    acc = warp_sum(acc);
+    if ((threadIdx.x & 31) == 0) out[i] = acc;
+  }
+  if (threadIdx.x == 0) *counter = 0;
+}
+
 // One element's group of lanes.
 template <int DIM, int P>
 struct NkLane {
   static constexpr int GL = nk_lanes<DIM, P>(), NP = Sh<DIM, P>::NP;
   int e, a;   // element (the last one for lanes past the end), node
   bool live;  // a node of an element
-  __device__ explicit NkLane(int K) {
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  __device__ explicit NkLane(int K, long long block = -1) {
+    const long long g = (block < 0 ? (long long)blockIdx.x : block) * blockDim.x + threadIdx.x;
     const long long el = g / GL;
     a = (int)(g % GL);
     live = el < K && a < NP;
@@ -195,7 +233,8 @@ __global__ void __launch_bounds__(kNkBlock) mass_factor_kernel(int K, const doub
 }
 
 // z = scale M(V)^{-1} x.  nrm2 given: x is divided by sqrt(*nrm2) first and
-// written to xn.  add: z is added to out instead of stored.
+// written to xn.  add: z is added to out instead of stored; otherwise *zz = <z, z>
+// (partial: one slot a block).  Blocks of lane groups in a grid-stride loop.
 template <int DIM, int P>
 __global__ void __launch_bounds__(kNkBlock) mass_apply_kernel(int K, const double* __restrict__ x,
                                                               const double* __restrict__ mats,
@@ -203,7 +242,8 @@ __global__ void __launch_bounds__(kNkBlock) mass_apply_kernel(int K, const doubl
                                                               const VolOps<DIM, P, double> ops, double scale,
                                                               const double* __restrict__ nrm2,
                                                               double* __restrict__ xn, double* __restrict__ out,
-                                                              int add) {
+                                                              int add, double* partial, double* zz,
+                                                              unsigned* counter) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV, GL = nk_lanes<DIM, P>();
   pdl_trigger();
@@ -211,39 +251,52 @@ __global__ void __launch_bounds__(kNkBlock) mass_apply_kernel(int K, const doubl
   nk_table<DIM, P>(t, ops);
   pdl_wait();
   after_wait(x, mats, nrm2);
-  const NkLane<DIM, P> L(K);
-  const size_t KN = (size_t)K * NP, o = (size_t)L.e * NP + L.a;
-  const double Jinv = geo[6 * (size_t)K + L.e];
+  const size_t KN = (size_t)K * NP;
   const double nrm = nrm2 ? 1.0 / sqrt(*nrm2) : 1.0;
-  double xr[NV], z[NV];
+  const long long blocks = ((long long)K * GL + kNkBlock - 1) / kNkBlock;
+  double acc = 0.0;
+  for (long long blk = blockIdx.x; blk < blocks; blk += gridDim.x) {
+    const NkLane<DIM, P> L(K, blk);
+    const size_t o = (size_t)L.e * NP + L.a;
+    const double Jinv = geo[6 * (size_t)K + L.e];
+    double xr[NV], z[NV];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    xr[v] = nrm * x[v * KN + o];
-    if (nrm2 && L.live) xn[v * KN + o] = xr[v];
-    xr[v] *= Jinv;
+    for (int v = 0; v < NV; ++v) {
+      xr[v] = nrm * x[v * KN + o];
+      if (nrm2 && L.live) xn[v * KN + o] = xr[v];
+      xr[v] *= Jinv;
+    }
+    z[0] = 0.0;
+#pragma unroll
+    for (int b = 0; b < NP; ++b) z[0] += t.Minv[L.a * NP + b] * from_lane<GL>(xr[0], b);
+#pragma unroll
+    for (int j = 1; j < NV; ++j) {
+#pragma unroll
+      for (int b = 0; b < NP; ++b)
+        xr[j] -= mats[((j * (size_t)K + L.e) * NP + b) * NP + L.a] * from_lane<GL>(z[0], b);
+      z[j] = 0.0;
+    }
+#pragma unroll
+    for (int b = 0; b < NP; ++b) {
+      const double m = mats[((size_t)L.e * NP + b) * NP + L.a];
+#pragma unroll
+      for (int j = 1; j < NV; ++j) z[j] += m * from_lane<GL>(xr[j], b);
+    }
+    if (L.live) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const size_t i = v * KN + o;
+        const double y = scale * z[v];
+        out[i] = add ? out[i] + y : y;
+        acc += y * y;
+      }
+    }
   }
-  z[0] = 0.0;
-#pragma unroll
-  for (int b = 0; b < NP; ++b) z[0] += t.Minv[L.a * NP + b] * from_lane<GL>(xr[0], b);
-#pragma unroll
-  for (int j = 1; j < NV; ++j) {
-#pragma unroll
-    for (int b = 0; b < NP; ++b)
-      xr[j] -= mats[((j * (size_t)K + L.e) * NP + b) * NP + L.a] * from_lane<GL>(z[0], b);
-    z[j] = 0.0;
-  }
-#pragma unroll
-  for (int b = 0; b < NP; ++b) {
-    const double m = mats[((size_t)L.e * NP + b) * NP + L.a];
-#pragma unroll
-    for (int j = 1; j < NV; ++j) z[j] += m * from_lane<GL>(xr[j], b);
-  }
-  if (!L.live) return;
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const size_t i = v * KN + o;
-    out[i] = add ? out[i] + scale * z[v] : scale * z[v];
-  }
+  if (add) return;
+  __shared__ double sh[kNkBlock / 32];
+  acc = block_sum_fixed(acc, sh);
+  if (threadIdx.x == 0) partial[blockIdx.x] = acc;
+  finish_sums(gridDim.x, 1, partial, zz, counter);
 }
 
 }  // namespace dgswe

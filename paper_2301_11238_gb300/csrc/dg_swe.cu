@@ -237,13 +237,16 @@ struct Impl final : Driver {
                    ph.h_floor);
     }
   }
+  // at most four blocks of 128 threads an SM: the sums of their squares have few
+  // partials, and a lane group takes its elements in turn
+  int mass_apply_blocks(dg_swe_ctx* c) override {
+    return (int)std::min<int64_t>(4 * 152, (c->mesh.K + kNkElements - 1) / kNkElements);
+  }
   void mass_apply(dg_swe_ctx* c, const double* x, const double* mats, double scale, const double* nrm2, double* xn,
-                  double* out, bool add, cudaStream_t s) override {
-    if constexpr (sizeof(R) == 8) {
-      const int K = (int)c->mesh.K;
-      launch_after(mass_apply_kernel<DIM, P>, (K + kNkElements - 1) / kNkElements, kNkBlock, 0, s, K, x, mats,
-                   c->at<double>(c->off.geo), vo, scale, nrm2, xn, out, add ? 1 : 0);
-    }
+                  double* out, bool add, double* partial, double* zz, unsigned* counter, cudaStream_t s) override {
+    if constexpr (sizeof(R) == 8)
+      launch_after(mass_apply_kernel<DIM, P>, mass_apply_blocks(c), kNkBlock, 0, s, (int)c->mesh.K, x, mats,
+                   c->at<double>(c->off.geo), vo, scale, nrm2, xn, out, add ? 1 : 0, partial, zz, counter);
   }
   void residual_from(dg_swe_ctx* c, const void* V, const void* E, const void* wflux, void* out,
                      cudaStream_t s) override {
