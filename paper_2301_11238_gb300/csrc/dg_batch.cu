@@ -124,8 +124,8 @@ __global__ void __launch_bounds__(256) mass_block_kernel(int K, int b0, const in
                                                          const R* __restrict__ V, const R* __restrict__ geo,
                                                          const double* __restrict__ wint,
                                                          double* __restrict__ partial) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(V);
   __shared__ double red[8];
   const int b = b0 + blockIdx.x;
@@ -151,8 +151,8 @@ __global__ void __launch_bounds__(256) mass_block_kernel(int K, int b0, const in
 static __global__ void mass_members_kernel(int first, int count, const int32_t* __restrict__ mblk,
                                            const int32_t* __restrict__ gid, const double* __restrict__ partial,
                                            int set_ref, DevScalars* __restrict__ sc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(partial);
   const int i = first + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;

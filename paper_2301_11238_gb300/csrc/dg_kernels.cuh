@@ -658,8 +658,8 @@ __global__ void __launch_bounds__(256, estep_min_blocks<R>()) estep_kernel(int K
                                                     const int8_t* __restrict__ nbrf, const R* __restrict__ fn,
                                                     const R* __restrict__ fsj, const EstepOps<DIM, P, R> ops,
                                                     const BCEntry<R>* __restrict__ bct) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(V);
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= K) return;
@@ -676,8 +676,8 @@ __global__ void __launch_bounds__(64) estep_split_kernel(int K, const double* __
                                                          const double* __restrict__ fn, const double* __restrict__ fsj,
                                                          const EstepOps<DIM, P, double> ops,
                                                          const BCEntry<double>* __restrict__ bct) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(V);
   const int g = blockIdx.x * blockDim.x + threadIdx.x, e = g / DIM, j = g % DIM;
   if (e >= K) return;
@@ -824,8 +824,8 @@ __global__ void __launch_bounds__(256, face_min_blocks<DIM, P, R>())
                                                    const Phys<R> ph0, const Phys<R>* __restrict__ ptab,
                                                    const int32_t* __restrict__ inst,
                                                    const BCEntry<R>* __restrict__ bct) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(V, E);
   constexpr int NFQ = Sh<DIM, P>::NFQ;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -900,8 +900,8 @@ __global__ void __launch_bounds__(256, face_pf_min_blocks<DIM, P, R>())
                    const R* __restrict__ fnrm, const R* __restrict__ fsj, R* __restrict__ wflux,
                    const FaceOps<DIM, P, R> ops, const Phys<R> ph0, const Phys<R>* __restrict__ ptab, const int32_t* __restrict__ inst,
                    const BCEntry<R>* __restrict__ bct) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(V, E);
   const int stride = gridDim.x * blockDim.x;
   int fc = blockIdx.x * blockDim.x + threadIdx.x;
@@ -950,8 +950,8 @@ __global__ void __launch_bounds__(256, estep_min_blocks<R>()) estep_pf_kernel(in
                                                        const int8_t* __restrict__ nbrf, const R* __restrict__ fn,
                                                        const R* __restrict__ fsj, const EstepOps<DIM, P, R> ops,
                                                        const BCEntry<R>* __restrict__ bct) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(V);
   constexpr int NF = Sh<DIM, P>::NF;
   const int stride = gridDim.x * blockDim.x;
@@ -1467,12 +1467,12 @@ __global__ void __launch_bounds__(256) __maxnreg__((volume_max_regs<DIM, P, R>()
                                                      const Phys<R> ph0, const Phys<R>* __restrict__ ptab,
                                                      const int32_t* __restrict__ inst, int mode, R c0, R c1,
                                                      const DevScalars* __restrict__ sc) {
-  pdl_trigger();
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV, NE = S::NE;
   __shared__ __align__(16) Fx tab[VolArgT<DIM, P, R>::TAB];
   vol_table<DIM, P, R>(tab, ops);
   pdl_wait();
+  pdl_trigger();
   after_wait(Vin, V0, E, wflux, sc);
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= K) return;
@@ -1519,10 +1519,10 @@ __global__ void __launch_bounds__(kSplitBlock) volume_split_kernel(
     const DevScalars* __restrict__ sc) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV, NE = S::NE, T = split_lanes<DIM, P>();
-  pdl_trigger();
   __shared__ __align__(16) Fx tab[FxTab<DIM, P>::SIZE];
   vol_table<DIM, P, double>(tab, ops);
   pdl_wait();
+  pdl_trigger();
   after_wait(Vin, V0, E, wflux, sc);
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   const bool live = g / T < K;
@@ -1557,8 +1557,8 @@ __global__ void __launch_bounds__(128) wetdry_stage_kernel(int K, const R* __res
                                                            const Phys<R>* __restrict__ ptab,
                                                            const int32_t* __restrict__ inst, R c0, R c1,
                                                            const DevScalars* __restrict__ sc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(Vin, V0, rbuf, sc);
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV;
@@ -1712,8 +1712,8 @@ __global__ void __launch_bounds__(256) volume_staged_kernel(int K, int F, const 
                                                             const Phys<R>* __restrict__ ptab,
                                                             const int32_t* __restrict__ inst, R c0, R c1,
                                                             DevScalars* sc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(Vin, V0, E, wflux);
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV, NE = S::NE;
@@ -1949,8 +1949,8 @@ template <int DIM, int P, typename R>
 __global__ void __launch_bounds__(256) dt_partial_kernel(int K, const R* __restrict__ V, const R* __restrict__ geo,
                                                          double gc, double h_floor, double cfl, double nu,
                                                          double* __restrict__ partial) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(V);
   __shared__ R red[8];
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1964,8 +1964,8 @@ __global__ void __launch_bounds__(256) dt_partial_kernel(int K, const R* __restr
 // step counter.  A negative partial latches DG_ERR_NONFINITE (4).
 static __global__ void dt_finalize_kernel(int nblocks, const double* __restrict__ partial, double fixed_dt,
                                    DevScalars* __restrict__ sc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(partial);
   __shared__ double red[32];
   double v = 1e300;
@@ -1990,8 +1990,8 @@ template <int NP, typename R>
 __global__ void __launch_bounds__(256) mass_partial_kernel(int K, const R* __restrict__ V, const R* __restrict__ geo,
                                                            const double* __restrict__ wint,
                                                            double* __restrict__ partial) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(V);
   __shared__ double red[8];
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2027,8 +2027,8 @@ __device__ __forceinline__ void two_sum(double a, double b, double& s, double& e
 // all of them took 70 clocks an addition, four additions a partial.)
 static __global__ void __launch_bounds__(256) mass_finalize_kernel(int nblocks, const double* __restrict__ partial,
                                                                    int set_ref, DevScalars* __restrict__ sc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(partial);
   __shared__ double sh[256], sl[256];
   const int t = threadIdx.x, per = (nblocks + 255) / 256;
@@ -2071,8 +2071,8 @@ __global__ void __launch_bounds__(256) dt_block_kernel(int K, const int64_t* __r
                                                        const R* __restrict__ V, const R* __restrict__ geo,
                                                        const double* __restrict__ iparm,
                                                        double* __restrict__ partial) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(V);
   __shared__ R red[8];
   const int b = blockIdx.x;
@@ -2092,8 +2092,8 @@ static __global__ void __launch_bounds__(256) dt_members_kernel(const int32_t* _
                                                                 const int32_t* __restrict__ gid,
                                                                 const double* __restrict__ partial,
                                                                 DevScalars* __restrict__ sc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(partial);
   __shared__ double red[8];
   const int i = blockIdx.x;
@@ -2115,8 +2115,8 @@ static __global__ void __launch_bounds__(256) dt_members_kernel(const int32_t* _
 }
 
 static __global__ void reset_scalars_kernel(int n, DevScalars* sc) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) reset_scalars(sc[i]);
 }
@@ -2228,8 +2228,8 @@ inline double max_bingham_slope(int reg, double sigma0, double gamma, double pap
 template <typename Rin, typename Rout>
 __global__ void __launch_bounds__(256) fields_kernel(int nf, size_t n, const Rin* __restrict__ in, size_t sin,
                                                      Rout* __restrict__ out, size_t sout) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(in);
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n)
@@ -2238,8 +2238,8 @@ __global__ void __launch_bounds__(256) fields_kernel(int nf, size_t n, const Rin
 
 template <typename Rin, typename Rout>
 __global__ void convert_kernel(size_t n, const Rin* __restrict__ in, Rout* __restrict__ out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(in);
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = (Rout)in[i];

@@ -1,13 +1,16 @@
 // Programmatic dependent launch: a kernel of the explicit path may start while
-// its predecessor in the stream drains.  pdl_trigger lets the successor's blocks
-// take the room that the last blocks of this grid leave free; pdl_wait holds a
-// thread until every earlier kernel of the chain has completed and its writes
-// are visible.  Every kernel launched with launch_after calls pdl_wait before it
-// reads or writes anything that another kernel touches (only its parameters,
-// operator tables among them, may come first), so completion is transitive along
-// the stream.
+// its predecessor in the stream drains.  pdl_wait holds a thread until every
+// earlier kernel of the chain has completed and its writes are visible; only then
+// pdl_trigger lets the successor's blocks take the room that this grid leaves
+// free, so at most one grid waits (with the trigger first, three or four wait,
+// and the places they hold spread a grid's blocks unevenly over the SMs: 1D FP64,
+// 11,726 intervals, p = 2, 77 -> 173 us a step).  Every kernel launched with
+// launch_after calls pdl_wait before it reads or writes anything that another
+// kernel touches (only its parameters, operator tables among them, may come
+// first), so completion is transitive along the stream.
 #pragma once
 #include <cuda_runtime.h>
+#include <type_traits>
 
 namespace dgswe {
 
@@ -23,10 +26,19 @@ __device__ __forceinline__ void after_wait(T&... p) {
   (hide_pointer(p), ...);
 }
 
-// Grids beyond the chip's room for threads (152 SMs of 2,048) start the plain
-// way: their last blocks gain nothing from company, and the successor's waiting
-// blocks cost them 1 % (2,097,152 FP32 triangles, p = 2), where 73,728 gain 6 %.
-constexpr size_t kPdlThreads = 152 * 2048;
+// Threads of the largest grid that starts this way.  A grid whose blocks take
+// their places while its predecessor drains is spread unevenly: two on one SM,
+// none on another.  An FP64 pass of about a block an SM is one long chain of
+// instructions and then takes up to twice as long (19,208 triangles, two steps,
+// no programmatic launch against all: p = 2 0.81 / 1.15 ms, wet/dry mode 0.37 /
+// 0.54 ms), so FP64 grids start this way up to a warp an SM (200 intervals, 16
+// steps: 0.81 / 0.85 ms).  FP32 passes are short, and the launch is a larger part
+// of them: four warps an SM (11,726 intervals, 16 steps, 0.455 ms against 0.492;
+// 19,602 triangles, four steps, 0.50 / 0.55 ms; 1 % slower at 2,097,152).
+template <typename T>
+constexpr bool is_fp32_data = std::is_same_v<std::remove_cv_t<std::remove_pointer_t<T>>, float>;
+template <typename... KA>
+constexpr size_t kPdlThreads = (is_fp32_data<KA> || ...) ? 152 * 128 : 152 * 32;
 
 template <typename... KA, typename... A>
 inline void launch_after(void (*kernel)(KA...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
@@ -39,7 +51,7 @@ inline void launch_after(void (*kernel)(KA...), unsigned grid, unsigned block, s
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = &at;
-  cfg.numAttrs = (size_t)grid * block <= kPdlThreads ? 1 : 0;
+  cfg.numAttrs = (size_t)grid * block <= kPdlThreads<KA...> ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
 }
 

@@ -30,8 +30,8 @@ inline size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 __global__ void __launch_bounds__(kVecBlock) dots_kernel(size_t n, const double* __restrict__ x,
                                                          const double* __restrict__ Y, double* __restrict__ partial,
                                                          double* __restrict__ out, unsigned* counter) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(x, Y);
   __shared__ double sh[kVecBlock / 32];
   const int i = blockIdx.y;
@@ -49,8 +49,8 @@ __global__ void __launch_bounds__(kVecBlock) multi_axpy_kernel(size_t n, int k, 
                                                                const double* __restrict__ Y, double* __restrict__ w,
                                                                double* __restrict__ partial, double* __restrict__ nrm2,
                                                                unsigned* counter) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(c, Y, w);
   __shared__ double sh[kVecBlock / 32];
   double acc = 0.0;
@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(kVecBlock) multi_axpy_kernel(size_t n, int k, 
 // out = sum_i c[i] Y_i
 __global__ void __launch_bounds__(kVecBlock) combine_kernel(size_t n, int k, const double* __restrict__ c,
                                                             const double* __restrict__ Y, double* __restrict__ out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(c, Y);
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x) {
     double s = 0.0;
@@ -82,8 +82,8 @@ __global__ void __launch_bounds__(kVecBlock) combine_kernel(size_t n, int k, con
 // y = a * x
 __global__ void __launch_bounds__(kVecBlock) scale_kernel(size_t n, double a, const double* __restrict__ x,
                                                           double* __restrict__ y) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(x);
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x)
     y[j] = a * x[j];
@@ -95,8 +95,8 @@ __global__ void __launch_bounds__(kVecBlock) fd_point_kernel(size_t n, const dou
                                                              const double* __restrict__ vn2,
                                                              const double* __restrict__ zn2, double* __restrict__ Vp,
                                                              double* __restrict__ eps_out) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   after_wait(V, z, vn2, zn2);
   const double eps = 1e-8 * (1.0 + sqrt(*vn2)) / sqrt(*zn2);
   if (blockIdx.x == 0 && threadIdx.x == 0) *eps_out = eps;
@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(kVecBlock) fd_point_kernel(size_t n, const dou
 }
 
 __global__ void advance_time_kernel(DevScalars* sc, double dt) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   sc->t += dt;
   sc->dt = dt;
   sc->dt_min = fmin(sc->dt_min, dt);

@@ -132,10 +132,10 @@ __global__ void __launch_bounds__(kNkBlock) be_time_kernel(int K, const double* 
                                                            const double* __restrict__ eps) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NQ = S::NQ, NV = S::NV, GL = nk_lanes<DIM, P>(), NS = (NQ + GL - 1) / GL;
-  pdl_trigger();
   __shared__ NkTab<DIM, P> t;
   nk_table<DIM, P>(t, ops);
   pdl_wait();
+  pdl_trigger();
   after_wait(V, Uold, R0, eps);
   const NkLane<DIM, P> L(K);
   const size_t KN = (size_t)K * NP, o = (size_t)L.e * NP + L.a;
@@ -184,10 +184,10 @@ __global__ void __launch_bounds__(kNkBlock) mass_factor_kernel(int K, const doub
                                                                const VolOps<DIM, P, double> ops, double h_floor) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NQ = S::NQ, NV = S::NV, GL = nk_lanes<DIM, P>(), NS = (NQ + GL - 1) / GL;
-  pdl_trigger();
   __shared__ NkTab<DIM, P> t;
   nk_table<DIM, P>(t, ops);
   pdl_wait();
+  pdl_trigger();
   after_wait(V);
   const NkLane<DIM, P> L(K);
   const size_t KN = (size_t)K * NP, o = (size_t)L.e * NP + L.a;
@@ -246,10 +246,10 @@ __global__ void __launch_bounds__(kNkBlock) mass_apply_kernel(int K, const doubl
                                                               unsigned* counter) {
   using S = Sh<DIM, P>;
   constexpr int NP = S::NP, NV = S::NV, GL = nk_lanes<DIM, P>();
-  pdl_trigger();
   __shared__ NkTab<DIM, P> t;
   nk_table<DIM, P>(t, ops);
   pdl_wait();
+  pdl_trigger();
   after_wait(x, mats, nrm2);
   const size_t KN = (size_t)K * NP;
   const double nrm = nrm2 ? 1.0 / sqrt(*nrm2) : 1.0;
