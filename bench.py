@@ -482,10 +482,10 @@ def implicit_main(args):
                        "linear_solver": args.solver, "newton_its_per_step": its,
                        "l2": "working set (a few hundred KB) is cache-resident by nature; not flushed",
                        "parallelism": f"replicas x{world}"},
-            "roofline": {"bound": "latency", "kernel": "implicit_kernel<1,0> (one thread block)",
+            "roofline": {"bound": "latency", "kernel": "implicit_kernel<1,0> (one cluster of thread blocks)",
                          "achieved": None, "peak": None, "unit": None, "frac": None, "traffic": None,
-                         "note": "one 100-element problem in one block: the Newton loop is a dependent "
-                                 "chain on one SM (the block-Thomas sweep is one warp)",
+                         "note": "one 100-element problem on one cluster of eight blocks: the Newton loop is "
+                                 "a dependent chain (block cyclic reduction, cluster barriers)",
                          "ms_per_time_step": total_ms / steps_timed},
             "cpu_baseline": cpu, "e2e": None, "gpu_launches": args.steps,
             "clocks": clk.summary(), "accuracy": acc,
@@ -817,6 +817,10 @@ def roofline(r, prec, G, args, peaks_derived, peaks_probe, batch_mode):
             "peak_source": (f"{'FP64' if rs == 8 else 'FP32'} pipe from unit counts: SMs x "
                             f"{2 if rs == 8 else 128} FMA lanes/SM/clk x 2 flop x {SM_MAX_MHZ:g} MHz"),
             "peak_probe": peaks_probe[key], "frac_of_probe": achieved_tf / peaks_probe[key],
+            # FP64 contractions run as integer multiply-adds beside the FP64 pipe: the
+            # algorithmic rate can exceed that pipe's peak
+            "contractions": ("integer pipe (block fixed point)" if rs == 8 else
+                             "tensor cores (split TF32)" if tcf else "FP32 pipe"),
             "traffic": traffic_record("volume_kernel", wl_key),
             "elements_per_launch": K,
             "algorithmic_flops_per_launch": flops, "algorithmic_bytes_per_launch": vbytes,
