@@ -2,7 +2,7 @@
 // and the pointwise HLL and central stress fluxes in floating point, written for
 // few FP64 instructions.  Included by dg_kernels.cuh.
 //
-// Bound by the FP64 pipe (84 % busy): about 101 operations a face point in 2D (175 with
+// Bound by the FP64 pipe (83 % busy): about 96 operations a face point in 2D (175 with
 // floating-point interpolation, IEEE division and square root and FP64
 // comparisons); comparisons, minima and maxima run on the integer pipe, the
 // reciprocal and roots start from the FP32 unit (dg_math64.cuh).  524,288

@@ -3,13 +3,13 @@
 //
 // What stays in floating point is the pointwise stress and flux (about 38
 // operations a volume point in 2D), the Cholesky solve and the stage update:
-// 695 FP64 instructions per element at p = 2 (counted) where the pass in
+// 500 FP64 instructions per element at p = 2 (counted) where the pass in
 // floating point took 2065 and kept the FP64 pipe 91 % busy; the contractions
 // (interpolation, metric transform, test functions, face lift, mass matrices)
 // are 1140 integer multiply-adds of three IMAD.WIDE each.  524,288 triangles,
 // p = 2: 1969 -> 834 us, p = 1 691 -> 402 us (with the wet/dry stage kernel);
 // 73,728 triangles, p = 2: 314 -> 159 us; 8,192: 84 -> 52 us.  The FP64 pipe is
-// 57 % busy then: few warps (168 to 240 registers a thread) wait for one
+// 50 % busy then: few warps (168 to 240 registers a thread) wait for one
 // another's chains.
 //
 //   pass 1  per volume point: interpolate V and the symmetric gradient, form
