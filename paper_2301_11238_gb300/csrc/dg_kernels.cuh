@@ -983,12 +983,16 @@ __global__ void __launch_bounds__(256, estep_min_blocks<R>()) estep_pf_kernel(in
   }
 }
 
-// Minimum (FP64: as integers, off the FP64 pipe; a NaN is then kept or skipped by
-// its bits, and a stage with one stays non-finite through its other sums).
-template <typename T>
-__device__ __forceinline__ T min_depth(T x, T y) { return fmin(x, y); }
-template <>
-__device__ __forceinline__ double min_depth<double>(double x, double y) { return min_f64(x, y); }
+// Minimum in a context of type R.  FP64: as integers, off the FP64 pipe (a NaN is
+// then kept or skipped by its bits, and a stage with one stays non-finite through
+// its other sums).  FP32 contexts, few of whose elements take FP64, keep fmin and
+// IEEE roots: the integer forms cost two registers and a resident block
+// (2,097,152 triangles, p = 1, four steps with transfers 4.76 -> 4.91 ms).
+template <typename R, typename T>
+__device__ __forceinline__ T min_depth(T x, T y) {
+  if constexpr (sizeof(R) == 8) return min_f64(x, y);
+  else return fmin(x, y);
+}
 
 // Unroll factor of the wet/dry stage's loops: full below 2D p = 3, none there.
 template <int DIM, int P>
@@ -1009,14 +1013,14 @@ __device__ __forceinline__ T limit_depth(T* h, const VolOps<DIM, P, R>& ops) {
 #pragma unroll (wd_unroll<DIM, P>())
   for (int a = 0; a < NP; ++a) {
     hbar += (T)ops.wavg[a] * h[a];
-    m = min_depth(m, h[a]);
+    m = min_depth<R>(m, h[a]);
   }
 #pragma unroll (wd_unroll<DIM, P>())
   for (int q = 0; q < NQ; ++q) {
     T hq = T(0);
 #pragma unroll (wd_unroll<DIM, P>())
     for (int a = 0; a < NP; ++a) hq += (T)ops.Vq[q * NP + a] * h[a];
-    m = min_depth(m, hq);
+    m = min_depth<R>(m, hq);
   }
 #pragma unroll (wd_unroll<DIM, P>())
   for (int f = 0; f < NF; ++f)
@@ -1025,7 +1029,7 @@ __device__ __forceinline__ T limit_depth(T* h, const VolOps<DIM, P, R>& ops) {
       T hf = T(0);
 #pragma unroll (wd_unroll<DIM, P>())
       for (int k = 0; k < NFP; ++k) hf += (T)ops.LfT[k * NFQ + mq] * h[face_node(DIM, P, f, k)];
-      m = min_depth(m, hf);
+      m = min_depth<R>(m, hf);
     }
   if (hbar <= T(0)) {
 #pragma unroll (wd_unroll<DIM, P>())
@@ -1135,7 +1139,7 @@ __device__ __forceinline__ void conservative_stage(const R (&Vn)[Sh<DIM, P>::NV]
     T d = Mh[a * NP + a];
 #pragma unroll (wd_unroll<DIM, P>())
     for (int c = 0; c < a; ++c) d -= Mh[a * NP + c] * Mh[a * NP + c];
-    dinv[a] = dg_rsqrt<T>(d);
+    dinv[a] = sizeof(R) == 8 ? dg_rsqrt<T>(d) : T(1) / sqrt(d);
   }
   const bool dry = hbar < hf;
 #pragma unroll (wd_unroll<DIM, P>())
