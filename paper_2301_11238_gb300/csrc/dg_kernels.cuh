@@ -383,7 +383,9 @@ __device__ __forceinline__ void q_normal(R h, const R* E, const R* n, const Phys
 // Per velocity component j the nodal values and the neighbours' traces share an
 // exponent; the reference derivatives and the lifted jumps w_f(a) =
 // sum_k LIFT_a,fk [u_j]_k / 2 stay integers and are combined with the element's
-// metric terms and sc n_i (one more exponent) before they return to doubles:
+// metric terms and sc n_i before they return to doubles.  Those of one direction i
+// share an exponent: on a stretched element the two directions differ by its aspect
+// ratio, and with one exponent for both the small one would lose that many bits.
 // 4 NP conversions and 9 products are the FP64 pipe's share (2D), of 417
 // FP64 instructions in floating point at p = 2.  524,288 triangles, p = 2:
 // 411 -> 180 us; p = 1: 167 -> 67 us; 8,192 triangles, p = 2: 20.6 -> 12.5 us.
@@ -415,21 +417,19 @@ __device__ __forceinline__ void estep_element_fx(int j0, int j1,
 #pragma unroll
     for (int i = 0; i < DIM; ++i) sn[f][i] = sc * fn[(f * DIM + i) * K + e];
   }
-  int eg = 0;
-#pragma unroll
-  for (int i = 0; i < DIM; ++i) {
-#pragma unroll
-    for (int r = 0; r < DIM; ++r) eg = max(eg, fx_exp(G[r][i]));
-#pragma unroll
-    for (int f = 0; f < NF; ++f) eg = max(eg, fx_exp(sn[f][i]));
-  }
+  int eg[DIM];
   Fx Gx[DIM][DIM], snx[NF][DIM];
 #pragma unroll
   for (int i = 0; i < DIM; ++i) {
+    eg[i] = 0;
 #pragma unroll
-    for (int r = 0; r < DIM; ++r) Gx[r][i] = fx_from<5>(G[r][i], eg);
+    for (int r = 0; r < DIM; ++r) eg[i] = max(eg[i], fx_exp(G[r][i]));
 #pragma unroll
-    for (int f = 0; f < NF; ++f) snx[f][i] = fx_from<5>(sn[f][i], eg);
+    for (int f = 0; f < NF; ++f) eg[i] = max(eg[i], fx_exp(sn[f][i]));
+#pragma unroll
+    for (int r = 0; r < DIM; ++r) Gx[r][i] = fx_from<5>(G[r][i], eg[i]);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) snx[f][i] = fx_from<5>(sn[f][i], eg[i]);
   }
   // one component at a time: both at once take 192 registers (p = 2) and half the warps
 #pragma unroll 1
@@ -480,7 +480,10 @@ __device__ __forceinline__ void estep_element_fx(int j0, int j1,
         gx[f][k].l = b.l - o.l;
       }
     // results in units of 2^(eu - 1079) 2^-cs 2^56 2^4 2^(eg - 1080) 2^56
-    const FxScale s = fx_scale(eu + eg - 2043 - ops.cs, eu <= kFxMaxExp && eg <= kFxMaxExp);
+    FxScale s[DIM];
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+      s[i] = fx_scale(eu + eg[i] - 2043 - ops.cs, eu <= kFxMaxExp && eg[i] <= kFxMaxExp);
 #pragma unroll (P == 3 ? 1 : 2)
     for (int a = 0; a < NP; ++a) {
       FxAcc dr{0, 0}, ds{0, 0}, out[DIM];
@@ -510,7 +513,7 @@ __device__ __forceinline__ void estep_element_fx(int j0, int j1,
         for (int i = 0; i < DIM; ++i) fx_mac(out[i], wx, snx[f][i]);
       }
 #pragma unroll
-      for (int i = 0; i < DIM; ++i) E[(DIM * i + j) * KN + (size_t)e * NP + a] = fx_to(fx_sum(out[i]), s);
+      for (int i = 0; i < DIM; ++i) E[(DIM * i + j) * KN + (size_t)e * NP + a] = fx_to(fx_sum(out[i]), s[i]);
     }
   }
 }
