@@ -1456,12 +1456,13 @@ __device__ __forceinline__ void volume_any(int e, int K, int F, const R* const (
 // Register cap of the direct volume kernel: 168, the most that keeps three
 // warps on each SM sub-partition (16,384 registers each), for FP32 at p = 3
 // (left to the compiler it took 171, and the p = 3 bump volume pass ran 0.40
-// instead of 0.30 ms) and FP64 triangles at p = 2 (230 registers left to the
+// instead of 0.30 ms), FP64 triangles at p = 2 (230 registers left to the
 // compiler: 1004 us against 929 on 524,288 triangles, with 156 bytes spilled; on
-// 8,192 triangles, one warp a sub-partition, 56 against 61 us).  Otherwise no cap.
+// 8,192 triangles, one warp a sub-partition, 56 against 61 us) and at p = 1 (170 left
+// to the compiler in the batch's form).  Otherwise no cap.
 template <int DIM, int P, typename R>
 constexpr int volume_max_regs() {
-  return (DIM == 2 && P == (sizeof(R) == 4 ? 3 : 2)) ? 168 : 255;
+  return (DIM == 2 && (sizeof(R) == 4 ? P == 3 : P <= 2)) ? 168 : 255;
 }
 
 // One thread per element; nodal values read straight from global memory.

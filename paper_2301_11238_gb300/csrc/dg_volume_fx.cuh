@@ -14,9 +14,13 @@
 //
 //   pass 1  per volume point: interpolate V and the symmetric gradient, form
 //           the flux tensor, the source and h for M_h; keep them (local memory)
-//           with the largest exponent of each kind
+//           with the largest exponent of each component
 //   pass 2  per volume point: metric transform J G (Q - F), test functions;
 //           the face fluxes are lifted into the same accumulators
+// Every component of the residual has a unit of its own, set by the largest of its
+// terms, and the metric terms of each direction have theirs: on stretched elements,
+// or with a momentum component far below the other, a unit for all would take bits
+// from the small ones.
 //   solve   M dh/dt = -r_h straight from the integer residual, then M_h and
 //           M_u dh/dt per volume point, Cholesky in floating point
 #pragma once
@@ -99,11 +103,26 @@ __device__ __forceinline__ long long lanes_sum(FxAcc v) {
   }
   return fx_sum(v);
 }
-template <int T>
-__device__ __forceinline__ int lanes_max(int v) {
+// (N exponents, two in a word)
+template <int T, int N>
+__device__ __forceinline__ void lanes_max(int (&v)[N]) {
+  if constexpr (T > 1) {
 #pragma unroll
-  for (int o = 1; o < T; o *= 2) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+    for (int i = 0; i < N; i += 2) {
+      unsigned w = (unsigned)v[i] | (i + 1 < N ? (unsigned)v[i + 1] << 16 : 0u);
+#pragma unroll
+      for (int o = 1; o < T; o *= 2) w = __vmaxu2(w, __shfl_xor_sync(0xffffffffu, w, o));
+      v[i] = (int)(w & 0xffffu);
+      if (i + 1 < N) v[i + 1] = (int)(w >> 16);
+    }
+  }
+}
+template <int N>
+__device__ __forceinline__ int largest(const int (&v)[N]) {
+  int m = v[0];
+#pragma unroll
+  for (int i = 1; i < N; ++i) m = max(m, v[i]);
+  return m;
 }
 
 // Arguments and modes as volume_element (dg_kernels.cuh).  T = 1: one thread per
@@ -134,7 +153,12 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
 
   double hu_s[NS][DIM], T_s[NS][NT], S_s[NS][DIM], u_s[NS][DIM];
   Fx hm_s[NS];
-  int eH = 0, eT = 0, eS = 0;  // largest exponents of h u, the flux tensor and the source
+  // largest exponents of each component of the flux (h u, then the tensor) and of the source
+  int eX[DIM + NT], eS[DIM];
+#pragma unroll
+  for (int c = 0; c < DIM + NT; ++c) eX[c] = 0;
+#pragma unroll
+  for (int j = 0; j < DIM; ++j) eS[j] = 0;
   // bound of the exponent of max(h, h_floor) at the volume points (Lebesgue constants below 4)
   int eM = 0;
   bool finite = true;
@@ -228,19 +252,18 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
         hu_s[i][j] = hu[j];
         S_s[i][j] = Sv[j];
         u_s[i][j] = Vq[1 + j];
-        eH = max(eH, fx_exp(hu[j]));
-        eS = max(eS, fx_exp(Sv[j]));
+        eX[j] = max(eX[j], fx_exp(hu[j]));
+        eS[j] = max(eS[j], fx_exp(Sv[j]));
       }
 #pragma unroll
       for (int c = 0; c < NT; ++c) {
         T_s[i][c] = Tq[c];
-        eT = max(eT, fx_exp(Tq[c]));
+        eX[DIM + c] = max(eX[DIM + c], fx_exp(Tq[c]));
       }
     }
   }
-  eH = lanes_max<T>(eH);
-  eT = lanes_max<T>(eT);
-  eS = lanes_max<T>(eS);
+  lanes_max<T>(eX);
+  lanes_max<T>(eS);
 
   // ---- pass 2: J times (metric transform, test functions, face lift)
   FxAcc r[NV][NP];
@@ -254,15 +277,19 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
   for (int k = 0; k < DIM; ++k)
 #pragma unroll
     for (int i = 0; i < DIM; ++i) JG[k][i] = J * geo[(2 * k + i) * K + e];
-  int eG = 0;
+  int eG[DIM];  // of each direction i
 #pragma unroll
-  for (int k = 0; k < DIM; ++k)
+  for (int i = 0; i < DIM; ++i) {
+    eG[i] = 0;
 #pragma unroll
-    for (int i = 0; i < DIM; ++i) eG = max(eG, fx_exp(JG[k][i]));
+    for (int k = 0; k < DIM; ++k) eG[i] = max(eG[i], fx_exp(JG[k][i]));
+  }
   const int eJ = fx_exp(J);
   // weighted face fluxes, in the owner's orientation
   double fv[NF][NV][NFQ];
-  int eW[2] = {0, 0};
+  int eW[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) eW[v] = 0;
   const size_t FQ = (size_t)F * NFQ;
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
@@ -276,16 +303,22 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       for (int m = 0; m < NFQ; ++m) {
         const double x = DG_LDC(COH, wflux, v * FQ + base + (own ? m : NFQ - 1 - m));
         fv[f][v][m] = __hiloint2double(__double2hiint(x) ^ (own ? 0 : (int)0x80000000u), __double2loint(x));
-        eW[v > 0] = max(eW[v > 0], fx_exp(x));
+        eW[v] = max(eW[v], fx_exp(x));
       }
   }
-  eW[0] = lanes_max<T>(eW[0]);
-  eW[1] = lanes_max<T>(eW[1]);
-  // one unit per group of rows (depth, momentum): operands below
-  // 2^(tot - 2043) in units of 2^(tot - 2101)
-  const int tot0 = max(eH + eG, eW[0] + 1021), tot1 = max(max(eT + eG, eS + eJ), eW[1] + 1021);
-  finite = finite && eH <= kFxMaxExp && eT <= kFxMaxExp && eS <= kFxMaxExp && eW[0] <= kFxMaxExp &&
-           eW[1] <= kFxMaxExp;
+  lanes_max<T>(eW);
+  // a unit for each row (depth, momentum components): its terms below 2^(tot - 2043)
+  // in units of 2^(tot - 2101).  flux_of: component of the flux in row v, direction i.
+  auto flux_of = [](int v, int i) { return v == 0 ? i : DIM + (v - 1 + i) % (NT + 1); };
+  int tot[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    tot[v] = eW[v] + 1021;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) tot[v] = max(tot[v], eX[flux_of(v, i)] + eG[i]);
+    if (v > 0) tot[v] = max(tot[v], eS[(v + DIM - 1) % DIM] + eJ);
+  }
+  finite = finite && max(max(largest(eX), largest(eS)), largest(eW)) <= kFxMaxExp;
 #pragma unroll
   for (int f = 0; f < NF; ++f)
 #pragma unroll
@@ -293,7 +326,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
 #pragma unroll
       for (int m = 0; m < NFQ; ++m) {
         if (T > 1 && f % T != tl) continue;
-        const Fx x = fx_from<5>(fv[f][v][m], (v > 0 ? tot1 : tot0) - 1021);
+        const Fx x = fx_from<5>(fv[f][v][m], tot[v] - 1021);
 #pragma unroll
         for (int k = 0; k < NFP; ++k) fx_mac(r[v][face_node(DIM, P, f, k)], x, ops.LfT[k * NFQ + m]);
       }
@@ -302,7 +335,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
 #pragma unroll
     for (int k = 0; k < DIM; ++k)
 #pragma unroll
-      for (int i = 0; i < DIM; ++i) JGx[k][i] = fx_from<5>(JG[k][i], eG);
+      for (int i = 0; i < DIM; ++i) JGx[k][i] = fx_from<5>(JG[k][i], eG[i]);
     const Fx Jx = fx_from<5>(-J, eJ);
     // at most 2 NFQ + 5 (DIM + 1) terms before the first fold, 5 (DIM + 1) after it
     static_assert(2 * S::NFQ <= 15, "the lift terms need a fold of their own");
@@ -324,7 +357,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
         Fx x[DIM];
 #pragma unroll
         for (int i = 0; i < DIM; ++i)
-          x[i] = v == 0 ? fx_from<5>(hu_s[k][i], tot0 - eG) : fx_from<5>(T_s[k][(v - 1 + i) % (NT + 1)], tot1 - eG);
+          x[i] = fx_from<5>(v == 0 ? hu_s[k][i] : T_s[k][(v - 1 + i) % (NT + 1)], tot[v] - eG[i]);
         FxAcc fr{0, 0}, fs{0, 0};
 #pragma unroll
         for (int i = 0; i < DIM; ++i) {
@@ -336,7 +369,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
         if constexpr (DIM == 2) fsx = fx_operand<61>(fx_sum(fs));
         if (v > 0) {
           FxAcc s{0, 0};
-          fx_mac(s, fx_from<5>(S_s[k][(v + DIM - 1) % DIM], tot1 - eJ), Jx);
+          fx_mac(s, fx_from<5>(S_s[k][(v + DIM - 1) % DIM], tot[v] - eJ), Jx);
           sx = fx_operand<61>(fx_sum(s));
         }
 #pragma unroll
@@ -353,7 +386,9 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
   for (int v = 0; v < NV; ++v)
 #pragma unroll
     for (int a = 0; a < NP; ++a) rs[v][a] = lanes_sum<T>(r[v][a]);
-  const FxScale s0 = fx_scale(tot0 - 2045 - ops.cs_w, finite), s1 = fx_scale(tot1 - 2045 - ops.cs_w, finite);
+  FxScale sr[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) sr[v] = fx_scale(tot[v] - 2045 - ops.cs_w, finite);
 
   // mode 2: the spatial residual r_V itself (physical scaling), for the
   // implicit integrators that assemble their own time term
@@ -362,14 +397,14 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
     for (int v = 0; v < NV; ++v)
 #pragma unroll
       for (int a = 0; a < NP; ++a)
-        if (live && (T == 1 || a % T == tl)) out[v * KN + eo + a] = fx_to(rs[v][a], v > 0 ? s1 : s0);
+        if (live && (T == 1 || a % T == tl)) out[v * KN + eo + a] = fx_to(rs[v][a], sr[v]);
     return;
   }
 
   // ---- mass solve, J dV/dt: x_h = -Minv r_h ; M_h x_u = -r_u - <psi, x_h u>
   double x[NV][NP], ru[DIM][NP];
   Fx dh[NP];
-  int kh = tot0 - 2045 - ops.cs_w;  // binary orders of what dh holds
+  int kh = tot[0] - 2045 - ops.cs_w;  // binary orders of what dh holds
   {
     // r_h brought up to full length (the fluxes mostly cancel in it)
     long long rh[NP];
@@ -379,7 +414,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       rh[a] = rs[0][a];
       m |= fx_mag(rh[a]);
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) ru[j][a] = fx_to(rs[1 + j][a], s1);
+      for (int j = 0; j < DIM; ++j) ru[j][a] = fx_to(rs[1 + j][a], sr[1 + j]);
     }
     int n = fx_norm(m);
     Fx rx[NP];
@@ -404,7 +439,9 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
     kh += 60 - n - ops.cs_v;
   }
   const FxScale sq = fx_scale(kh, finite);
-  int eZ = 0;
+  int eZ[DIM];
+#pragma unroll
+  for (int j = 0; j < DIM; ++j) eZ[j] = 0;
 #pragma unroll 1
   for (int q = tl, k = 0; q < NQ; q += T, ++k) {
     Fx row[NP];
@@ -417,12 +454,11 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
     for (int j = 0; j < DIM; ++j) {
       const double z = dq * u_s[k][j];
       u_s[k][j] = z;
-      eZ = max(eZ, fx_exp(z));
+      eZ[j] = max(eZ[j], fx_exp(z));
     }
   }
-  eZ = lanes_max<T>(eZ);
-  const FxScale sm = fx_scale(eM - 1024 - ops.cs_m, finite),
-                sz = fx_scale(eZ - 1024 - ops.cs_w, finite && eZ <= kFxMaxExp);
+  lanes_max<T>(eZ);
+  const FxScale sm = fx_scale(eM - 1024 - ops.cs_m, finite);
   // -r_u - <psi, x_h u>, and after it M_h (one after the other: their
   // accumulators together would take 132 registers at p = 2)
   {
@@ -443,15 +479,17 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       }
 #pragma unroll
       for (int j = 0; j < DIM; ++j) {
-        const Fx z = fx_from<5>(u_s[k][j], eZ);
+        const Fx z = fx_from<5>(u_s[k][j], eZ[j]);
 #pragma unroll
         for (int a = 0; a < NP; ++a) fx_mac(za[j][a], z, wm[a]);
       }
     }
 #pragma unroll
-    for (int j = 0; j < DIM; ++j)
+    for (int j = 0; j < DIM; ++j) {
+      const FxScale sz = fx_scale(eZ[j] - 1024 - ops.cs_w, finite && eZ[j] <= kFxMaxExp);
 #pragma unroll
       for (int a = 0; a < NP; ++a) ru[j][a] = fx_to(lanes_sum<T>(za[j][a]), sz) - ru[j][a];
+    }
   }
   FxAcc Ma[NM];
 #pragma unroll

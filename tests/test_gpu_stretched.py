@@ -65,3 +65,21 @@ def test_gradient(p, aspect, along, shear):
     V = rough_state(len(etov), p)
     _, E, (_, _, ref, mag) = both(coords, etov, p, V)
     assert max(worst(E, ref, mag)) < TOL
+
+
+@pytest.mark.parametrize("p", [1, 2, 3])
+@pytest.mark.parametrize("aspect", [1.0, 1e3, 1e6])
+@pytest.mark.parametrize("along", [0, 1])
+@pytest.mark.parametrize("flow", ["fast", "slow", "one way"])
+def test_residual(p, aspect, along, flow):
+    """fast: velocities of the wave speed's size; slow: the pressure is nearly all there is; one way: one
+    velocity component 1e-9 of the other."""
+    coords, etov = mesh(aspect, along, 0.5)
+    V = rough_state(len(etov), p)
+    if flow == "slow":
+        V[0] = 1.0
+        V[1:] *= 1e-7
+    if flow == "one way":
+        V[2 - along] *= 1e-9
+    dV, _, (ref, mag, _, _) = both(coords, etov, p, V)
+    assert max(worst(dV, ref, mag)) < TOL
