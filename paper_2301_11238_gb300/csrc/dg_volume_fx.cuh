@@ -152,15 +152,16 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
   const size_t eo = (size_t)e * NP;
 
   double hu_s[NS][DIM], T_s[NS][NT], S_s[NS][DIM], u_s[NS][DIM];
-  Fx hm_s[NS];
+  double hm_s[NS];
   // largest exponents of each component of the flux (h u, then the tensor) and of the source
   int eX[DIM + NT], eS[DIM];
 #pragma unroll
   for (int c = 0; c < DIM + NT; ++c) eX[c] = 0;
 #pragma unroll
   for (int j = 0; j < DIM; ++j) eS[j] = 0;
-  // bound of the exponent of max(h, h_floor) at the volume points (Lebesgue constants below 4)
-  int eM = 0;
+  // largest exponent of max(h, h_floor): of the points themselves, for where the depth
+  // is below the floor the nodal values can be far above what M_h holds
+  int eM[1] = {0};
   bool finite = true;
 
   {  // ---- pass 1
@@ -176,7 +177,6 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       for (int a = 0; a < NP; ++a) vx[v][a] = fx_from<5>(Vn[v][a], ev);
       sv[v] = fx_scale(ev - 1024 - ops.cs_v, ev <= kFxMaxExp);
       finite = finite && ev <= kFxMaxExp;
-      if (v == 0) eM = max(ev + 2, fx_exp(ph.h_floor));
     }
     if constexpr (DIM == 1) {
       int ed = 0;
@@ -228,7 +228,8 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
       const double h = Vq[0];
       // max(h, h_floor) as integers: h_floor > 0, so a negative h orders below it
       const double hm = __longlong_as_double(max(__double_as_longlong(h), __double_as_longlong(ph.h_floor)));
-      hm_s[i] = fx_from<5>(hm, eM);
+      hm_s[i] = hm;
+      eM[0] = max(eM[0], fx_exp(hm));
       double hu[DIM], Tq[NT], Sv[DIM];
 #pragma unroll
       for (int j = 0; j < DIM; ++j) hu[j] = -h * Vq[1 + j];
@@ -264,6 +265,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
   }
   lanes_max<T>(eX);
   lanes_max<T>(eS);
+  lanes_max<T>(eM);
 
   // ---- pass 2: J times (metric transform, test functions, face lift)
   FxAcc r[NV][NP];
@@ -458,7 +460,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
     }
   }
   lanes_max<T>(eZ);
-  const FxScale sm = fx_scale(eM - 1024 - ops.cs_m, finite);
+  const FxScale sm = fx_scale(eM[0] - 1024 - ops.cs_m, finite);
   // -r_u - <psi, x_h u>, and after it M_h (one after the other: their
   // accumulators together would take 132 registers at p = 2)
   {
@@ -498,7 +500,7 @@ __device__ __forceinline__ void volume_element_fx(int e, int K, int F,
   for (int q = tl, k = 0; q < NQ; q += T, ++k) {
     Fx mp[NM];
     fx_row<DIM, P, 4>(ops, tab, q, mp);
-    const Fx hm = hm_s[k];
+    const Fx hm = fx_from<5>(hm_s[k], eM[0]);
     if (NS > 15 && k % 12 == 0) {
 #pragma unroll
       for (int i = 0; i < NM; ++i) fx_fold(Ma[i]);

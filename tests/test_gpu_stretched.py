@@ -83,3 +83,25 @@ def test_residual(p, aspect, along, flow):
         V[2 - along] *= 1e-9
     dV, _, (ref, mag, _, _) = both(coords, etov, p, V)
     assert max(worst(dV, ref, mag)) < TOL
+
+
+@pytest.mark.parametrize("dim", [1, 2])
+@pytest.mark.parametrize("p", [1, 2, 3])
+@pytest.mark.parametrize("depth", [-1.0, -1e-3, 1e-9, "mixed"])
+def test_depth_below_the_floor(dim, p, depth):
+    """Elements whose depth is below the floor, alone and among wet ones: M_h then holds the floor, whatever
+    the size of the nodal depths."""
+    if dim == 1:
+        coords, etov = np.linspace(0.0, 1.0, 41).reshape(-1, 1), np.stack([np.arange(40), np.arange(1, 41)], 1)
+        etov = etov.astype(np.int32)
+    else:
+        coords, etov = mesh(1.0, 0, 0.0)
+    r = np.random.default_rng(p).uniform(-1, 1, (3, len(etov), p + 1 if dim == 1 else (p + 1) * (p + 2) // 2))
+    V = np.stack([1 + 0.1 * r[0], 0.3 + 0.2 * r[1], -0.2 + 0.2 * r[2]])[:dim + 1]
+    if depth == "mixed":
+        V[0, ::3] = 1e-9
+        V[0, 1::3] *= -0.01
+    else:
+        V[0] *= depth
+    dV, _, (ref, mag, _, _) = both(coords, etov, p, V)
+    assert max(worst(dV, ref, mag)) < TOL
