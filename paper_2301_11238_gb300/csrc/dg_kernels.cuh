@@ -1862,8 +1862,7 @@ __device__ __forceinline__ R block_min_flag(R v, R* red) {
   return v;
 }
 
-// A float near x (FP64: by the integer pipe; 0 or infinity outside the float range).
-__device__ __forceinline__ float near_f32(float x) { return x; }
+// A float near x, by the integer pipe; 0 or infinity outside the float range.
 __device__ __forceinline__ float near_f32(double x) {
   const int hi = __double2hiint(x);
   const int e = (hi >> 20) & 0x7ff;
@@ -1873,7 +1872,6 @@ __device__ __forceinline__ float near_f32(double x) {
 }
 __device__ __forceinline__ bool not_finite(float x) { return (__float_as_uint(x) & 0x7f800000u) == 0x7f800000u; }
 __device__ __forceinline__ bool not_finite(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
-__device__ __forceinline__ float sqrt_nonneg(float x) { return sqrtf(x); }
 __device__ __forceinline__ double sqrt_nonneg(double x) {
   return __double_as_longlong(x) == 0 ? 0.0 : sqrt_pos(x);
 }
@@ -1881,70 +1879,90 @@ __device__ __forceinline__ double sqrt_nonneg(double x) {
 template <typename R>
 __device__ __forceinline__ R huge_dt() { return sizeof(R) == 8 ? R(1e300) : R(3e38); }
 
-// Stable step of element e (see dg_swe_step), -1 for a non-finite state.  The
-// largest wave speed is found in two steps: fast single-precision speeds at all
-// nodes, then the speed in the state's precision at the nodes within 1e-5 of
-// their largest (usually one), so that the value is that of the plain maximum.
-// With the minimum on the integer pipe: FP64, 524,288 triangles, p = 2 179 -> 77 us
-// (bound by 84 FP64 root and sum instructions an element before); FP32, 2,097,152
-// triangles 81 -> 52 us (ten FP64 minima a warp before).
+// Stable step of element e (see dg_swe_step), -1 for a non-finite state: from the
+// largest wave speed over the nodes.  FP32 contexts take the speed of every node.
+// FP64, whose roots are the time here, finds the largest in two steps: fast
+// single-precision speeds at all nodes, then the speed in FP64 at the nodes within
+// 1e-5 of their largest, so that the value is that of the plain maximum.  In flow
+// these are one or two nodes, in still water of even depth all of them; everything
+// but the products and roots of a node's speed is kept off the FP64 pipe for their
+// sake.  524,288 triangles, p = 2, us in flow / in still water: FP64 43 / 99 (with
+// the nodes compared in FP64 61 / 186, the plain maximum 179), FP32 12.6 / 12.6 (in
+// two steps like FP64 14.5 / 20.7, with FP64 minima 24).
 template <int DIM, int P, typename R, bool COH = false>
 __device__ __forceinline__ R element_dt(size_t e, int K, const R* __restrict__ V, const R* __restrict__ geo, R gc,
                                         R h_floor, R cfl, R nu) {
   constexpr int NP = Sh<DIM, P>::NP;
   const size_t KN = (size_t)K * NP;
-  R h[NP], u[DIM][NP];
-  float l[NP], top = 0.f;
-  const float gcf = near_f32(gc), hf = near_f32(h_floor);
   bool bad = false;
-#pragma unroll
-  for (int a = 0; a < NP; ++a) {
-    h[a] = DG_LDC(COH, V, e * NP + a);
-    bad = bad || not_finite(h[a]);
-    float s2 = 0.f;
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) {
-      u[j][a] = DG_LDC(COH, V, (1 + j) * KN + e * NP + a);
-      bad = bad || not_finite(u[j][a]);
-      const float x = near_f32(u[j][a]);
-      s2 += x * x;
-    }
-    l[a] = dg_sqrt<float>(s2) + dg_sqrt<float>(gcf * fmaxf(near_f32(h[a]), hf));
-    top = fmaxf(top, l[a]);
-  }
-  if (bad) return R(-1);
-  const float near_top = top * (1.f - 1e-5f);
-  unsigned cand = 0;
-#pragma unroll
-  for (int a = 0; a < NP; ++a) cand |= l[a] < near_top ? 0u : 1u << a;
   R lam = R(0);
-  while (cand) {
-    const int c = __ffs(cand) - 1;
-    R hc = h[0], uc[DIM];
+  if constexpr (sizeof(R) == 4) {
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) uc[j] = u[j][0];
+    for (int a = 0; a < NP; ++a) {
+      const R h = DG_LDC(COH, V, e * NP + a);
+      R sp2 = R(0);
 #pragma unroll
-    for (int a = 1; a < NP; ++a)
-      if (a == c) {
-        hc = h[a];
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) uc[j] = u[j][a];
+      for (int j = 0; j < DIM; ++j) {
+        const R u = DG_LDC(COH, V, (1 + j) * KN + e * NP + a);
+        sp2 += u * u;
       }
-    cand &= cand - 1;
-    // nodes equal to this one give the same speed
-#pragma unroll
-    for (int a = 1; a < NP; ++a) {
-      bool same = h[a] == hc;
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) same = same && u[j][a] == uc[j];
-      if (same) cand &= ~(1u << a);
+      const R v = sqrtf(sp2) + sqrtf(gc * fmaxf(h, h_floor));
+      bad = bad || not_finite(h) || not_finite(v);
+      lam = fmaxf(lam, v);
     }
-    R sp2 = R(0);
+    if (bad) return R(-1);
+  } else {
+    R h[NP], u[DIM][NP];
+    float l[NP], top = 0.f;
+    const float gcf = near_f32(gc), hf = near_f32(h_floor);
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) sp2 += uc[j] * uc[j];
-    const R v = sqrt_nonneg(sp2) + sqrt_nonneg(gc * fmax(hc, h_floor));
-    if (not_finite(v)) return R(-1);
-    lam = fmax(lam, v);
+    for (int a = 0; a < NP; ++a) {
+      h[a] = DG_LDC(COH, V, e * NP + a);
+      bad = bad || not_finite(h[a]);
+      float s2 = 0.f;
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) {
+        u[j][a] = DG_LDC(COH, V, (1 + j) * KN + e * NP + a);
+        bad = bad || not_finite(u[j][a]);
+        const float x = near_f32(u[j][a]);
+        s2 += x * x;
+      }
+      l[a] = dg_sqrt<float>(s2) + dg_sqrt<float>(gcf * fmaxf(near_f32(h[a]), hf));
+      top = fmaxf(top, l[a]);
+    }
+    if (bad) return R(-1);
+    // all nodes where squares leave the single-precision range
+    const float near_top = top > 1e-13f && top < 1e18f ? top * (1.f - 1e-5f) : 0.f;
+    unsigned cand = 0;
+#pragma unroll
+    for (int a = 0; a < NP; ++a) cand |= l[a] < near_top ? 0u : 1u << a;
+    while (cand) {
+      const int c = __ffs(cand) - 1;
+      R hc = h[0], uc[DIM];
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) uc[j] = u[j][0];
+#pragma unroll
+      for (int a = 1; a < NP; ++a)
+        if (a == c) {
+          hc = h[a];
+#pragma unroll
+          for (int j = 0; j < DIM; ++j) uc[j] = u[j][a];
+        }
+      cand &= cand - 1;
+      // nodes equal to this one give the same speed
+#pragma unroll
+      for (int a = 1; a < NP; ++a) {
+        bool same = __double_as_longlong(h[a]) == __double_as_longlong(hc);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) same = same && __double_as_longlong(u[j][a]) == __double_as_longlong(uc[j]);
+        if (same) cand &= ~(1u << a);
+      }
+      R sp2 = uc[0] * uc[0];
+      if constexpr (DIM == 2) sp2 += uc[DIM - 1] * uc[DIM - 1];
+      const R v = sqrt_nonneg(sp2) + sqrt_nonneg(gc * max_pos(hc, h_floor));
+      if (not_finite(v)) return R(-1);
+      lam = max_pos(v, lam);
+    }
   }
   const R dx = geo[5 * (size_t)K + e];
   const R qq = R(2 * P + 1);
