@@ -243,7 +243,6 @@ dg_status dg_newton_set_workspace(dg_newton* k, void* ptr, size_t bytes) {
   if (!ptr || ((uintptr_t)ptr & 255) != 0 || bytes < k->ws_need)
     return nfail(k, DG_ERR_WORKSPACE, "workspace missing, misaligned or smaller than dg_newton_workspace_size");
   k->ws = static_cast<char*>(ptr);
-  NK(cudaMemsetAsync(k->ws + k->off.counter, 0, sizeof(unsigned), k->c->stream));
   return DG_OK;
 }
 
@@ -274,6 +273,8 @@ dg_status dg_newton_run(dg_newton* k, int64_t n_steps, dg_newton_stats* stats) {
   const unsigned G = x.grid;
   cudaStream_t s = x.s;
   std::vector<double> H((size_t)(m + 1) * m), g(m + 1), cs(m), sn(m), y(m);
+  // on the stream of this run, whatever the workspace and the last run left there
+  NK(cudaMemsetAsync(counter, 0, sizeof(unsigned), s));
   auto norm2 = [&](const double* v, double* slot, double& host) -> dg_status {
     x.dots(v, v, 1, slot);
     NK(cudaMemcpyAsync(hbuf, slot, sizeof(double), cudaMemcpyDeviceToHost, s));
