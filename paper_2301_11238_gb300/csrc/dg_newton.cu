@@ -130,7 +130,8 @@ struct dg_newton {
   dg_newton_stats st{};
   std::string err;
   // host side of the per-iteration read (pinned, so that the copy is one DMA and
-  // the call does not stage it)
+  // the call does not stage it; allocated by the first run, which synchronizes: a
+  // pinned allocation in init would break a capture under way)
   double* hbuf = nullptr;
   template <typename T>
   T* at(size_t o) const { return reinterpret_cast<T*>(ws + o); }
@@ -227,11 +228,6 @@ dg_status dg_newton_init(dg_swe_ctx* c, const dg_newton_params* p, dg_newton** o
   k->off.scal = take(S_COUNT * sizeof(double));
   k->off.counter = take(sizeof(unsigned));
   k->ws_need = o;
-  if (cudaHostAlloc((void**)&k->hbuf, (2 * (size_t)(k->m + 1) + 1) * sizeof(double), cudaHostAllocDefault) !=
-      cudaSuccess) {
-    cudaGetLastError();  // no device here: run needs one anyway
-    k->hbuf = nullptr;
-  }
   *out = k;
   return DG_OK;
 }
