@@ -19,7 +19,8 @@
  *    geometry, operators, scratch) lives in one caller-provided workspace of
  *    dg_swe_workspace_size() bytes (dg_swe_set_workspace), so a caller's
  *    allocator (e.g. PyTorch's) owns it.  Host memory is allocated in
- *    dg_swe_init and released in dg_swe_destroy.
+ *    dg_swe_init (and, pinned, a block of under 100 bytes for status reads in
+ *    dg_swe_set_workspace) and released in dg_swe_destroy.
  *  - Kernels run on the stream set by dg_swe_set_stream (default stream 0).
  *    Calls that only enqueue work return DG_OK at enqueue; device-side errors
  *    (non-finite state) are latched in a device status word and reported by

@@ -93,7 +93,7 @@ struct dg_batch {
   std::vector<cudaStream_t> side;     // capture streams of the groups after the first
   std::vector<cudaEvent_t> side_ev;
   cudaGraphExec_t g1 = nullptr, gN = nullptr;
-  DevScalars* h_sc = nullptr;  // host side of read_stats, one per instance
+  StatusBlock status;  // of read_stats, a scalar block per instance; allocated by dg_batch_set_workspace
   std::string err;
   template <typename T>
   T* at(size_t o) const { return reinterpret_cast<T*>(ws + o); }
@@ -571,12 +571,8 @@ void fields(int nf, size_t n, const void* in, size_t sin, void* out, size_t sout
 }
 
 dg_status read_stats(dg_batch* b, dg_swe_stats* st) {
-  // pinned, so that the copy is one DMA in the stream (a pageable one is staged)
-  if (!b->h_sc) BK(cudaHostAlloc((void**)&b->h_sc, b->n * sizeof(DevScalars), cudaHostAllocDefault));
-  const DevScalars* h = b->h_sc;
-  BK(cudaMemcpyAsync(b->h_sc, b->at<DevScalars>(b->off_sc), b->n * sizeof(DevScalars), cudaMemcpyDeviceToHost,
-                     b->stream));
-  BK(cudaStreamSynchronize(b->stream));
+  std::vector<DevScalars> h(b->n);
+  BK(read_status(b->status, h.data(), b->at<DevScalars>(b->off_sc), b->n * sizeof(DevScalars), b->stream));
   int bad = -1;
   for (int i = 0; i < b->n; ++i) {
     if (h[i].status && bad < 0) bad = i;
@@ -937,6 +933,7 @@ dg_status dg_batch_set_workspace(dg_batch* b, void* ptr, size_t bytes) {
   launch_after(reset_scalars_kernel, (b->n + 127) / 128, 128, 0, s, b->n, b->at<DevScalars>(b->off_sc));
   BK(cudaGetLastError());
   BK(cudaStreamSynchronize(s));
+  b->status.allocate(b->n * sizeof(DevScalars));
   return DG_OK;
 }
 
@@ -1208,7 +1205,6 @@ void dg_batch_destroy(dg_batch* b) {
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
   if (b->ev_join) cudaEventDestroy(b->ev_join);
   if (b->priv) cudaStreamDestroy(b->priv);
-  if (b->h_sc) cudaFreeHost(b->h_sc);
   delete b;
 }
 

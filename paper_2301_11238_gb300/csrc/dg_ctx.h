@@ -3,7 +3,9 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cstring>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -46,6 +48,32 @@ struct DriverDeleter {
   void operator()(Driver* d) const;
 };
 using DriverPtr = std::unique_ptr<Driver, DriverDeleter>;
+
+// Pinned host block for the status reads of a context, so that the copy is one DMA
+// in the stream (a pageable one is staged).  One reader at a time uses it; another
+// reader of the same context, or all if there is none, copies to its own memory.
+struct StatusBlock {
+  void* p = nullptr;
+  std::mutex mu;
+  void allocate(size_t bytes) {
+    if (!p && cudaHostAlloc(&p, bytes, cudaHostAllocDefault) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+  }
+  ~StatusBlock() {
+    if (p) cudaFreeHost(p);
+  }
+};
+// Copies n bytes at dev to host through the block and synchronizes the stream.
+inline cudaError_t read_status(StatusBlock& b, void* host, const void* dev, size_t n, cudaStream_t s) {
+  std::unique_lock<std::mutex> lk(b.mu, std::try_to_lock);
+  void* dst = b.p && lk.owns_lock() ? b.p : host;
+  cudaError_t e = cudaMemcpyAsync(dst, dev, n, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess && dst != host) std::memcpy(host, dst, n);
+  return e;
+}
 }  // namespace dgswe
 
 struct dg_swe_ctx {
@@ -70,7 +98,7 @@ struct dg_swe_ctx {
   cudaStream_t priv = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaGraphExec_t g1 = nullptr, gN = nullptr;
-  void* h_sc = nullptr;  // pinned host copy of the scalar block (read_scalars)
+  dgswe::StatusBlock status;  // of read_scalars; allocated by dg_swe_set_workspace
   dgswe::DriverPtr drv;
   std::string err;
 

@@ -351,11 +351,7 @@ dg_status capture(dg_swe_ctx* c, int nsteps, cudaGraphExec_t* out) {
 }
 
 dg_status read_scalars(dg_swe_ctx* c, DevScalars* h) {
-  // pinned, so that the copy is one DMA in the stream (a pageable one is staged)
-  if (!c->h_sc) CK(cudaHostAlloc(&c->h_sc, sizeof(DevScalars), cudaHostAllocDefault));
-  CK(cudaMemcpyAsync(c->h_sc, c->at<DevScalars>(c->off.sc), sizeof(DevScalars), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
-  *h = *static_cast<DevScalars*>(c->h_sc);
+  CK(read_status(c->status, h, c->at<DevScalars>(c->off.sc), sizeof(DevScalars), c->stream));
   return DG_OK;
 }
 
@@ -547,6 +543,7 @@ dg_status dg_swe_set_workspace(dg_swe_ctx* c, void* ptr, size_t bytes) {
   launch_after(reset_scalars_kernel, 1, 1, 0, s, 1, c->at<DevScalars>(c->off.sc));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));
+  c->status.allocate(sizeof(DevScalars));
   return DG_OK;
 }
 
@@ -871,7 +868,6 @@ void dg_swe_destroy(dg_swe_ctx* c) {
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->priv) cudaStreamDestroy(c->priv);
-  if (c->h_sc) cudaFreeHost(c->h_sc);
   delete c;
 }
 
