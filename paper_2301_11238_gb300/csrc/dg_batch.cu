@@ -15,6 +15,7 @@
 #include "dg_kernels.cuh"
 #include "dg_tc.cuh"
 #include "dg_persist.cuh"
+#include "dg_pointer.h"
 
 using namespace dgswe;
 
@@ -946,18 +947,19 @@ dg_status dg_batch_set_state(dg_batch* b, int i, const double* V, int on_device)
   const int64_t K = b->K_of[i], Np = b->Np_of[i], eb = g.ebase[mi];
   const int nV = g.dim + 1;
   cudaStream_t s = b->stream;
-  // one launch for a device state; a host state field by field
+  // one launch for a state in this device's memory; any other field by field
   const size_t n = (size_t)K * Np, ng = (size_t)g.K * Np;
   char* dst = b->ws + g.off.V[0] + (size_t)eb * Np * b->rsize;
-  if (on_device) {
+  const bool launch = on_device && (b->rsize == 4 || kernel_addressable(V));
+  if (launch) {
     if (b->rsize == 8) fields<double, double>(nV, n, V, n, dst, ng, s);
     else fields<double, float>(nV, n, V, n, dst, ng, s);
   }
-  for (int f = 0; f < nV && !on_device; ++f) {
+  for (int f = 0; f < nV && !launch; ++f) {
     char* df = dst + f * ng * b->rsize;
     const double* src = V + f * n;
     if (b->rsize == 8) {
-      BK(cudaMemcpyAsync(df, src, n * 8, cudaMemcpyHostToDevice, s));
+      BK(cudaMemcpyAsync(df, src, n * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
     } else {
       std::vector<float> h(src, src + n);
       BK(cudaMemcpyAsync(df, h.data(), n * 4, cudaMemcpyHostToDevice, s));
@@ -981,15 +983,16 @@ dg_status dg_batch_get_state(dg_batch* b, int i, double* V, int on_device) {
   cudaStream_t s = b->stream;
   const size_t n = (size_t)K * Np, ng = (size_t)g.K * Np;
   const char* src = b->ws + g.off.V[0] + (size_t)eb * Np * b->rsize;
-  if (on_device) {
+  const bool launch = on_device && (b->rsize == 4 || kernel_addressable(V));
+  if (launch) {
     if (b->rsize == 8) fields<double, double>(nV, n, src, ng, V, n, s);
     else fields<float, double>(nV, n, src, ng, V, n, s);
   }
-  for (int f = 0; f < nV && !on_device; ++f) {
+  for (int f = 0; f < nV && !launch; ++f) {
     const char* sf = src + f * ng * b->rsize;
     double* dst = V + f * n;
     if (b->rsize == 8) {
-      BK(cudaMemcpyAsync(dst, sf, n * 8, cudaMemcpyDeviceToHost, s));
+      BK(cudaMemcpyAsync(dst, sf, n * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     } else {
       std::vector<float> h(n);
       BK(cudaMemcpyAsync(h.data(), sf, n * 4, cudaMemcpyDeviceToHost, s));
