@@ -79,13 +79,22 @@ __device__ __forceinline__ void store_pairs(float* p, float2 (&v)[(NP + 1) / 2])
     for (int a = 0; a < NP; ++a) p[a] = comp(v, a);
   }
 }
-// sum_a row_a x_a
-template <int NH>
-__device__ __forceinline__ float dot_pairs(const float2* row, const float2 (&x)[NH]) {
-  float2 s = mul2(row[0], x[0]);
+// sum_a row_a x_a.  Up to three nodes one after the other: as many instructions as in
+// pairs, and one rounding less (rms error of dh/dt, 1D p = 1: 0.066 against 0.058
+// units of 2^-24 of its terms).
+template <int NP>
+__device__ __forceinline__ float dot_pairs(const float2* row, const float2 (&x)[(NP + 1) / 2]) {
+  [[maybe_unused]] constexpr int NH = (NP + 1) / 2;
+  if constexpr (NP <= 3) {
+    float s = fmaf(row[0].y, x[0].y, row[0].x * x[0].x);
+    if constexpr (NP == 3) s = fmaf(row[1].x, x[1].x, s);
+    return s;
+  } else {
+    float2 s = mul2(row[0], x[0]);
 #pragma unroll
-  for (int i = 1; i < NH; ++i) s = fma2(row[i], x[i], s);
-  return s.x + s.y;
+    for (int i = 1; i < NH; ++i) s = fma2(row[i], x[i], s);
+    return s.x + s.y;
+  }
 }
 
 // The element's nodal pairs: V, and the gradient components the stress needs
@@ -155,13 +164,13 @@ __device__ __forceinline__ void volume_element_f32(int e, int K, int F,
     const float2* lq = ops.Vq + q * NH;
     float Vq[NV], d[ND];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) Vq[v] = dot_pairs<NH>(lq, V2[v]);
+    for (int v = 0; v < NV; ++v) Vq[v] = dot_pairs<NP>(lq, V2[v]);
 #pragma unroll
-    for (int c = 0; c < ND; ++c) d[c] = dot_pairs<NH>(lq, E2[c]);
+    for (int c = 0; c < ND; ++c) d[c] = dot_pairs<NP>(lq, E2[c]);
     float Hr = 0.f, Hs = 0.f;
     if (has_bed) {
-      Hr = dot_pairs<NH>(ops.Drq + q * NH, H2);
-      if constexpr (DIM == 2) Hs = dot_pairs<NH>(ops.Dsq + q * NH, H2);
+      Hr = dot_pairs<NP>(ops.Drq + q * NH, H2);
+      if constexpr (DIM == 2) Hs = dot_pairs<NP>(ops.Dsq + q * NH, H2);
     }
     const float h = Vq[0], hr = h * ph.rho_inv, p = 0.5f * ph.gc * h * h;
     float fr[NV], fs[NV], Sv[DIM];
@@ -201,10 +210,12 @@ __device__ __forceinline__ void volume_element_f32(int e, int K, int F,
     }
   }
   const float J = geo[4 * K + e];
+  if constexpr (DIM == 2) {
 #pragma unroll
-  for (int v = 0; v < NV; ++v)
+    for (int v = 0; v < NV; ++v)
 #pragma unroll
-    for (int i = 0; i < NH; ++i) r[v][i] = mul2(r[v][i], both(J));
+      for (int i = 0; i < NH; ++i) r[v][i] = mul2(r[v][i], both(J));
+  }
 
   // ---- face terms <N^-, F_bar.n - Q_bar.n> (weights and sJ folded into wflux)
   const size_t FQ = (size_t)F * NFQ;
@@ -227,8 +238,19 @@ __device__ __forceinline__ void volume_element_f32(int e, int K, int F,
 #pragma unroll
       for (int v = 0; v < NV; ++v)
 #pragma unroll
-        for (int m = 0; m < NFQ; ++m) comp(r[v], a) += ops.o.LfT[k * NFQ + m] * fv[v][m];
+        for (int m = 0; m < NFQ; ++m) {
+          // 1D: one face value a node, added to J r in one rounding
+          float& x = comp(r[v], a);
+          if constexpr (DIM == 1) x = fmaf(x, J, ops.o.LfT[0] * fv[v][m]);
+          else x += ops.o.LfT[k * NFQ + m] * fv[v][m];
+        }
     }
+  }
+  if constexpr (DIM == 1) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+      for (int a = 1; a < NP - 1; ++a) comp(r[v], a) *= J;
   }
 
   // mode 2: the spatial residual r_V itself (physical scaling)
@@ -262,7 +284,7 @@ __device__ __forceinline__ void volume_element_f32(int e, int K, int F,
   } else {
     if constexpr (NP % 2 == 1) dV[0][NH - 1].y = 0.f;
 #pragma unroll
-    for (int a = 0; a < NP; ++a) comp(dV[0], a) = -Jinv * dot_pairs<NH>(ops.Minv + a * NH, r[0]);
+    for (int a = 0; a < NP; ++a) comp(dV[0], a) = -Jinv * dot_pairs<NP>(ops.Minv + a * NH, r[0]);
     float2 M[T::NMH], rhs[DIM][NH];
 #pragma unroll
     for (int i = 0; i < T::NMH; ++i) M[i] = both(0.f);
@@ -273,12 +295,12 @@ __device__ __forceinline__ void volume_element_f32(int e, int K, int F,
 #pragma unroll 1
     for (int q = 0; q < NQ; ++q) {
       const float2* lq = ops.Vq + q * NH;
-      const float hf = fmaxf(dot_pairs<NH>(lq, V2[0]), ph.h_floor), hd = -dot_pairs<NH>(lq, dV[0]);
+      const float hf = fmaxf(dot_pairs<NP>(lq, V2[0]), ph.h_floor), hd = -dot_pairs<NP>(lq, dV[0]);
 #pragma unroll
       for (int i = 0; i < T::NMH; ++i) M[i] = fma2(ops.MP[q * T::NMH + i], both(hf), M[i]);
 #pragma unroll
       for (int j = 0; j < DIM; ++j) {
-        const float2 z = both(hd * dot_pairs<NH>(lq, V2[1 + j]));
+        const float2 z = both(hd * dot_pairs<NP>(lq, V2[1 + j]));
 #pragma unroll
         for (int i = 0; i < NH; ++i) rhs[j][i] = fma2(ops.Wm[q * NH + i], z, rhs[j][i]);
       }
