@@ -489,11 +489,16 @@ dg_status capture(dg_batch* b, int nsteps, cudaGraphExec_t* out) {
   // 10.0 -> 7.5 ms).
   const size_t ng = b->groups.size();
   while (b->side.size() + 1 < ng) {
+    // a stream with its event, or neither: a capture after a failure finds them even
     cudaStream_t st = nullptr;
     cudaEvent_t ev = nullptr;
     BK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+    const cudaError_t ee = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (ee != cudaSuccess) {
+      cudaStreamDestroy(st);
+      return bcuda(b, ee, "cudaEventCreate");
+    }
     b->side.push_back(st);
-    BK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     b->side_ev.push_back(ev);
   }
   BK(cudaStreamBeginCapture(b->priv, cudaStreamCaptureModeThreadLocal));
