@@ -547,11 +547,12 @@ __device__ void linear_residual_f64(const ImplArgs& a, const Team& t) {
 template <int NB>
 __device__ void solve_f32(const ImplArgs& a, const double* b, float* x, const Team& t) {
   const BTri<float> A{a.Df, a.Lf, a.Uf, a.bf, a.K};
-  for (int i = t.tid; i < a.K * NB * NB; i += t.threads) {
+  const size_t nb = (size_t)a.K * NB, n = nb * NB;  // the blocks' entries can pass 2^31
+  for (size_t i = t.tid; i < n; i += t.threads) {
     a.Df[i] = (float)a.D[i];
     a.Lf[i] = (float)a.L[i];
     a.Uf[i] = (float)a.U[i];
-    if (i < a.K * NB) a.bf[i] = (float)b[i];
+    if (i < nb) a.bf[i] = (float)b[i];
   }
   cluster_sync();
   bcr_solve<float, NB>(A, x, t);
