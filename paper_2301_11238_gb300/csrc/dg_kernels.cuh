@@ -1058,7 +1058,7 @@ __device__ __forceinline__ T limit_depth(T* h, const VolOps<DIM, P, R>& ops) {
 // zero in a dry element; this one divides the new momentum by the new depth.
 // Computed in T: FP64 in FP64 contexts and for near-dry elements of FP32
 // contexts, FP32 for their wet elements (wetdry_stage_kernel chooses, as
-// mass_solve_dispatch does for the primitive stages); loops unrolled up to
+// the FP32 volume pass does for the primitive stages); loops unrolled up to
 // p = 2 (2D p = 3 keeps them rolled: unrolled, its arrays spilled 13 KB per
 // thread).  Runs in its own
 // kernel (wetdry_stage_kernel) after the volume pass has written r_V, so the
@@ -1167,97 +1167,6 @@ __device__ __forceinline__ void conservative_stage(const R (&Vn)[Sh<DIM, P>::NV]
   for (int i = 0; i < NV * NP; ++i) out[(i / NP) * KN + eo + i % NP] = (R)y[i];
 }
 
-// Primitive-variable mass solve of one element (Appendix A, dU/dV):
-// dV = -M(V)^{-1} r, i.e. M dh/dt = -r_h and M_h du/dt = -r_u - M_u dh/dt,
-// with M_h = <psi, max(h, h_floor) psi> and M_u = <psi, u psi> at the volume
-// quadrature points; r in physical scaling, Jinv = 1 / J.
-template <int DIM, int P, typename R>
-__device__ __forceinline__ void mass_solve_element(const R (&Vn)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
-                                                   const R (&r)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
-                                                   const VolOps<DIM, P, R>& ops, R h_floor, R Jinv,
-                                                   R (&dV)[Sh<DIM, P>::NV][Sh<DIM, P>::NP]) {
-  using S = Sh<DIM, P>;
-  constexpr int NP = S::NP, NQ = S::NQ;
-#pragma unroll
-  for (int a = 0; a < NP; ++a) {
-    R acc = R(0);
-#pragma unroll
-    for (int b = 0; b < NP; ++b) acc += ops.Minv[a * NP + b] * r[0][b];
-    dV[0][a] = -acc * Jinv;
-  }
-  R Mh[NP][NP];
-  R rhs[DIM][NP];
-#pragma unroll
-  for (int a = 0; a < NP; ++a) {
-#pragma unroll
-    for (int b = 0; b < NP; ++b) Mh[a][b] = R(0);
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) rhs[j][a] = -r[1 + j][a] * Jinv;
-  }
-#pragma unroll 1
-  for (int q = 0; q < NQ; ++q) {
-    R hq = R(0), hdq = R(0), uq[DIM];
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) uq[j] = R(0);
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      const R l = ops.Vq[q * NP + a];
-      hq += l * Vn[0][a];
-      hdq += l * dV[0][a];
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) uq[j] += l * Vn[1 + j][a];
-    }
-    const R wd = ops.wq[q] * hdq;
-    const R wh = ops.wq[q] * fmax(hq, h_floor);
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      const R la = ops.Vq[q * NP + a];
-      const R t = wh * la;
-#pragma unroll
-      for (int b = 0; b <= a; ++b) Mh[a][b] += t * ops.Vq[q * NP + b];
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) rhs[j][a] -= wd * uq[j] * la;
-    }
-  }
-  // Cholesky of the reference-scaled M_h (lower triangle); the diagonal is
-  // kept as reciprocals so the factorization and both triangular solves
-  // multiply instead of divide (NP divisions per element instead of
-  // NP (NP + 3) / 2 + 2 DIM NP).
-  R dinv[NP];
-#pragma unroll
-  for (int a = 0; a < NP; ++a) {
-#pragma unroll
-    for (int b = 0; b < a; ++b) {
-      R s = Mh[a][b];
-#pragma unroll
-      for (int c = 0; c < b; ++c) s -= Mh[a][c] * Mh[b][c];
-      Mh[a][b] = s * dinv[b];
-    }
-    R d = Mh[a][a];
-#pragma unroll
-    for (int c = 0; c < a; ++c) d -= Mh[a][c] * Mh[a][c];
-    dinv[a] = dg_rsqrt<R>(d);
-  }
-#pragma unroll
-  for (int j = 0; j < DIM; ++j) {
-    R y[NP];
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-      R s = rhs[j][a];
-#pragma unroll
-      for (int c = 0; c < a; ++c) s -= Mh[a][c] * y[c];
-      y[a] = s * dinv[a];
-    }
-#pragma unroll
-    for (int a = NP - 1; a >= 0; --a) {
-      R s = y[a];
-#pragma unroll
-      for (int c = a + 1; c < NP; ++c) s -= Mh[c][a] * dV[1 + j][c];
-      dV[1 + j][a] = s * dinv[a];
-    }
-  }
-}
-
 // Near-dry treatment of FP32 contexts: an element whose smallest nodal depth
 // is below h_dry (kDryFactor x h_floor) assembles and solves its h-weighted
 // mass matrix in FP64 (the depths at the quadrature points, M_h = <psi,
@@ -1267,8 +1176,8 @@ __device__ __forceinline__ void mass_solve_element(const R (&Vn)[Sh<DIM, P>::NV]
 // larger, and FP32 would lose their relative accuracy.  The FP64 solve runs
 // in loops over per-thread local arrays: it is rare (fronts and films only)
 // and must not add registers to the FP32 kernels' common path.  FP64
-// contexts and wet elements take the working-precision solve
-// (mass_solve_element), whose formulas this restates.
+// contexts and wet elements solve in their volume passes (dg_volume_fx.cuh,
+// dg_volume_f32.cuh), whose formulas this restates.
 constexpr double kDryFactor = 1000.0;
 
 template <int DIM, int P>
@@ -1357,25 +1266,6 @@ __device__ __forceinline__ void mass_solve_dry(const float (&Vn)[Sh<DIM, P>::NV]
   for (int v = 0; v < NV; ++v)
 #pragma unroll
     for (int a = 0; a < NP; ++a) dVout[v][a] = (float)dV[v * NP + a];
-}
-
-template <int DIM, int P, typename R>
-__device__ __forceinline__ void mass_solve_dispatch(const R (&Vn)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
-                                                    const R (&r)[Sh<DIM, P>::NV][Sh<DIM, P>::NP],
-                                                    const VolOps<DIM, P, R>& ops, const Phys<R>& ph, R Jinv,
-                                                    R (&dV)[Sh<DIM, P>::NV][Sh<DIM, P>::NP]) {
-  using S = Sh<DIM, P>;
-  constexpr int NP = S::NP;
-  if constexpr (sizeof(R) == 4) {
-    R hmin = Vn[0][0];
-#pragma unroll
-    for (int a = 1; a < NP; ++a) hmin = fmin(hmin, Vn[0][a]);
-    if (hmin < ph.h_dry) {
-      mass_solve_dry<DIM, P>(Vn, r, ops, ph.h_floor, Jinv, dV);
-      return;
-    }
-  }
-  mass_solve_element<DIM, P, R>(Vn, r, ops, ph.h_floor, Jinv, dV);
 }
 
 }  // namespace dgswe

@@ -22,7 +22,7 @@
 // item, so that no block claims further work.
 //
 // The per-element and per-face-point arithmetic is the graph form's own
-// (estep_element, face_item, volume_element); compiled into this kernel, some
+// (estep_element, face_item, volume_any); compiled into this kernel, some
 // multiply-adds may be fused differently, so results agree to rounding.  Data that another block writes during the launch (stage states, E,
 // face fluxes, tile bounds, dt) is read through L2 (ld.global.cg): the
 // producer's block barrier, fence and counter increment, and the consumer's

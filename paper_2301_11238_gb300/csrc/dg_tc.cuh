@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           // near-dry element (smallest nodal depth below h_dry): the whole
           // mass solve again in FP64 from the nodal values, as in the
-          // CUDA-core kernel (mass_solve_dispatch)
+          // CUDA-core pass (volume_element_f32)
           float hmin = Vin[eo];
 #pragma unroll
           for (int a = 1; a < NP; ++a) hmin = fminf(hmin, Vin[eo + a]);

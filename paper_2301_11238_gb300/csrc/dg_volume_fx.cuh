@@ -125,7 +125,7 @@ __device__ __forceinline__ int largest(const int (&v)[N]) {
   return m;
 }
 
-// Arguments and modes as volume_element (dg_kernels.cuh).  T = 1: one thread per
+// Arguments and modes as volume_any (dg_kernels.cuh).  T = 1: one thread per
 // element.  T = 2, 4: T neighbouring lanes share one (tl: the thread's place
 // among them; all lanes of a warp come here, live = false for those past the
 // last element): each takes every T-th volume point and face, the integer sums
