@@ -1776,9 +1776,10 @@ __device__ __forceinline__ R huge_dt() { return sizeof(R) == 8 ? R(1e300) : R(3e
 // 1e-5 of their largest, so that the value is that of the plain maximum.  In flow
 // these are one or two nodes, in still water of even depth all of them; everything
 // but the products and roots of a node's speed is kept off the FP64 pipe for their
-// sake.  524,288 triangles, p = 2, us in flow / in still water: FP64 43 / 99 (with
-// the nodes compared in FP64 61 / 186, the plain maximum 179), FP32 12.6 / 12.6 (in
-// two steps like FP64 14.5 / 20.7, with FP64 minima 24).
+// sake.  524,288 triangles, us in flow / in still water: FP64 p = 2 39 / 109 (with the
+// nodes compared in FP64 58 / 213, the plain maximum 178), p = 3 55 / 172 (84 / 466,
+// 281); FP32 p = 2 8.3 / 10.3 (in two steps like FP64 9.9 / 20.5, with FP64 minima
+// 14.5 / 16.4), p = 3 12.5 / 16.5 (12.5 / 43, 19.5 / 20.7).
 template <int DIM, int P, typename R, bool COH = false>
 __device__ __forceinline__ R element_dt(size_t e, int K, const R* __restrict__ V, const R* __restrict__ geo, R gc,
                                         R h_floor, R cfl, R nu) {
@@ -1786,33 +1787,34 @@ __device__ __forceinline__ R element_dt(size_t e, int K, const R* __restrict__ V
   const size_t KN = (size_t)K * NP;
   bool bad = false;
   R lam = R(0);
+  R h[NP], u[DIM][NP];
+#pragma unroll
+  for (int a = 0; a < NP; ++a) {
+    h[a] = DG_LDC(COH, V, e * NP + a);
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) u[j][a] = DG_LDC(COH, V, (1 + j) * KN + e * NP + a);
+  }
   if constexpr (sizeof(R) == 4) {
+    // (the loads stand before the roots, whose slow paths are branches)
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
-      const R h = DG_LDC(COH, V, e * NP + a);
       R sp2 = R(0);
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) {
-        const R u = DG_LDC(COH, V, (1 + j) * KN + e * NP + a);
-        sp2 += u * u;
-      }
-      const R v = sqrtf(sp2) + sqrtf(gc * fmaxf(h, h_floor));
-      bad = bad || not_finite(h) || not_finite(v);
+      for (int j = 0; j < DIM; ++j) sp2 += u[j][a] * u[j][a];
+      const R v = sqrtf(sp2) + sqrtf(gc * fmaxf(h[a], h_floor));
+      bad = bad || not_finite(h[a]) || not_finite(v);
       lam = fmaxf(lam, v);
     }
     if (bad) return R(-1);
   } else {
-    R h[NP], u[DIM][NP];
     float l[NP], top = 0.f;
     const float gcf = near_f32(gc), hf = near_f32(h_floor);
 #pragma unroll
     for (int a = 0; a < NP; ++a) {
-      h[a] = DG_LDC(COH, V, e * NP + a);
       bad = bad || not_finite(h[a]);
       float s2 = 0.f;
 #pragma unroll
       for (int j = 0; j < DIM; ++j) {
-        u[j][a] = DG_LDC(COH, V, (1 + j) * KN + e * NP + a);
         bad = bad || not_finite(u[j][a]);
         const float x = near_f32(u[j][a]);
         s2 += x * x;
