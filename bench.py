@@ -284,8 +284,10 @@ def traffic_record(kernel, workload):
             rec = json.load(f)
     except Exception:
         return None
-    src = os.path.join(ROOT, "paper_2301_11238_gb300", "csrc", "dg_kernels.cuh")
-    h = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for f in ("dg_kernels.cuh", "dg_fixed.cuh", "dg_math64.cuh", "dg_volume_f32.cuh", "dg_volume_fx.cuh"):
+        h.update(open(os.path.join(ROOT, "paper_2301_11238_gb300", "csrc", f), "rb").read())
+    h = h.hexdigest()[:16]
     r = rec.get(f"{kernel}|{workload}")
     if not r or r.get("source_sha") != h:
         return None

@@ -388,7 +388,7 @@ __device__ __forceinline__ void q_normal(R h, const R* E, const R* n, const Phys
 // ratio, and with one exponent for both the small one would lose that many bits.
 // 4 NP conversions and 9 products are the FP64 pipe's share (2D), of 417
 // FP64 instructions in floating point at p = 2.  524,288 triangles, p = 2:
-// 411 -> 180 us; p = 1: 167 -> 67 us; 8,192 triangles, p = 2: 20.6 -> 12.5 us.
+// 411 -> 121 us; p = 1: 167 -> 64 us; 8,192 triangles, p = 2: 20.6 -> 10.5 us.
 // The components j0 .. j1 - 1 (small meshes: one a thread).
 template <int DIM, int P, bool COH, bool PRE>
 __device__ __forceinline__ void estep_element_fx(int j0, int j1,
@@ -1399,12 +1399,13 @@ __global__ void __launch_bounds__(256) __maxnreg__((volume_max_regs<DIM, P, R>()
 // the longer chain of one.  Four lanes against a thread per
 // element, triangles, us: p = 2: 128 elements 42 / 57, 4,608 41 / 52, 9,522
 // 48 / 53; p = 1: 9,522 16 / 18; p = 3: 512 95 / 197, 9,522 139 / 220; intervals,
-// p = 1: 200 elements 9.4 / 10.9.
+// p = 1: 200 elements 9.4 / 10.9 (both sides before the rows' own units, which add
+// up to 4 %).
 constexpr int kSplitBlock = 64;
 constexpr int64_t kOneWarpEach = 152 * 4 * 32;  // threads that fill every sub-partition once
 template <int DIM, int P>
 constexpr int split_lanes() {
-  return Sh<DIM, P>::NQ < 3 ? 2 : 4;  // no more lanes than volume points
+  return Sh<DIM, P>::NQ < 3 ? 2 : 4;  // two for the two points of 1D p = 1
 }
 inline bool volume_split(int64_t K) { return K * 2 <= kOneWarpEach; }
 

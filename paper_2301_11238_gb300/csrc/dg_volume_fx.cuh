@@ -7,8 +7,8 @@
 // floating point took 2065 and kept the FP64 pipe 91 % busy; the contractions
 // (interpolation, metric transform, test functions, face lift, mass matrices)
 // are 1140 integer multiply-adds of three IMAD.WIDE each.  524,288 triangles,
-// p = 2: 1969 -> 834 us, p = 1 691 -> 402 us (with the wet/dry stage kernel);
-// 73,728 triangles, p = 2: 314 -> 159 us; 8,192: 84 -> 52 us.  The FP64 pipe is
+// p = 2: 1969 -> 844 us, p = 1 691 -> 403 us (with the wet/dry stage kernel);
+// 73,728 triangles, p = 2: 314 -> 160 us; 8,192: 84 -> 47 us.  The FP64 pipe is
 // 50 % busy then: few warps (168 to 240 registers a thread) wait for one
 // another's chains.
 //
@@ -17,12 +17,13 @@
 //           with the largest exponent of each component
 //   pass 2  per volume point: metric transform J G (Q - F), test functions;
 //           the face fluxes are lifted into the same accumulators
+//   solve   M dh/dt = -r_h straight from the integer residual, then M_h and
+//           M_u dh/dt per volume point, Cholesky in floating point
+//
 // Every component of the residual has a unit of its own, set by the largest of its
 // terms, and the metric terms of each direction have theirs: on stretched elements,
 // or with a momentum component far below the other, a unit for all would take bits
 // from the small ones.
-//   solve   M dh/dt = -r_h straight from the integer residual, then M_h and
-//           M_u dh/dt per volume point, Cholesky in floating point
 #pragma once
 
 namespace dgswe {
